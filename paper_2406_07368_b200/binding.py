@@ -1,13 +1,18 @@
-"""ctypes binding of libla_b200.so: argument marshalling only.
+"""Python binding of libla_b200.so: argument marshalling only.
 
 The methods carry the names of the C entry points declared in include/la.h and take torch
 tensors where the C side takes device pointers.  Every step of the layer runs inside the
 library's CUDA kernels; torch supplies device memory and streams.  There is no fallback: if the
 shared library is missing or a call fails, an exception is raised.
+
+The calls of a model's inner loop (prefill, decode, verify, accept, commit) go through _host.so, which checks the
+tensors and allocates missing outputs in C++: a small call is bound by this work, not by its kernel (csrc/host.cpp).
+Everything else is ctypes.
 """
 from __future__ import annotations
 
 import ctypes as C
+import importlib
 import os
 from dataclasses import dataclass
 
@@ -15,6 +20,7 @@ import torch
 
 _LIB_PATH = os.path.join(os.path.dirname(os.path.abspath(__file__)), "libla_b200.so")
 _lib = None
+_host = None
 
 LA_OK, LA_ERR_INVALID_ARG, LA_ERR_UNSUPPORTED, LA_ERR_CUDA, LA_ERR_BAD_TREE, LA_ERR_TIMEOUT, LA_ERR_TOO_LARGE = range(7)
 LA_PHI = {"elu1": 0, "relu": 1}
@@ -88,6 +94,20 @@ def lib() -> C.CDLL:
     return _lib
 
 
+def _host_module():
+    """The native side of the binding; raises if it has not been built."""
+    global _host
+    if _host is None:
+        lib()                                    # the library it links against, or the error that says it is missing
+        try:
+            _host = importlib.import_module("._host", __package__)
+        except ImportError as e:
+            raise RuntimeError("_host.so is missing or does not load: build it with `python -m "
+                               f"{__package__}.build` (there is no CPU or eager fallback): {e}") from e
+        _host.set_error(LaError)
+    return _host
+
+
 def status_str(code: int) -> str:
     return lib().la_status_str(int(code)).decode()
 
@@ -144,9 +164,12 @@ class Context:
         with torch.cuda.device(self.device):
             torch.cuda.current_stream()          # make sure the device context exists
             _check("la_create", lib().la_create(C.byref(cfg), C.byref(self._h)))
+        self._plan = _host_module().Plan(self._h.value, H, d, conv_taps, max_depth, io == "bf16")
 
     def close(self) -> None:
         if self._h:
+            if hasattr(self, "_plan"):
+                self._plan.close()
             lib().la_destroy(self._h)
             self._h = C.c_void_p()
 
@@ -164,37 +187,13 @@ class Context:
                      torch.zeros(B, self.H, self.W - 1, self.d, dtype=self.dtype, device=dev),
                      torch.zeros(B, dtype=torch.int64, device=dev))
 
-    def _check_state(self, st: State, B: int) -> None:
-        _ptr(st.S, torch.float32, (B, self.H, self.d, self.d), "state.S")
-        _ptr(st.z, torch.float32, (B, self.H, self.d), "state.z")
-        _ptr(st.win, self.dtype, (B, self.H, self.W - 1, self.d), "state.win")
-        _ptr(st.pos, torch.int64, (B,), "state.pos")
-
     # -- entry points ----------------------------------------------------------------------
     def la_prefill(self, q, k, v, conv_w, state: State, init_state: bool = False, out=None, stream=None):
-        B, H, T, d = q.shape
-        shp = (B, self.H, T, self.d)
-        out = torch.empty(shp, dtype=self.dtype, device=q.device) if out is None else out
-        self._check_state(state, B)
-        cs = state.c()
-        _check("la_prefill", lib().la_prefill(
-            self._h, B, T, _ptr(q, self.dtype, shp, "q"), _ptr(k, self.dtype, shp, "k"), _ptr(v, self.dtype, shp, "v"),
-            _ptr(conv_w, torch.float32, (self.H, self.d, self.W), "conv_w"), int(bool(init_state)), C.byref(cs),
-            _ptr(out, self.dtype, shp, "o"), _stream(stream)))
-        return out
+        return self._plan.prefill(q, k, v, conv_w, state, init_state, out, stream)
 
     def la_prefill_grouped(self, q, k, v, conv_w, state: State, group: int, alpha: float, softmax_scale: float,
                            init_state: bool = False, out=None, stream=None):
-        B, H, T, d = q.shape
-        shp = (B, self.H, T, self.d)
-        out = torch.empty(shp, dtype=self.dtype, device=q.device) if out is None else out
-        self._check_state(state, B)
-        cs = state.c()
-        _check("la_prefill_grouped", lib().la_prefill_grouped(
-            self._h, B, T, _ptr(q, self.dtype, shp, "q"), _ptr(k, self.dtype, shp, "k"), _ptr(v, self.dtype, shp, "v"),
-            _ptr(conv_w, torch.float32, (self.H, self.d, self.W), "conv_w"), int(group), float(alpha),
-            float(softmax_scale), int(bool(init_state)), C.byref(cs), _ptr(out, self.dtype, shp, "o"), _stream(stream)))
-        return out
+        return self._plan.prefill_grouped(q, k, v, conv_w, state, group, alpha, softmax_scale, init_state, out, stream)
 
     def la_prefill_grouped_max_group(self) -> int:
         return int(lib().la_prefill_grouped_max_group(self._h))
@@ -224,71 +223,20 @@ class Context:
         return S, z
 
     def la_decode_step(self, q, k, v, conv_w, state: State, out=None, stream=None):
-        B = q.shape[0]
-        shp = (B, self.H, self.d)
-        out = torch.empty(shp, dtype=self.dtype, device=q.device) if out is None else out
-        self._check_state(state, B)
-        cs = state.c()
-        _check("la_decode_step", lib().la_decode_step(
-            self._h, B, _ptr(q, self.dtype, shp, "q"), _ptr(k, self.dtype, shp, "k"), _ptr(v, self.dtype, shp, "v"),
-            _ptr(conv_w, torch.float32, (self.H, self.d, self.W), "conv_w"), C.byref(cs),
-            _ptr(out, self.dtype, shp, "o"), _stream(stream)))
-        return out
+        return self._plan.decode_step(q, k, v, conv_w, state, out, stream)
 
     def la_verify_tree(self, q, k, v, parent, conv_w, state: State, out=None, stream=None):
-        B, H, N, d = q.shape
-        shp = (B, self.H, N, self.d)
-        out = torch.empty(shp, dtype=self.dtype, device=q.device) if out is None else out
-        self._check_state(state, B)
-        cs = state.c()
-        _check("la_verify_tree", lib().la_verify_tree(
-            self._h, B, N, _ptr(q, self.dtype, shp, "q"), _ptr(k, self.dtype, shp, "k"), _ptr(v, self.dtype, shp, "v"),
-            _ptr(parent, torch.int32, (B, N), "parent"),
-            _ptr(conv_w, torch.float32, (self.H, self.d, self.W), "conv_w"), C.byref(cs),
-            _ptr(out, self.dtype, shp, "o"), _stream(stream)))
-        return out
+        return self._plan.verify_tree(q, k, v, parent, conv_w, state, out, stream)
 
     def la_commit(self, k, v, parent, accept_node, state: State, path_out=None, commit_len=None, stream=None):
-        B, H, N, d = k.shape
-        shp = (B, self.H, N, self.d)
-        if path_out is None:
-            path_out = torch.full((B, self.max_depth), -1, dtype=torch.int32, device=k.device)
-        if commit_len is None:
-            commit_len = torch.zeros(B, dtype=torch.int32, device=k.device)
-        self._check_state(state, B)
-        cs = state.c()
-        _check("la_commit", lib().la_commit(
-            self._h, B, N, _ptr(k, self.dtype, shp, "k"), _ptr(v, self.dtype, shp, "v"),
-            _ptr(parent, torch.int32, (B, N), "parent"), _ptr(accept_node, torch.int32, (B,), "accept_node"),
-            C.byref(cs), _ptr(path_out, torch.int32, (B, self.max_depth), "path_out"),
-            _ptr(commit_len, torch.int32, (B,), "commit_len"), _stream(stream)))
-        return path_out, commit_len
+        return self._plan.commit(k, v, parent, accept_node, state, path_out, commit_len, stream)
 
     def la_accept_greedy(self, parent, draft_token, pred_root, pred, accept_node=None, accept_len=None,
                          next_token=None, stream=None):
-        B, N = parent.shape
-        dev = parent.device
-        accept_node = torch.empty(B, dtype=torch.int32, device=dev) if accept_node is None else accept_node
-        accept_len = torch.empty(B, dtype=torch.int32, device=dev) if accept_len is None else accept_len
-        next_token = torch.empty(B, dtype=torch.int32, device=dev) if next_token is None else next_token
-        _check("la_accept_greedy", lib().la_accept_greedy(
-            self._h, B, N, _ptr(parent, torch.int32, (B, N), "parent"),
-            _ptr(draft_token, torch.int32, (B, N), "draft_token"), _ptr(pred_root, torch.int32, (B,), "pred_root"),
-            _ptr(pred, torch.int32, (B, N), "pred"), _ptr(accept_node, torch.int32, (B,), "accept_node"),
-            _ptr(accept_len, torch.int32, (B,), "accept_len"), _ptr(next_token, torch.int32, (B,), "next_token"),
-            _stream(stream)))
-        return accept_node, accept_len, next_token
+        return self._plan.accept_greedy(parent, draft_token, pred_root, pred, accept_node, accept_len, next_token, stream)
 
     def la_accept_threshold(self, parent, score, thresh, accept_node=None, accept_len=None, stream=None):
-        B, N = parent.shape
-        dev = parent.device
-        accept_node = torch.empty(B, dtype=torch.int32, device=dev) if accept_node is None else accept_node
-        accept_len = torch.empty(B, dtype=torch.int32, device=dev) if accept_len is None else accept_len
-        _check("la_accept_threshold", lib().la_accept_threshold(
-            self._h, B, N, _ptr(parent, torch.int32, (B, N), "parent"), _ptr(score, torch.float32, (B, N), "score"),
-            _ptr(thresh, torch.float32, (B, N), "thresh"), _ptr(accept_node, torch.int32, (B,), "accept_node"),
-            _ptr(accept_len, torch.int32, (B,), "accept_len"), _stream(stream)))
-        return accept_node, accept_len
+        return self._plan.accept_threshold(parent, score, thresh, accept_node, accept_len, stream)
 
     def la_selftest_wait_timeout(self, limit_us: int, stream=None) -> int:
         """Runs the bounded-wait self-test; returns the nanoseconds the wait took (see include/la.h)."""

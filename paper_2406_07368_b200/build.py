@@ -1,4 +1,5 @@
-"""Builds libla_b200.so in-tree with nvcc for sm_100a (cross-compiles without a GPU)."""
+"""Builds libla_b200.so in-tree with nvcc for sm_100a (cross-compiles without a GPU), and beside it _host.so, the native
+side of the Python binding (g++ against torch's headers)."""
 from __future__ import annotations
 
 import os
@@ -11,6 +12,7 @@ ROOT = os.path.dirname(PKG)
 CSRC = os.path.join(PKG, "csrc")
 OBJ = os.path.join(PKG, "_build")
 LIB = os.path.join(PKG, "libla_b200.so")
+HOST = os.path.join(PKG, "_host.so")
 SOURCES = ["la_api.cu", "decode.cu", "prefill_simt.cu", "prefill_tc.cu", "prefill_grouped.cu", "seqpar.cu", "verify.cu", "verify_tc.cu", "commit.cu", "accept.cu", "selftest.cu"]
 FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
          "-Xcompiler", "-fPIC", "-I", os.path.join(ROOT, "include"), "-I", CSRC]
@@ -28,6 +30,24 @@ def _newer(target: str, deps: list[str]) -> bool:
         return False
     t = os.path.getmtime(target)
     return all(os.path.getmtime(d) <= t for d in deps)
+
+
+def _build_host(deps: list[str]) -> None:
+    """_host.so: links against libla_b200.so (found beside it) and the torch libraries of the running interpreter."""
+    src = os.path.join(CSRC, "host.cpp")
+    if _newer(HOST, [src, *deps]):
+        return
+    import sysconfig
+
+    from torch.utils import cpp_extension
+    inc = [f"-I{d}" for d in (*cpp_extension.include_paths("cuda"), sysconfig.get_paths()["include"], os.path.join(ROOT, "include"), CSRC)]
+    libs = [f"-L{d}" for d in cpp_extension.library_paths("cuda")]
+    cmd = [os.environ.get("CXX", "g++"), "-O2", "-std=c++17", "-fPIC", "-shared", src, "-o", HOST, *inc, *libs, f"-L{PKG}",
+           "-lla_b200", "-ltorch_python", "-ltorch_cuda", "-ltorch_cpu", "-ltorch", "-lc10_cuda", "-lc10", "-Wl,-rpath,$ORIGIN"]
+    r = subprocess.run(cmd, capture_output=True, text=True)
+    if r.returncode != 0:
+        sys.stderr.write(r.stdout + r.stderr)
+        raise RuntimeError("g++ failed on host.cpp")
 
 
 def build(verbose: bool = False, force: bool = False) -> str:
@@ -60,6 +80,7 @@ def build(verbose: bool = False, force: bool = False) -> str:
         if r.returncode != 0:
             sys.stderr.write(r.stdout + r.stderr)
             raise RuntimeError("link failed")
+    _build_host([h for h in headers if h.endswith(".h")] + ([LIB] if force else []))
     return LIB
 
 

@@ -5,6 +5,7 @@
 // The loads of the state are issued first, so that they are in flight while the path is rebuilt and the path
 // tokens are gathered.
 #include "la_common.cuh"
+#include "la_internal.h"
 
 namespace la {
 
@@ -25,7 +26,7 @@ __global__ void __launch_bounds__(256)
 commit_kernel(const T* __restrict__ k, const T* __restrict__ v, const int32_t* __restrict__ parent,
               const int32_t* __restrict__ accept, float* __restrict__ S, float* __restrict__ z, T* __restrict__ win,
               int64_t* __restrict__ pos, int32_t* __restrict__ path_out, int32_t* __restrict__ commit_len, int* status,
-              int H, int N, int W, int max_depth) {
+              int H, int N, int W, int max_depth, int fresh) {
   constexpr int TPR = D / 4, RPP = 256 / TPR, ROWS = D / kCommitSplit, PASSES = ROWS / RPP;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   float (*fk)[D] = reinterpret_cast<float (*)[D]>(smem_raw);
@@ -66,6 +67,11 @@ commit_kernel(const T* __restrict__ k, const T* __restrict__ v, const int32_t* _
   __syncthreads();
   if (sm.bad) {
     if (t == 0) report(status, LA_ERR_BAD_TREE);
+    if (h == 0 && part == 0) {             // buffers whose contents nobody has seen yet
+      if (fresh & LA_FRESH_PATH)
+        for (int i = t; i < max_depth; i += 256) path_out[(size_t)b * max_depth + i] = -1;
+      if ((fresh & LA_FRESH_LEN) && t == 0) commit_len[b] = 0;
+    }
     return;
   }
   const int L = sm.len;
@@ -114,7 +120,7 @@ commit_kernel(const T* __restrict__ k, const T* __restrict__ v, const int32_t* _
 
 template <typename T, int D, int PHI>
 static cudaError_t launch_t(la_ctx* ctx, int B, int N, const void* k, const void* v, const int32_t* parent,
-                            const int32_t* accept, const la_state& st, int32_t* path_out, int32_t* commit_len,
+                            const int32_t* accept, const la_state& st, int32_t* path_out, int32_t* commit_len, int fresh,
                             cudaStream_t s) {
   const la_config& c = ctx->cfg;
   auto kern = commit_kernel<T, D, PHI>;
@@ -123,27 +129,27 @@ static cudaError_t launch_t(la_ctx* ctx, int B, int N, const void* k, const void
   if (e != cudaSuccess) return e;
   ctx->launches += 1;
   return launch_pdl(kern, dim3(B * c.H * kCommitSplit), dim3(256), smem, s, (const T*)k, (const T*)v, parent, accept, st.S,
-                    st.z, (T*)st.win, st.pos, path_out, commit_len, ctx->d_status, c.H, N, c.conv_taps, c.max_depth);
+                    st.z, (T*)st.win, st.pos, path_out, commit_len, ctx->d_status, c.H, N, c.conv_taps, c.max_depth, fresh);
 }
 
 template <typename T, int D>
 static cudaError_t launch_phi(la_ctx* ctx, int B, int N, const void* k, const void* v, const int32_t* parent,
-                              const int32_t* accept, const la_state& st, int32_t* path_out, int32_t* commit_len,
+                              const int32_t* accept, const la_state& st, int32_t* path_out, int32_t* commit_len, int fresh,
                               cudaStream_t s) {
   return ctx->cfg.phi == LA_PHI_ELU1
-             ? launch_t<T, D, LA_PHI_ELU1>(ctx, B, N, k, v, parent, accept, st, path_out, commit_len, s)
-             : launch_t<T, D, LA_PHI_RELU>(ctx, B, N, k, v, parent, accept, st, path_out, commit_len, s);
+             ? launch_t<T, D, LA_PHI_ELU1>(ctx, B, N, k, v, parent, accept, st, path_out, commit_len, fresh, s)
+             : launch_t<T, D, LA_PHI_RELU>(ctx, B, N, k, v, parent, accept, st, path_out, commit_len, fresh, s);
 }
 
 cudaError_t launch_commit(la_ctx* ctx, int B, int N, const void* k, const void* v, const int32_t* parent,
-                          const int32_t* accept, const la_state& st, int32_t* path_out, int32_t* commit_len,
+                          const int32_t* accept, const la_state& st, int32_t* path_out, int32_t* commit_len, int fresh,
                           cudaStream_t s) {
   const la_config& c = ctx->cfg;
   if (c.io_dtype == LA_F32)
-    return c.d == 64 ? launch_phi<float, 64>(ctx, B, N, k, v, parent, accept, st, path_out, commit_len, s)
-                     : launch_phi<float, 128>(ctx, B, N, k, v, parent, accept, st, path_out, commit_len, s);
-  return c.d == 64 ? launch_phi<__nv_bfloat16, 64>(ctx, B, N, k, v, parent, accept, st, path_out, commit_len, s)
-                   : launch_phi<__nv_bfloat16, 128>(ctx, B, N, k, v, parent, accept, st, path_out, commit_len, s);
+    return c.d == 64 ? launch_phi<float, 64>(ctx, B, N, k, v, parent, accept, st, path_out, commit_len, fresh, s)
+                     : launch_phi<float, 128>(ctx, B, N, k, v, parent, accept, st, path_out, commit_len, fresh, s);
+  return c.d == 64 ? launch_phi<__nv_bfloat16, 64>(ctx, B, N, k, v, parent, accept, st, path_out, commit_len, fresh, s)
+                   : launch_phi<__nv_bfloat16, 128>(ctx, B, N, k, v, parent, accept, st, path_out, commit_len, fresh, s);
 }
 
 }  // namespace la

@@ -4,6 +4,7 @@
 #include <new>
 
 #include "la_common.cuh"
+#include "la_internal.h"
 
 namespace {
 
@@ -201,13 +202,19 @@ la_status la_verify_tree(la_ctx* ctx, int32_t B, int32_t N, const void* q, const
 
 la_status la_commit(la_ctx* ctx, int32_t B, int32_t N, const void* k, const void* v, const int32_t* parent,
                     const int32_t* accept_node, la_state* st, int32_t* path_out, int32_t* commit_len, void* stream) {
+  return la_commit_fresh(ctx, B, N, k, v, parent, accept_node, st, path_out, commit_len, 0, stream);
+}
+
+la_status la_commit_fresh(la_ctx* ctx, int32_t B, int32_t N, const void* k, const void* v, const int32_t* parent,
+                          const int32_t* accept_node, la_state* st, int32_t* path_out, int32_t* commit_len, int fresh,
+                          void* stream) {
   if (!ctx || B < 1 || N < 1 || !good(k) || !good(v) || !parent || !accept_node || !path_out || !commit_len)
     return LA_ERR_INVALID_ARG;
   if (N > ctx->cfg.max_nodes) return LA_ERR_INVALID_ARG;
   if (!state_ok(ctx, st)) return LA_ERR_INVALID_ARG;
   DeviceGuard g(ctx->device);
   if (!g.ok) return LA_ERR_CUDA;
-  return la::launch_commit(ctx, B, N, k, v, parent, accept_node, *st, path_out, commit_len,
+  return la::launch_commit(ctx, B, N, k, v, parent, accept_node, *st, path_out, commit_len, fresh,
                            static_cast<cudaStream_t>(stream)) == cudaSuccess
              ? LA_OK
              : LA_ERR_CUDA;

@@ -130,7 +130,7 @@ cudaError_t launch_prefill_simt(la_ctx* ctx, int B, int T, const void* q, const 
 cudaError_t launch_verify(la_ctx* ctx, int B, int N, const void* q, const void* k, const void* v,
                           const int32_t* parent, const float* w, const la_state& st, void* o, cudaStream_t s);
 cudaError_t launch_commit(la_ctx* ctx, int B, int N, const void* k, const void* v, const int32_t* parent,
-                          const int32_t* accept, const la_state& st, int32_t* path_out, int32_t* commit_len,
+                          const int32_t* accept, const la_state& st, int32_t* path_out, int32_t* commit_len, int fresh,
                           cudaStream_t s);
 // Tensor-core prefill (bf16, d = 128).  Sets *handled to false when the shape is not covered.
 cudaError_t launch_prefill_tc(la_ctx* ctx, int B, int T, const void* q, const void* k, const void* v,

@@ -1,0 +1,63 @@
+"""The native side of the binding: what it refuses, and the output buffers it makes."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2406_07368_b200 import binding, workloads as wl
+
+pytestmark = pytest.mark.gpu
+
+
+def _inputs(io="bf16", B=2, H=2, d=128, N=8, W=3):
+    ctx = binding.Context(H, d, W, "elu1", 0.0, io, max_nodes=16, max_depth=4)
+    q, k, v = (torch.from_numpy(x).to(ctx.dtype).cuda() for x in wl.qkv(11, (B, H, N, d), 1.0, io))
+    w = torch.from_numpy(wl.conv_weights(11, H, d, W)).cuda()
+    return ctx, q, k, v, w, ctx.new_state(B)
+
+
+def test_refusals():
+    ctx, q, k, v, w, st = _inputs()
+    for bad, what in ((q.float(), "dtype"), (q[:, :, :5], "contiguous"), (q.cpu(), "CUDA"), (q[:1], "shape")):
+        with pytest.raises(ValueError, match=what):
+            ctx.la_prefill(q, bad, v, w, st)
+    with pytest.raises(ValueError, match="state.S"):
+        ctx.la_prefill(q[:1].contiguous(), k[:1].contiguous(), v[:1].contiguous(), w, st)
+    with pytest.raises(ValueError):
+        ctx.la_decode_step(q, k, v, w, st)                       # one dimension too many
+    with pytest.raises(TypeError):
+        ctx.la_prefill("q", k, v, w, st)
+    with pytest.raises(binding.LaError) as e:                    # a missing tensor is the library's to refuse
+        ctx.la_prefill(q, None, v, w, st)
+    assert e.value.code == binding.LA_ERR_INVALID_ARG
+    ctx.close()
+    with pytest.raises(binding.LaError) as e:
+        ctx.la_prefill(q, k, v, w, st)
+    assert e.value.code == binding.LA_ERR_INVALID_ARG
+
+
+@pytest.mark.parametrize("given_path", [False, True])
+@pytest.mark.parametrize("given_len", [False, True])
+def test_commit_outputs_of_skipped_sequences(given_path, given_len):
+    """A malformed tree leaves the caller's buffers alone; buffers the binding makes read "no path, length 0"."""
+    ctx, q, k, v, w, st = _inputs()
+    parent = np.stack([wl.chain_tree(8)] * 2)
+    parent[1, 2] = 5                                             # parent after child
+    dirty = torch.full((1 << 16,), 77, dtype=torch.int32, device="cuda")
+    del dirty                                                    # what a new buffer gets is not zero by luck
+    path = torch.full((2, 4), 55, dtype=torch.int32, device="cuda") if given_path else None
+    length = torch.full((2,), 55, dtype=torch.int32, device="cuda") if given_len else None
+    path, length = ctx.la_commit(k, v, torch.from_numpy(parent).cuda(), torch.full((2,), 2, dtype=torch.int32, device="cuda"),
+                                 st, path_out=path, commit_len=length)
+    assert ctx.la_last_device_status() == binding.LA_ERR_BAD_TREE
+    assert path.tolist() == [[0, 1, 2, -1], [55] * 4 if given_path else [-1] * 4]
+    assert length.tolist() == [3, 55 if given_len else 0]
+
+
+def test_calls_on_a_given_stream():
+    ctx, q, k, v, w, st = _inputs()
+    want = ctx.la_prefill(q, k, v, w, st)
+    st2, out, s = ctx.new_state(2), torch.empty_like(q), torch.cuda.Stream()
+    s.wait_stream(torch.cuda.current_stream())
+    got = ctx.la_prefill(q, k, v, w, st2, out=out, stream=s)
+    s.synchronize()
+    assert torch.equal(got, want)
