@@ -125,7 +125,7 @@ static cudaError_t launch_t(la_ctx* ctx, int B, int N, const void* k, const void
   const la_config& c = ctx->cfg;
   auto kern = commit_kernel<T, D, PHI>;
   const size_t smem = (size_t)2 * c.max_depth * D * sizeof(float) + sizeof(CommitTables);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem((const void*)kern, ctx->device);
   if (e != cudaSuccess) return e;
   ctx->launches += 1;
   return launch_pdl(kern, dim3(B * c.H * kCommitSplit), dim3(256), smem, s, (const T*)k, (const T*)v, parent, accept, st.S,

@@ -1,4 +1,5 @@
 // C boundary: argument validation, dispatch to the kernel launchers, status handling.
+#include <atomic>
 #include <cmath>
 #include <cstdlib>
 #include <new>
@@ -34,6 +35,28 @@ struct DeviceGuard {
 };
 
 }  // namespace
+
+namespace la {
+
+cudaError_t allow_smem(const void* kern, int device) {
+  // Kernels already set, as an insert-only hash table without locks; a key is the kernel's address mixed with the device.
+  static std::atomic<uintptr_t> seen[1024];
+  const uintptr_t key = reinterpret_cast<uintptr_t>(kern) ^ ((uintptr_t)(device + 1) << 52);
+  size_t at = (size_t)((key * 0x9E3779B97F4A7C15ull) >> 54);
+  for (int probe = 0; probe < 1024; ++probe, at = (at + 1) & 1023) {
+    uintptr_t x = seen[at].load(std::memory_order_acquire);
+    if (x == key) return cudaSuccess;
+    if (x) continue;
+    int most = 0;
+    cudaError_t e = cudaDeviceGetAttribute(&most, cudaDevAttrMaxSharedMemoryPerBlockOptin, device);
+    if (e == cudaSuccess) e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, most);
+    if (e != cudaSuccess) return e;
+    if (seen[at].compare_exchange_strong(x, key, std::memory_order_acq_rel) || x == key) return cudaSuccess;
+  }
+  return cudaErrorUnknown;   // (more kernels times devices than places: does not happen)
+}
+
+}  // namespace la
 
 extern "C" {
 

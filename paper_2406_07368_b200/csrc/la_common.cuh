@@ -108,9 +108,10 @@ struct la_ctx {
   size_t ws_bytes;
 };
 
-// Launch with programmatic stream serialization allowed (see pdl_wait above).
+// Launch, with programmatic stream serialization allowed if asked for (see pdl_wait above).
 template <typename... KArgs, typename... Args>
-static inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args) {
+static inline cudaError_t launch_maybe_pdl(bool pdl, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                           Args... args) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = grid;
   cfg.blockDim = block;
@@ -120,9 +121,20 @@ static inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 blo
   attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
   attr[0].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = 1;
+  cfg.numAttrs = pdl ? 1 : 0;
   return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
 }
+template <typename... KArgs, typename... Args>
+static inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args) {
+  return launch_maybe_pdl(true, kern, grid, block, smem, s, args...);
+}
+
+namespace la {
+// Lets a kernel without static shared memory use all the dynamic shared memory an SM has.  Set once per kernel and
+// device (and to the same value for everybody: contexts of different sizes share the kernels), since the call costs as
+// much as the checks of a whole entry point; `device` is the current one.
+cudaError_t allow_smem(const void* kern, int device);
+}  // namespace la
 
 // Kernel launchers (one per translation unit).  All return the cudaError_t of the launch.
 namespace la {

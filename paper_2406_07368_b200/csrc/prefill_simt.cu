@@ -430,7 +430,7 @@ static cudaError_t launch_t(la_ctx* ctx, int B, int Tlen, const void* q, const v
   const la_config& c = ctx->cfg;
   auto kern = prefill_simt_kernel<T, D, PHI>;
   const size_t smem = Sh::bytes(c.conv_taps);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem((const void*)kern, ctx->device);
   if (e != cudaSuccess) return e;
   // CTAs per chain, each a segment of whole chunks: a whole cluster, until the chains alone fill half of the places for
   // CTAs.  (d = 64, 1000 tokens, us by CTAs per chain: 48 chains 196 with 1, 126 with 2, 94 with 4, 67 with 8; 192 chains

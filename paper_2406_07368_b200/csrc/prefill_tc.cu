@@ -6,7 +6,7 @@
 // chain in tiles of 128 tokens:
 //     O = phi(Q) S_prev + (P o M) V,   den = phi(Q) . z_prev + rowsum(P o M),   S += phi(K)^T V,   z += colsum phi(K).
 // The matrix products run on the tensor cores, and z rides along with them: V is extended by a column of ones
-// ([S | z] += phi(K)^T [V | 1], a 16-column unswizzled operand block), and the K tile by a row that holds z_prev, so
+// ([S | z] += phi(K)^T [V | 1], one product of 144 columns), and the K tile by a row that holds z_prev, so
 // that the score product delivers phi(q) . z_prev as one more column of P.  The row sums of the masked P are taken
 // by the threads that mask it.  Per tile n:
 //
@@ -16,17 +16,18 @@
 //            [S | z] += phi(K)^T [V | 1]               (fp32 in TMEM for the whole chain)
 //            O = phi(Q) S_prev                         (S_prev is a bf16 copy in shared memory)
 //   group A  phi on K of tile n+1 (K is double-buffered), while the tensor cores form the scores;
-//            P -> causal mask, row sums (+ the z column), bf16 -> TMEM (the A operand of the next product);
-//            the rows of v before the next tile -> a halo buffer;  S -> bf16 copy, z -> the K buffer of tile n+1
+//            P -> causal mask, row sums (+ the z column), bf16 -> TMEM (the A operand of the next product)
+//   group B  S -> bf16 copy, z -> the K buffer of tile n+1 (long windows: group A)
 //   tcgen05  O += (P o M) V
 //   group B  o = O / (den + eps) + conv(V) -> the tile's V buffer;  TMA stores it to global memory
 // (More than 5 taps: a second epilogue, which forms the tap sums by channel pair and stages the outputs in the tile's
 // K buffer; three-branch mode, GRP: the score product on the raw q and k and a causal softmax instead of the mask.)
 //
-// Four roles run concurrently: group A (warps 8-15), group B (warps 0-7), warp 16, whose elected lane issues
-// every MMA and the Q loads, and warp 17, one lane of which issues the V loads and the output stores (a store has
+// Five roles run concurrently: group A (warps 8-15), group B (warps 0-7), warp 16, whose elected lane issues
+// every MMA and the Q loads, warp 17, one lane of which issues the V loads and the output stores (a store has
 // to have read its buffer before the buffer is reloaded: that wait must not hold up the products) and another the
-// K reloads.  While group B finishes tile n, group A already works on tile n+1.  Every wait on an mbarrier is bounded; when one runs out the CTA
+// K reloads, and warp 18, which copies aside the rows of v that the convolution reaches back to.  While group B finishes
+// tile n, group A already works on tile n+1.  Every wait on an mbarrier is bounded; when one runs out the CTA
 // records LA_ERR_TIMEOUT, stops issuing work, frees its TMEM and returns.
 #include <cuda.h>
 
@@ -42,8 +43,8 @@ constexpr int D = 128;
 constexpr int TILE = 128;
 constexpr int kThreadsB = 256;                     // group B: warps 0-7
 constexpr int kThreadsA = 256;                     // group A: warps 8-15
-constexpr int kCtrlWarp = 16, kCopyWarp = 17;
-constexpr int kThreads = 576;
+constexpr int kCtrlWarp = 16, kCopyWarp = 17, kHaloWarp = 18;
+constexpr int kThreads = 640;
 constexpr uint32_t BOX_BYTES = 128 * 128;          // 128 rows x 64 bf16
 constexpr uint32_t TILE_BYTES = 2 * BOX_BYTES;
 // A K buffer carries 8 more rows below the 128 token rows of each box, the first of which (row 128) holds z_prev as
@@ -57,15 +58,27 @@ constexpr uint32_t KBUF_BYTES = 2 * KBOX_BYTES;
 // has been read.  The masked P goes back as packed bf16 pairs
 // into the columns its own fp32 values came from: each thread overwrites only columns of its own row that it has
 // already read (row r, tokens 64 hf + 32 qq ... + 31 -> columns 64 hf + 16 qq ... + 15).
-constexpr uint32_t P_COL = 0, QZ_COL = 128, O_COL = 144, S_COL = 272, FQ_COL = 400 /* 64 columns */, Z_COL = 464,
+constexpr uint32_t P_COL = 0, QZ_COL = 128, O_COL = 144, S_COL = 272, Z_COL = S_COL + 128, FQ_COL = 416 /* 64 columns */,
                    TMEM_COLS = 512;
 
-// shared-memory map (offsets from a 1024-byte aligned base)
-constexpr uint32_t OFF_Q = 0, OFF_V0 = TILE_BYTES, /* second V buffer at 2 * TILE_BYTES */ OFF_S = 3 * TILE_BYTES,
-                   OFF_K0 = 4 * TILE_BYTES, OFF_K1 = OFF_K0 + KBUF_BYTES,
-                   OFF_ONES = OFF_K1 + KBUF_BYTES, // [128 x 16] bf16, column 0 = 1: the extension of V
-                   OFF_DEN = OFF_ONES + 4096,      // [2][2][128] fp32: halves of the denominator of tile n in slot n & 1
-                   OFF_SMALL = OFF_DEN + 2048;
+// Shared-memory map (offsets from a 1024-byte aligned base).  The boxes of the two V buffers lie so that the block of
+// ones that extends V to [V | 1] is the third box of both: buffer 0 in steps of one box, buffer 1 in steps of three, with
+// Q in between.  [S | z] += phi(K)^T [V | 1] is then one product of 144 columns.  (As a product of its own, 16 columns
+// wide, the extension cost as many cycles of the tensor cores as any: they take ~75 per instruction from 16 columns to
+// 128, and every one of them reads phi(K) again: 1030 cycles per tile for the two, 616 for the one.)
+constexpr uint32_t OFF_S = 0, OFF_K0 = TILE_BYTES, OFF_K1 = OFF_K0 + KBUF_BYTES, OFF_VQ = OFF_K1 + KBUF_BYTES,
+                   OFF_Q = OFF_VQ + BOX_BYTES, OFF_ONES = OFF_VQ + 6 * BOX_BYTES;
+static_assert(OFF_VQ % 1024 == 0, "swizzled boxes");
+__host__ __device__ constexpr uint32_t vstep(uint32_t par) { return par ? 3 * BOX_BYTES : BOX_BYTES; }   // between a buffer's boxes
+__host__ __device__ constexpr uint32_t vbox(uint32_t par, uint32_t half) {
+  return OFF_VQ + (par ? 0u : 4 * BOX_BYTES) + half * vstep(par);
+}
+// The ones: a 128-byte-swizzled box of 128 rows of which the first 16 columns count (z3), or, where the taps of a long
+// window leave no room for that, a block of 16 unswizzled columns (a product of its own, columns S_COL + 128 ...).
+__host__ __device__ constexpr uint32_t ones_bytes(bool z3) { return z3 ? BOX_BYTES : 4096u; }
+// [2][2][128] fp32: halves of the denominator of tile n in slot n & 1
+__host__ __device__ constexpr uint32_t off_den(bool z3) { return OFF_ONES + ones_bytes(z3); }
+__host__ __device__ constexpr uint32_t off_small(bool z3) { return off_den(z3) + 2048; }
 
 struct Small {
   unsigned long long bars[20];
@@ -80,28 +93,37 @@ struct Small {
 // after O = phi(Q) S_prev; after O += P V (MMA_O0 / MMA_O1, tiles alternate).
 // A barrier that one role waits on while another role can run a tile ahead exists once per tile parity, so that a
 // waiter is never more than one phase behind.
-enum { B_FULL_K0 = 0, B_FULL_V0 = 1, B_FULL_V1 = 2, B_MMA_P = 3, B_MMA_S = 4, B_MMA_O0 = 5, B_MMA_O1 = 6, B_PHI = 7,
+enum { B_FULL_K0 = 0, B_FULL_V0 = 1, B_FULL_V1 = 2, B_MMA_P = 3, B_MMA_S0 = 4, B_MMA_O0 = 5, B_MMA_O1 = 6, B_PHI = 7,
        B_PDONE = 8, B_SB = 9, B_EPI0 = 10, B_EPI1 = 11, B_MMA_Q = 12, B_FULL_Q = 13, B_FULL_K1 = 14, B_STAGED0 = 15,
-       B_STAGED1 = 16, B_HALO = 17, kNumBars = 18 };
+       B_STAGED1 = 16, B_HALO0 = 17, B_HALO1 = 18, B_MMA_S1 = 19, kNumBars = 20 };
+static_assert(kNumBars <= 20, "Small::bars");
 
-__host__ __device__ constexpr uint32_t off_w() { return OFF_SMALL + (uint32_t)((sizeof(Small) + 15) / 16 * 16); }
-__host__ __device__ inline uint32_t off_halo(int W) { return off_w() + (uint32_t)W * D * 4; }
-// Three halo buffers (the rows of v before a tile, for the convolution).  Where group B fills them itself, tile n reads
-// buffer n & 1 and fills the other; where group A fills them (short windows of the exact layer), tile n reads buffer
-// n % 3 and group A fills (n + 1) % 3 meanwhile, which the epilogue of tile n - 1 no longer reads.
-__host__ __device__ inline uint32_t smem_bytes(int W) { return off_halo(W) + 3u * (uint32_t)(W > 1 ? W - 1 : 1) * D * 2 + 1024; }
+__host__ __device__ constexpr uint32_t off_w(bool z3) { return off_small(z3) + (uint32_t)((sizeof(Small) + 15) / 16 * 16); }
+// Short windows: nine halo buffers, rows of v that lie before 32 rows of a tile, for the convolution.  Buffers 0-2: the
+// rows before tile n in n % 3; 3-8: the rows before rows 32, 64 and 96 of a tile, by the tile's parity.  Rows lie as in a
+// V box (64 channels each, 128-byte swizzle; the row number counted back from the 32 rows: -1, -2, ...).
+__host__ __device__ inline uint32_t off_halo(int W) { return (off_w(true) + (uint32_t)W * D * 4 + 127u) & ~127u; }
+__host__ __device__ inline uint32_t halo_bytes(int W) { return (uint32_t)(W - 1) * 256u; }
+__device__ __forceinline__ uint32_t halo_at(int i, int c16, int W) {   // row i (0 = oldest), 16-byte piece c16 of 16
+  return (uint32_t)(c16 >> 3) * (uint32_t)(W - 1) * 128u + (uint32_t)i * 128u + (uint32_t)(((c16 & 7) ^ ((i - (W - 1)) & 7)) << 4);
+}
+__host__ __device__ inline uint32_t smem_bytes(int W) { return off_halo(W) + 9u * halo_bytes(W) + 1024; }
 // The three-branch mode keeps 4 KB more behind the halo rows: z before the tile as fp32 [128], the halves of
 // phi(q) . z [2][128], and each half-row's running maximum and sum of the softmax [2][128] x 2.
 constexpr uint32_t kGrpScratch = 4096;
 // The epilogue for longer tap windows ("long" below) keeps the taps padded with zeros to whole groups of 8 and ONE
 // halo buffer, updated in place, of as many rows as the padded taps reach back (the rows before the window stay 0).
+constexpr uint32_t kMaxSmem = 227u * 1024u;
 __host__ __device__ inline uint32_t long_taps(int W) { return ((uint32_t)W + 7u) & ~7u; }
-__host__ __device__ inline uint32_t off_halo_long(int W) { return off_w() + long_taps(W) * D * 4; }
-__host__ __device__ inline uint32_t smem_bytes_long(int W) { return off_halo_long(W) + (long_taps(W) - 1) * D * 2 + 1024; }
-__host__ __device__ inline uint32_t off_grp(int W, bool lng = false) {
-  return ((lng ? smem_bytes_long(W) : smem_bytes(W)) - 1024 + 15u) & ~15u;
+__host__ __device__ inline bool z3_long(int W, bool grp) {
+  return off_w(true) + long_taps(W) * D * 4 + (long_taps(W) - 1) * D * 2 + 1024 + (grp ? kGrpScratch + 16u : 0u) <= kMaxSmem;
 }
-__host__ __device__ inline uint32_t smem_bytes_grp(int W, bool lng = false) { return off_grp(W, lng) + kGrpScratch + 1024; }
+__host__ __device__ inline uint32_t off_halo_long(int W, bool grp) { return off_w(z3_long(W, grp)) + long_taps(W) * D * 4; }
+__host__ __device__ inline uint32_t smem_bytes_long(int W, bool grp) { return off_halo_long(W, grp) + (long_taps(W) - 1) * D * 2 + 1024; }
+__host__ __device__ inline uint32_t off_grp(int W, bool lng) {
+  return ((lng ? smem_bytes_long(W, true) : smem_bytes(W)) - 1024 + 15u) & ~15u;
+}
+__host__ __device__ inline uint32_t smem_bytes_grp(int W, bool lng) { return off_grp(W, lng) + kGrpScratch + 1024; }
 // Which windows take the long epilogue: above 5 taps it is the faster of the two (measured on 128 chains of 2048
 // tokens: 6 taps 126 us either way, 8 taps 132 against 154 us, 16 taps 126 against 254, 32 taps 162 against 686).
 // The three-branch mode compiles the short epilogue for 3 taps only.
@@ -129,11 +151,6 @@ __device__ __forceinline__ float ex2(float x) {
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
-__device__ __forceinline__ void sync_half_b(int hf) {
-  if (hf) asm volatile("bar.sync 4, 128;" ::: "memory");
-  else asm volatile("bar.sync 3, 128;" ::: "memory");
-}
-
 __device__ __forceinline__ void tma_load(uint32_t dst, const CUtensorMap* map, int x, int y, int z, uint32_t bar) {
   asm volatile(
       "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
@@ -192,6 +209,76 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
         "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]),          \
         "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])           \
       : "memory")
+
+// Fragments of 8 rows x 8 columns: 16 TMEM lanes x 8 G columns at once; register 4 g + 2 i + e of lane l holds row
+// (l >> 2) + 8 i, column 8 g + 2 (l & 3) + e.  Four lanes then hold 32 consecutive bytes of an fp32 row, one sector of
+// global memory: the layout in which a state moves between TMEM and HBM (with a row per lane every access touched 32
+// cache lines, 16 bytes each: 3 us to write one 64 KB state, as long as a tile takes).
+#define LA_TMEM_LD_FRAG8(taddr, r)                                                                               \
+  asm volatile(                                                                                                  \
+      "tcgen05.ld.sync.aligned.16x256b.x8.b32 "                                                                  \
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "                                  \
+      "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"                  \
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),          \
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15]),    \
+        "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23]),  \
+        "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])   \
+      : "r"(taddr)                                                                                               \
+      : "memory")
+#define LA_TMEM_ST_FRAG8(taddr, r)                                                                               \
+  asm volatile(                                                                                                  \
+      "tcgen05.st.sync.aligned.16x256b.x8.b32 [%0], "                                                            \
+      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "                                 \
+      "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};"                         \
+      ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),      \
+        "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]),            \
+        "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]),          \
+        "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])           \
+      : "memory")
+#define LA_TMEM_LD_FRAG4(taddr, r)                                                                               \
+  asm volatile(                                                                                                  \
+      "tcgen05.ld.sync.aligned.16x256b.x4.b32 "                                                                  \
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"                           \
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),          \
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])     \
+      : "r"(taddr)                                                                                               \
+      : "memory")
+// Global side of a fragment of 64 columns; `p` is this lane's first element (row l >> 2, column 2 (l & 3)) of a [..][128]
+// matrix.
+__device__ __forceinline__ void frag_load(const float* p, uint32_t (&r)[32]) {
+#pragma unroll
+  for (int g = 0; g < 8; ++g)
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const float2 x = *reinterpret_cast<const float2*>(p + i * 8 * D + 8 * g);
+      r[4 * g + 2 * i] = __float_as_uint(x.x);
+      r[4 * g + 2 * i + 1] = __float_as_uint(x.y);
+    }
+}
+__device__ __forceinline__ void frag_add(uint32_t (&r)[32], const uint32_t (&x)[32]) {
+#pragma unroll
+  for (int e = 0; e < 32; ++e) r[e] = __float_as_uint(__uint_as_float(r[e]) + __uint_as_float(x[e]));
+}
+__device__ __forceinline__ void frag_store(float* p, const uint32_t (&r)[32]) {
+#pragma unroll
+  for (int g = 0; g < 8; ++g)
+#pragma unroll
+    for (int i = 0; i < 2; ++i)
+      *reinterpret_cast<float2*>(p + i * 8 * D + 8 * g) =
+          make_float2(__uint_as_float(r[4 * g + 2 * i]), __uint_as_float(r[4 * g + 2 * i + 1]));
+}
+// 8 x 8 matrices of bf16 between shared memory and the same fragments: lane l names the 16-byte row l & 7 of matrix l >> 3.
+__device__ __forceinline__ void ldmatrix4(uint32_t a, uint32_t (&r)[4]) {
+  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
+               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3])
+               : "r"(a)
+               : "memory");
+}
+__device__ __forceinline__ void stmatrix4(uint32_t a, const uint32_t (&r)[4]) {
+  asm volatile("stmatrix.sync.aligned.m8n8.x4.shared.b16 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(r[0]), "r"(r[1]), "r"(r[2]),
+               "r"(r[3])
+               : "memory");
+}
 
 __device__ __forceinline__ uint32_t tmem_ld1(uint32_t taddr) {
   uint32_t v;
@@ -286,28 +373,8 @@ template <int PHI> __device__ __forceinline__ uint4 phi8(uint4 u) {
 __device__ __forceinline__ uint32_t swz(int row, int cc) { return (uint32_t)row * 128u + (uint32_t)((cc ^ (row & 7)) << 4); }
 
 // ---- the kernel ------------------------------------------------------------------------------------
-// Convolution part of the epilogue for one 8-channel chunk: acc[e] += sum_t w[t][ch] v_{row-t}[ch], two channels per
-// packed fp32 multiply-add (each half is the IEEE fused multiply-add of the scalar instruction).
+// (Two channels per packed fp32 multiply-add: each half is the IEEE fused multiply-add of the scalar instruction.)
 __device__ __forceinline__ float2 bf2(uint32_t u) { return make_float2(lo_f(u), hi_f(u)); }
-template <int WT>
-__device__ __forceinline__ void conv8(float2* acc, int W, int r, int cc, int ch0, const unsigned char* Vbox,
-                                      const __nv_bfloat16* halo, const float* wsm) {
-  const int taps = WT > 0 ? WT : W;
-#pragma unroll
-  for (int t = 0; t < taps; ++t) {
-    const int row = r - t;
-    uint4 u;
-    if (row >= 0) u = *reinterpret_cast<const uint4*>(Vbox + swz(row, cc));
-    else u = *reinterpret_cast<const uint4*>(halo + (W - 1 + row) * D + ch0);
-    const float4 w0 = *reinterpret_cast<const float4*>(wsm + t * D + ch0);
-    const float4 w1 = *reinterpret_cast<const float4*>(wsm + t * D + ch0 + 4);
-    acc[0] = __ffma2_rn(make_float2(w0.x, w0.y), bf2(u.x), acc[0]);
-    acc[1] = __ffma2_rn(make_float2(w0.z, w0.w), bf2(u.y), acc[1]);
-    acc[2] = __ffma2_rn(make_float2(w1.x, w1.y), bf2(u.z), acc[2]);
-    acc[3] = __ffma2_rn(make_float2(w1.z, w1.w), bf2(u.w), acc[3]);
-  }
-}
-
 // Long-window epilogue: one thread owns a pair of channels and 32 consecutive rows of the tile, in four blocks of 8.
 // conv_block adds one group of 8 taps to the 8 sums of block BLK: the 15 rows of v that those taps reach are each
 // read once, as one packed pair, and feed up to 8 of the sums.  Where the rows come from is fixed at compile time:
@@ -409,20 +476,26 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
                   const float* __restrict__ w, float* __restrict__ S, float* __restrict__ z,
                   __nv_bfloat16* __restrict__ win, int64_t* __restrict__ pos,
                   int* status, int H, int Ttot, int W, float eps, int init, int nseg,
-                  int seg_len, float* __restrict__ S_fin, float* __restrict__ z_fin, float alpha, float sm_scale,
-                  int tstep) {
+                  int seg_len, const float* __restrict__ S_seg, const float* __restrict__ z_seg,
+                  const __nv_bfloat16* __restrict__ win_seg, int prefixed, const __nv_bfloat16* __restrict__ vg, float alpha,
+                  float sm_scale, int tstep, int early) {
   extern __shared__ unsigned char smem_dyn[];
   // (an offset into the array rather than an integer cast: the compiler then knows that these are shared-memory
   // addresses: 32-bit arithmetic, ld.shared / st.shared)
   unsigned char* smem = smem_dyn + ((1024u - (smem_u32(smem_dyn) & 1023u)) & 1023u);
   const uint32_t sbase = smem_u32(smem);
-  Small& sm = *reinterpret_cast<Small*>(smem + OFF_SMALL);
   constexpr bool LONG = WT < 0;                  // the epilogue for longer tap windows
-  constexpr bool HALO_A = !GRP && WT > 0;        // group A copies the rows before the next tile aside (it has the time)
-  float* wsm = reinterpret_cast<float*>(smem + off_w());                       // [W][128] ([W up to a multiple of 8][128] if LONG)
-  // two halo buffers [W-1][128], oldest row first: tile n reads buffer n&1 and writes buffer (n+1)&1 (LONG: one buffer)
-  __nv_bfloat16* halo0 = reinterpret_cast<__nv_bfloat16*>(smem + (LONG ? off_halo_long(W) : off_halo(W)));
-  const int halo_elems = (W > 1 ? W - 1 : 1) * D;
+  // Who copies the state between two tiles: group B has the time beside an elu + 1 (which keeps group A busy), group A beside
+  // a ReLU or a long window (which keeps group B busy).
+  constexpr bool SNAP_A = LONG || (PHI == LA_PHI_RELU && !GRP);
+  // Of the 128 rows of phi(K) group B takes the last 16 KB, beside an elu + 1 with a short window: group A's loop (phi(Q),
+  // phi(K), mask) is the longest there, and group B had 2 K of a tile's 5.9 K cycles to spare.  (128 chains of 2048 tokens,
+  // 3 taps: 71 us with none, 65.4 with 2, 64.6 with 3, 65.8 with 4.)
+  constexpr int KB = SNAP_A || GRP ? 0 : 3;
+  const bool z3 = LONG ? z3_long(W, GRP) : true; // z rides in the state update's product
+  Small& sm = *reinterpret_cast<Small*>(smem + off_small(z3));
+  float* wsm = reinterpret_cast<float*>(smem + off_w(z3));                     // [W][128] ([W up to a multiple of 8][128] if LONG)
+  __nv_bfloat16* halo0 = reinterpret_cast<__nv_bfloat16*>(smem + (LONG ? off_halo_long(W, GRP) : off_halo(W)));
   volatile int* abort = &sm.abort;
   // three-branch mode only: z before the tile (fp32), the halves of phi(q) . z, the halves of the softmax statistics
   float* zs = reinterpret_cast<float*>(smem + off_grp(W, LONG));               // [128]
@@ -431,10 +504,25 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
   const bool use_glob = GRP && alpha != 0.f;     // alpha = 0: the global branch is switched off altogether
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  // A launch covers BH chains cut into nseg segments of seg_len tokens (nseg = 1: whole chains).  Unit u owns
-  // tokens [y0, y0 + T) of chain bh; state, window and z of a unit are addressed by u.
-  const int u = blockIdx.x, bh = u / nseg, h = bh % H;
-  const int y0 = (u % nseg) * seg_len, T = min(seg_len, Ttot - y0);
+  // A launch covers BH chains cut into nseg segments of seg_len tokens (nseg = 1: whole chains).  This block owns
+  // tokens [y0, y0 + T) of chain bh.  Whole chains start from the caller's state.  Of a chain that was cut, segment
+  // sg > 0 starts from the sums of the segments before it (the first of which holds the caller's state too; `prefixed`:
+  // slot sg - 1 holds them added up) and from the values of v before it, segment 0 from the copy of the caller's state
+  // that the pre-pass left in the last slot; only the last segment writes a state, the caller's.
+  const int bh = blockIdx.x / nseg, sg = blockIdx.x % nseg, h = bh % H;
+  const int y0 = sg * seg_len, T = min(seg_len, Ttot - y0);
+  const bool has_in = init || sg > 0, writes_state = sg == nseg - 1;
+  const int nsum = sg > 0 && !prefixed ? sg : 1;  // how many parts the incoming state has
+  const size_t slot = nseg > 1 ? (size_t)bh * nseg + (sg == 0 ? nseg - 1 : prefixed ? sg - 1 : 0) : (size_t)bh;
+  const float* S_in = (nseg > 1 ? S_seg : S) + slot * D * D;
+  const float* z_in = (nseg > 1 ? z_seg : z) + slot * D;
+  const __nv_bfloat16* win_in = sg > 0 ? vg + ((size_t)bh * Ttot + y0 - (W - 1)) * D
+                                       : (nseg > 1 ? win_seg : win) + (size_t)bh * (W - 1) * D;
+  auto z_start = [&](int a) {
+    float x = z_in[a];
+    for (int j = 1; j < nsum; ++j) x += z_in[j * D + a];
+    return x;
+  };
   // tstep: tokens per tile, 128 except for three-branch groups shorter than that, which take one partly filled tile
   // each (the TMA boxes are then tstep rows high; the rows below hold zeros or values that the causal mask discards).
   const int nchunks = (T + tstep - 1) / tstep;
@@ -442,27 +530,45 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
   const uint32_t bar0 = smem_u32(&sm.bars[0]);    // barrier i lives at bar0 + 8 i
 
   // ---- set-up ----
-  if (tid == 0) {
+  if (tid == kCopyWarp * 32) {
     mbar_init((bar0 + 8u * (B_FULL_K0)), 1);
     mbar_init((bar0 + 8u * (B_FULL_K1)), 1);
     mbar_init((bar0 + 8u * (B_FULL_Q)), 1);
     mbar_init((bar0 + 8u * (B_FULL_V0)), 1);
     mbar_init((bar0 + 8u * (B_FULL_V1)), 1);
     mbar_init((bar0 + 8u * (B_MMA_P)), 1);
-    mbar_init((bar0 + 8u * (B_MMA_S)), 1);
+    mbar_init((bar0 + 8u * (B_MMA_S0)), 1);
+    mbar_init((bar0 + 8u * (B_MMA_S1)), 1);
     mbar_init((bar0 + 8u * (B_MMA_O0)), 1);
     mbar_init((bar0 + 8u * (B_MMA_O1)), 1);
     mbar_init((bar0 + 8u * (B_PHI)), kThreadsA);
     mbar_init((bar0 + 8u * (B_PDONE)), kThreadsA);
-    mbar_init((bar0 + 8u * (B_SB)), kThreadsA);
+    mbar_init((bar0 + 8u * (B_SB)), SNAP_A ? kThreadsA : kThreadsB);
     mbar_init((bar0 + 8u * (B_EPI0)), kThreadsB);
     mbar_init((bar0 + 8u * (B_EPI1)), kThreadsB);
     mbar_init((bar0 + 8u * (B_MMA_Q)), 1);
     mbar_init((bar0 + 8u * (B_STAGED0)), kThreadsB);
     mbar_init((bar0 + 8u * (B_STAGED1)), kThreadsB);
-    mbar_init((bar0 + 8u * (B_HALO)), kThreadsA);
+    mbar_init((bar0 + 8u * (B_HALO0)), 32);
+    mbar_init((bar0 + 8u * (B_HALO1)), 32);
     sm.abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    // the first tiles are requested at once (nothing below touches the rows that they bring)
+    pdl_wait();
+    for (int n = 0; n < 2 && n < nchunks; ++n) {
+      const uint32_t kb = sbase + (n ? OFF_K1 : OFF_K0), kbar = bar0 + 8u * (n ? B_FULL_K1 : B_FULL_K0), vbar = bar0 + 8u * (B_FULL_V0 + n);
+      mbar_expect_tx(kbar, tile_tx);
+      tma_load(kb, &mk, 0, y0 + n * tstep, bh, kbar);
+      tma_load(kb + KBOX_BYTES, &mk, 64, y0 + n * tstep, bh, kbar);
+      if (n == 0) {
+        mbar_expect_tx((bar0 + 8u * (B_FULL_Q)), tile_tx);
+        tma_load(sbase + OFF_Q, &mq, 0, y0, bh, (bar0 + 8u * (B_FULL_Q)));
+        tma_load(sbase + OFF_Q + BOX_BYTES, &mq, 64, y0, bh, (bar0 + 8u * (B_FULL_Q)));
+      }
+      mbar_expect_tx(vbar, tile_tx);
+      tma_load(sbase + vbox(n, 0), &mv, 0, y0 + n * tstep, bh, vbar);
+      tma_load(sbase + vbox(n, 1), &mv, 64, y0 + n * tstep, bh, vbar);
+    }
   }
   if (warp == kCtrlWarp) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sm.tmem_base)),
@@ -470,32 +576,36 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
+  float* denbuf = reinterpret_cast<float*>(smem + off_den(z3));
+  for (int idx = tid; idx < (int)ones_bytes(z3) / 16; idx += kThreads)         // the block of ones <- 0
+    reinterpret_cast<uint4*>(smem + OFF_ONES)[idx] = make_uint4(0u, 0u, 0u, 0u);
+  if (GRP && tstep < TILE) {                                                   // partly filled tiles: rows tstep-127 of V <- 0
+    const int per_box = (TILE - tstep) * 8;                                    // 16-byte pieces per box
+    for (int idx = tid; idx < 4 * per_box; idx += kThreads)
+      reinterpret_cast<uint4*>(smem + vbox((idx / per_box) >> 1, (idx / per_box) & 1) + tstep * 128)[idx % per_box] = make_uint4(0u, 0u, 0u, 0u);
+  }
+  for (int idx = tid; idx < 4 * 1024 / 16; idx += kThreads)                    // rows 128-135 of the four K boxes <- 0
+    reinterpret_cast<uint4*>(smem + OFF_K0 + (idx >> 6) * KBOX_BYTES + BOX_BYTES)[idx & 63] = make_uint4(0u, 0u, 0u, 0u);
+  pdl_wait();                                     // everything above touched shared memory and TMEM only
+  if (early) pdl_trigger();
   for (int idx = tid; idx < (LONG ? (int)long_taps(W) : W) * D; idx += kThreads)
     wsm[idx] = idx < W * D ? w[((size_t)h * D + (idx % D)) * W + idx / D] : 0.f;
   if (LONG) {                                    // [long_taps - 1][128]: zeros, then the W-1 rows of the window
     const int lead = ((int)long_taps(W) - W) * D;
     for (int idx = tid; idx < ((int)long_taps(W) - 1) * D; idx += kThreads)
-      halo0[idx] = init && idx >= lead ? win[(size_t)u * (W - 1) * D + idx - lead] : __float2bfloat16_rn(0.f);
-  } else
-  for (int idx = tid; idx < (W - 1) * D; idx += kThreads)
-    halo0[idx] = init ? win[(size_t)u * (W - 1) * D + idx] : __float2bfloat16_rn(0.f);
-  float* denbuf = reinterpret_cast<float*>(smem + OFF_DEN);
-  for (int idx = tid; idx < 4096 / 16; idx += kThreads)                        // the 16-column block of ones <- 0
-    reinterpret_cast<uint4*>(smem + OFF_ONES)[idx] = make_uint4(0u, 0u, 0u, 0u);
-  if (GRP && tstep < TILE) {                                                   // partly filled tiles: rows tstep-127 of V <- 0
-    const int per_box = (TILE - tstep) * 8;                                    // 16-byte pieces per box
-    for (int idx = tid; idx < 4 * per_box; idx += kThreads)
-      reinterpret_cast<uint4*>(smem + OFF_V0 + (idx / per_box) * BOX_BYTES + tstep * 128)[idx % per_box] = make_uint4(0u, 0u, 0u, 0u);
+      halo0[idx] = has_in && idx >= lead ? win_in[idx - lead] : __float2bfloat16_rn(0.f);
+  } else {
+    for (int idx = tid; idx < (W - 1) * 16; idx += kThreads)
+      *reinterpret_cast<uint4*>(smem + off_halo(W) + halo_at(idx >> 4, idx & 15, W)) =
+          has_in ? reinterpret_cast<const uint4*>(win_in)[idx] : make_uint4(0u, 0u, 0u, 0u);
   }
-  for (int idx = tid; idx < 4 * 1024 / 16; idx += kThreads)                    // rows 128-135 of the four K boxes <- 0
-    reinterpret_cast<uint4*>(smem + OFF_K0 + (idx >> 6) * KBOX_BYTES + BOX_BYTES)[idx & 63] = make_uint4(0u, 0u, 0u, 0u);
   __syncthreads();
   if (tid < TILE) {
-    *reinterpret_cast<__nv_bfloat16*>(smem + OFF_ONES + ext_offset(tid, 0)) = __float2bfloat16_rn(1.f);
-    if (GRP) zs[tid] = init ? z[(size_t)u * D + tid] : 0.f;
-    else if (init)                                // z before tile 0: row 128 of the first K buffer (feature tid)
+    *reinterpret_cast<__nv_bfloat16*>(smem + OFF_ONES + (z3 ? swz(tid, 0) : ext_offset(tid, 0))) = __float2bfloat16_rn(1.f);
+    if (GRP) zs[tid] = has_in ? z_start(tid) : 0.f;
+    else if (has_in)                                // z before tile 0: row 128 of the first K buffer (feature tid)
       *reinterpret_cast<__nv_bfloat16*>(smem + OFF_K0 + (tid >> 6) * KBOX_BYTES + BOX_BYTES + (tid & 63) * 2) =
-          __float2bfloat16_rn(z[(size_t)u * D + tid]);
+          __float2bfloat16_rn(z_start(tid));
   }
   fence_proxy_async();
   tc_fence_before();
@@ -503,21 +613,122 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
   tc_fence_after();
   const uint32_t tmem = sm.tmem_base;
 
+  if (has_in && warp < 16) {
+    // The incoming state: fp32 into TMEM and a bf16 copy into shared memory (z: the row in the K buffer is in place).
+    // Both groups share it out, 16 rows x 64 columns per warp.
+    const int q4 = warp & 3, hf = (warp >> 2) & 1, r0 = 32 * q4 + 16 * (warp >> 3);
+    const float* Sg = S_in + (size_t)(r0 + (lane >> 2)) * D + 64 * hf + 2 * (lane & 3);
+    uint32_t v[32], x[32];
+    frag_load(Sg, v);
+    for (int j = 1; j < nsum; ++j) {                // the sums of the segments before this one
+      frag_load(Sg + (size_t)j * D * D, x);
+      frag_add(v, x);
+    }
+    LA_TMEM_ST_FRAG8(tmem + ((uint32_t)r0 << 16) + S_COL + 64 * hf, v);
+#pragma unroll
+    for (int g = 0; g < 8; ++g)
+#pragma unroll
+      for (int i = 0; i < 2; ++i)
+        *reinterpret_cast<uint32_t*>(smem + OFF_S + hf * BOX_BYTES + swz(r0 + (lane >> 2) + 8 * i, g) + 4 * (lane & 3)) =
+            pack2(__uint_as_float(v[4 * g + 2 * i]), __uint_as_float(v[4 * g + 2 * i + 1]));
+    if (warp < 4) {                                 // z, and zeros in the other columns of its block (32 rows per warp)
+      const uint32_t zaddr = tmem + ((uint32_t)(32 * q4) << 16) + Z_COL;
+      tmem_st1(zaddr, __float_as_uint(z_start(32 * q4 + lane)));
+#pragma unroll
+      for (int c = 1; c < 16; ++c) tmem_st1(zaddr + c, 0u);
+    }
+    tmem_wait_st();
+    fence_proxy_async();
+    tc_fence_before();
+    asm volatile("bar.sync 6, 512;" ::: "memory");
+    tc_fence_after();
+  }
+
+  // phi on rows 16 I0 ... 16 I1 - 1 of the K tile of tile m, in place, by 256 threads (ta); rows at or beyond the end of the
+  // sequence become zero
+  auto phi_k = [&](auto i0c, auto i1c, int m, int ta) {
+    constexpr int I0 = decltype(i0c)::value, I1 = decltype(i1c)::value, NI = I1 - I0;
+    if constexpr (NI > 0) {
+      const int valid = min(tstep, T - m * tstep);
+      const int ct = ta & 15, rg = ta >> 4;                     // chunk column 0..15, row group 0..15
+      unsigned char* Kb = smem + ((m & 1) ? OFF_K1 : OFF_K0) + (ct >> 3) * KBOX_BYTES;
+      uint4 x[NI];                                              // all loads first: they do not wait for the stores
+#pragma unroll
+      for (int i = 0; i < NI; ++i) x[i] = *reinterpret_cast<const uint4*>(Kb + swz(rg + 16 * (I0 + i), ct & 7));
+#pragma unroll
+      for (int i = 0; i < NI; ++i) {
+        const int j = rg + 16 * (I0 + i);
+        *reinterpret_cast<uint4*>(Kb + swz(j, ct & 7)) = j < valid ? phi8<PHI>(x[i]) : make_uint4(0u, 0u, 0u, 0u);
+      }
+    }
+  };
+  using K0c = std::integral_constant<int, 0>;
+  using KAc = std::integral_constant<int, 8 - KB>;
+  using K8c = std::integral_constant<int, 8>;
+
+  // S and z after tile n: the bf16 copy and the z row for the next tile, or the final state to global memory.  256 threads
+  // (row r, 64 columns each): group B or group A.
+  auto snapshot = [&](int n, int r, int hf, uint32_t lane_addr, bool& ok) {
+    const uint32_t par = n & 1;
+    const bool last = n + 1 == nchunks;
+    unsigned char* Sb = smem + OFF_S + hf * BOX_BYTES;
+    // ---- S_n: bf16 copy for the next tile, or the final state to global memory ----
+    // S_n is final after MMA_S; the old copy may be overwritten once O = phi(Q) S_prev has read it
+    ok = ok && mbar_wait((bar0 + 8u * (par ? B_MMA_S1 : B_MMA_S0)), (n >> 1) & 1, abort) && mbar_wait((bar0 + 8u * (B_MMA_Q)), par, abort);
+    ok = __all_sync(0xffffffffu, ok);
+    if (ok) {
+      tc_fence_after();
+      uint32_t zbits = 0u;
+      if (hf == 0) zbits = tmem_ld1(tmem + lane_addr + Z_COL);
+      if (!last) {
+#pragma unroll
+        for (int qq = 0; qq < 2; ++qq) {
+          uint32_t v[32];
+          LA_TMEM_LD32(tmem + lane_addr + S_COL + 64 * hf + 32 * qq, v);
+          tmem_wait_ld();
+#pragma unroll
+          for (int c = 0; c < 4; ++c) *reinterpret_cast<uint4*>(Sb + swz(r, 4 * qq + c)) = pack8(v + 8 * c);
+        }
+      } else if (writes_state) {
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {             // rows 16 i ... 16 i + 15 of this warp's 32
+          uint32_t v[32];
+          LA_TMEM_LD_FRAG8(tmem + lane_addr + ((uint32_t)(16 * i) << 16) + S_COL + 64 * hf, v);
+          tmem_wait_ld();
+          frag_store(S + (size_t)bh * D * D + (size_t)((r & ~31) + 16 * i + (lane >> 2)) * D + 64 * hf + 2 * (lane & 3), v);
+        }
+      } else {
+        tmem_wait_ld();                           // zbits
+      }
+      if (hf == 0) {
+        const float zz = __uint_as_float(zbits);
+        if (last) {
+          if (writes_state) z[(size_t)bh * D + r] = zz;
+        } else if (GRP) {
+          zs[r] = zz;                             // fp32, for phi(q) . z of the next tile
+        } else {                                  // row 128 of the K buffer of tile n+1
+          *reinterpret_cast<__nv_bfloat16*>(smem + (((n + 1) & 1) ? OFF_K1 : OFF_K0) + (r >> 6) * KBOX_BYTES + BOX_BYTES +
+                                            (r & 63) * 2) = __float2bfloat16_rn(zz);
+        }
+      }
+    }
+    fence_proxy_async();
+    tc_fence_before();
+    mbar_arrive((bar0 + 8u * (B_SB)));
+  };
+
   if (warp == kCtrlWarp) {
     // =============================== MMA issue, the Q and K loads (one lane) ===============================
     if (lane == 0) {
       bool ok = true;
-      mbar_expect_tx((bar0 + 8u * (B_FULL_Q)), tile_tx);
-      tma_load(sbase + OFF_Q, &mq, 0, y0, bh, (bar0 + 8u * (B_FULL_Q)));
-      tma_load(sbase + OFF_Q + BOX_BYTES, &mq, 64, y0, bh, (bar0 + 8u * (B_FULL_Q)));
       for (int n = 0; n < nchunks; ++n) {
         const uint32_t par = n & 1;
-        const uint32_t vbuf = sbase + OFF_V0 + par * TILE_BYTES;
+        const uint32_t vbuf = sbase + vbox(par, 0);
         const uint32_t kbuf = sbase + (par ? OFF_K1 : OFF_K0);
-        const bool has_state = init || n > 0;
+        const bool has_state = has_in || n > 0;
         // low descriptor words of step 0: K read along its rows (K-major), K, V and the S copy down their rows
         const uint32_t k_km = desc_lo(kbuf, 16u);
-        const uint32_t k_mn = desc_lo(kbuf, KBOX_BYTES), v_mn = desc_lo(vbuf, BOX_BYTES), s_mn = desc_lo(sbase + OFF_S, BOX_BYTES);
+        const uint32_t k_mn = desc_lo(kbuf, KBOX_BYTES), v_mn = desc_lo(vbuf, vstep(par)), s_mn = desc_lo(sbase + OFF_S, BOX_BYTES);
         if (GRP) {
           // scores of the raw q and k, both operands from shared memory as TMA delivered them; group A applies phi
           // only once this product is complete
@@ -531,7 +742,9 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
                      idesc(false, false, 128), ks > 0);
           mma_commit((bar0 + 8u * (B_MMA_P)));
         }
-        ok = mbar_wait((bar0 + 8u * (B_PHI)), par, abort);   // phi(Q) of tile n is in TMEM, phi(K) in place
+        // phi(Q) of tile n is in TMEM, phi(K) in place; the copy of S and z before tile n are complete (after n + 1 arrivals:
+        // from here on the update may change S)
+        ok = mbar_wait((bar0 + 8u * (B_PHI)), par, abort) && mbar_wait((bar0 + 8u * (B_SB)), par, abort);
         if (!ok) break;
         tc_fence_after();
         // The Q buffer has been read by then (phi(Q) lives in TMEM): its reload, which sets the pace, goes out first.
@@ -554,14 +767,13 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
 #pragma unroll
         for (int ks = 0; ks < 8; ++ks) {     // [S | z] += phi(K)^T [V | 1]
           const uint64_t kd = desc64(k_mn + kstep_mnmajor(ks));
-          mma_bf16(tmem + S_COL, kd, desc64(v_mn + kstep_mnmajor(ks)), idesc(true, true, 128), has_state || ks > 0);
-          mma_bf16(tmem + Z_COL, kd, desc_ext(sbase + OFF_ONES, ks), idesc(true, true, 16), has_state || ks > 0);
+          mma_bf16(tmem + S_COL, kd, desc64(v_mn + kstep_mnmajor(ks)), z3 ? idesc(true, true, 144) : idesc(true, true, 128),
+                   has_state || ks > 0);
+          if (!z3) mma_bf16(tmem + Z_COL, kd, desc_ext(sbase + OFF_ONES, ks), idesc(true, true, 16), has_state || ks > 0);
         }
-        mma_commit((bar0 + 8u * (B_MMA_S)));
-        // the bf16 copy of S before tile n is complete after n + 1 arrivals; the accumulator is free once the
-        // epilogue of tile n-1 has read it
-        ok = mbar_wait((bar0 + 8u * (B_SB)), par, abort);
-        if (ok && n >= 1) ok = mbar_wait((bar0 + 8u * (B_EPI0 + (par ^ 1))), ((n - 1) >> 1) & 1, abort);
+        mma_commit((bar0 + 8u * (par ? B_MMA_S1 : B_MMA_S0)));
+        // the accumulator is free once the epilogue of tile n-1 has read it
+        if (n >= 1) ok = mbar_wait((bar0 + 8u * (B_EPI0 + (par ^ 1))), ((n - 1) >> 1) & 1, abort);
         if (!ok) break;
         tc_fence_after();
         if (has_state && (!GRP || use_glob)) {
@@ -584,28 +796,17 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
       }
     }
   } else if (warp == kCopyWarp) {
-    // =============================== the first K loads, the V loads, output stores (one lane) ===============================
+    // =============================== V reloads and output stores (lane 0), K reloads (lane 1) ===============================
     // A lane of its own, so that waiting for a store to have read its buffer never holds up the issue of products.
     if (lane == 0) {
       bool ok = true;
-      for (int n = 0; n < 2 && n < nchunks; ++n) {
-        const uint32_t kb = sbase + (n ? OFF_K1 : OFF_K0), kbar = bar0 + 8u * (n ? B_FULL_K1 : B_FULL_K0);
-        mbar_expect_tx(kbar, tile_tx);
-        tma_load(kb, &mk, 0, y0 + n * tstep, bh, kbar);
-        tma_load(kb + KBOX_BYTES, &mk, 64, y0 + n * tstep, bh, kbar);
-      }
-      for (int n = 0; n < 2 && n < nchunks; ++n) {
-        mbar_expect_tx((bar0 + 8u * (B_FULL_V0 + n)), tile_tx);
-        tma_load(sbase + OFF_V0 + n * TILE_BYTES, &mv, 0, y0 + n * tstep, bh, (bar0 + 8u * (B_FULL_V0 + n)));
-        tma_load(sbase + OFF_V0 + n * TILE_BYTES + BOX_BYTES, &mv, 64, y0 + n * tstep, bh, (bar0 + 8u * (B_FULL_V0 + n)));
-      }
       for (int n = 0; n < nchunks; ++n) {
         const uint32_t par = n & 1;
         // the outputs of tile n are staged in its V buffer: store them; once they have been read the buffer takes
         // tile n+2
         ok = mbar_wait((bar0 + 8u * (B_STAGED0 + par)), (n >> 1) & 1, abort);
         if (!ok) break;
-        const uint32_t vb = sbase + OFF_V0 + par * TILE_BYTES;
+        const uint32_t vb = sbase + vbox(par, 0), vb1 = sbase + vbox(par, 1);
         if (LONG) {
           // the outputs wait in the token rows of this tile's K buffer; every tap has been taken from its V buffer
           const uint32_t kb = sbase + (par ? OFF_K1 : OFF_K0), kbar = bar0 + 8u * (par ? B_FULL_K1 : B_FULL_K0);
@@ -615,7 +816,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
           if (n + 2 < nchunks) {
             mbar_expect_tx((bar0 + 8u * (B_FULL_V0 + par)), tile_tx);
             tma_load(vb, &mv, 0, y0 + (n + 2) * tstep, bh, (bar0 + 8u * (B_FULL_V0 + par)));
-            tma_load(vb + BOX_BYTES, &mv, 64, y0 + (n + 2) * tstep, bh, (bar0 + 8u * (B_FULL_V0 + par)));
+            tma_load(vb1, &mv, 64, y0 + (n + 2) * tstep, bh, (bar0 + 8u * (B_FULL_V0 + par)));
             tma_wait_read();
             mbar_expect_tx(kbar, tile_tx);
             tma_load(kb, &mk, 0, y0 + (n + 2) * tstep, bh, kbar);
@@ -624,13 +825,13 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
           continue;
         }
         tma_store(&mo, 0, y0 + n * tstep, bh, vb);               // rows past the end of the sequence are clipped
-        tma_store(&mo, 64, y0 + n * tstep, bh, vb + BOX_BYTES);
+        tma_store(&mo, 64, y0 + n * tstep, bh, vb1);
         tma_commit();
         if (n + 2 < nchunks) {
           tma_wait_read();
           mbar_expect_tx((bar0 + 8u * (B_FULL_V0 + par)), tile_tx);
           tma_load(vb, &mv, 0, y0 + (n + 2) * tstep, bh, (bar0 + 8u * (B_FULL_V0 + par)));
-          tma_load(vb + BOX_BYTES, &mv, 64, y0 + (n + 2) * tstep, bh, (bar0 + 8u * (B_FULL_V0 + par)));
+          tma_load(vb1, &mv, 64, y0 + (n + 2) * tstep, bh, (bar0 + 8u * (B_FULL_V0 + par)));
         }
       }
       tma_wait_all();                             // every store is complete before the CTA exits
@@ -640,14 +841,45 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
       // should have to stand by for that moment.
       for (int n = 0; n + 2 < nchunks; ++n) {
         const uint32_t par = n & 1;
-        if (!mbar_wait((bar0 + 8u * (B_MMA_S)), par, abort)) break;
+        if (!mbar_wait((bar0 + 8u * (par ? B_MMA_S1 : B_MMA_S0)), (n >> 1) & 1, abort)) break;
         const uint32_t kbuf = sbase + (par ? OFF_K1 : OFF_K0), kbar = bar0 + 8u * (par ? B_FULL_K1 : B_FULL_K0);
         mbar_expect_tx(kbar, tile_tx);
         tma_load(kbuf, &mk, 0, y0 + (n + 2) * tstep, bh, kbar);
         tma_load(kbuf + KBOX_BYTES, &mk, 64, y0 + (n + 2) * tstep, bh, kbar);
       }
     }
-  } else if (warp >= 8) {
+  } else if (warp == kHaloWarp) {
+    // =============================== the rows of v before every 32 rows (short windows) ===============================
+    // The epilogue overwrites V with the outputs 32 rows at a time, without waiting for its other warps: what the taps of
+    // the next 32 rows (or of the next tile) reach back to is copied aside first.
+    if constexpr (WT > 1) {
+      bool ok = true;
+      for (int n = 0; n < nchunks; ++n) {
+        const uint32_t par = n & 1;
+        const int valid = min(tstep, T - n * tstep);
+        ok = ok && mbar_wait((bar0 + 8u * (B_FULL_V0 + par)), (n >> 1) & 1, abort);
+        ok = __all_sync(0xffffffffu, ok);
+        if (ok) {
+          unsigned char* hb = smem + off_halo(WT);
+          uint4 x[2 * (WT - 1)];
+#pragma unroll
+          for (int m = 0; m < 2 * (WT - 1); ++m) {          // piece lane & 15 of rows 2 m, 2 m + 1 of the 4 (W - 1)
+            const int j = 2 * m + (lane >> 4), blk = j / (WT - 1), i = j % (WT - 1);
+            const int row = (blk < 3 ? 32 * (blk + 1) : valid) - (WT - 1) + i;
+            x[m] = row >= 0 ? *reinterpret_cast<const uint4*>(smem + vbox(par, (lane & 15) >> 3) + swz(row, lane & 7))
+                            : *reinterpret_cast<const uint4*>(hb + (n % 3) * halo_bytes(WT) + halo_at(row + WT - 1, lane & 15, WT));
+          }
+#pragma unroll
+          for (int m = 0; m < 2 * (WT - 1); ++m) {
+            const int j = 2 * m + (lane >> 4), blk = j / (WT - 1), i = j % (WT - 1);
+            const int buf = blk < 3 ? 3 + 3 * (int)par + blk : (n + 1) % 3;
+            *reinterpret_cast<uint4*>(hb + buf * halo_bytes(WT) + halo_at(i, lane & 15, WT)) = x[m];
+          }
+        }
+        mbar_arrive((bar0 + 8u * (B_HALO0 + par)));
+      }
+    }
+  } else if (warp >= 8 && warp < 16) {
     // =============================== group A: phi, P, [S|z] snapshot (256 threads) ===============================
     const int ta = tid - kThreadsB;               // 0..255
     const int wa = warp - 8;                      // 0..7
@@ -655,59 +887,14 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
     const int hf = wa >> 2;                       // column half
     const uint32_t lane_addr = (uint32_t)(32 * (wa & 3)) << 16;
     unsigned char* Qb = smem + OFF_Q + hf * BOX_BYTES;
-    unsigned char* Sb = smem + OFF_S + hf * BOX_BYTES;
-    float* Sg = S + (size_t)u * D * D + (size_t)r * D + 64 * hf;
-    // Where the state after this unit goes: its own slot, or -- for the last segment of a chain that was cut -- the
-    // caller's state (the pre-pass does not visit last segments: nobody starts from their sums).
-    const bool to_caller = nseg > 1 && (u % nseg) == nseg - 1;
-    float* Sout = to_caller ? S_fin + (size_t)bh * D * D + (size_t)r * D + 64 * hf : Sg;
-    float* zout = to_caller ? z_fin + (size_t)bh * D : z + (size_t)u * D;
     bool ok = true;
 
-    if (init) {   // S -> TMEM (fp32) and bf16 copy in shared memory (z was copied during set-up)
-#pragma unroll
-      for (int qq = 0; qq < 2; ++qq) {
-        uint32_t v[32];
-#pragma unroll
-        for (int e = 0; e < 32; e += 4) {
-          const float4 x = *reinterpret_cast<const float4*>(Sg + 32 * qq + e);
-          v[e] = __float_as_uint(x.x); v[e + 1] = __float_as_uint(x.y);
-          v[e + 2] = __float_as_uint(x.z); v[e + 3] = __float_as_uint(x.w);
-        }
-        LA_TMEM_ST32(tmem + lane_addr + S_COL + 64 * hf + 32 * qq, v);
-#pragma unroll
-        for (int c = 0; c < 4; ++c) *reinterpret_cast<uint4*>(Sb + swz(r, 4 * qq + c)) = pack8(v + 8 * c);
-      }
-      if (hf == 0) {
-        tmem_st1(tmem + lane_addr + Z_COL, __float_as_uint(z[(size_t)u * D + r]));
-#pragma unroll
-        for (int c = 1; c < 16; ++c) tmem_st1(tmem + lane_addr + Z_COL + c, 0u);
-      }
-      tmem_wait_st();
-    }
-    fence_proxy_async();
-    tc_fence_before();
-    mbar_arrive((bar0 + 8u * (B_SB)));                       // phase 0: the state before tile 0 is in place
+    if (SNAP_A) mbar_arrive((bar0 + 8u * (B_SB)));           // phase 0: the state before tile 0 is in place
 
-    // phi on the K tile of tile m, in place; rows at or beyond the end of the sequence become zero
-    auto phi_k = [&](int m, bool go) {
-      if (!go) return;
-      const int valid = min(tstep, T - m * tstep);
-      const int ct = ta & 15, rg = ta >> 4;                     // chunk column 0..15, row group 0..15
-      unsigned char* Kb = smem + ((m & 1) ? OFF_K1 : OFF_K0) + (ct >> 3) * KBOX_BYTES;
-      uint4 x[8];                                               // all eight loads first: they do not wait for the stores
-#pragma unroll
-      for (int i = 0; i < 8; ++i) x[i] = *reinterpret_cast<const uint4*>(Kb + swz(rg + 16 * i, ct & 7));
-#pragma unroll
-      for (int i = 0; i < 8; ++i) {
-        const int j = rg + 16 * i;
-        *reinterpret_cast<uint4*>(Kb + swz(j, ct & 7)) = j < valid ? phi8<PHI>(x[i]) : make_uint4(0u, 0u, 0u, 0u);
-      }
-    };
     if (!GRP) {
       ok = mbar_wait((bar0 + 8u * (B_FULL_K0)), 0, abort);
       ok = __all_sync(0xffffffffu, ok);
-      phi_k(0, ok);
+      if (ok) phi_k(K0c{}, KAc{}, 0, ta);
     }
 
     for (int n = 0; n < nchunks; ++n) {
@@ -716,10 +903,10 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
 
       // ---- phi on Q in place (phi on K of this tile was done one iteration earlier) ----
       ok = ok && mbar_wait((bar0 + 8u * (B_FULL_Q)), par, abort);
+      if (GRP) ok = ok && mbar_wait((bar0 + 8u * (B_SB)), par, abort);       // z before tile n is in place
       ok = __all_sync(0xffffffffu, ok);
-      if (GRP) sync_group_a();                    // z of the previous snapshot (written by other threads) is in place
-      // phi(q) of row r, this thread's 64 channels: 32 packed pairs = 32 TMEM columns of lane r.  (The products of
-      // tile n-1 that read these columns are complete: the snapshot at the end of the previous iteration waited for them.)
+      if (GRP) sync_group_a();                    // every thread is done with the halves of the last tile (dgh, mlh)
+      // phi(q) of row r, this thread's 64 channels: 32 packed pairs = 32 TMEM columns of lane r.
       uint32_t fq[32];
       if (ok) {
 #pragma unroll
@@ -727,6 +914,13 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
           const uint4 f = phi8<PHI>(*reinterpret_cast<const uint4*>(Qb + swz(r, cc)));
           fq[4 * cc] = f.x; fq[4 * cc + 1] = f.y; fq[4 * cc + 2] = f.z; fq[4 * cc + 3] = f.w;
         }
+      }
+      if (!SNAP_A) {                              // the products of tile n-1 that read these columns are complete
+        if (n > 0) ok = ok && mbar_wait((bar0 + 8u * (B_MMA_Q)), par ^ 1, abort);
+        ok = __all_sync(0xffffffffu, ok);
+        tc_fence_after();
+      }
+      if (ok) {
         LA_TMEM_ST32(tmem + lane_addr + FQ_COL + 32 * hf, fq);
         if (GRP) {                                // this half of phi(q) . z_prev, z in fp32
           float dg = 0.f;
@@ -745,7 +939,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
         ok = ok && mbar_wait((bar0 + 8u * (par ? B_FULL_K1 : B_FULL_K0)), (n >> 1) & 1, abort) &&
              mbar_wait((bar0 + 8u * (B_MMA_P)), par, abort);
         ok = __all_sync(0xffffffffu, ok);
-        phi_k(n, ok);
+        if (ok) phi_k(K0c{}, K8c{}, n, ta);
       }
       fence_proxy_async();                        // (phi(K) of this tile, written one iteration earlier)
       tc_fence_before();
@@ -758,7 +952,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
       if (!GRP && !LONG && !last) {
         ok = ok && mbar_wait((bar0 + 8u * (((n + 1) & 1) ? B_FULL_K1 : B_FULL_K0)), ((n + 1) >> 1) & 1, abort);
         ok = __all_sync(0xffffffffu, ok);
-        phi_k(n + 1, ok);
+        if (ok) phi_k(K0c{}, KAc{}, n + 1, ta);
       }
 
       // ---- P: causal mask, packed bf16 -> TMEM ----
@@ -836,7 +1030,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
         const float m = fmaxf(m_run, oth.x);                    // finite: the row's own column lies in one of the halves
         const float l = l_run * ex2(m_run - m) + oth.y * ex2(oth.x - m);
         const float den = dgh[r] + dgh[D + r] + eps;
-        const bool has_g = use_glob && (init || n > 0) && den != 0.f;
+        const bool has_g = use_glob && (has_in || n > 0) && den != 0.f;
         const float rs = has_g ? den / alpha : 1.f;
         const float f = rs / l;
         if (ok) {
@@ -871,68 +1065,12 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
       if (!GRP && LONG && !last) {                // long-window epilogue: phi on K of the next tile after the mask
         ok = ok && mbar_wait((bar0 + 8u * (((n + 1) & 1) ? B_FULL_K1 : B_FULL_K0)), ((n + 1) >> 1) & 1, abort);
         ok = __all_sync(0xffffffffu, ok);
-        phi_k(n + 1, ok);
+        if (ok) phi_k(K0c{}, KAc{}, n + 1, ta);
       }
 
-      // ---- the rows of v before the next tile: the last W-1 of (halo ++ valid rows of this tile's V), 16 bytes per
-      //      thread, in the time this group would otherwise wait for the state update ----
-      if (HALO_A) {
-        ok = ok && mbar_wait((bar0 + 8u * (B_FULL_V0 + par)), (n >> 1) & 1, abort);
-        ok = __all_sync(0xffffffffu, ok);
-        if (ok) {
-          const int valid = min(tstep, T - n * tstep);
-          const __nv_bfloat16* halo = halo0 + (n % 3) * halo_elems;
-          __nv_bfloat16* halo_next = halo0 + ((n + 1) % 3) * halo_elems;
-          const unsigned char* Vt = smem + OFF_V0 + par * TILE_BYTES;
-          for (int idx = ta; idx < 16 * (W - 1); idx += kThreadsA) {
-            const int i = idx >> 4, c16 = idx & 15, src = valid + i;
-            uint4 x;
-            if (src < W - 1) x = *reinterpret_cast<const uint4*>(halo + src * D + 8 * c16);
-            else x = *reinterpret_cast<const uint4*>(Vt + (c16 >> 3) * BOX_BYTES + swz(src - (W - 1), c16 & 7));
-            *reinterpret_cast<uint4*>(halo_next + i * D + 8 * c16) = x;
-          }
-        }
-        mbar_arrive((bar0 + 8u * (B_HALO)));
-      }
-
-      // ---- S_n: bf16 copy for the next tile, or the final state to global memory ----
-      // S_n is final after MMA_S; the old copy may be overwritten once O = phi(Q) S_prev has read it
-      ok = ok && mbar_wait((bar0 + 8u * (B_MMA_S)), par, abort) && mbar_wait((bar0 + 8u * (B_MMA_Q)), par, abort);
-      ok = __all_sync(0xffffffffu, ok);
-      if (ok) {
-        tc_fence_after();
-        uint32_t zbits = 0u;
-        if (hf == 0) zbits = tmem_ld1(tmem + lane_addr + Z_COL);
-#pragma unroll
-        for (int qq = 0; qq < 2; ++qq) {
-          uint32_t v[32];
-          LA_TMEM_LD32(tmem + lane_addr + S_COL + 64 * hf + 32 * qq, v);
-          tmem_wait_ld();
-          if (last) {
-#pragma unroll
-            for (int e = 0; e < 32; e += 4)
-              *reinterpret_cast<float4*>(Sout + 32 * qq + e) =
-                  make_float4(__uint_as_float(v[e]), __uint_as_float(v[e + 1]), __uint_as_float(v[e + 2]),
-                              __uint_as_float(v[e + 3]));
-          } else {
-#pragma unroll
-            for (int c = 0; c < 4; ++c) *reinterpret_cast<uint4*>(Sb + swz(r, 4 * qq + c)) = pack8(v + 8 * c);
-          }
-        }
-        if (hf == 0) {
-          const float zz = __uint_as_float(zbits);
-          if (last) zout[r] = zz;
-          else if (GRP) zs[r] = zz;               // fp32, for phi(q) . z of the next tile
-          else                                    // row 128 of the K buffer of tile n+1 (its token rows are in place already)
-            *reinterpret_cast<__nv_bfloat16*>(smem + (((n + 1) & 1) ? OFF_K1 : OFF_K0) + (r >> 6) * KBOX_BYTES + BOX_BYTES +
-                                              (r & 63) * 2) = __float2bfloat16_rn(zz);
-        }
-      }
-      fence_proxy_async();
-      tc_fence_before();
-      mbar_arrive((bar0 + 8u * (B_SB)));
+      if (SNAP_A) snapshot(n, r, hf, lane_addr, ok);
     }
-  } else {
+  } else if (warp < 8) {
     // =============================== group B: epilogue (256 threads) ===============================
     const int r = 32 * (warp & 3) + lane;         // tile row = TMEM lane
     const int hf = warp >> 2;                     // column half
@@ -948,17 +1086,18 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
       // longer grows with rows x taps x 16 bytes, and the V buffer is never written.
       const int cp = tid & 63, jq = tid >> 6;
       const int cc = (cp & 31) >> 2;                                         // 16-byte piece of the pair in its box row
-      const uint32_t colv = (uint32_t)(cp >> 5) * BOX_BYTES + (uint32_t)(cp & 3) * 4u + (uint32_t)jq * 4096u;
+      const uint32_t colv = (uint32_t)(cp & 3) * 4u + (uint32_t)jq * 4096u;
       const uint32_t colk = (uint32_t)(cp >> 5) * KBOX_BYTES + (uint32_t)(cp & 3) * 4u + (uint32_t)jq * 4096u;
       const int lead = (int)long_taps(W) - W;                                // rows of zeros at the head of the halo
-      const uint32_t hcol = sbase + off_halo_long(W) + 4u * cp;
+      const uint32_t hcol = sbase + off_halo_long(W, GRP) + 4u * cp;
       const uint32_t hend = hcol + (long_taps(W) - 1) * (D * 2);
-      const uint32_t wcol = sbase + off_w() + 8u * cp;
+      const uint32_t wcol = sbase + off_w(z3) + 8u * cp;
       const int ngroups = (W + 7) >> 3;
       for (int n = 0; n < nchunks; ++n) {
         const uint32_t par = n & 1;
+        if (!early && n + 1 == nchunks) pdl_trigger();
         const int valid = min(tstep, T - n * tstep);
-        const uint32_t vthr = sbase + OFF_V0 + par * TILE_BYTES + colv;       // this thread's column at its first row
+        const uint32_t vthr = sbase + vbox(par, cp >> 5) + colv;       // this thread's column at its first row
         unsigned char* stage = smem + (par ? OFF_K1 : OFF_K0);
         ok = ok && mbar_wait((bar0 + 8u * (B_MMA_O0 + par)), (n >> 1) & 1, abort);   // also: every product that reads K or V is done
         ok = __all_sync(0xffffffffu, ok);
@@ -1022,95 +1161,108 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
         mbar_arrive((bar0 + 8u * (B_STAGED0 + par)));
       }
     } else
+    {
+    // 32 rows x 64 channels per warp, as 8 x 8 fragments: a lane holds two channels of rows l >> 2, + 8, + 16, + 24 per
+    // fragment column, so that one 8-byte load of a tap serves eight multiply-adds (with a row per lane every tap was
+    // loaded for two).  ldmatrix brings v of row r - t for all rows at once; the outputs take the place of the V rows,
+    // which no other warp reads (the halo buffers hold what reaches across), so that no barrier is needed.
+    constexpr int WN = WT > 0 ? WT : 1;
+    const int q4 = warp & 3;
+    const uint32_t waddr = sbase + off_w(true) + 4u * (64 * hf + 2 * (lane & 3));
+    if (KB > 0) {                                 // this group's share of the first K tile
+      ok = mbar_wait((bar0 + 8u * (B_FULL_K0)), 0, abort);
+      ok = __all_sync(0xffffffffu, ok);
+      if (ok) phi_k(KAc{}, K8c{}, 0, tid);
+      fence_proxy_async();
+    }
+    if (!SNAP_A) mbar_arrive((bar0 + 8u * (B_SB)));  // phase 0: the state before tile 0 is in place
     for (int n = 0; n < nchunks; ++n) {
       const uint32_t par = n & 1;
       const int valid = min(tstep, T - n * tstep);
-      const unsigned char* Vt = smem + OFF_V0 + par * TILE_BYTES;
-      // rows before this tile, addressed so that row -1 is the last of W-1 rows
-      const __nv_bfloat16* halo = halo0 + (HALO_A ? n % 3 : (int)par) * halo_elems;
-      __nv_bfloat16* halo_next = halo0 + (par ^ 1) * halo_elems;    // rows before the next tile
-      ok = ok && mbar_wait((bar0 + 8u * (B_FULL_V0 + par)), (n >> 1) & 1, abort);
-      // (HALO_A: group A has read the last rows of this tile's V, and with that filled the halo of the tile before)
-      if (HALO_A) ok = ok && mbar_wait((bar0 + 8u * (B_HALO)), par, abort);
-      ok = __all_sync(0xffffffffu, ok);
-      if (ok && !HALO_A) {
-        // next halo <- last W-1 rows of (halo ++ valid rows of V), 16 bytes (8 channels) per thread; each half of the
-        // group copies its own 64 channels
-        const unsigned char* Vc = Vt + hf * BOX_BYTES;
-        for (int idx = tid & 127; idx < 8 * (W - 1); idx += 128) {
-          const int i = idx >> 3, c8 = idx & 7, src = valid + i;
-          uint4 x;
-          if (src < W - 1) x = *reinterpret_cast<const uint4*>(halo + src * D + 64 * hf + 8 * c8);
-          else x = *reinterpret_cast<const uint4*>(Vc + swz(src - (W - 1), c8));
-          *reinterpret_cast<uint4*>(halo_next + i * D + 64 * hf + 8 * c8) = x;
-        }
+      if (!early && n + 1 == nchunks) pdl_trigger();
+      if (KB > 0 && n + 1 < nchunks) {            // (announced, like the state, by the arrival in snapshot)
+        ok = ok && mbar_wait((bar0 + 8u * (((n + 1) & 1) ? B_FULL_K1 : B_FULL_K0)), ((n + 1) >> 1) & 1, abort);
+        ok = __all_sync(0xffffffffu, ok);
+        if (ok) phi_k(KAc{}, K8c{}, n + 1, tid);
       }
+      if (!SNAP_A) snapshot(n, r, hf, lane_addr, ok);
+      uint32_t vrow[WN];                          // row lane - t of the warp's 32: this lane's address for ldmatrix, chunk 0
+      {
+        const uint32_t vb = sbase + vbox(par, hf) + 4096u * q4;
+        const uint32_t he = sbase + off_halo(WN) + (q4 == 0 ? n % 3 : 2 + 3 * par + q4) * halo_bytes(WN) + (hf + 1) * (WN - 1) * 128u;
+#pragma unroll
+        for (int t = 0; t < WN; ++t) vrow[t] = (lane >= t ? vb : he) + (uint32_t)((lane - t) * 128) + (uint32_t)(((lane - t) & 7) << 4);
+      }
+      ok = ok && mbar_wait((bar0 + 8u * (B_FULL_V0 + par)), (n >> 1) & 1, abort);
+      if (WN > 1) ok = ok && mbar_wait((bar0 + 8u * (B_HALO0 + par)), (n >> 1) & 1, abort);
       ok = ok && mbar_wait((bar0 + 8u * (B_MMA_O0 + par)), (n >> 1) & 1, abort);   // also: every product that reads V is done
       ok = __all_sync(0xffffffffu, ok);
-      // The outputs leave through the V buffer of this tile, 16-byte column by column: a column is overwritten (same
-      // swizzled layout) once every thread of this half has taken its taps from it, so that a thread holds one
-      // column of outputs at a time; the control lane then stores whole rows with one TMA store per box.  The two
-      // halves of the group (64 channels each) share nothing and synchronise separately.
-      // The accumulator is read 32 columns at a time; each load is issued as early as its registers are free, so
-      // that its latency passes behind the barrier and the arithmetic in between.
-      uint32_t v[32];
       if (ok) {
         tc_fence_after();
-        LA_TMEM_LD32(tmem + lane_addr + O_COL + 64 * hf, v);
-      }
-      if (!HALO_A) sync_half_b(hf);               // the next halo is complete before any row of V is overwritten
-      float rden = 0.f;
-      if (ok) {
-        // row sum of the masked P + phi(q) . z_prev, both halves gathered by the masking threads
-        const float den = denbuf[(par * 2) * D + r] + denbuf[(par * 2 + 1) * D + r];
-        rden = 1.f / (den + (GRP ? 0.f : eps));   // (three-branch mode: the masking threads left the finished factor)
-      }
-      unsigned char* Ob = smem + OFF_V0 + par * TILE_BYTES + hf * BOX_BYTES;
+        const uint32_t oaddr = tmem + lane_addr + O_COL + 64 * hf;
+        uint32_t a0[16], a1[16];                  // rows 0-15 and 16-31
+        LA_TMEM_LD_FRAG4(oaddr, a0);
+        LA_TMEM_LD_FRAG4(oaddr + (16u << 16), a1);
+        float rden[4];
 #pragma unroll
-      for (int qq = 0; qq < 2; ++qq) {
-        if (ok) tmem_wait_ld();
-        if (qq == 1) {
-          tc_fence_before();
-          mbar_arrive((bar0 + 8u * (B_EPI0 + par)));         // this accumulator has been read
+        for (int m = 0; m < 4; ++m) {
+          // row sum of the masked P + phi(q) . z_prev, both halves gathered by the masking threads
+          const float* dr = denbuf + par * 2 * D + 32 * q4 + (lane >> 2) + 8 * m;
+          rden[m] = 1.f / (dr[0] + dr[D] + (GRP ? 0.f : eps));  // (three-branch mode: those left the finished factor)
         }
 #pragma unroll
-        for (int c2 = 0; c2 < 2; ++c2) {          // two columns per barrier
-          uint4 outp[2];
+        for (int qq = 0; qq < 2; ++qq) {
+          tmem_wait_ld();
 #pragma unroll
-          for (int j = 0; j < 2; ++j) {
-            const int c = 2 * c2 + j;
-            const int cc = 4 * qq + c;                          // chunk inside this half's box
-            const int ch0 = 64 * hf + 8 * cc;                   // first channel of the chunk
-            outp[j] = make_uint4(0u, 0u, 0u, 0u);
-            if (ok && r < valid) {                              // rows past the tile's tokens stage zeros
-              float2 acc[4];
+          for (int g = 0; g < 4; ++g) {
+            const int cc = 4 * qq + g;
+            float2 acc[4];
 #pragma unroll
-              for (int e = 0; e < 4; ++e)
-                acc[e] = __fmul2_rn(make_float2(__uint_as_float(v[8 * c + 2 * e]), __uint_as_float(v[8 * c + 2 * e + 1])),
-                                    make_float2(rden, rden));
-              conv8<WT>(acc, W, r, cc, ch0, Vt + hf * BOX_BYTES, halo, wsm);
-              outp[j] = make_uint4(pack2(acc[0].x, acc[0].y), pack2(acc[1].x, acc[1].y), pack2(acc[2].x, acc[2].y),
-                                   pack2(acc[3].x, acc[3].y));
+            for (int m = 0; m < 4; ++m) {
+              const uint32_t* src = (m < 2 ? a0 : a1) + 4 * g + 2 * (m & 1);
+              acc[m] = __fmul2_rn(make_float2(__uint_as_float(src[0]), __uint_as_float(src[1])), make_float2(rden[m], rden[m]));
             }
-          }
-          if (qq == 0 && c2 == 1 && ok)           // the first 32 columns have been used: fetch the other 32
-            LA_TMEM_LD32(tmem + lane_addr + O_COL + 64 * hf + 32, v);
-          sync_half_b(hf);                        // these two columns of this half have been read by all of its rows
-          if (ok) {
 #pragma unroll
-            for (int j = 0; j < 2; ++j) *reinterpret_cast<uint4*>(Ob + swz(r, 4 * qq + 2 * c2 + j)) = outp[j];
+            for (int t = 0; t < WN; ++t) {
+              uint32_t u[4];
+              ldmatrix4(vrow[t] ^ (uint32_t)(cc << 4), u);
+              const float2 wt = lds_f2(waddr + t * (D * 4) + cc * 32);
+#pragma unroll
+              for (int m = 0; m < 4; ++m) acc[m] = __ffma2_rn(wt, bf2(u[m]), acc[m]);
+            }
+            uint32_t out[4];
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+              out[m] = pack2(acc[m].x, acc[m].y);
+              // a partly filled tile stays zero below its tokens
+              if (GRP && 32 * q4 + (lane >> 2) + 8 * m >= valid) out[m] = 0u;
+            }
+            stmatrix4(vrow[0] ^ (uint32_t)(cc << 4), out);
+          }
+          if (qq == 0) {
+            LA_TMEM_LD_FRAG4(oaddr + 32, a0);
+            LA_TMEM_LD_FRAG4(oaddr + 32 + (16u << 16), a1);
+            tmem_wait_ld();
+            tc_fence_before();
+            mbar_arrive((bar0 + 8u * (B_EPI0 + par)));         // this accumulator has been read
           }
         }
+      } else {
+        mbar_arrive((bar0 + 8u * (B_EPI0 + par)));
       }
       fence_proxy_async();
       mbar_arrive((bar0 + 8u * (B_STAGED0 + par)));
     }
+    }
     sync_group_b();                               // both halves of the last halo are complete
-    if (ok && tid < D) {
-      // the window to carry on: the last W-1 values of (incoming window ++ this unit's v)
-      const __nv_bfloat16* halo = halo0 + (LONG ? ((int)long_taps(W) - W) * D : (HALO_A ? nchunks % 3 : nchunks & 1) * halo_elems);
-      for (int i = 0; i < W - 1; ++i) win[((size_t)u * (W - 1) + i) * D + tid] = halo[i * D + tid];
-      if (tid == 0 && h == 0 && nseg == 1) pos[bh / H] = (init ? pos[bh / H] : 0) + T;
+    if (ok && tid < D && writes_state) {
+      // the window to carry on: the last W-1 values of (incoming window ++ this block's v)
+      const unsigned char* halo = smem + off_halo(W) + nchunks % 3 * halo_bytes(W);
+      for (int i = 0; i < W - 1; ++i)
+        win[((size_t)bh * (W - 1) + i) * D + tid] =
+            LONG ? halo0[((int)long_taps(W) - W + i) * D + tid]
+                 : *reinterpret_cast<const __nv_bfloat16*>(halo + halo_at(i, tid >> 3, W) + (tid & 7) * 2);
+      if (tid == 0 && h == 0) pos[bh / H] = (init ? pos[bh / H] : 0) + Ttot;
     }
   }
 
@@ -1131,10 +1283,14 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
 // ---- sequence split: local state of a segment ------------------------------------------------------
 // For chains too few to fill the GPU the sequence is cut into segments that run as separate CTAs.  This
 // kernel computes, for one segment, only its own contribution [dS | dz] = sum phi(k) [v | 1]^T (K and V are
-// read, phi applied to K, one product per tile) and stores it in fp32.  A prefix sum over the segments
-// (prefix_kernel) turns the contributions into the state each segment starts from.
+// read, phi applied to K, one product per tile) and stores it in fp32.  In the main pass every segment adds up the
+// contributions of those before it.
 constexpr int kStateThreads = 288;       // 8 compute warps + 1 issue warp
-constexpr uint32_t ST_OFF_K = 0, ST_OFF_V = 2 * TILE_BYTES, ST_OFF_ONES = 4 * TILE_BYTES, ST_OFF_SMALL = ST_OFF_ONES + 4096;
+// (K buffer 1, then V buffer 1 around K buffer 0, V buffer 0 and the ones, which are the third box of both V buffers as
+// in the main kernel)
+constexpr uint32_t ST_OFF_VQ = TILE_BYTES, ST_OFF_ONES = ST_OFF_VQ + 6 * BOX_BYTES, ST_OFF_SMALL = ST_OFF_ONES + BOX_BYTES;
+__host__ __device__ constexpr uint32_t st_kbuf(uint32_t b) { return b ? 0u : ST_OFF_VQ + BOX_BYTES; }
+__host__ __device__ constexpr uint32_t st_vbox(uint32_t b, uint32_t half) { return ST_OFF_VQ + (b ? 0u : 4 * BOX_BYTES) + half * vstep(b); }
 constexpr uint32_t kStateSmem = ST_OFF_SMALL + 256 + 1024;
 enum { SB_FULL_K0 = 0, SB_FULL_K1, SB_FULL_V0, SB_FULL_V1, SB_PHI, SB_MMA, kStateBars };
 
@@ -1142,7 +1298,8 @@ template <int PHI>
 __global__ void __launch_bounds__(kStateThreads, 1)
 segment_state_kernel(const __grid_constant__ CUtensorMap mk, const __grid_constant__ CUtensorMap mv,
                      float* __restrict__ S_out, float* __restrict__ z_out, int* status, int Ttot, int nseg,
-                     int seg_len, int nrun) {
+                     int seg_len, int nrun, int init, const float* __restrict__ S, const float* __restrict__ z,
+                     const __nv_bfloat16* __restrict__ win, __nv_bfloat16* __restrict__ win_copy, int W) {
   extern __shared__ unsigned char smem_dyn[];
   // (an offset into the array rather than an integer cast: the compiler then knows that these are shared-memory
   // addresses: 32-bit arithmetic, ld.shared / st.shared)
@@ -1171,10 +1328,12 @@ segment_state_kernel(const __grid_constant__ CUtensorMap mk, const __grid_consta
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  for (int idx = tid; idx < 4096 / 16; idx += kStateThreads)
+  for (int idx = tid; idx < (int)BOX_BYTES / 16; idx += kStateThreads)
     reinterpret_cast<uint4*>(smem + ST_OFF_ONES)[idx] = make_uint4(0u, 0u, 0u, 0u);
+  pdl_wait();                                     // everything above touched shared memory and TMEM only
+  pdl_trigger();
   __syncthreads();
-  if (tid < TILE) *reinterpret_cast<__nv_bfloat16*>(smem + ST_OFF_ONES + ext_offset(tid, 0)) = __float2bfloat16_rn(1.f);
+  if (tid < TILE) *reinterpret_cast<__nv_bfloat16*>(smem + ST_OFF_ONES + swz(tid, 0)) = __float2bfloat16_rn(1.f);
   fence_proxy_async();
   tc_fence_before();
   __syncthreads();
@@ -1187,23 +1346,22 @@ segment_state_kernel(const __grid_constant__ CUtensorMap mk, const __grid_consta
       auto load_tile = [&](int n) {
         const uint32_t b2 = n & 1;
         mbar_expect_tx((bar0 + 8u * (SB_FULL_K0 + b2)), TILE_BYTES);
-        tma_load(sbase + ST_OFF_K + b2 * TILE_BYTES, &mk, 0, y0 + n * TILE, bh, (bar0 + 8u * (SB_FULL_K0 + b2)));
-        tma_load(sbase + ST_OFF_K + b2 * TILE_BYTES + BOX_BYTES, &mk, 64, y0 + n * TILE, bh, (bar0 + 8u * (SB_FULL_K0 + b2)));
+        tma_load(sbase + st_kbuf(b2), &mk, 0, y0 + n * TILE, bh, (bar0 + 8u * (SB_FULL_K0 + b2)));
+        tma_load(sbase + st_kbuf(b2) + BOX_BYTES, &mk, 64, y0 + n * TILE, bh, (bar0 + 8u * (SB_FULL_K0 + b2)));
         mbar_expect_tx((bar0 + 8u * (SB_FULL_V0 + b2)), TILE_BYTES);
-        tma_load(sbase + ST_OFF_V + b2 * TILE_BYTES, &mv, 0, y0 + n * TILE, bh, (bar0 + 8u * (SB_FULL_V0 + b2)));
-        tma_load(sbase + ST_OFF_V + b2 * TILE_BYTES + BOX_BYTES, &mv, 64, y0 + n * TILE, bh, (bar0 + 8u * (SB_FULL_V0 + b2)));
+        tma_load(sbase + st_vbox(b2, 0), &mv, 0, y0 + n * TILE, bh, (bar0 + 8u * (SB_FULL_V0 + b2)));
+        tma_load(sbase + st_vbox(b2, 1), &mv, 64, y0 + n * TILE, bh, (bar0 + 8u * (SB_FULL_V0 + b2)));
       };
       for (int n = 0; n < 2 && n < nchunks; ++n) load_tile(n);
       for (int n = 0; n < nchunks; ++n) {
         const uint32_t b2 = n & 1;
         if (!mbar_wait((bar0 + 8u * (SB_PHI)), n & 1, abort) || !mbar_wait((bar0 + 8u * (SB_FULL_V0 + b2)), (n >> 1) & 1, abort)) break;
         tc_fence_after();
+        const uint32_t k_mn = desc_lo(sbase + st_kbuf(b2), BOX_BYTES), v_mn = desc_lo(sbase + st_vbox(b2, 0), vstep(b2));
 #pragma unroll
-        for (int ks = 0; ks < 8; ++ks) {     // [dS | dz] += phi(K)^T [V | 1]
-          const uint64_t kd = desc_mnmajor(sbase + ST_OFF_K + b2 * TILE_BYTES, ks);
-          mma_bf16(tmem + SCOL, kd, desc_mnmajor(sbase + ST_OFF_V + b2 * TILE_BYTES, ks), idesc(true, true, 128), n > 0 || ks > 0);
-          mma_bf16(tmem + ZCOL, kd, desc_ext(sbase + ST_OFF_ONES, ks), idesc(true, true, 16), n > 0 || ks > 0);
-        }
+        for (int ks = 0; ks < 8; ++ks)       // [dS | dz] += phi(K)^T [V | 1]
+          mma_bf16(tmem + SCOL, desc64(k_mn + kstep_mnmajor(ks)), desc64(v_mn + kstep_mnmajor(ks)), idesc(true, true, 144),
+                   n > 0 || ks > 0);
         mma_commit((bar0 + 8u * (SB_MMA)));
         if (!mbar_wait((bar0 + 8u * (SB_MMA)), n & 1, abort)) break;       // both buffers of this tile are free
         if (n + 2 < nchunks) load_tile(n + 2);
@@ -1217,7 +1375,7 @@ segment_state_kernel(const __grid_constant__ CUtensorMap mk, const __grid_consta
       ok = __all_sync(0xffffffffu, ok);
       if (ok) {
         const int ct = tid & 15, rg = tid >> 4;
-        unsigned char* Kb = smem + ST_OFF_K + (n & 1) * TILE_BYTES + (ct >> 3) * BOX_BYTES;
+        unsigned char* Kb = smem + st_kbuf(n & 1) + (ct >> 3) * BOX_BYTES;
         uint4 x[8];                                             // all eight loads first: they do not wait for the stores
 #pragma unroll
         for (int i = 0; i < 8; ++i) x[i] = *reinterpret_cast<const uint4*>(Kb + swz(rg + 16 * i, ct & 7));
@@ -1238,22 +1396,37 @@ segment_state_kernel(const __grid_constant__ CUtensorMap mk, const __grid_consta
       tc_fence_after();
       const int r = 32 * (warp & 3) + lane, hf = warp >> 2;
       const uint32_t lane_addr = (uint32_t)(32 * (warp & 3)) << 16;
-      float* Sg = S_out + (size_t)u * D * D + (size_t)r * D + 64 * hf;
+      // Where the chain continues a state, its first segment adds that state to its sums and leaves a copy (with the
+      // window) for the main pass, whose last segments overwrite the caller's.
+      const bool base = init && sg == 0;
+      const size_t copy = (size_t)bh * nseg + nseg - 1;
+      const size_t at = (size_t)(32 * (warp & 3) + (lane >> 2)) * D + 64 * hf + 2 * (lane & 3);
 #pragma unroll
-      for (int qq = 0; qq < 2; ++qq) {
-        uint32_t v[32];
-        LA_TMEM_LD32(tmem + lane_addr + SCOL + 64 * hf + 32 * qq, v);
+      for (int i = 0; i < 2; ++i) {                 // rows 16 i ... 16 i + 15 of this warp's 32
+        uint32_t v[32], x[32];
+        if (base) frag_load(S + (size_t)bh * D * D + at + 16 * i * D, x);
+        LA_TMEM_LD_FRAG8(tmem + lane_addr + ((uint32_t)(16 * i) << 16) + SCOL + 64 * hf, v);
         tmem_wait_ld();
-#pragma unroll
-        for (int e = 0; e < 32; e += 4)
-          *reinterpret_cast<float4*>(Sg + 32 * qq + e) = make_float4(__uint_as_float(v[e]), __uint_as_float(v[e + 1]),
-                                                                     __uint_as_float(v[e + 2]), __uint_as_float(v[e + 3]));
+        if (base) {
+          frag_store(S_out + copy * D * D + at + 16 * i * D, x);
+          frag_add(v, x);
+        }
+        frag_store(S_out + (size_t)u * D * D + at + 16 * i * D, v);
       }
       if (hf == 0) {
         const uint32_t zz = tmem_ld1(tmem + lane_addr + ZCOL);
         tmem_wait_ld();
-        z_out[(size_t)u * D + r] = __uint_as_float(zz);
+        float x = __uint_as_float(zz);
+        if (base) {
+          const float c = z[(size_t)bh * D + r];
+          z_out[copy * D + r] = c;
+          x += c;
+        }
+        z_out[(size_t)u * D + r] = x;
       }
+      if (base)
+        for (int idx = tid; idx < (W - 1) * D; idx += 256)
+          win_copy[(size_t)bh * (W - 1) * D + idx] = win[(size_t)bh * (W - 1) * D + idx];
     }
   }
   tc_fence_before();
@@ -1269,61 +1442,40 @@ segment_state_kernel(const __grid_constant__ CUtensorMap mk, const __grid_consta
   }
 }
 
-// Exclusive prefix over the segments of one chain, in place: on return S_seg[bh][s] / z_seg[bh][s] hold the state
-// segment s starts from and win_seg its incoming window; win / pos of the caller get their final values here, S / z
-// of the caller are written by the last segment's block of the main pass (the sums of last segments are not
-// computed beforehand, so their slots are not read).
-// grid = (BH, d*d / 1024), 256 threads, four consecutive elements of S per thread.
+// The sums of the segments 0 ... s of a chain into slot s, in place (s < nseg - 1).
+// grid = (BH, d*d / 1024), 256 threads, four consecutive elements of S per thread; loads in batches of sixteen slots, all
+// in flight at once, only the additions are sequential.
 __global__ void __launch_bounds__(256)
-prefix_kernel(float* __restrict__ S_seg, float* __restrict__ z_seg, __nv_bfloat16* __restrict__ win_seg,
-              const __nv_bfloat16* __restrict__ v, float* __restrict__ S, float* __restrict__ z,
-              __nv_bfloat16* __restrict__ win, int64_t* __restrict__ pos, int H, int Ttot, int W, int nseg, int seg_len,
-              int init) {
+prefix_kernel(float* __restrict__ S_seg, float* __restrict__ z_seg, int nseg) {
   const int bh = blockIdx.x, e4 = (blockIdx.y * 256 + threadIdx.x) * 4;
-  // Loads in batches of sixteen segments, all in flight at once; only the additions are sequential.
-  float4 run = init ? *reinterpret_cast<const float4*>(S + (size_t)bh * D * D + e4) : make_float4(0.f, 0.f, 0.f, 0.f);
-  for (int sg0 = 0; sg0 < nseg; sg0 += 16) {
+  pdl_wait();
+  pdl_trigger();
+  float* Sp = S_seg + (size_t)bh * nseg * D * D + e4;
+  float4 run = make_float4(0.f, 0.f, 0.f, 0.f);
+  for (int s0 = 0; s0 < nseg - 1; s0 += 16) {
     float4 d[16];
 #pragma unroll
     for (int j = 0; j < 16; ++j)
-      if (sg0 + j < nseg - 1) d[j] = *reinterpret_cast<const float4*>(S_seg + ((size_t)bh * nseg + sg0 + j) * D * D + e4);
+      if (s0 + j < nseg - 1) d[j] = *reinterpret_cast<const float4*>(Sp + (size_t)(s0 + j) * D * D);
 #pragma unroll
     for (int j = 0; j < 16; ++j)
-      if (sg0 + j < nseg) {
-        *reinterpret_cast<float4*>(S_seg + ((size_t)bh * nseg + sg0 + j) * D * D + e4) = run;
-        if (sg0 + j < nseg - 1) { run.x += d[j].x; run.y += d[j].y; run.z += d[j].z; run.w += d[j].w; }
+      if (s0 + j < nseg - 1) {
+        run.x += d[j].x, run.y += d[j].y, run.z += d[j].z, run.w += d[j].w;
+        *reinterpret_cast<float4*>(Sp + (size_t)(s0 + j) * D * D) = run;
       }
   }
   if (blockIdx.y == 0 && threadIdx.x < D) {
-    const int c = threadIdx.x;
-    float rz = init ? z[(size_t)bh * D + c] : 0.f;
-    for (int sg0 = 0; sg0 < nseg; sg0 += 8) {
-      float d[8];
+    float* zp = z_seg + (size_t)bh * nseg * D + threadIdx.x;
+    float rz = 0.f;
+    for (int s0 = 0; s0 < nseg - 1; s0 += 16) {
+      float d[16];
 #pragma unroll
-      for (int j = 0; j < 8; ++j)
-        if (sg0 + j < nseg - 1) d[j] = z_seg[((size_t)bh * nseg + sg0 + j) * D + c];
+      for (int j = 0; j < 16; ++j)
+        if (s0 + j < nseg - 1) d[j] = zp[(size_t)(s0 + j) * D];
 #pragma unroll
-      for (int j = 0; j < 8; ++j)
-        if (sg0 + j < nseg) {
-          z_seg[((size_t)bh * nseg + sg0 + j) * D + c] = rz;
-          if (sg0 + j < nseg - 1) rz += d[j];
-        }
+      for (int j = 0; j < 16; ++j)
+        if (s0 + j < nseg - 1) zp[(size_t)(s0 + j) * D] = rz += d[j];
     }
-    if (c == 0 && bh % H == 0) pos[bh / H] = (init ? pos[bh / H] : 0) + Ttot;
-  }
-  // Incoming windows: the W-1 values of v before each segment; before the first one the caller's window or zeros.
-  // One element per thread over all blocks of this chain.  The thread that reads the caller's window entry (i, c)
-  // is also the one that overwrites it with the final window: the last W-1 values of v (Ttot >= W-1 whenever the
-  // split is used).
-  const int per_chain = nseg * (W - 1) * D;
-  for (int idx = blockIdx.y * 256 + threadIdx.x; idx < per_chain; idx += gridDim.y * 256) {
-    const int c = idx % D, i = (idx / D) % (W - 1), sg = idx / (D * (W - 1));
-    const int t = sg * seg_len - (W - 1) + i;
-    __nv_bfloat16 x = __float2bfloat16_rn(0.f);
-    if (t >= 0) x = v[((size_t)bh * Ttot + t) * D + c];
-    else if (init) x = win[((size_t)bh * (W - 1) + i) * D + c];          // sg == 0: t = i - (W-1)
-    win_seg[(((size_t)bh * nseg + sg) * (W - 1) + i) * D + c] = x;
-    if (sg == 0) win[((size_t)bh * (W - 1) + i) * D + c] = v[((size_t)bh * Ttot + Ttot - (W - 1) + i) * D + c];
   }
 }
 
@@ -1360,16 +1512,23 @@ static bool make_map(CUtensorMap* m, const void* base, int BH, int T, int box_ro
 
 }  // namespace tc
 
+// What the chains of a launch start from and how they are cut (one piece per chain: everything null).
+struct Split {
+  int nseg = 1, seg_len = 0;
+  const float *S = nullptr, *z = nullptr;
+  const __nv_bfloat16* win = nullptr;
+  int prefixed = 0;
+};
+
 template <int PHI>
-static cudaError_t launch_w(const la_config& c, int units, int T, const CUtensorMap& mq, const CUtensorMap& mk,
-                            const CUtensorMap& mv, const CUtensorMap& mo, const float* w, int init, float* S, float* z,
-                            __nv_bfloat16* win, int64_t* pos, int* status, int nseg, int seg_len,
-                            float* S_fin, float* z_fin, cudaStream_t s, bool grouped = false, float alpha = 1.f,
-                            float sm_scale = 1.f, int tstep = tc::TILE) {
+static cudaError_t launch_w(la_ctx* ctx, int BH, int T, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
+                            const CUtensorMap& mo, const void* v, const float* w, int init, const la_state& st,
+                            const Split& sp, cudaStream_t s, bool grouped = false, float alpha = 1.f, float sm_scale = 1.f,
+                            int tstep = tc::TILE) {
+  const la_config& c = ctx->cfg;
   const bool lng = tc::long_epilogue(c.conv_taps, grouped);
-  const size_t smem = grouped ? tc::smem_bytes_grp(c.conv_taps, lng) : lng ? tc::smem_bytes_long(c.conv_taps) : tc::smem_bytes(c.conv_taps);
-  void (*kern)(CUtensorMap, CUtensorMap, CUtensorMap, CUtensorMap, const float*, float*, float*, __nv_bfloat16*, int64_t*,
-               int*, int, int, int, float, int, int, int, float*, float*, float, float, int);
+  const size_t smem = grouped ? tc::smem_bytes_grp(c.conv_taps, lng) : lng ? tc::smem_bytes_long(c.conv_taps, false) : tc::smem_bytes(c.conv_taps);
+  auto kern = tc::prefill_tc_kernel<PHI, 3>;
   if (grouped) {
     kern = lng ? tc::prefill_tc_kernel<PHI, -1, true> : tc::prefill_tc_kernel<PHI, 3, true>;
   } else
@@ -1381,32 +1540,51 @@ static cudaError_t launch_w(const la_config& c, int units, int T, const CUtensor
     case 5: kern = tc::prefill_tc_kernel<PHI, 5>; break;
     default: kern = tc::prefill_tc_kernel<PHI, -1>; break;
   }
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem((const void*)kern, ctx->device);
   if (e != cudaSuccess) return e;
-  kern<<<dim3(units), dim3(tc::kThreads), smem, s>>>(mq, mk, mv, mo, w, S, z, win, pos, status, c.H, T,
-                                                     c.conv_taps, c.eps, init, nseg, seg_len, S_fin, z_fin, alpha, sm_scale, tstep);
-  return cudaGetLastError();
+  ctx->launches += 1;
+  const int units = BH * sp.nseg;
+  // Programmatic dependent launch where this launch and the one behind it fit on the SMs together (that one's set-up then
+  // runs beside this one's tiles), and behind the pre-pass.  Not for fuller grids: the blocks that start early take the
+  // SMs that the launch before left idle (128 chains of 2048 tokens, 3 taps: 70 against 65 us).
+  const int early = 2 * units <= ctx->sm_count;
+  return launch_maybe_pdl(early || sp.nseg > 1, kern, dim3(units), dim3(tc::kThreads), smem, s, mq, mk, mv, mo, w, st.S, st.z,
+                          (__nv_bfloat16*)st.win, st.pos, ctx->d_status, c.H, T, c.conv_taps, c.eps, init, sp.nseg,
+                          sp.nseg > 1 ? sp.seg_len : T, sp.S, sp.z, sp.win, sp.prefixed, (const __nv_bfloat16*)v, alpha,
+                          sm_scale, tstep, early);
+}
+static cudaError_t launch_phi(la_ctx* ctx, int BH, int T, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
+                              const CUtensorMap& mo, const void* v, const float* w, int init, const la_state& st,
+                              const Split& sp, cudaStream_t s, bool grouped = false, float alpha = 1.f, float sm_scale = 1.f,
+                              int tstep = tc::TILE) {
+  return ctx->cfg.phi == LA_PHI_ELU1
+             ? launch_w<LA_PHI_ELU1>(ctx, BH, T, mq, mk, mv, mo, v, w, init, st, sp, s, grouped, alpha, sm_scale, tstep)
+             : launch_w<LA_PHI_RELU>(ctx, BH, T, mq, mk, mv, mo, v, w, init, st, sp, s, grouped, alpha, sm_scale, tstep);
 }
 
 // Segments per chain for a launch of BH chains of T tokens: 1 unless the chains are too few to fill the GPU and
-// long enough to cut (every segment a multiple of 128 tokens, at least 1024).
+// long enough to cut (every segment a multiple of 128 tokens).
+constexpr int kSplitMinTiles = 6;
+// Up to this many segments per chain the blocks of the main pass add up the sums before them as they load their state;
+// beyond it a launch of its own forms the prefixes.
+constexpr int kSumInPlace = 4;
 static void plan_split(const la_ctx* ctx, int BH, int T, int* nseg, int* seg_len) {
   *nseg = 1;
   *seg_len = T;
-  if (2 * BH > ctx->sm_count || T < 2048) return;
+  const int tiles = (T + tc::TILE - 1) / tc::TILE;
+  if (2 * BH > ctx->sm_count || tiles < kSplitMinTiles) return;
   // One wave of thread blocks: as many segments per chain as fit on the SMs at once.  (Measured on 32 chains of
   // 32768 tokens: 4 segments per chain 418 us, 9 segments (two waves) 432 us, 13: 456, 18: 483 -- a second wave
   // never fills as well as the first, and every segment costs a 64 KB state written and read back.)
-  int n = std::min(ctx->sm_count / BH, T / 1024);
-  if (n < 2) return;
-  const int len = ((T + n - 1) / n + tc::TILE - 1) / tc::TILE * tc::TILE;
-  n = (T + len - 1) / len;
+  int n = std::min(ctx->sm_count / BH, tiles);
+  const int per = (tiles + n - 1) / n;
+  n = (tiles + per - 1) / per;
   if (n < 2) return;
   *nseg = n;
-  *seg_len = len;
+  *seg_len = per * tc::TILE;
 }
 static size_t split_bytes(const la_config& c, int BH, int nseg) {
-  return (size_t)BH * nseg * ((size_t)tc::D * tc::D * 4 + tc::D * 4 + (size_t)(c.conv_taps > 1 ? c.conv_taps - 1 : 1) * tc::D * 2);
+  return (size_t)BH * ((size_t)nseg * (tc::D * tc::D + tc::D) * 4 + (size_t)(c.conv_taps > 1 ? c.conv_taps - 1 : 1) * tc::D * 2);
 }
 
 size_t prefill_workspace_bytes(const la_ctx* ctx, int B, int T) {
@@ -1422,47 +1600,40 @@ cudaError_t launch_prefill_tc(la_ctx* ctx, int B, int T, const void* q, const vo
   const la_config& c = ctx->cfg;
   *handled = false;
   if (c.io_dtype != LA_BF16 || c.d != tc::D) return cudaSuccess;
-  if ((tc::long_epilogue(c.conv_taps) ? tc::smem_bytes_long(c.conv_taps) : tc::smem_bytes(c.conv_taps)) > 227u * 1024u)
+  if ((tc::long_epilogue(c.conv_taps) ? tc::smem_bytes_long(c.conv_taps, false) : tc::smem_bytes(c.conv_taps)) > tc::kMaxSmem)
     return cudaSuccess;                                                  // (does not happen up to LA_MAX_TAPS)
   const int BH = B * c.H;
   CUtensorMap mq, mk, mv, mo;
   if (!tc::make_map(&mq, q, BH, T) || !tc::make_map(&mk, k, BH, T) || !tc::make_map(&mv, v, BH, T) ||
       !tc::make_map(&mo, o, BH, T))
     return cudaErrorNotSupported;   // the driver cannot encode tensor maps: reported, never a silent slow path
-  int nseg, seg_len;
-  plan_split(ctx, BH, T, &nseg, &seg_len);
-  if (nseg > 1 && (ctx->ws == nullptr || ctx->ws_bytes < split_bytes(c, BH, nseg) || T < c.conv_taps)) nseg = 1, seg_len = T;
-  const bool elu = c.phi == LA_PHI_ELU1;
-  cudaError_t e;
-  if (nseg == 1) {
-    e = elu ? launch_w<LA_PHI_ELU1>(c, BH, T, mq, mk, mv, mo, w, init, st.S, st.z, (__nv_bfloat16*)st.win, st.pos,
-                                    ctx->d_status, 1, T, nullptr, nullptr, s)
-            : launch_w<LA_PHI_RELU>(c, BH, T, mq, mk, mv, mo, w, init, st.S, st.z, (__nv_bfloat16*)st.win, st.pos,
-                                    ctx->d_status, 1, T, nullptr, nullptr, s);
-    ctx->launches += 1;
-    *handled = true;
-    return e;
-  }
-  // Sequence split: local states of all segments, prefix over the segments, then every segment as its own CTA.
-  const int units = BH * nseg;
-  float* S_seg = static_cast<float*>(ctx->ws);
-  float* z_seg = S_seg + (size_t)units * tc::D * tc::D;
-  __nv_bfloat16* win_seg = reinterpret_cast<__nv_bfloat16*>(z_seg + (size_t)units * tc::D);
-  auto skern = elu ? tc::segment_state_kernel<LA_PHI_ELU1> : tc::segment_state_kernel<LA_PHI_RELU>;
-  e = cudaFuncSetAttribute(skern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::kStateSmem);
-  if (e != cudaSuccess) return e;
-  skern<<<dim3(BH * (nseg - 1)), dim3(tc::kStateThreads), tc::kStateSmem, s>>>(mk, mv, S_seg, z_seg, ctx->d_status, T, nseg,
-                                                                               seg_len, nseg - 1);
-  tc::prefix_kernel<<<dim3(BH, tc::D * tc::D / 1024), dim3(256), 0, s>>>(S_seg, z_seg, win_seg, (const __nv_bfloat16*)v, st.S,
-                                                                          st.z, (__nv_bfloat16*)st.win, st.pos, c.H, T,
-                                                                          c.conv_taps, nseg, seg_len, init);
-  e = elu ? launch_w<LA_PHI_ELU1>(c, units, T, mq, mk, mv, mo, w, 1, S_seg, z_seg, win_seg, st.pos, ctx->d_status, nseg,
-                                  seg_len, st.S, st.z, s)
-          : launch_w<LA_PHI_RELU>(c, units, T, mq, mk, mv, mo, w, 1, S_seg, z_seg, win_seg, st.pos, ctx->d_status, nseg,
-                                  seg_len, st.S, st.z, s);
-  ctx->launches += 3;
   *handled = true;
-  return e;
+  Split sp;
+  plan_split(ctx, BH, T, &sp.nseg, &sp.seg_len);
+  if (sp.nseg > 1 && (ctx->ws == nullptr || ctx->ws_bytes < split_bytes(c, BH, sp.nseg) || T < c.conv_taps)) sp = Split();
+  if (sp.nseg > 1) {
+    // Sequence split: the sums of all segments but the last, then every segment as its own CTA.
+    const int nseg = sp.nseg, units = BH * nseg;
+    float* S_seg = static_cast<float*>(ctx->ws);
+    float* z_seg = S_seg + (size_t)units * tc::D * tc::D;
+    __nv_bfloat16* win_seg = reinterpret_cast<__nv_bfloat16*>(z_seg + (size_t)units * tc::D);
+    sp.S = S_seg, sp.z = z_seg, sp.win = win_seg;
+    auto skern = c.phi == LA_PHI_ELU1 ? tc::segment_state_kernel<LA_PHI_ELU1> : tc::segment_state_kernel<LA_PHI_RELU>;
+    cudaError_t e = allow_smem((const void*)skern, ctx->device);
+    if (e != cudaSuccess) return e;
+    ctx->launches += 1;
+    e = launch_maybe_pdl(true, skern, dim3(BH * (nseg - 1)), dim3(tc::kStateThreads), tc::kStateSmem, s, mk, mv, S_seg, z_seg,
+                         ctx->d_status, T, nseg, sp.seg_len, nseg - 1, init, (const float*)st.S, (const float*)st.z,
+                         (const __nv_bfloat16*)st.win, win_seg, c.conv_taps);
+    if (e != cudaSuccess) return e;
+    if (nseg > kSumInPlace) {
+      sp.prefixed = 1;
+      ctx->launches += 1;
+      e = launch_pdl(tc::prefix_kernel, dim3(BH, tc::D * tc::D / 1024), dim3(256), 0, s, S_seg, z_seg, nseg);
+      if (e != cudaSuccess) return e;
+    }
+  }
+  return launch_phi(ctx, BH, T, mq, mk, mv, mo, v, w, init, st, sp, s);
 }
 
 // The three-branch block on the tensor cores: bf16 io, d = 128, groups of 32 to 128 tokens (one tile per group, partly
@@ -1474,20 +1645,14 @@ cudaError_t launch_prefill_grouped_tc(la_ctx* ctx, int B, int T, const void* q, 
   const la_config& c = ctx->cfg;
   *handled = false;
   if (c.io_dtype != LA_BF16 || c.d != tc::D || group < 32 || group > tc::TILE) return cudaSuccess;
-  if (tc::smem_bytes_grp(c.conv_taps, tc::long_epilogue(c.conv_taps, true)) > 227u * 1024u) return cudaSuccess;
+  if (tc::smem_bytes_grp(c.conv_taps, tc::long_epilogue(c.conv_taps, true)) > tc::kMaxSmem) return cudaSuccess;
   const int BH = B * c.H;
   CUtensorMap mq, mk, mv, mo;
   if (!tc::make_map(&mq, q, BH, T, group) || !tc::make_map(&mk, k, BH, T, group) || !tc::make_map(&mv, v, BH, T, group) ||
       !tc::make_map(&mo, o, BH, T, group))
     return cudaErrorNotSupported;
-  cudaError_t e = c.phi == LA_PHI_ELU1
-                      ? launch_w<LA_PHI_ELU1>(c, BH, T, mq, mk, mv, mo, w, init, st.S, st.z, (__nv_bfloat16*)st.win, st.pos,
-                                              ctx->d_status, 1, T, nullptr, nullptr, s, true, alpha, scale, group)
-                      : launch_w<LA_PHI_RELU>(c, BH, T, mq, mk, mv, mo, w, init, st.S, st.z, (__nv_bfloat16*)st.win, st.pos,
-                                              ctx->d_status, 1, T, nullptr, nullptr, s, true, alpha, scale, group);
-  ctx->launches += 1;
   *handled = true;
-  return e;
+  return launch_phi(ctx, BH, T, mq, mk, mv, mo, v, w, init, st, Split(), s, true, alpha, scale, group);
 }
 
 // The sums of one segment on the tensor cores (bf16 io, d = 128): the kernel of the sequence split with one segment
@@ -1501,12 +1666,13 @@ cudaError_t launch_segment_state_tc(la_ctx* ctx, int B, int T, const void* k, co
   CUtensorMap mk, mv;
   if (!tc::make_map(&mk, k, BH, T) || !tc::make_map(&mv, v, BH, T)) return cudaErrorNotSupported;
   auto skern = c.phi == LA_PHI_ELU1 ? tc::segment_state_kernel<LA_PHI_ELU1> : tc::segment_state_kernel<LA_PHI_RELU>;
-  cudaError_t e = cudaFuncSetAttribute(skern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)tc::kStateSmem);
-  if (e != cudaSuccess) return e;
-  skern<<<dim3(BH), dim3(tc::kStateThreads), tc::kStateSmem, s>>>(mk, mv, dS, dz, ctx->d_status, T, 1, T, 1);
-  ctx->launches += 1;
   *handled = true;
-  return cudaGetLastError();
+  cudaError_t e = allow_smem((const void*)skern, ctx->device);
+  if (e != cudaSuccess) return e;
+  ctx->launches += 1;
+  return launch_maybe_pdl(false, skern, dim3(BH), dim3(tc::kStateThreads), tc::kStateSmem, s, mk, mv, dS, dz, ctx->d_status, T,
+                          1, T, 1, 0, (const float*)nullptr, (const float*)nullptr, (const __nv_bfloat16*)nullptr,
+                          (__nv_bfloat16*)nullptr, c.conv_taps);
 }
 
 }  // namespace la

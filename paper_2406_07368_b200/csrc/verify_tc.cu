@@ -764,7 +764,7 @@ cudaError_t launch_verify_tc(la_ctx* ctx, int B, int N, const void* q, const voi
                   ? (elu ? vtc::verify_tc_kernel<LA_PHI_ELU1, false> : vtc::verify_tc_kernel<LA_PHI_RELU, false>)
                   : (elu ? vtc::verify_tc_kernel<LA_PHI_ELU1, true> : vtc::verify_tc_kernel<LA_PHI_RELU, true>);
   const uint32_t smem = vtc::smem_bytes(c.conv_taps);
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = allow_smem((const void*)kern, ctx->device);
   if (e != cudaSuccess) return e;
   e = launch_pdl(kern, dim3(std::min(BH, ctx->sm_count)), dim3(vtc::kThreads), smem, s, ms, mv,
                  (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, parent, w, (const float*)st.z,

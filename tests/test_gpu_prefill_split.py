@@ -1,0 +1,48 @@
+"""The prefill cut along the sequence with few segments per chain (their sums are added up by the blocks of the main pass
+as they load their state), at the smallest lengths that are cut, ragged and not, fresh and continuing."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import la_oracle as orc
+from paper_2406_07368_b200 import binding, workloads as wl
+from tests._util import rel_err
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("H,T,W,first", [(36, 768, 3, 0), (36, 641, 3, 70), (74, 700, 1, 130), (37, 769, 5, 3), (40, 900, 32, 33),
+                                         (49, 2000, 2, 0)])
+def test_split_with_few_segments(H, T, W, first):
+    """`first` tokens in a call of their own, then T in one that is cut; against the oracle on all of them (bf16: 2e-2, the
+    tolerance of every tensor-core path) and against the same call without the workspace (only the order of fp32 sums and
+    the roundings behind it differ: a few bf16 ulps)."""
+    d, io = 128, "bf16"
+    q, k, v = wl.qkv(H + T, (1, H, first + T, d), d ** -0.5, io, v_mean=0.5)
+    w = wl.conv_weights(5, H, d, W)
+    dev = lambda x: torch.from_numpy(np.ascontiguousarray(x)).to(torch.bfloat16).cuda()   # noqa: E731
+    wd = torch.from_numpy(w).cuda()
+    ctx = binding.Context(H, d, W, "elu1", 0.0, io)
+    outs, states = [], []
+    for lend in (True, False):
+        st = ctx.new_state(1)
+        need = ctx.la_prefill_workspace_bytes(1, T)
+        assert need > 0
+        ctx.la_set_workspace(None)
+        if first:
+            ctx.la_prefill(dev(q[:, :, :first]), dev(k[:, :, :first]), dev(v[:, :, :first]), wd, st)
+        if lend:
+            ctx.la_set_workspace(torch.full((need,), 0xff, dtype=torch.uint8, device="cuda"))
+        n0 = ctx.la_launch_count()
+        outs.append(ctx.la_prefill(dev(q[:, :, first:]), dev(k[:, :, first:]), dev(v[:, :, first:]), wd, st, init_state=first > 0))
+        assert ctx.la_launch_count() - n0 == (2 if lend else 1)
+        states.append(st)
+    assert ctx.la_last_device_status() == binding.LA_OK
+    want, ost = orc.prefill_quadratic(q, k, v, w, "elu1", 0.0)
+    got = outs[0].float().cpu().numpy()
+    assert rel_err(got, want[:, :, first:]) < 2e-2
+    assert rel_err(got, outs[1].float().cpu().numpy()) < 1.2e-2
+    for st in states:
+        assert rel_err(st.S.cpu().numpy(), ost.S) < 2e-2 and rel_err(st.z.cpu().numpy(), ost.z) < 2e-2
+        assert st.pos.tolist() == [first + T]
+    assert torch.equal(states[0].win, states[1].win)
