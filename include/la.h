@@ -150,10 +150,11 @@ la_status la_prefill(la_ctx* ctx, int32_t B, int32_t T, const void* q, const voi
  *                  W-1 values of v, pos the token count
  *   other arguments as for la_prefill.
  *
- * Kernels: bf16 io with d = 128 and groups of 32 to 128 tokens run on the tensor cores, one 128-row tile per group
- * (a shorter group leaves the rest of its tile empty; the probabilities of the softmax are rounded to bf16 there
- * before they multiply v).  Everything else runs on the CUDA cores in fp32 (a register-tiled kernel, one thread
- * block per (batch, head)), several times slower per token. */
+ * Kernels: bf16 io with d = 128 and groups of 32 to 128 tokens run on the tensor cores: groups of 32 and 64 share
+ * 128-row tiles, any other group has one of its own and leaves the rest of it empty (the probabilities of the softmax
+ * are rounded to bf16 there before they multiply v).  Few chains of a long sequence are cut along the sequence as in
+ * la_prefill, with the same workspace (la_set_workspace).  Everything else runs on the CUDA cores in fp32 (a
+ * register-tiled kernel, one thread block per (batch, head)), several times slower per token. */
 la_status la_prefill_grouped(la_ctx* ctx, int32_t B, int32_t T, const void* q, const void* k, const void* v,
                              const float* conv_w, int32_t group, float alpha, float softmax_scale, int32_t init_state,
                              la_state* st /*host struct*/, void* o, void* stream);
@@ -315,8 +316,8 @@ la_status la_clear_device_status(la_ctx* ctx, void* stream);
  * they apply: bf16 io, d = 128), 1 = always the fp32 CUDA-core kernels.  For testing one kernel against the other. */
 la_status la_set_prefill_kernel(la_ctx* ctx, int32_t which);
 
-/* Optional workspace for la_prefill.  With few (batch, head) chains and a long sequence -- fewer chains
- * than half the SMs, T >= 2048 -- the grouped processing of Sec. 4.1 is also cut along the sequence:
+/* Optional workspace for la_prefill (and la_prefill_grouped on the tensor cores).  With few (batch, head) chains and a long sequence -- fewer chains
+ * than half the SMs, T > 640 -- the grouped processing of Sec. 4.1 is also cut along the sequence:
  * every segment first computes its own sum of phi(k) v^T, a prefix over the segments gives each its
  * starting state (the cumulative sum of Sec. 4.1 taken at segment level), and all segments then run
  * as independent thread blocks.  That needs la_prefill_workspace_bytes(ctx, B, T) bytes of device

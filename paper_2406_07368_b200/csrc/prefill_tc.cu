@@ -81,7 +81,7 @@ __host__ __device__ constexpr uint32_t off_den(bool z3) { return OFF_ONES + ones
 __host__ __device__ constexpr uint32_t off_small(bool z3) { return off_den(z3) + 2048; }
 
 struct Small {
-  unsigned long long bars[20];
+  unsigned long long bars[22];
   uint32_t tmem_base;
   int abort;
   int pad[2];
@@ -95,8 +95,9 @@ struct Small {
 // waiter is never more than one phase behind.
 enum { B_FULL_K0 = 0, B_FULL_V0 = 1, B_FULL_V1 = 2, B_MMA_P = 3, B_MMA_S0 = 4, B_MMA_O0 = 5, B_MMA_O1 = 6, B_PHI = 7,
        B_PDONE = 8, B_SB = 9, B_EPI0 = 10, B_EPI1 = 11, B_MMA_Q = 12, B_FULL_Q = 13, B_FULL_K1 = 14, B_STAGED0 = 15,
-       B_STAGED1 = 16, B_HALO0 = 17, B_HALO1 = 18, B_MMA_S1 = 19, kNumBars = 20 };
-static_assert(kNumBars <= 20, "Small::bars");
+       B_STAGED1 = 16, B_HALO0 = 17, B_HALO1 = 18, B_MMA_S1 = 19,
+       B_MMA_L = 20 /* the scores against earlier groups of the tile */, kNumBars = 21 };
+static_assert(kNumBars <= 22, "Small::bars");
 
 __host__ __device__ constexpr uint32_t off_w(bool z3) { return off_small(z3) + (uint32_t)((sizeof(Small) + 15) / 16 * 16); }
 // Short windows: nine halo buffers, rows of v that lie before 32 rows of a tile, for the convolution.  Buffers 0-2: the
@@ -146,6 +147,8 @@ __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence:
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void sync_group_b() { asm volatile("bar.sync 2, 256;" ::: "memory"); }
 __device__ __forceinline__ void sync_group_a() { asm volatile("bar.sync 5, 256;" ::: "memory"); }
+template <int N> __device__ __forceinline__ void regs_up() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
+template <int N> __device__ __forceinline__ void regs_down() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
 __device__ __forceinline__ float ex2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
@@ -181,6 +184,16 @@ __device__ __forceinline__ void mma_bf16_ts(uint32_t d_tmem, uint32_t a_tmem, ui
       "setp.ne.b32 p, %4, 0;\n\t"
       "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
       ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"((uint32_t)acc)
+      : "memory");
+}
+// ... and with the first `off` lanes (0, 32, 64 or 96) of the accumulator left as they are.
+__device__ __forceinline__ void mma_bf16_ts_below(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc, bool acc, int off) {
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, {%5, %6, %7, %8}, p;\n\t}"
+      ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"((uint32_t)acc), "r"(off > 0 ? ~0u : 0u), "r"(off > 32 ? ~0u : 0u),
+        "r"(off > 64 ? ~0u : 0u), "r"(0u)
       : "memory");
 }
 __device__ __forceinline__ void mma_commit(uint32_t bar) {
@@ -295,6 +308,22 @@ __device__ __forceinline__ void tmem_st1(uint32_t taddr, uint32_t v) {
       ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),      \
         "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])             \
       : "memory")
+
+#define LA_TMEM_LD16(taddr, r)                                                                                   \
+  asm volatile(                                                                                                  \
+      "tcgen05.ld.sync.aligned.32x32b.x16.b32 "                                                                  \
+      "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"                           \
+      : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),          \
+        "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])     \
+      : "r"(taddr)                                                                                               \
+      : "memory")
+__device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* r) {
+  asm volatile("tcgen05.st.sync.aligned.32x32b.x8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"r"(taddr), "r"(r[0]),
+               "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
+               : "memory");
+}
+// TMEM column (from P_COL) where the packed bf16 of token c, a multiple of 16, begins.
+__device__ __forceinline__ uint32_t pk_col(int c) { return (uint32_t)((c & 64) + ((c & 63) >> 1)); }
 
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
@@ -465,11 +494,16 @@ __device__ __forceinline__ uint4 pack8(const uint32_t* v) {
                     pack2(__uint_as_float(v[4]), __uint_as_float(v[5])), pack2(__uint_as_float(v[6]), __uint_as_float(v[7])));
 }
 
-// GRP: the three-branch block of Sec. 4.1 with the group equal to the 128-token tile: the score product runs on the raw
-// q and k and its rows go through a causal softmax (left branch); the products with the state of the earlier tiles are
-// the group-exclusive linear attention (middle branch: there is no intra-tile linear term); both land in one
-// accumulator, the probabilities pre-scaled by (phi(q).z_prev + eps) / alpha so that one row factor finishes both.
-template <int PHI, int WT, bool GRP = false>
+// GM > 0 (GRP): the three-branch block of Sec. 4.1.  The score product runs on the raw q and k and its rows go through a
+// causal softmax inside their group (left branch); the products with the state of the earlier tiles are the
+// group-exclusive linear attention (middle branch); both land in one accumulator, the probabilities pre-scaled by
+// (phi(q).z + eps) / alpha so that one row factor finishes both.
+// GM = 1: one group per tile (partly filled where the group is shorter than 128), no intra-tile linear term.
+// GM = 2 (MULTI): 128 / gsz groups of gsz = 32 or 64 tokens per tile.  A row then also meets the earlier groups of its
+// tile, linearly: a product per group, phi(Q) with phi(K) of that group, puts those scores in the place of the raw ones
+// that nobody needs (the accumulator's other lanes are masked off), and they join P unscaled.  (One partly filled tile
+// per group of 64 took 200 us on 128 chains of 2048 tokens, as long per tile as a full one.)
+template <int PHI, int WT, int GM = 0>
 __global__ void __launch_bounds__(kThreads, 1)
 prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant__ CUtensorMap mk,
                   const __grid_constant__ CUtensorMap mv, const __grid_constant__ CUtensorMap mo,
@@ -478,12 +512,13 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
                   int* status, int H, int Ttot, int W, float eps, int init, int nseg,
                   int seg_len, const float* __restrict__ S_seg, const float* __restrict__ z_seg,
                   const __nv_bfloat16* __restrict__ win_seg, int prefixed, const __nv_bfloat16* __restrict__ vg, float alpha,
-                  float sm_scale, int tstep, int early) {
+                  float sm_scale, int tstep, int gsz, int early) {
   extern __shared__ unsigned char smem_dyn[];
   // (an offset into the array rather than an integer cast: the compiler then knows that these are shared-memory
   // addresses: 32-bit arithmetic, ld.shared / st.shared)
   unsigned char* smem = smem_dyn + ((1024u - (smem_u32(smem_dyn) & 1023u)) & 1023u);
   const uint32_t sbase = smem_u32(smem);
+  constexpr bool GRP = GM > 0, MULTI = GM == 2;
   constexpr bool LONG = WT < 0;                  // the epilogue for longer tap windows
   // Who copies the state between two tiles: group B has the time beside an elu + 1 (which keeps group A busy), group A beside
   // a ReLU or a long window (which keeps group B busy).
@@ -492,6 +527,11 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
   // phi(K), mask) is the longest there, and group B had 2 K of a tile's 5.9 K cycles to spare.  (128 chains of 2048 tokens,
   // 3 taps: 71 us with none, 65.4 with 2, 64.6 with 3, 65.8 with 4.)
   constexpr int KB = SNAP_A || GRP ? 0 : 3;
+  // Long windows and the three-branch mode: registers per thread once the roles have traded theirs.  256 threads of group
+  // A, 256 of group B and 128 others were launched with 96 each: 2 kRegsA + 2 kRegsB + 64 = 5 x 96.
+  constexpr bool TRADE = LONG || GRP;
+  constexpr int kRegsA = LONG && !MULTI ? 96 : LONG ? 104 : 112, kRegsB = 208 - kRegsA;
+  static_assert(kThreadsA == 256 && kThreadsB == 256 && kThreads == 640, "register split");
   const bool z3 = LONG ? z3_long(W, GRP) : true; // z rides in the state update's product
   Small& sm = *reinterpret_cast<Small*>(smem + off_small(z3));
   float* wsm = reinterpret_cast<float*>(smem + off_w(z3));                     // [W][128] ([W up to a multiple of 8][128] if LONG)
@@ -539,6 +579,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
     mbar_init((bar0 + 8u * (B_MMA_P)), 1);
     mbar_init((bar0 + 8u * (B_MMA_S0)), 1);
     mbar_init((bar0 + 8u * (B_MMA_S1)), 1);
+    mbar_init((bar0 + 8u * (B_MMA_L)), 1);
     mbar_init((bar0 + 8u * (B_MMA_O0)), 1);
     mbar_init((bar0 + 8u * (B_MMA_O1)), 1);
     mbar_init((bar0 + 8u * (B_PHI)), kThreadsA);
@@ -717,6 +758,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
     mbar_arrive((bar0 + 8u * (B_SB)));
   };
 
+  if (warp >= 16) {
+  if (TRADE) regs_down<64>();
   if (warp == kCtrlWarp) {
     // =============================== MMA issue, the Q and K loads (one lane) ===============================
     if (lane == 0) {
@@ -752,6 +795,16 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
           mbar_expect_tx((bar0 + 8u * (B_FULL_Q)), tile_tx);
           tma_load(sbase + OFF_Q, &mq, 0, y0 + (n + 1) * tstep, bh, (bar0 + 8u * (B_FULL_Q)));
           tma_load(sbase + OFF_Q + BOX_BYTES, &mq, 64, y0 + (n + 1) * tstep, bh, (bar0 + 8u * (B_FULL_Q)));
+        }
+        if (MULTI) {                       // the scores of rows gsz (c + 1) ... 127 against the tokens of group c of this tile
+          if (use_glob)
+            for (int c = 0; c + 1 < TILE / gsz; ++c)
+#pragma unroll
+              for (int ks = 0; ks < 8; ++ks)
+                mma_bf16_ts_below(tmem + P_COL + gsz * c, tmem + FQ_COL + 8 * ks,
+                                  desc64(k_km + (((uint32_t)(gsz * c) * 128u) >> 4) + kstep_kmajor(ks, KBOX_BYTES)),
+                                  idesc(false, false, (uint32_t)gsz), ks > 0, gsz * (c + 1));
+          mma_commit((bar0 + 8u * (B_MMA_L)));
         }
         if (!GRP) {
 #pragma unroll
@@ -879,8 +932,10 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
         mbar_arrive((bar0 + 8u * (B_HALO0 + par)));
       }
     }
-  } else if (warp >= 8 && warp < 16) {
+  }
+  } else if (warp >= 8) {
     // =============================== group A: phi, P, [S|z] snapshot (256 threads) ===============================
+    if (TRADE && kRegsA > 96) regs_up<kRegsA>();
     const int ta = tid - kThreadsB;               // 0..255
     const int wa = warp - 8;                      // 0..7
     const int r = 32 * (wa & 3) + lane;           // tile row = TMEM lane
@@ -908,6 +963,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
       if (GRP) sync_group_a();                    // every thread is done with the halves of the last tile (dgh, mlh)
       // phi(q) of row r, this thread's 64 channels: 32 packed pairs = 32 TMEM columns of lane r.
       uint32_t fq[32];
+      float dg = 0.f;
       if (ok) {
 #pragma unroll
         for (int cc = 0; cc < 8; ++cc) {
@@ -923,13 +979,12 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
       if (ok) {
         LA_TMEM_ST32(tmem + lane_addr + FQ_COL + 32 * hf, fq);
         if (GRP) {                                // this half of phi(q) . z_prev, z in fp32
-          float dg = 0.f;
 #pragma unroll
           for (int e = 0; e < 32; e += 2) {
             const float4 z4 = *reinterpret_cast<const float4*>(zs + 64 * hf + 2 * e);
             dg = fmaf(lo_f(fq[e]), z4.x, fmaf(hi_f(fq[e]), z4.y, fmaf(lo_f(fq[e + 1]), z4.z, fmaf(hi_f(fq[e + 1]), z4.w, dg))));
           }
-          dgh[hf * D + r] = dg;
+          if (!MULTI) dgh[hf * D + r] = dg;
         }
         tmem_wait_st();
       }
@@ -992,7 +1047,78 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
         denbuf[(par * 2 + hf) * D + r] = dpart;
         tmem_wait_st();
       }
-      if (GRP) {
+      if constexpr (MULTI) {
+        // ---- P: causal softmax inside the row's group (the two threads of a row take half of its columns each), the
+        // linear scores against the earlier groups of the tile, zeros behind the group.  Everything a row has is read
+        // before the barrier and written, packed, after it.
+        const float c2 = sm_scale * 1.4426950408889634f;       // scores -> exponents of two
+        const int b0 = 32 * (wa & 3) / gsz * gsz, hw = gsz >> 1, d0 = b0 + hw * hf, l0 = (b0 >> 1) * hf;   // warp-uniform
+        float m_run = -INFINITY, l_run = 0.f;
+        uint32_t v[32], lp[24];
+        if (ok) {
+          tc_fence_after();
+          if (hw == 32) LA_TMEM_LD32(tmem + P_COL + lane_addr + d0, v);
+          else LA_TMEM_LD16(tmem + P_COL + lane_addr + d0, v);
+          tmem_wait_ld();
+#pragma unroll
+          for (int e = 0; e < 32; ++e) {
+            v[e] = __float_as_uint((e < 16 || hw == 32) && d0 + e <= r ? __uint_as_float(v[e]) * c2 : -INFINITY);
+            m_run = fmaxf(m_run, __uint_as_float(v[e]));
+          }
+          if (m_run > -INFINITY) {
+#pragma unroll
+            for (int e = 0; e < 32; ++e) l_run += ex2(__uint_as_float(v[e]) - m_run);
+          }
+        }
+        if (use_glob && b0 > 0) {
+          ok = ok && mbar_wait((bar0 + 8u * (B_MMA_L)), par, abort);
+          ok = __all_sync(0xffffffffu, ok);
+        }
+#pragma unroll
+        for (int c = 0; c < 3; ++c)                             // 16 of this thread's b0 / 2 linear scores at a time
+          if (32 * c < b0) {
+            uint32_t x[16];
+#pragma unroll
+            for (int e = 0; e < 16; ++e) x[e] = 0u;
+            if (ok && use_glob) {
+              tc_fence_after();
+              LA_TMEM_LD16(tmem + P_COL + lane_addr + l0 + 16 * c, x);
+              tmem_wait_ld();
+            }
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+              lp[8 * c + e] = pack2(__uint_as_float(x[2 * e]), __uint_as_float(x[2 * e + 1]));
+              dg += __uint_as_float(x[2 * e]) + __uint_as_float(x[2 * e + 1]);
+            }
+          }
+        mlh[hf * D + r] = make_float2(m_run, l_run);
+        dgh[hf * D + r] = dg;
+        tc_fence_before();
+        sync_group_a();
+        const float2 oth = mlh[(hf ^ 1) * D + r];
+        const float m = fmaxf(m_run, oth.x);                    // finite: the row's own column lies in one of the halves
+        const float l = l_run * ex2(m_run - m) + oth.y * ex2(oth.x - m);
+        const float den = dgh[r] + dgh[D + r] + eps;
+        const bool has_g = use_glob && (has_in || n > 0 || b0 > 0) && den != 0.f;
+        const float rs = has_g ? den / alpha : 1.f, f = rs / l;
+        if (ok) {
+          tc_fence_after();
+          const uint32_t pbase = tmem + P_COL + lane_addr;
+          uint32_t pk[16];
+#pragma unroll
+          for (int e = 0; e < 16; ++e)
+            pk[e] = pack2(ex2(__uint_as_float(v[2 * e]) - m) * f, ex2(__uint_as_float(v[2 * e + 1]) - m) * f);
+          if (hw == 32) LA_TMEM_ST16(pbase + pk_col(d0), pk);
+          else tmem_st8(pbase + pk_col(d0), pk);
+#pragma unroll
+          for (int c = 0; c < 3; ++c)
+            if (32 * c < b0) tmem_st8(pbase + pk_col(l0 + 16 * c), lp + 8 * c);
+          const uint32_t zero[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
+          for (int c = b0 + gsz + 16 * hf; c < TILE; c += 32) tmem_st8(pbase + pk_col(c), zero);
+          denbuf[(par * 2 + hf) * D + r] = hf == 0 ? rs : 0.f;
+          tmem_wait_st();
+        }
+      } else if (GRP) {
         // ---- P: causal softmax along the rows.  A row's 128 columns belong to two threads (halves): each takes the
         // running maximum and sum of its half, the halves meet through shared memory, and a second pass writes
         // exp(s - max) / sum back as bf16 -- times (phi(q) . z_prev + eps) / alpha where the global branch is alive, so
@@ -1070,8 +1196,9 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
 
       if (SNAP_A) snapshot(n, r, hf, lane_addr, ok);
     }
-  } else if (warp < 8) {
+  } else {
     // =============================== group B: epilogue (256 threads) ===============================
+    if (TRADE && kRegsB > 96) regs_up<kRegsB>();
     const int r = 32 * (warp & 3) + lane;         // tile row = TMEM lane
     const int hf = warp >> 2;                     // column half
     const uint32_t lane_addr = (uint32_t)(32 * (warp & 3)) << 16;
@@ -1524,13 +1651,14 @@ template <int PHI>
 static cudaError_t launch_w(la_ctx* ctx, int BH, int T, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
                             const CUtensorMap& mo, const void* v, const float* w, int init, const la_state& st,
                             const Split& sp, cudaStream_t s, bool grouped = false, float alpha = 1.f, float sm_scale = 1.f,
-                            int tstep = tc::TILE) {
+                            int tstep = tc::TILE, int gsz = 0) {
   const la_config& c = ctx->cfg;
   const bool lng = tc::long_epilogue(c.conv_taps, grouped);
   const size_t smem = grouped ? tc::smem_bytes_grp(c.conv_taps, lng) : lng ? tc::smem_bytes_long(c.conv_taps, false) : tc::smem_bytes(c.conv_taps);
   auto kern = tc::prefill_tc_kernel<PHI, 3>;
   if (grouped) {
-    kern = lng ? tc::prefill_tc_kernel<PHI, -1, true> : tc::prefill_tc_kernel<PHI, 3, true>;
+    kern = gsz ? (lng ? tc::prefill_tc_kernel<PHI, -1, 2> : tc::prefill_tc_kernel<PHI, 3, 2>)
+               : (lng ? tc::prefill_tc_kernel<PHI, -1, 1> : tc::prefill_tc_kernel<PHI, 3, 1>);
   } else
   switch (c.conv_taps) {     // short windows: the tap loop unrolled; the others: the long epilogue
     case 1: kern = tc::prefill_tc_kernel<PHI, 1>; break;
@@ -1551,37 +1679,38 @@ static cudaError_t launch_w(la_ctx* ctx, int BH, int T, const CUtensorMap& mq, c
   return launch_maybe_pdl(early || sp.nseg > 1, kern, dim3(units), dim3(tc::kThreads), smem, s, mq, mk, mv, mo, w, st.S, st.z,
                           (__nv_bfloat16*)st.win, st.pos, ctx->d_status, c.H, T, c.conv_taps, c.eps, init, sp.nseg,
                           sp.nseg > 1 ? sp.seg_len : T, sp.S, sp.z, sp.win, sp.prefixed, (const __nv_bfloat16*)v, alpha,
-                          sm_scale, tstep, early);
+                          sm_scale, tstep, gsz, early);
 }
 static cudaError_t launch_phi(la_ctx* ctx, int BH, int T, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
                               const CUtensorMap& mo, const void* v, const float* w, int init, const la_state& st,
                               const Split& sp, cudaStream_t s, bool grouped = false, float alpha = 1.f, float sm_scale = 1.f,
-                              int tstep = tc::TILE) {
+                              int tstep = tc::TILE, int gsz = 0) {
   return ctx->cfg.phi == LA_PHI_ELU1
-             ? launch_w<LA_PHI_ELU1>(ctx, BH, T, mq, mk, mv, mo, v, w, init, st, sp, s, grouped, alpha, sm_scale, tstep)
-             : launch_w<LA_PHI_RELU>(ctx, BH, T, mq, mk, mv, mo, v, w, init, st, sp, s, grouped, alpha, sm_scale, tstep);
+             ? launch_w<LA_PHI_ELU1>(ctx, BH, T, mq, mk, mv, mo, v, w, init, st, sp, s, grouped, alpha, sm_scale, tstep, gsz)
+             : launch_w<LA_PHI_RELU>(ctx, BH, T, mq, mk, mv, mo, v, w, init, st, sp, s, grouped, alpha, sm_scale, tstep, gsz);
 }
 
 // Segments per chain for a launch of BH chains of T tokens: 1 unless the chains are too few to fill the GPU and
-// long enough to cut (every segment a multiple of 128 tokens).
+// long enough to cut (every segment a whole number of tiles).
 constexpr int kSplitMinTiles = 6;
 // Up to this many segments per chain the blocks of the main pass add up the sums before them as they load their state;
 // beyond it a launch of its own forms the prefixes.
 constexpr int kSumInPlace = 4;
-static void plan_split(const la_ctx* ctx, int BH, int T, int* nseg, int* seg_len) {
+static void plan_split(const la_ctx* ctx, int BH, int T, int* nseg, int* seg_len, int tile = tc::TILE) {
   *nseg = 1;
   *seg_len = T;
-  const int tiles = (T + tc::TILE - 1) / tc::TILE;
+  int tiles = (T + tc::TILE - 1) / tc::TILE;
   if (2 * BH > ctx->sm_count || tiles < kSplitMinTiles) return;
   // One wave of thread blocks: as many segments per chain as fit on the SMs at once.  (Measured on 32 chains of
   // 32768 tokens: 4 segments per chain 418 us, 9 segments (two waves) 432 us, 13: 456, 18: 483 -- a second wave
   // never fills as well as the first, and every segment costs a 64 KB state written and read back.)
   int n = std::min(ctx->sm_count / BH, tiles);
+  tiles = (T + tile - 1) / tile;               // (shorter tiles, of the three-branch block, never mean more segments)
   const int per = (tiles + n - 1) / n;
   n = (tiles + per - 1) / per;
   if (n < 2) return;
   *nseg = n;
-  *seg_len = per * tc::TILE;
+  *seg_len = per * tile;
 }
 static size_t split_bytes(const la_config& c, int BH, int nseg) {
   return (size_t)BH * ((size_t)nseg * (tc::D * tc::D + tc::D) * 4 + (size_t)(c.conv_taps > 1 ? c.conv_taps - 1 : 1) * tc::D * 2);
@@ -1595,21 +1724,13 @@ size_t prefill_workspace_bytes(const la_ctx* ctx, int B, int T) {
   return nseg > 1 ? split_bytes(c, B * c.H, nseg) : 0;
 }
 
-cudaError_t launch_prefill_tc(la_ctx* ctx, int B, int T, const void* q, const void* k, const void* v, const float* w,
-                              int init, const la_state& st, void* o, cudaStream_t s, bool* handled) {
+// Cuts the chains where that pays and the workspace allows it: launches what forms the segments' starting states.  `tile`:
+// tokens per tile of the main pass; mk, mv: maps with boxes of 128 rows.
+static cudaError_t launch_split(la_ctx* ctx, int BH, int T, int tile, const CUtensorMap& mk, const CUtensorMap& mv, int init,
+                                const la_state& st, Split* out, cudaStream_t s) {
+  Split& sp = *out;
   const la_config& c = ctx->cfg;
-  *handled = false;
-  if (c.io_dtype != LA_BF16 || c.d != tc::D) return cudaSuccess;
-  if ((tc::long_epilogue(c.conv_taps) ? tc::smem_bytes_long(c.conv_taps, false) : tc::smem_bytes(c.conv_taps)) > tc::kMaxSmem)
-    return cudaSuccess;                                                  // (does not happen up to LA_MAX_TAPS)
-  const int BH = B * c.H;
-  CUtensorMap mq, mk, mv, mo;
-  if (!tc::make_map(&mq, q, BH, T) || !tc::make_map(&mk, k, BH, T) || !tc::make_map(&mv, v, BH, T) ||
-      !tc::make_map(&mo, o, BH, T))
-    return cudaErrorNotSupported;   // the driver cannot encode tensor maps: reported, never a silent slow path
-  *handled = true;
-  Split sp;
-  plan_split(ctx, BH, T, &sp.nseg, &sp.seg_len);
+  plan_split(ctx, BH, T, &sp.nseg, &sp.seg_len, tile);
   if (sp.nseg > 1 && (ctx->ws == nullptr || ctx->ws_bytes < split_bytes(c, BH, sp.nseg) || T < c.conv_taps)) sp = Split();
   if (sp.nseg > 1) {
     // Sequence split: the sums of all segments but the last, then every segment as its own CTA.
@@ -1633,12 +1754,32 @@ cudaError_t launch_prefill_tc(la_ctx* ctx, int B, int T, const void* q, const vo
       if (e != cudaSuccess) return e;
     }
   }
+  return cudaSuccess;
+}
+
+cudaError_t launch_prefill_tc(la_ctx* ctx, int B, int T, const void* q, const void* k, const void* v, const float* w,
+                              int init, const la_state& st, void* o, cudaStream_t s, bool* handled) {
+  const la_config& c = ctx->cfg;
+  *handled = false;
+  if (c.io_dtype != LA_BF16 || c.d != tc::D) return cudaSuccess;
+  if ((tc::long_epilogue(c.conv_taps) ? tc::smem_bytes_long(c.conv_taps, false) : tc::smem_bytes(c.conv_taps)) > tc::kMaxSmem)
+    return cudaSuccess;                                                  // (does not happen up to LA_MAX_TAPS)
+  const int BH = B * c.H;
+  CUtensorMap mq, mk, mv, mo;
+  if (!tc::make_map(&mq, q, BH, T) || !tc::make_map(&mk, k, BH, T) || !tc::make_map(&mv, v, BH, T) ||
+      !tc::make_map(&mo, o, BH, T))
+    return cudaErrorNotSupported;   // the driver cannot encode tensor maps: reported, never a silent slow path
+  *handled = true;
+  Split sp;
+  const cudaError_t e = launch_split(ctx, BH, T, tc::TILE, mk, mv, init, st, &sp, s);
+  if (e != cudaSuccess) return e;
   return launch_phi(ctx, BH, T, mq, mk, mv, mo, v, w, init, st, sp, s);
 }
 
-// The three-branch block on the tensor cores: bf16 io, d = 128, groups of 32 to 128 tokens (one tile per group, partly
-// filled below 128: a group of 64 runs the tensor cores half empty and still beats the CUDA-core kernel seven times;
-// below 32 that kernel takes over), and few enough taps for the 4 KB of extra shared memory.  Sets *handled to false otherwise (the CUDA-core kernel takes those).
+// The three-branch block on the tensor cores: bf16 io, d = 128, groups of 32 to 128 tokens (groups of 32 and 64 share
+// tiles of 128; any other has a tile of its own, partly filled, which still beats the CUDA-core kernel several times;
+// below 32 that kernel takes over), and few enough taps for the 4 KB of extra shared memory.  Sets *handled to false
+// otherwise (the CUDA-core kernel takes those).
 cudaError_t launch_prefill_grouped_tc(la_ctx* ctx, int B, int T, const void* q, const void* k, const void* v, const float* w,
                                       int group, float alpha, float scale, int init, const la_state& st, void* o,
                                       cudaStream_t s, bool* handled) {
@@ -1647,12 +1788,16 @@ cudaError_t launch_prefill_grouped_tc(la_ctx* ctx, int B, int T, const void* q, 
   if (c.io_dtype != LA_BF16 || c.d != tc::D || group < 32 || group > tc::TILE) return cudaSuccess;
   if (tc::smem_bytes_grp(c.conv_taps, tc::long_epilogue(c.conv_taps, true)) > tc::kMaxSmem) return cudaSuccess;
   const int BH = B * c.H;
-  CUtensorMap mq, mk, mv, mo;
-  if (!tc::make_map(&mq, q, BH, T, group) || !tc::make_map(&mk, k, BH, T, group) || !tc::make_map(&mv, v, BH, T, group) ||
-      !tc::make_map(&mo, o, BH, T, group))
+  const int gsz = group == 32 || group == 64 ? group : 0, tile = gsz ? tc::TILE : group;
+  CUtensorMap mq, mk, mv, mo, mk1, mv1;
+  if (!tc::make_map(&mq, q, BH, T, tile) || !tc::make_map(&mk, k, BH, T, tile) || !tc::make_map(&mv, v, BH, T, tile) ||
+      !tc::make_map(&mo, o, BH, T, tile) || (tile != tc::TILE && (!tc::make_map(&mk1, k, BH, T) || !tc::make_map(&mv1, v, BH, T))))
     return cudaErrorNotSupported;
   *handled = true;
-  return launch_phi(ctx, BH, T, mq, mk, mv, mo, v, w, init, st, Split(), s, true, alpha, scale, group);
+  Split sp;
+  const cudaError_t e = launch_split(ctx, BH, T, tile, tile != tc::TILE ? mk1 : mk, tile != tc::TILE ? mv1 : mv, init, st, &sp, s);
+  if (e != cudaSuccess) return e;
+  return launch_phi(ctx, BH, T, mq, mk, mv, mo, v, w, init, st, sp, s, true, alpha, scale, tile, gsz);
 }
 
 // The sums of one segment on the tensor cores (bf16 io, d = 128): the kernel of the sequence split with one segment

@@ -1,0 +1,61 @@
+"""The three-branch block with several groups per 128-token tile (groups of 32 and 64 on the tensor cores), at the edges of
+groups and tiles, and cut along the sequence."""
+import numpy as np
+import pytest
+import torch
+
+from oracle import la_oracle as orc
+from paper_2406_07368_b200 import binding, workloads as wl
+from tests._util import TOL, rel_err
+
+pytestmark = pytest.mark.gpu
+
+
+def _run(C, T, W, phi, eps, alpha, first=0, B=1, H=3, workspace=False):
+    d, io = 128, "bf16"
+    q, k, v = wl.qkv(41 + T, (B, H, first + T, d), 0.5, io, v_mean=1.0)
+    w = wl.conv_weights(41, H, d, W)
+    dev = lambda x: torch.from_numpy(np.ascontiguousarray(x)).to(torch.bfloat16).cuda()   # noqa: E731
+    wd = torch.from_numpy(w).cuda()
+    ctx = binding.Context(H, d, W, phi, eps, io)
+    st = ctx.new_state(B)
+    args = (C, alpha, d ** -0.5)
+    if first:
+        ctx.la_prefill_grouped(dev(q[:, :, :first]), dev(k[:, :, :first]), dev(v[:, :, :first]), wd, st, *args)
+    if workspace:
+        need = ctx.la_prefill_workspace_bytes(B, T)
+        assert need > 0
+        ctx.la_set_workspace(torch.full((need,), 0xff, dtype=torch.uint8, device="cuda"))
+    n0 = ctx.la_launch_count()
+    o = ctx.la_prefill_grouped(dev(q[:, :, first:]), dev(k[:, :, first:]), dev(v[:, :, first:]), wd, st, *args,
+                               init_state=first > 0)
+    launches = ctx.la_launch_count() - n0
+    assert ctx.la_last_device_status() == binding.LA_OK
+    want, ost = orc.prefill_grouped_block(q, k, v, w, phi, eps, C, alpha, d ** -0.5)
+    got = o.float().cpu().numpy()
+    assert rel_err(got, want[:, :, first:]) < TOL[io]
+    for a in range(0, T, C):                                     # group by group: one wrong group cannot hide
+        assert rel_err(got[:, :, a:a + C], want[:, :, first + a:first + a + C]) < TOL[io], a
+    assert rel_err(st.S.cpu().numpy(), ost.S) < TOL[io] and rel_err(st.z.cpu().numpy(), ost.z) < TOL[io]
+    assert st.pos.tolist() == [first + T] * B
+    np.testing.assert_array_equal(st.win.float().cpu().numpy(), ost.win)
+    return launches
+
+
+@pytest.mark.parametrize("C", [32, 64])
+@pytest.mark.parametrize("T", [1, 31, 32, 33, 63, 65, 96, 127, 128, 129, 161, 390])
+def test_edges(C, T):
+    _run(C, T, 3, "elu1", 0.0, 0.8)
+
+
+@pytest.mark.parametrize("C,W,phi,eps,alpha,first", [(32, 8, "elu1", 0.0, 1.0, 0), (64, 1, "relu", 1e-6, 0.7, 64),
+                                                     (32, 3, "relu", 1e-6, 1.3, 96), (64, 3, "elu1", 0.0, 0.0, 128),
+                                                     (32, 16, "elu1", 0.0, 0.0, 32)])
+def test_options_and_continuation(C, W, phi, eps, alpha, first):
+    _run(C, 300, W, phi, eps, alpha, first)
+
+
+@pytest.mark.parametrize("C,T,first,H", [(64, 900, 0, 36), (32, 770, 64, 2), (128, 1000, 0, 3), (100, 1200, 100, 40)])
+def test_cut_along_the_sequence(C, T, first, H):
+    """With a workspace: packed groups, one group per tile, and partly filled tiles (100 tokens)."""
+    assert _run(C, T, 3, "elu1", 0.0, 1.0, first, H=H, workspace=True) > 1
