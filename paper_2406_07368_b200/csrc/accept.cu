@@ -15,6 +15,8 @@ accept_greedy_kernel(const int32_t* __restrict__ parent, const int32_t* __restri
   __shared__ int s_par[kAcceptWarps][LA_MAX_NODES], s_draft[kAcceptWarps][LA_MAX_NODES], s_pred[kAcceptWarps][LA_MAX_NODES];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int b = blockIdx.x * kAcceptWarps + warp;
+  pdl_wait();                                          // the kernel before this one in the stream may still be running
+  pdl_trigger();
   if (b >= B) return;                                  // whole warps leave: no block-wide barrier below
   for (int n = lane; n < N; n += 32) {
     s_par[warp][n] = parent[(size_t)b * N + n];
@@ -64,6 +66,8 @@ accept_threshold_kernel(const int32_t* __restrict__ parent, const float* __restr
   __shared__ unsigned char s_pass[kAcceptWarps][LA_MAX_NODES];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int b = blockIdx.x * kAcceptWarps + warp;
+  pdl_wait();                                          // the kernel before this one in the stream may still be running
+  pdl_trigger();
   if (b >= B) return;                                  // whole warps leave: no block-wide barrier below
   for (int n = lane; n < N; n += 32) {
     s_par[warp][n] = parent[(size_t)b * N + n];
@@ -100,19 +104,17 @@ accept_threshold_kernel(const int32_t* __restrict__ parent, const float* __restr
 
 cudaError_t launch_accept_threshold(la_ctx* ctx, int B, int N, const int32_t* parent, const float* score, const float* thresh,
                                     int32_t* accept_node, int32_t* accept_len, cudaStream_t s) {
-  accept_threshold_kernel<<<dim3((B + kAcceptWarps - 1) / kAcceptWarps), dim3(32 * kAcceptWarps), 0, s>>>(
-      parent, score, thresh, accept_node, accept_len, ctx->d_status, B, N);
   ctx->launches += 1;
-  return cudaGetLastError();
+  return launch_pdl(accept_threshold_kernel, dim3((B + kAcceptWarps - 1) / kAcceptWarps), dim3(32 * kAcceptWarps), 0, s, parent,
+                    score, thresh, accept_node, accept_len, ctx->d_status, B, N);
 }
 
 cudaError_t launch_accept(la_ctx* ctx, int B, int N, const int32_t* parent, const int32_t* draft, const int32_t* pred_root,
                           const int32_t* pred, int32_t* accept_node, int32_t* accept_len, int32_t* next_token,
                           cudaStream_t s) {
-  accept_greedy_kernel<<<dim3((B + kAcceptWarps - 1) / kAcceptWarps), dim3(32 * kAcceptWarps), 0, s>>>(
-      parent, draft, pred_root, pred, accept_node, accept_len, next_token, ctx->d_status, B, N);
   ctx->launches += 1;
-  return cudaGetLastError();
+  return launch_pdl(accept_greedy_kernel, dim3((B + kAcceptWarps - 1) / kAcceptWarps), dim3(32 * kAcceptWarps), 0, s, parent,
+                    draft, pred_root, pred, accept_node, accept_len, next_token, ctx->d_status, B, N);
 }
 
 }  // namespace la

@@ -43,10 +43,11 @@ commit_kernel(const T* __restrict__ k, const T* __restrict__ v, const int32_t* _
 #pragma unroll
   for (int m = 0; m < PASSES; ++m) s[m] = __ldcs(reinterpret_cast<const float4*>(Sb + (size_t)(rg + RPP * m) * D + c4));
 
+  const int acc_node = t == 0 ? accept[b] : 0;   // (in flight with the tree, not behind it)
   if (t < N) sm.par[t] = parent[(size_t)b * N + t];
   __syncthreads();
   if (t == 0) {
-    int a = accept[b], L = 0, bad = 0;
+    int a = acc_node, L = 0, bad = 0;
     if (a < -1 || a >= N) bad = 1;
     int m = bad ? -1 : a;
     while (m >= 0) {                       // m strictly decreases: terminates
@@ -108,11 +109,19 @@ commit_kernel(const T* __restrict__ k, const T* __restrict__ v, const int32_t* _
     float zz = z[(size_t)bh * D + t];
     for (int l = 0; l < L; ++l) zz += fk[l][t];
     z[(size_t)bh * D + t] = zz;
-    // window <- last W-1 entries of (window ++ v_path); ascending, source index above target
-    T* wb = win + (size_t)bh * (W - 1) * D;
-    for (int i = 0; i < W - 1; ++i) {
-      const int src = L + i;
-      wb[(size_t)i * D + t] = src < W - 1 ? wb[(size_t)src * D + t] : from_f32<T>(vv[src - (W - 1)][t]);
+    // window <- last W-1 entries of (window ++ v_path); ascending, source index above target.  Eight rows at a time, their
+    // loads in flight together (row by row, each waited for the store before it: 4 us at 8 taps).
+    T* wb = win + (size_t)bh * (W - 1) * D + t;
+    for (int i0 = 0; i0 < W - 1; i0 += 8) {
+      T x[8];
+#pragma unroll
+      for (int i = 0; i < 8; ++i) {
+        const int src = L + i0 + i;
+        if (i0 + i < W - 1) x[i] = src < W - 1 ? wb[(size_t)src * D] : from_f32<T>(vv[src - (W - 1)][t]);
+      }
+#pragma unroll
+      for (int i = 0; i < 8; ++i)
+        if (i0 + i < W - 1) wb[(size_t)(i0 + i) * D] = x[i];
     }
   }
   if (h == 0 && part == 0 && t == 0) pos[b] += L;

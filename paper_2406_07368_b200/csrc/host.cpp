@@ -79,6 +79,22 @@ void* ptr(PyObject* o, at::ScalarType dtype, Shape shape, const char* name) {
   return t.data_ptr();
 }
 
+// Small int32 outputs of one call that the caller did not bring share one allocation (a trip through the allocator costs a
+// fifth of a launch); each starts on a 64-byte boundary of it.
+struct Pool {
+  at::Tensor base;
+  int64_t used = 0;
+  at::Tensor take(const at::Tensor& like, Shape shape, int64_t room) {
+    if (!base.defined()) base = at::detail::empty_cuda({room}, at::kInt, like.device(), std::nullopt);
+    at::Tensor t = at::detail::make_tensor<at::TensorImpl>(c10::Storage(base.storage()), base.key_set(), base.dtype());
+    t.unsafeGetTensorImpl()->set_storage_offset(used);
+    t.unsafeGetTensorImpl()->set_sizes_contiguous(at::IntArrayRef(shape));
+    used += padded(t.numel());
+    return t;
+  }
+  static int64_t padded(int64_t n) { return (n + 15) & ~int64_t(15); }
+};
+
 // The given tensor, or a new one on the device of `like`.  Holds the reference that is returned to Python.
 struct Out {
   PyObject* obj = nullptr;
@@ -90,6 +106,18 @@ struct Out {
       obj = given;
     } else {
       at::Tensor t = at::detail::empty_cuda(at::IntArrayRef(shape), dtype, like.device(), std::nullopt);
+      p = t.data_ptr();
+      obj = THPVariable_Wrap(std::move(t));
+      if (!obj) throw Raised();
+    }
+  }
+  Out(PyObject* given, const at::Tensor& like, Shape shape, const char* name, Pool& pool, int64_t room) {
+    if (given != Py_None) {
+      p = ptr(given, at::kInt, shape, name);
+      Py_INCREF(given);
+      obj = given;
+    } else {
+      at::Tensor t = pool.take(like, shape, room);
       p = t.data_ptr();
       obj = THPVariable_Wrap(std::move(t));
       if (!obj) throw Raised();
@@ -277,7 +305,9 @@ PyObject* commit(PyObject* self, PyObject* const* a, Py_ssize_t n) {
     // Buffers made here have no earlier contents to keep: the kernel fills them for skipped sequences too (-1 and 0),
     // which takes the place of two fill launches.
     const int fresh = (a[5] == Py_None ? LA_FRESH_PATH : 0) | (a[6] == Py_None ? LA_FRESH_LEN : 0);
-    Out path(a[5], k, at::kInt, {B, p->max_depth}, "path_out"), len(a[6], k, at::kInt, {B}, "commit_len");
+    Pool pool;
+    const int64_t room = Pool::padded(B * p->max_depth) + Pool::padded(B);
+    Out path(a[5], k, {B, p->max_depth}, "path_out", pool, room), len(a[6], k, {B}, "commit_len", pool, room);
     void* s = stream_of(a[7]);
     check("la_commit", unlocked([&] {
             return la_commit_fresh(p->ctx, (int32_t)B, (int32_t)N, kp, vp, parent, accept, &st.st, (int32_t*)path.p,
@@ -296,8 +326,10 @@ PyObject* accept_greedy(PyObject* self, PyObject* const* a, Py_ssize_t n) {
     const int32_t* draft = (const int32_t*)ptr(a[1], at::kInt, {B, N}, "draft_token");
     const int32_t* root = (const int32_t*)ptr(a[2], at::kInt, {B}, "pred_root");
     const int32_t* pred = (const int32_t*)ptr(a[3], at::kInt, {B, N}, "pred");
-    Out node(a[4], par, at::kInt, {B}, "accept_node"), len(a[5], par, at::kInt, {B}, "accept_len"),
-        next(a[6], par, at::kInt, {B}, "next_token");
+    Pool pool;
+    const int64_t room = 3 * Pool::padded(B);
+    Out node(a[4], par, {B}, "accept_node", pool, room), len(a[5], par, {B}, "accept_len", pool, room),
+        next(a[6], par, {B}, "next_token", pool, room);
     void* s = stream_of(a[7]);
     check("la_accept_greedy", unlocked([&] {
             return la_accept_greedy(p->ctx, (int32_t)B, (int32_t)N, parent, draft, root, pred, (int32_t*)node.p, (int32_t*)len.p,
@@ -320,7 +352,9 @@ PyObject* accept_threshold(PyObject* self, PyObject* const* a, Py_ssize_t n) {
     const int32_t* parent = (const int32_t*)ptr(a[0], at::kInt, {B, N}, "parent");
     const float* score = (const float*)ptr(a[1], at::kFloat, {B, N}, "score");
     const float* thresh = (const float*)ptr(a[2], at::kFloat, {B, N}, "thresh");
-    Out node(a[3], par, at::kInt, {B}, "accept_node"), len(a[4], par, at::kInt, {B}, "accept_len");
+    Pool pool;
+    const int64_t room = 2 * Pool::padded(B);
+    Out node(a[3], par, {B}, "accept_node", pool, room), len(a[4], par, {B}, "accept_len", pool, room);
     void* s = stream_of(a[5]);
     check("la_accept_threshold", unlocked([&] {
             return la_accept_threshold(p->ctx, (int32_t)B, (int32_t)N, parent, score, thresh, (int32_t*)node.p, (int32_t*)len.p, s);

@@ -238,15 +238,12 @@ __device__ __forceinline__ void mma_commit(uint32_t bar) {
         "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]), "=r"(r[29]), "=r"(r[30]), "=r"(r[31])   \
       : "r"(taddr)                                                                                               \
       : "memory")
-#define LA_TMEM_ST_FRAG8(taddr, r)                                                                               \
+#define LA_TMEM_ST_FRAG4(taddr, r)                                                                               \
   asm volatile(                                                                                                  \
-      "tcgen05.st.sync.aligned.16x256b.x8.b32 [%0], "                                                            \
-      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, "                                 \
-      "%17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31, %32};"                         \
+      "tcgen05.st.sync.aligned.16x256b.x4.b32 [%0], "                                                            \
+      "{%1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16};"                                 \
       ::"r"(taddr), "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]),      \
-        "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]),            \
-        "r"(r[16]), "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]),          \
-        "r"(r[24]), "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31])           \
+        "r"(r[8]), "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15])             \
       : "memory")
 #define LA_TMEM_LD_FRAG4(taddr, r)                                                                               \
   asm volatile(                                                                                                  \
@@ -659,19 +656,35 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
     // Both groups share it out, 16 rows x 64 columns per warp.
     const int q4 = warp & 3, hf = (warp >> 2) & 1, r0 = 32 * q4 + 16 * (warp >> 3);
     const float* Sg = S_in + (size_t)(r0 + (lane >> 2)) * D + 64 * hf + 2 * (lane & 3);
-    uint32_t v[32], x[32];
-    frag_load(Sg, v);
-    for (int j = 1; j < nsum; ++j) {                // the sums of the segments before this one
-      frag_load(Sg + (size_t)j * D * D, x);
-      frag_add(v, x);
+#pragma unroll
+    for (int hh = 0; hh < 2; ++hh) {                // 32 columns at a time; two of the parts in flight
+      uint32_t v[16], x[16];
+      auto load = [&](int j, uint32_t (&y)[16]) {
+#pragma unroll
+        for (int g = 0; g < 4; ++g)
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            const float2 t = *reinterpret_cast<const float2*>(Sg + (size_t)j * D * D + i * 8 * D + 32 * hh + 8 * g);
+            y[4 * g + 2 * i] = __float_as_uint(t.x);
+            y[4 * g + 2 * i + 1] = __float_as_uint(t.y);
+          }
+      };
+      load(0, v);
+      if (nsum > 1) load(1, x);
+#pragma unroll 1
+      for (int j = 1; j < nsum; ++j) {              // the sums of the segments before this one
+#pragma unroll
+        for (int e = 0; e < 16; ++e) v[e] = __float_as_uint(__uint_as_float(v[e]) + __uint_as_float(x[e]));
+        if (j + 1 < nsum) load(j + 1, x);
+      }
+      LA_TMEM_ST_FRAG4(tmem + ((uint32_t)r0 << 16) + S_COL + 64 * hf + 32 * hh, v);
+#pragma unroll
+      for (int g = 0; g < 4; ++g)
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+          *reinterpret_cast<uint32_t*>(smem + OFF_S + hf * BOX_BYTES + swz(r0 + (lane >> 2) + 8 * i, 4 * hh + g) + 4 * (lane & 3)) =
+              pack2(__uint_as_float(v[4 * g + 2 * i]), __uint_as_float(v[4 * g + 2 * i + 1]));
     }
-    LA_TMEM_ST_FRAG8(tmem + ((uint32_t)r0 << 16) + S_COL + 64 * hf, v);
-#pragma unroll
-    for (int g = 0; g < 8; ++g)
-#pragma unroll
-      for (int i = 0; i < 2; ++i)
-        *reinterpret_cast<uint32_t*>(smem + OFF_S + hf * BOX_BYTES + swz(r0 + (lane >> 2) + 8 * i, g) + 4 * (lane & 3)) =
-            pack2(__uint_as_float(v[4 * g + 2 * i]), __uint_as_float(v[4 * g + 2 * i + 1]));
     if (warp < 4) {                                 // z, and zeros in the other columns of its block (32 rows per warp)
       const uint32_t zaddr = tmem + ((uint32_t)(32 * q4) << 16) + Z_COL;
       tmem_st1(zaddr, __float_as_uint(z_start(32 * q4 + lane)));
@@ -707,13 +720,11 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
   using KAc = std::integral_constant<int, 8 - KB>;
   using K8c = std::integral_constant<int, 8>;
 
-  // S and z after tile n: the bf16 copy and the z row for the next tile, or the final state to global memory.  256 threads
-  // (row r, 64 columns each): group B or group A.
+  // S and z after tile n, which is not the last: the bf16 copy and the z row for the next tile.  256 threads (row r, 64
+  // columns each): group B or group A.
   auto snapshot = [&](int n, int r, int hf, uint32_t lane_addr, bool& ok) {
     const uint32_t par = n & 1;
-    const bool last = n + 1 == nchunks;
     unsigned char* Sb = smem + OFF_S + hf * BOX_BYTES;
-    // ---- S_n: bf16 copy for the next tile, or the final state to global memory ----
     // S_n is final after MMA_S; the old copy may be overwritten once O = phi(Q) S_prev has read it
     ok = ok && mbar_wait((bar0 + 8u * (par ? B_MMA_S1 : B_MMA_S0)), (n >> 1) & 1, abort) && mbar_wait((bar0 + 8u * (B_MMA_Q)), par, abort);
     ok = __all_sync(0xffffffffu, ok);
@@ -721,31 +732,17 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
       tc_fence_after();
       uint32_t zbits = 0u;
       if (hf == 0) zbits = tmem_ld1(tmem + lane_addr + Z_COL);
-      if (!last) {
 #pragma unroll
-        for (int qq = 0; qq < 2; ++qq) {
-          uint32_t v[32];
-          LA_TMEM_LD32(tmem + lane_addr + S_COL + 64 * hf + 32 * qq, v);
-          tmem_wait_ld();
+      for (int qq = 0; qq < 2; ++qq) {
+        uint32_t v[32];
+        LA_TMEM_LD32(tmem + lane_addr + S_COL + 64 * hf + 32 * qq, v);
+        tmem_wait_ld();
 #pragma unroll
-          for (int c = 0; c < 4; ++c) *reinterpret_cast<uint4*>(Sb + swz(r, 4 * qq + c)) = pack8(v + 8 * c);
-        }
-      } else if (writes_state) {
-#pragma unroll
-        for (int i = 0; i < 2; ++i) {             // rows 16 i ... 16 i + 15 of this warp's 32
-          uint32_t v[32];
-          LA_TMEM_LD_FRAG8(tmem + lane_addr + ((uint32_t)(16 * i) << 16) + S_COL + 64 * hf, v);
-          tmem_wait_ld();
-          frag_store(S + (size_t)bh * D * D + (size_t)((r & ~31) + 16 * i + (lane >> 2)) * D + 64 * hf + 2 * (lane & 3), v);
-        }
-      } else {
-        tmem_wait_ld();                           // zbits
+        for (int c = 0; c < 4; ++c) *reinterpret_cast<uint4*>(Sb + swz(r, 4 * qq + c)) = pack8(v + 8 * c);
       }
       if (hf == 0) {
         const float zz = __uint_as_float(zbits);
-        if (last) {
-          if (writes_state) z[(size_t)bh * D + r] = zz;
-        } else if (GRP) {
+        if (GRP) {
           zs[r] = zz;                             // fp32, for phi(q) . z of the next tile
         } else {                                  // row 128 of the K buffer of tile n+1
           *reinterpret_cast<__nv_bfloat16*>(smem + (((n + 1) & 1) ? OFF_K1 : OFF_K0) + (r >> 6) * KBOX_BYTES + BOX_BYTES +
@@ -1194,7 +1191,29 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
         if (ok) phi_k(K0c{}, KAc{}, n + 1, ta);
       }
 
-      if (SNAP_A) snapshot(n, r, hf, lane_addr, ok);
+      if (SNAP_A && !last) snapshot(n, r, hf, lane_addr, ok);
+    }
+
+    // ---- the final state to global memory (this group has nothing else to do after the last tile) ----
+    {
+      const int n = nchunks - 1;
+      ok = ok && mbar_wait((bar0 + 8u * ((n & 1) ? B_MMA_S1 : B_MMA_S0)), (n >> 1) & 1, abort);
+      ok = __all_sync(0xffffffffu, ok);
+      if (ok && writes_state) {
+        tc_fence_after();
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {             // rows 16 i ... 16 i + 15 of this warp's 32
+          uint32_t v[32];
+          LA_TMEM_LD_FRAG8(tmem + lane_addr + ((uint32_t)(16 * i) << 16) + S_COL + 64 * hf, v);
+          tmem_wait_ld();
+          frag_store(S + (size_t)bh * D * D + (size_t)((r & ~31) + 16 * i + (lane >> 2)) * D + 64 * hf + 2 * (lane & 3), v);
+        }
+        if (hf == 0) {
+          const uint32_t zbits = tmem_ld1(tmem + lane_addr + Z_COL);
+          tmem_wait_ld();
+          z[(size_t)bh * D + r] = __uint_as_float(zbits);
+        }
+      }
     }
   } else {
     // =============================== group B: epilogue (256 threads) ===============================
@@ -1312,7 +1331,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
         ok = __all_sync(0xffffffffu, ok);
         if (ok) phi_k(KAc{}, K8c{}, n + 1, tid);
       }
-      if (!SNAP_A) snapshot(n, r, hf, lane_addr, ok);
+      if (!SNAP_A && n + 1 < nchunks) snapshot(n, r, hf, lane_addr, ok);
       uint32_t vrow[WN];                          // row lane - t of the warp's 32: this lane's address for ldmatrix, chunk 0
       {
         const uint32_t vb = sbase + vbox(par, hf) + 4096u * q4;
