@@ -30,7 +30,15 @@ namespace vtc {
 constexpr int D = 128, NMAX = LA_MAX_NODES;
 constexpr int kMaxTaps = 4;                        // taps whose gathers run as tensor-core products
 constexpr int kExtTaps = LA_MAX_TAPS - kMaxTaps;   // the others: gathered by the CUDA cores in the epilogue
-constexpr int kThreadsX = 256, kThreadsY = 256, kCtrlWarp = 16, kTreeWarp = 17, kThreads = 576;
+constexpr int kThreadsX = 256, kThreadsY = 256, kThreadsC = 128, kCtrlWarp = 16, kTreeWarp = 17 /* and 18 */, kLoadWarp = 19,
+              kConvWarp = 20;
+// More than four taps (EXT): warps 18-23 as well.  Up to four taps one tree warp and group X, which then rounds the state
+// too, are enough; six more warps only made the set-up longer (512 units, 3 taps: 18.6 us against 19.9).
+__host__ __device__ constexpr int threads(bool ext) { return ext ? 768 : 576; }
+// Registers per thread once the roles have traded theirs (EXT): the launch gives everyone 80, per scheduler 6 warps of
+// them, and 2 x 72 + 2 x 112 + 64 + 48 is the same number.
+constexpr int kRegsX = 72, kRegsY = 112, kRegsCtl = 64, kRegsC = 48;
+static_assert(2 * kRegsX + 2 * kRegsY + kRegsCtl + kRegsC == 6 * 80, "register split");
 constexpr uint32_t S_BYTES = 128 * 128 * 4;        // the fp32 state of one unit, row-major
 constexpr uint32_t SB_BOX = 128 * 128;             // 128 rows x 64 bf16
 constexpr uint32_t Q_BOX = NMAX * 128;             // 64 rows x 64 bf16
@@ -43,24 +51,23 @@ __host__ __device__ constexpr uint32_t acc_col(int t) { return (t & 1) ? 384u : 
 struct alignas(16) Tab {
   unsigned long long mask[2][NMAX];                // bit m of mask[n]: m is n or an ancestor of n
   float qz[2][NMAX];                               // phi(q_n) . z
-  int bad[2];                                      // a parent index was out of range
-  int pad0[2];
+  int bad[2][2];                                   // a parent index was out of range (one flag per tree warp)
   float den_part[2][NMAX];                         // masked row sums of P, one per column half
   float rden[NMAX];                                // 1 / (denominator + eps)
-  int par[NMAX];                                   // the parent array (private to the tree warp)
+  int par[2][NMAX];                                // the parent array (a copy per tree warp)
   unsigned short ext[2][kExtTaps][NMAX];           // where in a box of the V copy tap 4 + j of node n reads its row
                                                    // (row * 128 + ((row & 7) << 4); W > 4 only)
 };
 struct alignas(16) Ctl {
-  unsigned long long bars[12];
+  unsigned long long bars[14];
   uint32_t tmem_base;
   int abort;
 };
-// XDONE comes as a pair indexed by the unit parity (phase t >> 1); every other barrier completes once per unit
+// XDONE and TREE (EXT: the tree warps; else they arrive on XDONE) are pairs indexed by the unit parity (phase t >> 1); every other barrier completes once per unit
 // (phase t), and the protocol lets none complete again before the waiters of its previous phase have passed.
 // XT (more than four taps only): group Y has taken the values of the later taps from the V copy and its tables.
-enum { B_FULL_S = 0, B_FULL_V, B_XDONE0, B_XDONE1, B_SCONV, B_P, B_PS, B_SG, B_PMDONE, B_O, B_EPI, B_XT, kNumBars };
-static_assert(kNumBars <= 12, "Ctl::bars");
+enum { B_FULL_S = 0, B_FULL_V, B_XDONE0, B_XDONE1, B_SCONV, B_P, B_PS, B_SG, B_PMDONE, B_O, B_EPI, B_XT, B_TREE0, B_TREE1, kNumBars };
+static_assert(kNumBars <= 14, "Ctl::bars");
 constexpr uint32_t OFF_S = 0;                               // S as it lies in memory (fp32, rows = features)
 constexpr uint32_t OFF_SB = OFF_S + S_BYTES;                // S as bf16: two boxes of 64 channels, rows = features
 constexpr uint32_t OFF_QB = OFF_SB + 2 * SB_BOX;            // phi(Q) as bf16: two boxes of 64 features
@@ -87,6 +94,8 @@ __device__ __forceinline__ void mbar_init(uint32_t bar, uint32_t count) {
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
+template <int N> __device__ __forceinline__ void regs_up() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
+template <int N> __device__ __forceinline__ void regs_down() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
 __device__ __forceinline__ void sync_y() { asm volatile("bar.sync 2, 256;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -166,17 +175,18 @@ __device__ __forceinline__ uint32_t pack2(float a, float b) {
 }
 
 // Persistent kernel: CTA i handles units i, i + gridDim.x, ...  Roles:
-//   group X (warps 0-7)  unit t: phi(q), phi(k) as bf16 operands, phi(q) . z; rounds S to bf16;
-//   warp 17              unit t: walks the tree; writes the tree masks, the selection matrices and the window rows;
+//   group X (warps 0-7)  unit t: phi(q), phi(k) as bf16 operands, phi(q) . z; rounds S to bf16 (EXT: warps 20-23 do);
+//   warp 17 (EXT: and 18) unit t: walks the tree; writes the tree masks, the selection matrices and the window rows;
 //   warp 16 (one lane)   TMA of S and V; every tcgen05.mma;
 //   group Y (warps 8-15) masks the scores, forms the denominators, and writes the outputs.
 template <int PHI, bool EXT>   // EXT: more than kMaxTaps live taps
-__global__ void __launch_bounds__(kThreads, 1)
+__global__ void __launch_bounds__(threads(EXT), 1)
 verify_tc_kernel(const __grid_constant__ CUtensorMap ms, const __grid_constant__ CUtensorMap mv,
                  const __nv_bfloat16* __restrict__ q, const __nv_bfloat16* __restrict__ k,
                  const int32_t* __restrict__ parent, const float* __restrict__ w, const float* __restrict__ z,
                  const __nv_bfloat16* __restrict__ win, __nv_bfloat16* __restrict__ o, int* status, int H, int N, int W,
                  float eps, int units) {
+  constexpr int kThreads = threads(EXT);
   extern __shared__ unsigned char smem_dyn[];
   // (an offset into the array rather than an integer cast: the compiler then knows that these are shared-memory
   // addresses: 32-bit arithmetic, ld.shared / st.shared)
@@ -192,12 +202,30 @@ verify_tc_kernel(const __grid_constant__ CUtensorMap ms, const __grid_constant__
   for (int i = 0; i < kNumBars; ++i) bar[i] = smem_u32(&ctl.bars[i]);
 
   // ---- set-up: barriers, TMEM, the constant parts of the operands ----
-  if (tid == 0) {
+  auto load_s = [&](int t) {   // the committed state of unit t, 128 x 128 fp32 in one copy
+    const int u = (int)blockIdx.x + t * (int)gridDim.x;
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar[B_FULL_S]), "r"(S_BYTES) : "memory");
+    asm volatile(
+        "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
+        ::"r"(sbase + OFF_S), "l"(&ms), "r"(0), "r"(u * D), "r"(bar[B_FULL_S])
+        : "memory");
+  };
+  auto load_v = [&](int t) {   // the draft values of unit t: two boxes of 64 channels x 64 nodes (rows past N: zeros)
+    const int u = (int)blockIdx.x + t * (int)gridDim.x;
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar[B_FULL_V]), "r"(2 * Q_BOX) : "memory");
+#pragma unroll
+    for (int x = 0; x < 2; ++x)
+      asm volatile(
+          "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
+          ::"r"(sbase + OFF_V + x * V_BOX), "l"(&mv), "r"(64 * x), "r"(0), "r"(u), "r"(bar[B_FULL_V])
+          : "memory");
+  };
+  if (tid == (EXT ? kLoadWarp * 32 : 0)) {
     mbar_init(bar[B_FULL_S], 1);
     mbar_init(bar[B_FULL_V], 1);
-    mbar_init(bar[B_XDONE0], kThreadsX + 32);
-    mbar_init(bar[B_XDONE1], kThreadsX + 32);
-    mbar_init(bar[B_SCONV], kThreadsX);
+    mbar_init(bar[B_XDONE0], kThreadsX + (EXT ? 0 : 32));
+    mbar_init(bar[B_XDONE1], kThreadsX + (EXT ? 0 : 32));
+    mbar_init(bar[B_SCONV], EXT ? kThreadsC : kThreadsX);
     mbar_init(bar[B_P], 1);
     mbar_init(bar[B_PS], 1);
     mbar_init(bar[B_SG], 1);
@@ -205,8 +233,15 @@ verify_tc_kernel(const __grid_constant__ CUtensorMap ms, const __grid_constant__
     mbar_init(bar[B_O], 1);
     mbar_init(bar[B_EPI], kThreadsY);
     mbar_init(bar[B_XT], kThreadsY);
+    mbar_init(bar[B_TREE0], 64);
+    mbar_init(bar[B_TREE1], 64);
     ctl.abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    if (EXT) {                               // the first unit is requested at once: nothing below touches where it lands
+      pdl_wait();
+      load_s(0);
+      load_v(0);
+    }
   }
   // selection matrices and masked scores start as zeros; so do the 16 window rows below the draft rows of V
   for (uint32_t i = tid; i < (OFF_TAB - OFF_SEL) / 16; i += kThreads)
@@ -226,35 +261,43 @@ verify_tc_kernel(const __grid_constant__ CUtensorMap ms, const __grid_constant__
   pdl_wait();                                // everything above touched shared memory and TMEM only
   pdl_trigger();
 
+  auto round_s = [&](int a) {                // row a of S to bf16 in the operand layout (rows = features), 4 channels per lane
+    const float4 s4 = *reinterpret_cast<const float4*>(smem + OFF_S + a * 512 + lane * 16);
+    *reinterpret_cast<uint2*>(smem + OFF_SB + (lane >> 4) * SB_BOX + swz(a, (lane & 15) >> 1) + (lane & 1) * 8) =
+        make_uint2(pack2(s4.x, s4.y), pack2(s4.z, s4.w));
+  };
+  if (EXT && warp >= kConvWarp) {
+    // =============================== group C: the bf16 copy of S of unit t ===============================
+    if (EXT) regs_down<kRegsC>();
+    bool ok = true;
+    for (int t = 0; t < nloc; ++t) {
+      // the copy of unit t - 1 has been read; S of unit t has landed
+      if (t >= 1) ok = ok && mbar_wait(bar[B_PS], (t - 1) & 1, abort);
+      ok = ok && mbar_wait(bar[B_FULL_S], t & 1, abort);
+      ok = __all_sync(0xffffffffu, ok);
+      if (ok) {
+#pragma unroll 4
+        for (int it = 0; it < 32; ++it) round_s(warp - kConvWarp + 4 * it);
+      }
+      proxy_fence();
+      mbar_arrive(bar[B_SCONV]);
+    }
+  } else if (warp >= 16) {
+  if (EXT) regs_down<kRegsCtl>();
   if (warp == kCtrlWarp) {
     // =============================== TMA and the tensor cores (one lane) ===============================
     if (lane == 0) {
-      auto load_s = [&](int t) {   // the committed state of unit t, 128 x 128 fp32 in one copy
-        const int u = (int)blockIdx.x + t * (int)gridDim.x;
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar[B_FULL_S]), "r"(S_BYTES) : "memory");
-        asm volatile(
-            "cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3}], [%4];"
-            ::"r"(sbase + OFF_S), "l"(&ms), "r"(0), "r"(u * D), "r"(bar[B_FULL_S])
-            : "memory");
-      };
-      auto load_v = [&](int t) {   // the draft values of unit t: two boxes of 64 channels x 64 nodes (rows past N: zeros)
-        const int u = (int)blockIdx.x + t * (int)gridDim.x;
-        asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar[B_FULL_V]), "r"(2 * Q_BOX) : "memory");
-#pragma unroll
-        for (int x = 0; x < 2; ++x)
-          asm volatile(
-              "cp.async.bulk.tensor.3d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], [%5];"
-              ::"r"(sbase + OFF_V + x * V_BOX), "l"(&mv), "r"(64 * x), "r"(0), "r"(u), "r"(bar[B_FULL_V])
-              : "memory");
-      };
       constexpr uint32_t kIdP = idesc(false, false), kIdV = idesc(true, false);
-      load_s(0);
-      load_v(0);
+      if (!EXT) {
+        load_s(0);
+        load_v(0);
+      }
       for (int t = 0; t < nloc; ++t) {
         const uint32_t par = t & 1;
         if (!mbar_wait(bar[B_XDONE0 + par], (t >> 1) & 1, abort)) break;
         tc_fence_after();
-        const bool good = tab.bad[par] == 0;
+        // (EXT: a malformed tree is found out later, by group Y: the products are in bounds whatever the tree says)
+        const bool good = EXT || (tab.bad[par][0] | tab.bad[par][1]) == 0;
         if (good) {
 #pragma unroll
           for (int ks = 0; ks < 8; ++ks) {     // P[n][m]: 16 values of the feature index per step
@@ -277,6 +320,7 @@ verify_tc_kernel(const __grid_constant__ CUtensorMap ms, const __grid_constant__
         // G of unit t - 1 has been read (this unit's accumulator was last read two units ago)
         if (t >= 1 && !mbar_wait(bar[B_EPI], (t - 1) & 1, abort)) break;
         if (!mbar_wait(bar[B_FULL_V], par, abort)) break;
+        if (EXT && !mbar_wait(bar[B_TREE0 + par], (t >> 1) & 1, abort)) break;
         tc_fence_after();
         if (good) {
           // G_j[c][n], the value tap j reads for node n, for all taps at once: the selection matrices lie one after
@@ -306,8 +350,110 @@ verify_tc_kernel(const __grid_constant__ CUtensorMap ms, const __grid_constant__
         if (t + 1 < nloc) load_v(t + 1);
       }
     }
+  } else if (EXT && warp < kLoadWarp) {
+    // =============================== the tree of unit t, more than four taps (two warps, one node per lane) ===============================
+    // (One warp with two nodes per lane was the longest loop of all: 2 K cycles for the walk and 2-2.7 K for the writes
+    // of a unit's 5.2-6.9 K, and the score product waited for it.)
+    const int tw = warp - kTreeWarp, n = lane + 32 * tw;    // this lane's node
+    // Sel_0 is the identity: tap 0 reads the node's own value
+    *reinterpret_cast<unsigned short*>(smem + OFF_SEL + swz(n, n >> 3) + (n & 7) * 2) = 0x3F80;
+    uint32_t prev[3];                                       // where the ones of this lane's node were put for the last unit
+#pragma unroll
+    for (int i = 0; i < 3; ++i) prev[i] = 0xffffffffu;
+    bool ok = true;
+    // the parents, requested one unit ahead (right after the previous unit's walk)
+    auto load_par = [&](int t2, int& p0, int& p1) {
+      const int b2 = ((int)blockIdx.x + t2 * (int)gridDim.x) / H;
+      p0 = lane < N ? parent[(size_t)b2 * N + lane] : -1;
+      p1 = lane + 32 < N ? parent[(size_t)b2 * N + lane + 32] : -1;
+    };
+    int pn0 = -1, pn1 = -1;
+    if (nloc > 0) load_par(0, pn0, pn1);
+    for (int t = 0; t < nloc; ++t) {
+      const int u = (int)blockIdx.x + t * (int)gridDim.x, par = t & 1;
+      tab.par[tw][lane] = pn0;
+      tab.par[tw][lane + 32] = pn1;
+      // the committed window, W - 1 rows of 16 pieces of 16 bytes shared out over the two warps, four loads in flight
+      const uint4* wsrc = reinterpret_cast<const uint4*>(win + (size_t)u * (W - 1) * D);
+      const int wtotal = (W - 1) * 16;
+      uint4 wq[4];
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        if (n + 64 * i < wtotal) wq[i] = wsrc[n + 64 * i];
+      __syncwarp();
+      // ---- each lane follows the parents of its node (integer work) and notes where taps 4 .. W-1 read: the ancestor at
+      //      distance j while the chain lasts, then rows of the committed window, newest first.  (This parity's table
+      //      was last read two units ago, and the wait for that lies an iteration back.) ----
+      unsigned long long mask = 0ull;
+      int depth = 0, anc[3] = {0, 0, 0};
+      bool good = true;
+      for (int m = n < N ? n : -1; m >= 0;) {               // every step lowers m: at most N iterations
+        mask |= 1ull << m;
+        if (depth == 1) anc[0] = m;
+        if (depth == 2) anc[1] = m;
+        if (depth == 3) anc[2] = m;
+        if (depth >= kMaxTaps && depth < W)
+          tab.ext[par][depth - kMaxTaps][n] = (unsigned short)(m * 128 + ((m & 7) << 4));
+        ++depth;
+        const int p = tab.par[tw][m];
+        if (p < -1 || p >= m) {
+          good = false;
+          break;
+        }
+        m = p;
+      }
+      const bool bad_any = __any_sync(0xffffffffu, !good);
+      // behind the chain: window rows; nodes past N are read like the others and never stored: any row will do
+      for (int kk = max(n < N ? depth : 0, kMaxTaps); kk < W; ++kk) {
+        const int row = n < N ? NMAX + kk - depth : 0;
+        tab.ext[par][kk - kMaxTaps][n] = (unsigned short)(row * 128 + ((row & 7) << 4));
+      }
+      __syncwarp();
+      if (t + 1 < nloc) load_par(t + 1, pn0, pn1);           // in flight during the waits and the writes below
+
+      // ---- the selection matrices of unit t - 1 have been consumed by the products, its window rows and V copy by
+      //      group Y (and with them everything issued before: this parity's tables were last read two units ago) ----
+      if (t >= 1) ok = ok && mbar_wait(bar[B_SG], (t - 1) & 1, abort) && mbar_wait(bar[B_XT], (t - 1) & 1, abort);
+      ok = __all_sync(0xffffffffu, ok);
+      if (ok) {
+        if (lane == 0) tab.bad[par][tw] = bad_any ? 1 : 0;
+        tab.mask[par][n] = mask;
+#pragma unroll
+        for (int j = 1; j < kMaxTaps; ++j) {                // one entry per (node, tap): clear the last unit's, set this unit's
+          uint32_t& pv = prev[j - 1];
+          if (pv != 0xffffffffu) *reinterpret_cast<unsigned short*>(smem + pv) = 0;
+          pv = 0xffffffffu;
+          if (n < N) {
+            if (j < depth) {
+              const int a = anc[j - 1];
+              pv = OFF_SEL + j * Q_BOX + swz(n, a >> 3) + (a & 7) * 2;
+            } else {                                        // behind the chain: the committed window, newest row first
+              pv = OFF_SELW + selw_offset(64 * j + n, j - depth);
+            }
+            *reinterpret_cast<unsigned short*>(smem + pv) = 0x3F80;
+          }
+        }
+        // the window below the draft rows of both channel halves, newest row first: row NMAX + p holds the value
+        // p + 1 steps behind the first draft token
+        for (int base = 0; base < wtotal; base += 256) {
+          if (base > 0) {
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+              if (base + n + 64 * i < wtotal) wq[i] = wsrc[base + n + 64 * i];
+          }
+#pragma unroll
+          for (int i = 0; i < 4; ++i) {
+            const int idx = base + n + 64 * i;               // row idx >> 4 of the window (oldest first), channels 8 (idx & 15) ...
+            if (idx < wtotal)
+              *reinterpret_cast<uint4*>(smem + OFF_V + ((idx & 15) >> 3) * V_BOX + swz(NMAX + (W - 2) - (idx >> 4), idx & 7)) = wq[i];
+          }
+        }
+      }
+      proxy_fence();
+      mbar_arrive(bar[B_TREE0 + par]);
+    }
   } else if (warp == kTreeWarp) {
-    // =============================== the tree of unit t (one warp, nodes lane and lane + 32) ===============================
+    // =============================== the tree of unit t, up to four taps (one warp, nodes lane and lane + 32) ===============================
     for (int n = lane; n < NMAX; n += 32)                   // Sel_0 is the identity: tap 0 reads the node's own value
       *reinterpret_cast<unsigned short*>(smem + OFF_SEL + swz(n, n >> 3) + (n & 7) * 2) = 0x3F80;
     uint32_t prev[2][3];                                    // where the ones of this lane's nodes were put for the last unit
@@ -324,27 +470,17 @@ verify_tc_kernel(const __grid_constant__ CUtensorMap ms, const __grid_constant__
     if (nloc > 0) load_par(0, pn0, pn1);
     for (int t = 0; t < nloc; ++t) {
       const int u = (int)blockIdx.x + t * (int)gridDim.x, par = t & 1;
-      tab.par[lane] = pn0;
-      tab.par[lane + 32] = pn1;
+      tab.par[0][lane] = pn0;
+      tab.par[0][lane + 32] = pn1;
       uint32_t wv[6];                                       // the committed window (up to three rows: W <= 4) in flight early
 #pragma unroll
       for (int i = 0; i < 6; ++i) {
         const int idx = lane + 32 * i;
-        wv[i] = (!EXT && idx < 64 * (W - 1)) ? *reinterpret_cast<const uint32_t*>(win + (size_t)u * (W - 1) * D + 2 * idx)
-                                                      : 0u;
+        wv[i] = idx < 64 * (W - 1) ? *reinterpret_cast<const uint32_t*>(win + (size_t)u * (W - 1) * D + 2 * idx) : 0u;
       }
-      // more than four taps: the window is up to 31 rows, 16 bytes per lane and load, 8 loads in flight at a time
-      const uint4* wsrc = reinterpret_cast<const uint4*>(win + (size_t)u * (W - 1) * D);
-      const int wtotal = EXT ? (W - 1) * 16 : 0;
-      uint4 wq[8];
-#pragma unroll
-      for (int i = 0; i < 8; ++i)
-        if (EXT && lane + 32 * i < wtotal) wq[i] = wsrc[lane + 32 * i];
       __syncwarp();
       // ---- each lane follows the parents of its two nodes (integer work), both chains in one loop so that their
-      //      loads overlap.  With more than four taps the walk also notes where taps 4 .. W-1 read: the ancestor at
-      //      distance j while the chain lasts, then rows of the committed window, newest first.  (This parity's table
-      //      was last read two units ago, and the wait for that lies an iteration back.) ----
+      //      loads overlap ----
       unsigned long long mask[2] = {0ull, 0ull};
       int depth[2] = {0, 0}, anc[2][3] = {{0, 0, 0}, {0, 0, 0}};
       bool good = true;
@@ -358,10 +494,8 @@ verify_tc_kernel(const __grid_constant__ CUtensorMap ms, const __grid_constant__
             if (depth[s2] == 1) anc[s2][0] = m;
             if (depth[s2] == 2) anc[s2][1] = m;
             if (depth[s2] == 3) anc[s2][2] = m;
-            if (EXT && depth[s2] >= kMaxTaps && depth[s2] < W)
-              tab.ext[par][depth[s2] - kMaxTaps][lane + 32 * s2] = (unsigned short)(m * 128 + ((m & 7) << 4));
             ++depth[s2];
-            const int p = tab.par[m];
+            const int p = tab.par[0][m];
             if (p < -1 || p >= m) {
               good = false;
               mm[s2] = -1;
@@ -372,30 +506,15 @@ verify_tc_kernel(const __grid_constant__ CUtensorMap ms, const __grid_constant__
         }
       }
       const bool bad_any = __any_sync(0xffffffffu, !good);
-      if (EXT) {
-#pragma unroll
-        for (int s2 = 0; s2 < 2; ++s2) {
-          const int n = lane + 32 * s2;
-          // behind the chain: window rows; nodes past N are read like the others and never stored: any row will do
-          for (int kk = max(n < N ? depth[s2] : 0, kMaxTaps); kk < W; ++kk) {
-            const int row = n < N ? NMAX + kk - depth[s2] : 0;
-            tab.ext[par][kk - kMaxTaps][n] = (unsigned short)(row * 128 + ((row & 7) << 4));
-          }
-        }
-      }
       __syncwarp();
       if (t + 1 < nloc) load_par(t + 1, pn0, pn1);           // in flight during the waits and the writes below
-
-      // ---- the selection matrices and the window rows of unit t - 1 have been consumed      __syncwarp();
 
       // ---- the selection matrices and the window rows of unit t - 1 have been consumed (and with them everything
       //      issued before: this parity's tables were last read two units ago) ----
       if (t >= 1) ok = ok && mbar_wait(bar[B_SG], (t - 1) & 1, abort);
-      // with more than four taps group Y reads the window rows and the V copy of unit t - 1 as well
-      if (EXT && t >= 1) ok = ok && mbar_wait(bar[B_XT], (t - 1) & 1, abort);
       ok = __all_sync(0xffffffffu, ok);
       if (ok) {
-        if (lane == 0) tab.bad[par] = bad_any ? 1 : 0;
+        if (lane < 2) tab.bad[par][lane] = bad_any ? 1 : 0;
 #pragma unroll
         for (int s2 = 0; s2 < 2; ++s2) {
           const int n = lane + 32 * s2;
@@ -418,34 +537,20 @@ verify_tc_kernel(const __grid_constant__ CUtensorMap ms, const __grid_constant__
         }
         // the window below the draft rows of both channel halves, newest row first: row NMAX + p holds the value
         // p + 1 steps behind the first draft token
-        if (!EXT) {
 #pragma unroll
-          for (int i = 0; i < 6; ++i) {
-            const int idx = lane + 32 * i, p = (W - 2) - (idx >> 6), c2 = (idx & 63) * 2;
-            if (idx < 64 * (W - 1))
-              *reinterpret_cast<uint32_t*>(smem + OFF_V + (c2 >> 6) * V_BOX + swz(NMAX + p, (c2 & 63) >> 3) + (c2 & 7) * 2) = wv[i];
-          }
-        } else {
-          for (int base = 0; base < wtotal; base += 256) {
-            if (base > 0) {
-#pragma unroll
-              for (int i = 0; i < 8; ++i)
-                if (base + lane + 32 * i < wtotal) wq[i] = wsrc[base + lane + 32 * i];
-            }
-#pragma unroll
-            for (int i = 0; i < 8; ++i) {
-              const int idx = base + lane + 32 * i;          // row idx >> 4 of the window (oldest first), channels 8 (idx & 15) ...
-              if (idx < wtotal)
-                *reinterpret_cast<uint4*>(smem + OFF_V + ((idx & 15) >> 3) * V_BOX + swz(NMAX + (W - 2) - (idx >> 4), idx & 7)) = wq[i];
-            }
-          }
+        for (int i = 0; i < 6; ++i) {
+          const int idx = lane + 32 * i, p = (W - 2) - (idx >> 6), c2 = (idx & 63) * 2;
+          if (idx < 64 * (W - 1))
+            *reinterpret_cast<uint32_t*>(smem + OFF_V + (c2 >> 6) * V_BOX + swz(NMAX + p, (c2 & 63) >> 3) + (c2 & 7) * 2) = wv[i];
         }
       }
       proxy_fence();
       mbar_arrive(bar[B_XDONE0 + par]);
     }
+  }
   } else if (warp < 8) {
     // =============================== group X: phi(q), phi(k) and the bf16 copy of S of unit t ===============================
+    if (EXT) regs_down<kRegsX>();
     bool ok = true;
     uint2 pq[8], pk[8];
     float4 z4;
@@ -515,23 +620,20 @@ verify_tc_kernel(const __grid_constant__ CUtensorMap ms, const __grid_constant__
       mbar_arrive(bar[B_XDONE0 + par]);
       if (t + 1 < nloc) load_qk(t + 1);                      // in flight during the conversion below
 
-      // ---- S of unit t has landed: round it to bf16 in the operand layout (rows = features, channels contiguous) ----
-      ok = ok && mbar_wait(bar[B_FULL_S], par, abort);
-      ok = __all_sync(0xffffffffu, ok);
-      if (ok) {
+      if (!EXT) {                                            // S of unit t has landed: round it to bf16
+        ok = ok && mbar_wait(bar[B_FULL_S], par, abort);
+        ok = __all_sync(0xffffffffu, ok);
+        if (ok) {
 #pragma unroll 8
-        for (int it = 0; it < 16; ++it) {
-          const int a = warp + 8 * it;                         // row a, channels 4 lane .. 4 lane + 3
-          const float4 s4 = *reinterpret_cast<const float4*>(smem + OFF_S + a * 512 + lane * 16);
-          *reinterpret_cast<uint2*>(smem + OFF_SB + (lane >> 4) * SB_BOX + swz(a, (lane & 15) >> 1) + (lane & 1) * 8) =
-              make_uint2(pack2(s4.x, s4.y), pack2(s4.z, s4.w));
+          for (int it = 0; it < 16; ++it) round_s(warp + 8 * it);
         }
+        proxy_fence();
+        mbar_arrive(bar[B_SCONV]);
       }
-      proxy_fence();
-      mbar_arrive(bar[B_SCONV]);
     }
-  } else if (warp < 16) {
+  } else {
     // =============================== group Y: finish unit t ===============================
+    if (EXT) regs_up<kRegsY>();
     const int ty = tid - kThreadsX, wy = warp - 8;
     const int q4 = wy & 3;                                   // this warp reads TMEM lanes 32 q4 .. 32 q4 + 31
     const int c = 32 * q4 + lane, n0 = 32 * (wy >> 2);       // epilogue: channel c, nodes n0 .. n0 + 31
@@ -552,10 +654,11 @@ verify_tc_kernel(const __grid_constant__ CUtensorMap ms, const __grid_constant__
           wext[e] = wh[(e & (D - 1)) * W + (e >> 7)];
       }
 
+      if (EXT) ok = ok && mbar_wait(bar[B_TREE0 + par], (t >> 1) & 1, abort);
       ok = ok && mbar_wait(bar[B_XDONE0 + par], (t >> 1) & 1, abort) && mbar_wait(bar[B_P], par, abort);
       ok = __all_sync(0xffffffffu, ok);
       tc_fence_after();
-      const bool good = ok && tab.bad[par] == 0;
+      const bool good = ok && (tab.bad[par][0] | tab.bad[par][1]) == 0;
       // ---- scores under the tree mask: lane = node n, this warp's half of the columns m ----
       if (good && q4 < 2) {
         const int n = 32 * q4 + lane, hc = wy >> 2;
@@ -766,7 +869,7 @@ cudaError_t launch_verify_tc(la_ctx* ctx, int B, int N, const void* q, const voi
   const uint32_t smem = vtc::smem_bytes(c.conv_taps);
   cudaError_t e = allow_smem((const void*)kern, ctx->device);
   if (e != cudaSuccess) return e;
-  e = launch_pdl(kern, dim3(std::min(BH, ctx->sm_count)), dim3(vtc::kThreads), smem, s, ms, mv,
+  e = launch_pdl(kern, dim3(std::min(BH, ctx->sm_count)), dim3(vtc::threads(c.conv_taps > vtc::kMaxTaps)), smem, s, ms, mv,
                  (const __nv_bfloat16*)q, (const __nv_bfloat16*)k, parent, w, (const float*)st.z,
                  (const __nv_bfloat16*)st.win, (__nv_bfloat16*)o, ctx->d_status, c.H, N, c.conv_taps, c.eps, BH);
   ctx->launches += 1;
