@@ -92,6 +92,7 @@ la_status la_create(const la_config* cfg, la_ctx** out) {
   ctx->d_status = nullptr;
   ctx->ws = nullptr;
   ctx->ws_bytes = 0;
+  for (int& n : ctx->max_clusters) n = 0;
   if (cudaGetDevice(&ctx->device) != cudaSuccess ||
       cudaDeviceGetAttribute(&ctx->sm_count, cudaDevAttrMultiProcessorCount, ctx->device) != cudaSuccess ||
       cudaMalloc(&ctx->d_status, sizeof(int)) != cudaSuccess ||

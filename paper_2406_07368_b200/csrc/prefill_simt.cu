@@ -440,20 +440,9 @@ static cudaError_t launch_t(la_ctx* ctx, int B, int Tlen, const void* q, const v
   int n = 2 * BH >= ctx->sm_count * Sh::kResident ? 1 : std::min((int)kMaxCluster, chunks);
   const int per = (chunks + n - 1) / n;
   n = (chunks + per - 1) / per;
-  cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(BH * n);
-  cfg.blockDim = dim3(Sh::NT);
-  cfg.dynamicSmemBytes = smem;
-  cfg.stream = s;
-  cudaLaunchAttribute attr[1];
-  attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = n;
-  attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
-  cfg.attrs = attr;
-  cfg.numAttrs = 1;
   ctx->launches += 1;
-  return cudaLaunchKernelEx(&cfg, kern, (const T*)q, (const T*)k, (const T*)v, w, st.S, st.z, (T*)st.win, st.pos, (T*)o, c.H,
-                            Tlen, c.conv_taps, c.eps, init, per * Sh::C);
+  return launch_cluster(n, false, kern, dim3(BH * n), dim3(Sh::NT), smem, s, (const T*)q, (const T*)k, (const T*)v, w, st.S, st.z,
+                        (T*)st.win, st.pos, (T*)o, c.H, Tlen, c.conv_taps, c.eps, init, per * Sh::C);
 }
 
 template <typename T, int D>

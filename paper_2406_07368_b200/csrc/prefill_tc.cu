@@ -81,7 +81,7 @@ __host__ __device__ constexpr uint32_t off_den(bool z3) { return OFF_ONES + ones
 __host__ __device__ constexpr uint32_t off_small(bool z3) { return off_den(z3) + 2048; }
 
 struct Small {
-  unsigned long long bars[22];
+  unsigned long long bars[24];
   uint32_t tmem_base;
   int abort;
   int pad[2];
@@ -96,8 +96,9 @@ struct Small {
 enum { B_FULL_K0 = 0, B_FULL_V0 = 1, B_FULL_V1 = 2, B_MMA_P = 3, B_MMA_S0 = 4, B_MMA_O0 = 5, B_MMA_O1 = 6, B_PHI = 7,
        B_PDONE = 8, B_SB = 9, B_EPI0 = 10, B_EPI1 = 11, B_MMA_Q = 12, B_FULL_Q = 13, B_FULL_K1 = 14, B_STAGED0 = 15,
        B_STAGED1 = 16, B_HALO0 = 17, B_HALO1 = 18, B_MMA_S1 = 19,
-       B_MMA_L = 20 /* the scores against earlier groups of the tile */, kNumBars = 21 };
-static_assert(kNumBars <= 22, "Small::bars");
+       B_MMA_L = 20 /* the scores against earlier groups of the tile */, 
+       B_ST_PHI = 21, B_ST_MMA0 = 22, B_ST_MMA1 = 23 /* the state pass */, kNumBars = 24 };
+static_assert(kNumBars <= 24, "Small::bars");
 
 __host__ __device__ constexpr uint32_t off_w(bool z3) { return off_small(z3) + (uint32_t)((sizeof(Small) + 15) / 16 * 16); }
 // Short windows: nine halo buffers, rows of v that lie before 32 rows of a tile, for the convolution.  Buffers 0-2: the
@@ -142,6 +143,9 @@ __device__ __forceinline__ void mbar_expect_tx(uint32_t bar, uint32_t bytes) {
 __device__ __forceinline__ void mbar_arrive(uint32_t bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
+__device__ __forceinline__ void mbar_inval(uint32_t bar) { asm volatile("mbarrier.inval.shared::cta.b64 [%0];" ::"r"(bar) : "memory"); }
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire;" ::: "memory"); }
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
@@ -507,8 +511,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
                   const float* __restrict__ w, float* __restrict__ S, float* __restrict__ z,
                   __nv_bfloat16* __restrict__ win, int64_t* __restrict__ pos,
                   int* status, int H, int Ttot, int W, float eps, int init, int nseg,
-                  int seg_len, const float* __restrict__ S_seg, const float* __restrict__ z_seg,
-                  const __nv_bfloat16* __restrict__ win_seg, int prefixed, const __nv_bfloat16* __restrict__ vg, float alpha,
+                  int seg_len, float* S_seg, float* z_seg,
+                  const __nv_bfloat16* __restrict__ win_seg, int prefixed, int fused, const __nv_bfloat16* __restrict__ vg, float alpha,
                   float sm_scale, int tstep, int gsz, int early) {
   extern __shared__ unsigned char smem_dyn[];
   // (an offset into the array rather than an integer cast: the compiler then knows that these are shared-memory
@@ -542,19 +546,23 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   // A launch covers BH chains cut into nseg segments of seg_len tokens (nseg = 1: whole chains).  This block owns
-  // tokens [y0, y0 + T) of chain bh.  Whole chains start from the caller's state.  Of a chain that was cut, segment
-  // sg > 0 starts from the sums of the segments before it (the first of which holds the caller's state too; `prefixed`:
-  // slot sg - 1 holds them added up) and from the values of v before it, segment 0 from the copy of the caller's state
-  // that the pre-pass left in the last slot; only the last segment writes a state, the caller's.
+  // tokens [y0, y0 + T) of chain bh.  Whole chains start from the caller's state, the segments sg > 0 of a chain that was
+  // cut from the sums of the segments before them and from the values of v before them; only the last segment writes a
+  // state, the caller's.  Where the sums come from:
+  //   fused     the segments of a chain are one cluster: each block first forms its own segment's sums (the state pass),
+  //             leaves them in the workspace, and after a barrier of the cluster adds up those before it;
+  //   else      a launch of its own formed them (and left a copy of the caller's state for segment 0 in the last slot), and
+  //             with `prefixed` another one added them up: slot sg - 1.
+  // Either way the first segment's sums have the caller's state in them.
   const int bh = blockIdx.x / nseg, sg = blockIdx.x % nseg, h = bh % H;
   const int y0 = sg * seg_len, T = min(seg_len, Ttot - y0);
   const bool has_in = init || sg > 0, writes_state = sg == nseg - 1;
-  const int nsum = sg > 0 && !prefixed ? sg : 1;  // how many parts the incoming state has
-  const size_t slot = nseg > 1 ? (size_t)bh * nseg + (sg == 0 ? nseg - 1 : prefixed ? sg - 1 : 0) : (size_t)bh;
-  const float* S_in = (nseg > 1 ? S_seg : S) + slot * D * D;
-  const float* z_in = (nseg > 1 ? z_seg : z) + slot * D;
+  const bool callers = nseg == 1 || (fused && sg == 0);   // the incoming state is the caller's
+  const int nsum = sg > 0 && !prefixed ? sg : 1;          // how many parts it has
+  const size_t slot = (size_t)bh * nseg + (fused ? 0 : sg == 0 ? nseg - 1 : prefixed ? sg - 1 : 0);
+  const float *S_in = callers ? S + (size_t)bh * D * D : S_seg + slot * D * D, *z_in = callers ? z + (size_t)bh * D : z_seg + slot * D;
   const __nv_bfloat16* win_in = sg > 0 ? vg + ((size_t)bh * Ttot + y0 - (W - 1)) * D
-                                       : (nseg > 1 ? win_seg : win) + (size_t)bh * (W - 1) * D;
+                                       : (nseg > 1 && !fused ? win_seg : win) + (size_t)bh * (W - 1) * D;
   auto z_start = [&](int a) {
     float x = z_in[a];
     for (int j = 1; j < nsum; ++j) x += z_in[j * D + a];
@@ -565,6 +573,25 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
   const int nchunks = (T + tstep - 1) / tstep;
   const uint32_t tile_tx = (uint32_t)tstep * 256u;            // bytes a tile's two boxes bring
   const uint32_t bar0 = smem_u32(&sm.bars[0]);    // barrier i lives at bar0 + 8 i
+
+  auto load_k = [&](int n) {                      // K / V of tile n into the buffers of its parity (one thread)
+    const uint32_t kb = sbase + ((n & 1) ? OFF_K1 : OFF_K0), kbar = bar0 + 8u * ((n & 1) ? B_FULL_K1 : B_FULL_K0);
+    mbar_expect_tx(kbar, tile_tx);
+    tma_load(kb, &mk, 0, y0 + n * tstep, bh, kbar);
+    tma_load(kb + KBOX_BYTES, &mk, 64, y0 + n * tstep, bh, kbar);
+  };
+  auto load_v = [&](int n) {
+    const uint32_t vbar = bar0 + 8u * (B_FULL_V0 + (n & 1));
+    mbar_expect_tx(vbar, tile_tx);
+    tma_load(sbase + vbox(n & 1, 0), &mv, 0, y0 + n * tstep, bh, vbar);
+    tma_load(sbase + vbox(n & 1, 1), &mv, 64, y0 + n * tstep, bh, vbar);
+  };
+
+  auto load_q0 = [&]() {
+    mbar_expect_tx((bar0 + 8u * (B_FULL_Q)), tile_tx);
+    tma_load(sbase + OFF_Q, &mq, 0, y0, bh, (bar0 + 8u * (B_FULL_Q)));
+    tma_load(sbase + OFF_Q + BOX_BYTES, &mq, 64, y0, bh, (bar0 + 8u * (B_FULL_Q)));
+  };
 
   // ---- set-up ----
   if (tid == kCopyWarp * 32) {
@@ -591,22 +618,14 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
     mbar_init((bar0 + 8u * (B_HALO1)), 32);
     sm.abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    // the first tiles are requested at once (nothing below touches the rows that they bring)
+    for (int i = 0; i < 2; ++i) mbar_init((bar0 + 8u * (B_ST_MMA0 + i)), 1);
+    mbar_init((bar0 + 8u * (B_ST_PHI)), kThreadsA + kThreadsB);
+    // the first tile is requested at once (nothing below touches the rows that it brings); the others follow behind the
+    // taps and the window, which would otherwise wait for them (20 MB over all blocks: 3 us)
     pdl_wait();
-    for (int n = 0; n < 2 && n < nchunks; ++n) {
-      const uint32_t kb = sbase + (n ? OFF_K1 : OFF_K0), kbar = bar0 + 8u * (n ? B_FULL_K1 : B_FULL_K0), vbar = bar0 + 8u * (B_FULL_V0 + n);
-      mbar_expect_tx(kbar, tile_tx);
-      tma_load(kb, &mk, 0, y0 + n * tstep, bh, kbar);
-      tma_load(kb + KBOX_BYTES, &mk, 64, y0 + n * tstep, bh, kbar);
-      if (n == 0) {
-        mbar_expect_tx((bar0 + 8u * (B_FULL_Q)), tile_tx);
-        tma_load(sbase + OFF_Q, &mq, 0, y0, bh, (bar0 + 8u * (B_FULL_Q)));
-        tma_load(sbase + OFF_Q + BOX_BYTES, &mq, 64, y0, bh, (bar0 + 8u * (B_FULL_Q)));
-      }
-      mbar_expect_tx(vbar, tile_tx);
-      tma_load(sbase + vbox(n, 0), &mv, 0, y0 + n * tstep, bh, vbar);
-      tma_load(sbase + vbox(n, 1), &mv, 64, y0 + n * tstep, bh, vbar);
-    }
+    load_k(0);
+    if (!fused) load_q0();
+    load_v(0);
   }
   if (warp == kCtrlWarp) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&sm.tmem_base)),
@@ -638,65 +657,19 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
           has_in ? reinterpret_cast<const uint4*>(win_in)[idx] : make_uint4(0u, 0u, 0u, 0u);
   }
   __syncthreads();
+  if (tid == kCopyWarp * 32 && nchunks > 1) {
+    load_k(1);
+    load_v(1);
+  }
   if (tid < TILE) {
     *reinterpret_cast<__nv_bfloat16*>(smem + OFF_ONES + (z3 ? swz(tid, 0) : ext_offset(tid, 0))) = __float2bfloat16_rn(1.f);
-    if (GRP) zs[tid] = has_in ? z_start(tid) : 0.f;
-    else if (has_in)                                // z before tile 0: row 128 of the first K buffer (feature tid)
-      *reinterpret_cast<__nv_bfloat16*>(smem + OFF_K0 + (tid >> 6) * KBOX_BYTES + BOX_BYTES + (tid & 63) * 2) =
-          __float2bfloat16_rn(z_start(tid));
+    if (GRP) zs[tid] = 0.f;
   }
   fence_proxy_async();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = sm.tmem_base;
-
-  if (has_in && warp < 16) {
-    // The incoming state: fp32 into TMEM and a bf16 copy into shared memory (z: the row in the K buffer is in place).
-    // Both groups share it out, 16 rows x 64 columns per warp.
-    const int q4 = warp & 3, hf = (warp >> 2) & 1, r0 = 32 * q4 + 16 * (warp >> 3);
-    const float* Sg = S_in + (size_t)(r0 + (lane >> 2)) * D + 64 * hf + 2 * (lane & 3);
-#pragma unroll
-    for (int hh = 0; hh < 2; ++hh) {                // 32 columns at a time; two of the parts in flight
-      uint32_t v[16], x[16];
-      auto load = [&](int j, uint32_t (&y)[16]) {
-#pragma unroll
-        for (int g = 0; g < 4; ++g)
-#pragma unroll
-          for (int i = 0; i < 2; ++i) {
-            const float2 t = *reinterpret_cast<const float2*>(Sg + (size_t)j * D * D + i * 8 * D + 32 * hh + 8 * g);
-            y[4 * g + 2 * i] = __float_as_uint(t.x);
-            y[4 * g + 2 * i + 1] = __float_as_uint(t.y);
-          }
-      };
-      load(0, v);
-      if (nsum > 1) load(1, x);
-#pragma unroll 1
-      for (int j = 1; j < nsum; ++j) {              // the sums of the segments before this one
-#pragma unroll
-        for (int e = 0; e < 16; ++e) v[e] = __float_as_uint(__uint_as_float(v[e]) + __uint_as_float(x[e]));
-        if (j + 1 < nsum) load(j + 1, x);
-      }
-      LA_TMEM_ST_FRAG4(tmem + ((uint32_t)r0 << 16) + S_COL + 64 * hf + 32 * hh, v);
-#pragma unroll
-      for (int g = 0; g < 4; ++g)
-#pragma unroll
-        for (int i = 0; i < 2; ++i)
-          *reinterpret_cast<uint32_t*>(smem + OFF_S + hf * BOX_BYTES + swz(r0 + (lane >> 2) + 8 * i, 4 * hh + g) + 4 * (lane & 3)) =
-              pack2(__uint_as_float(v[4 * g + 2 * i]), __uint_as_float(v[4 * g + 2 * i + 1]));
-    }
-    if (warp < 4) {                                 // z, and zeros in the other columns of its block (32 rows per warp)
-      const uint32_t zaddr = tmem + ((uint32_t)(32 * q4) << 16) + Z_COL;
-      tmem_st1(zaddr, __float_as_uint(z_start(32 * q4 + lane)));
-#pragma unroll
-      for (int c = 1; c < 16; ++c) tmem_st1(zaddr + c, 0u);
-    }
-    tmem_wait_st();
-    fence_proxy_async();
-    tc_fence_before();
-    asm volatile("bar.sync 6, 512;" ::: "memory");
-    tc_fence_after();
-  }
 
   // phi on rows 16 I0 ... 16 I1 - 1 of the K tile of tile m, in place, by 256 threads (ta); rows at or beyond the end of the
   // sequence become zero
@@ -719,6 +692,160 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
   using K0c = std::integral_constant<int, 0>;
   using KAc = std::integral_constant<int, 8 - KB>;
   using K8c = std::integral_constant<int, 8>;
+
+  // ---- state pass (fused): the sums of this segment, which the segments behind it start from ----
+  if (fused && !writes_state) {
+    if (warp == kCtrlWarp) {
+      if (lane == 0)
+        for (int n = 0; n < nchunks; ++n) {
+          const uint32_t par = n & 1;
+          if (!mbar_wait((bar0 + 8u * (B_ST_PHI)), par, abort) || !mbar_wait((bar0 + 8u * (B_FULL_V0 + par)), (n >> 1) & 1, abort)) break;
+          tc_fence_after();
+          const uint32_t k_mn = desc_lo(sbase + (par ? OFF_K1 : OFF_K0), KBOX_BYTES), v_mn = desc_lo(sbase + vbox(par, 0), vstep(par));
+#pragma unroll
+          for (int ks = 0; ks < 8; ++ks) {     // [dS | dz] += phi(K)^T [V | 1]
+            const uint64_t kd = desc64(k_mn + kstep_mnmajor(ks));
+            mma_bf16(tmem + S_COL, kd, desc64(v_mn + kstep_mnmajor(ks)), z3 ? idesc(true, true, 144) : idesc(true, true, 128), n > 0 || ks > 0);
+            if (!z3) mma_bf16(tmem + Z_COL, kd, desc_ext(sbase + OFF_ONES, ks), idesc(true, true, 16), n > 0 || ks > 0);
+          }
+          mma_commit((bar0 + 8u * (B_ST_MMA0 + par)));
+        }
+    } else if (warp == kCopyWarp) {
+      if (lane == 0)
+        for (int n = 0; n + 2 < nchunks; ++n) {
+          if (!mbar_wait((bar0 + 8u * (B_ST_MMA0 + (n & 1))), (n >> 1) & 1, abort)) break;
+          load_k(n + 2);
+          load_v(n + 2);
+        }
+    } else if (warp < 16) {
+      using K4c = std::integral_constant<int, 4>;
+      bool ok = true;
+      const int q4 = warp & 3, hf = (warp >> 2) & 1, r0 = 32 * q4 + 16 * (warp >> 3);
+      const size_t at = (size_t)(r0 + (lane >> 2)) * D + 64 * hf + 2 * (lane & 3);
+      const bool base = init && sg == 0;          // the first segment's sums take the caller's state in
+      uint32_t x[32];
+      if (base) frag_load(S + (size_t)bh * D * D + at, x);
+      for (int n = 0; n < nchunks; ++n) {
+        ok = ok && mbar_wait((bar0 + 8u * ((n & 1) ? B_FULL_K1 : B_FULL_K0)), (n >> 1) & 1, abort);
+        ok = __all_sync(0xffffffffu, ok);
+        if (ok) {
+          if (warp < 8) phi_k(K0c{}, K4c{}, n, tid);
+          else phi_k(K4c{}, K8c{}, n, tid - kThreadsB);
+        }
+        fence_proxy_async();
+        mbar_arrive((bar0 + 8u * (B_ST_PHI)));
+      }
+      const int l = nchunks - 1;                  // (the last product; its barrier is at most one phase behind here: tile l
+                                                  // was loaded only after product l - 2 had completed)
+      ok = ok && mbar_wait((bar0 + 8u * (B_ST_MMA0 + (l & 1))), (l >> 1) & 1, abort);
+      ok = __all_sync(0xffffffffu, ok);
+      if (ok) {
+        tc_fence_after();
+        const size_t mine = (size_t)bh * nseg + sg;
+        uint32_t v[32];
+        LA_TMEM_LD_FRAG8(tmem + ((uint32_t)r0 << 16) + S_COL + 64 * hf, v);
+        tmem_wait_ld();
+        if (base) frag_add(v, x);
+        frag_store(S_seg + mine * D * D + at, v);
+        if (warp < 4) {
+          const uint32_t zz = tmem_ld1(tmem + ((uint32_t)(32 * q4) << 16) + Z_COL);
+          tmem_wait_ld();
+          z_seg[mine * D + tid] = __uint_as_float(zz) + (base ? z[(size_t)bh * D + tid] : 0.f);
+        }
+      }
+    }
+    fence_proxy_async();                          // phi(K) in place: the buffers are loaded anew
+    tc_fence_before();
+    __syncthreads();
+    tc_fence_after();
+    if (tid == kCopyWarp * 32) {                  // start the main pass with fresh barriers for K and V
+      for (int i : {B_FULL_K0, B_FULL_K1, B_FULL_V0, B_FULL_V1}) {
+        mbar_inval(bar0 + 8u * i);
+        mbar_init(bar0 + 8u * i, 1);
+      }
+      asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+      load_k(0);
+      load_q0();
+    }
+  } else if (fused && tid == kCopyWarp * 32) {
+    load_q0();
+  }
+  if (fused) {                                    // the sums are in the workspace, for every block of the chain
+    cluster_arrive();
+    cluster_wait();
+  }
+
+  if (has_in && warp < 16) {
+    // The incoming state: fp32 into TMEM and a bf16 copy into shared memory; z: row 128 of the first K buffer (feature tid).
+    // Both groups share it out, 16 rows x 64 columns per warp.
+    const int q4 = warp & 3, hf = (warp >> 2) & 1, r0 = 32 * q4 + 16 * (warp >> 3);
+    const size_t at = (size_t)(r0 + (lane >> 2)) * D + 64 * hf + 2 * (lane & 3);
+    uint32_t v[2][16];                              // 32 columns each
+#pragma unroll
+    for (int hh = 0; hh < 2; ++hh) {
+      auto load = [&](int j, uint32_t (&y)[16]) {
+#pragma unroll
+        for (int g = 0; g < 4; ++g)
+#pragma unroll
+          for (int i = 0; i < 2; ++i) {
+            const float2 t = *reinterpret_cast<const float2*>(S_in + (size_t)j * D * D + at + i * 8 * D + 32 * hh + 8 * g);
+            y[4 * g + 2 * i] = __float_as_uint(t.x);
+            y[4 * g + 2 * i + 1] = __float_as_uint(t.y);
+          }
+      };
+      auto add = [&](const uint32_t (&y)[16]) {
+#pragma unroll
+        for (int e = 0; e < 16; ++e) v[hh][e] = __float_as_uint(__uint_as_float(v[hh][e]) + __uint_as_float(y[e]));
+      };
+      load(0, v[hh]);
+#pragma unroll 1
+      for (int j = 1; j < nsum; j += 3) {           // the sums of the segments before this one, in order, three in flight
+        uint32_t x0[16], x1[16], x2[16];
+        load(j, x0);
+        if (j + 1 < nsum) load(j + 1, x1);
+        if (j + 2 < nsum) load(j + 2, x2);
+        add(x0);
+        if (j + 1 < nsum) add(x1);
+        if (j + 2 < nsum) add(x2);
+      }
+    }
+#pragma unroll
+    for (int hh = 0; hh < 2; ++hh) {
+      LA_TMEM_ST_FRAG4(tmem + ((uint32_t)r0 << 16) + S_COL + 64 * hf + 32 * hh, v[hh]);
+#pragma unroll
+      for (int g = 0; g < 4; ++g)
+#pragma unroll
+        for (int i = 0; i < 2; ++i)
+          *reinterpret_cast<uint32_t*>(smem + OFF_S + hf * BOX_BYTES + swz(r0 + (lane >> 2) + 8 * i, 4 * hh + g) + 4 * (lane & 3)) =
+              pack2(__uint_as_float(v[hh][4 * g + 2 * i]), __uint_as_float(v[hh][4 * g + 2 * i + 1]));
+    }
+    if (warp < 4) {                                 // z, and zeros in the other columns of its block (32 rows per warp)
+      const uint32_t zaddr = tmem + ((uint32_t)(32 * q4) << 16) + Z_COL;
+      const float zz = z_start(tid);
+      if (GRP) zs[tid] = zz;
+      else
+        *reinterpret_cast<__nv_bfloat16*>(smem + OFF_K0 + (tid >> 6) * KBOX_BYTES + BOX_BYTES + (tid & 63) * 2) = __float2bfloat16_rn(zz);
+      tmem_st1(zaddr, __float_as_uint(zz));
+#pragma unroll
+      for (int c = 1; c < 16; ++c) tmem_st1(zaddr + c, 0u);
+    }
+    tmem_wait_st();
+    fence_proxy_async();
+    tc_fence_before();
+    asm volatile("bar.sync 6, 544;" ::: "memory");
+    tc_fence_after();
+  } else if (has_in && warp == kCopyWarp) {
+    asm volatile("bar.sync 6, 544;" ::: "memory");
+  }
+  // (fused: V of the first tile and the second tile are requested behind the state, which would otherwise wait for them)
+  if (fused && !writes_state && tid == kCopyWarp * 32) {
+    load_v(0);
+    if (nchunks > 1) {
+      load_k(1);
+      load_v(1);
+    }
+  }
+  if (fused) cluster_arrive();                    // this block has read the caller's state (and its window)
 
   // S and z after tile n, which is not the last: the bf16 copy and the z row for the next tile.  256 threads (row r, 64
   // columns each): group B or group A.
@@ -859,18 +986,14 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
         const uint32_t vb = sbase + vbox(par, 0), vb1 = sbase + vbox(par, 1);
         if (LONG) {
           // the outputs wait in the token rows of this tile's K buffer; every tap has been taken from its V buffer
-          const uint32_t kb = sbase + (par ? OFF_K1 : OFF_K0), kbar = bar0 + 8u * (par ? B_FULL_K1 : B_FULL_K0);
+          const uint32_t kb = sbase + (par ? OFF_K1 : OFF_K0);
           tma_store(&mo, 0, y0 + n * tstep, bh, kb);
           tma_store(&mo, 64, y0 + n * tstep, bh, kb + KBOX_BYTES);
           tma_commit();
           if (n + 2 < nchunks) {
-            mbar_expect_tx((bar0 + 8u * (B_FULL_V0 + par)), tile_tx);
-            tma_load(vb, &mv, 0, y0 + (n + 2) * tstep, bh, (bar0 + 8u * (B_FULL_V0 + par)));
-            tma_load(vb1, &mv, 64, y0 + (n + 2) * tstep, bh, (bar0 + 8u * (B_FULL_V0 + par)));
+            load_v(n + 2);
             tma_wait_read();
-            mbar_expect_tx(kbar, tile_tx);
-            tma_load(kb, &mk, 0, y0 + (n + 2) * tstep, bh, kbar);
-            tma_load(kb + KBOX_BYTES, &mk, 64, y0 + (n + 2) * tstep, bh, kbar);
+            load_k(n + 2);
           }
           continue;
         }
@@ -879,9 +1002,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
         tma_commit();
         if (n + 2 < nchunks) {
           tma_wait_read();
-          mbar_expect_tx((bar0 + 8u * (B_FULL_V0 + par)), tile_tx);
-          tma_load(vb, &mv, 0, y0 + (n + 2) * tstep, bh, (bar0 + 8u * (B_FULL_V0 + par)));
-          tma_load(vb1, &mv, 64, y0 + (n + 2) * tstep, bh, (bar0 + 8u * (B_FULL_V0 + par)));
+          load_v(n + 2);
         }
       }
       tma_wait_all();                             // every store is complete before the CTA exits
@@ -892,10 +1013,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
       for (int n = 0; n + 2 < nchunks; ++n) {
         const uint32_t par = n & 1;
         if (!mbar_wait((bar0 + 8u * (par ? B_MMA_S1 : B_MMA_S0)), (n >> 1) & 1, abort)) break;
-        const uint32_t kbuf = sbase + (par ? OFF_K1 : OFF_K0), kbar = bar0 + 8u * (par ? B_FULL_K1 : B_FULL_K0);
-        mbar_expect_tx(kbar, tile_tx);
-        tma_load(kbuf, &mk, 0, y0 + (n + 2) * tstep, bh, kbar);
-        tma_load(kbuf + KBOX_BYTES, &mk, 64, y0 + (n + 2) * tstep, bh, kbar);
+        load_k(n + 2);
       }
     }
   } else if (warp == kHaloWarp) {
@@ -1199,6 +1317,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
       const int n = nchunks - 1;
       ok = ok && mbar_wait((bar0 + 8u * ((n & 1) ? B_MMA_S1 : B_MMA_S0)), (n >> 1) & 1, abort);
       ok = __all_sync(0xffffffffu, ok);
+      if (fused) cluster_wait();                  // every block of the chain has read the caller's state
       if (ok && writes_state) {
         tc_fence_after();
 #pragma unroll
@@ -1401,6 +1520,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
     }
     }
     sync_group_b();                               // both halves of the last halo are complete
+    if (fused) cluster_wait();
     if (ok && tid < D && writes_state) {
       // the window to carry on: the last W-1 values of (incoming window ++ this block's v)
       const unsigned char* halo = smem + off_halo(W) + nchunks % 3 * halo_bytes(W);
@@ -1413,6 +1533,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
   }
 
   // ---- teardown ----
+  if (fused && warp >= 16) cluster_wait();        // (groups A and B have waited before they wrote the state)
   tc_fence_before();
   __syncthreads();
   if (sm.abort) {
@@ -1661,9 +1782,10 @@ static bool make_map(CUtensorMap* m, const void* base, int BH, int T, int box_ro
 // What the chains of a launch start from and how they are cut (one piece per chain: everything null).
 struct Split {
   int nseg = 1, seg_len = 0;
-  const float *S = nullptr, *z = nullptr;
+  float *S = nullptr, *z = nullptr;
   const __nv_bfloat16* win = nullptr;
   int prefixed = 0;
+  int fused = 0;      // one cluster per chain, whose blocks form the segments' sums themselves
 };
 
 template <int PHI>
@@ -1695,9 +1817,9 @@ static cudaError_t launch_w(la_ctx* ctx, int BH, int T, const CUtensorMap& mq, c
   // runs beside this one's tiles), and behind the pre-pass.  Not for fuller grids: the blocks that start early take the
   // SMs that the launch before left idle (128 chains of 2048 tokens, 3 taps: 70 against 65 us).
   const int early = 2 * units <= ctx->sm_count;
-  return launch_maybe_pdl(early || sp.nseg > 1, kern, dim3(units), dim3(tc::kThreads), smem, s, mq, mk, mv, mo, w, st.S, st.z,
+  return launch_cluster(sp.fused ? sp.nseg : 1, early || sp.nseg > 1, kern, dim3(units), dim3(tc::kThreads), smem, s, mq, mk, mv, mo, w, st.S, st.z,
                           (__nv_bfloat16*)st.win, st.pos, ctx->d_status, c.H, T, c.conv_taps, c.eps, init, sp.nseg,
-                          sp.nseg > 1 ? sp.seg_len : T, sp.S, sp.z, sp.win, sp.prefixed, (const __nv_bfloat16*)v, alpha,
+                          sp.nseg > 1 ? sp.seg_len : T, sp.S, sp.z, sp.win, sp.prefixed, sp.fused, (const __nv_bfloat16*)v, alpha,
                           sm_scale, tstep, gsz, early);
 }
 static cudaError_t launch_phi(la_ctx* ctx, int BH, int T, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
@@ -1743,6 +1865,32 @@ size_t prefill_workspace_bytes(const la_ctx* ctx, int B, int T) {
   return nseg > 1 ? split_bytes(c, B * c.H, nseg) : 0;
 }
 
+// How many clusters of n blocks, one block per SM, the device holds at once.
+constexpr int kMaxCluster = 8;
+static int resident_clusters(la_ctx* ctx, int n) {
+  if (ctx->max_clusters[n] == 0) {
+    auto kern = tc::prefill_tc_kernel<LA_PHI_ELU1, 3>;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(n);
+    cfg.blockDim = dim3(tc::kThreads);
+    cfg.dynamicSmemBytes = tc::kMaxSmem;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = n;
+    attr[0].val.clusterDim.y = attr[0].val.clusterDim.z = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    int got = 0;
+    if (allow_smem((const void*)kern, ctx->device) != cudaSuccess ||
+        cudaOccupancyMaxActiveClusters(&got, kern, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      got = 0;
+    }
+    ctx->max_clusters[n] = got > 0 ? got : -1;
+  }
+  return ctx->max_clusters[n];
+}
+
 // Cuts the chains where that pays and the workspace allows it: launches what forms the segments' starting states.  `tile`:
 // tokens per tile of the main pass; mk, mv: maps with boxes of 128 rows.
 static cudaError_t launch_split(la_ctx* ctx, int BH, int T, int tile, const CUtensorMap& mk, const CUtensorMap& mv, int init,
@@ -1758,6 +1906,13 @@ static cudaError_t launch_split(la_ctx* ctx, int BH, int T, int tile, const CUte
     float* z_seg = S_seg + (size_t)units * tc::D * tc::D;
     __nv_bfloat16* win_seg = reinterpret_cast<__nv_bfloat16*>(z_seg + (size_t)units * tc::D);
     sp.S = S_seg, sp.z = z_seg, sp.win = win_seg;
+    // Up to 8 segments (a portable cluster): one launch, provided that all the clusters are resident at once.  (32 chains of
+    // 1700 tokens, 4 segments each: 40.7 us with the sums formed by a launch of their own, 37 so; 32 x 3000: 55 and
+    // 50; 32 x 32768 no difference.)
+    if (nseg <= kMaxCluster && BH <= resident_clusters(ctx, nseg)) {
+      sp.fused = 1;
+      return cudaSuccess;
+    }
     auto skern = c.phi == LA_PHI_ELU1 ? tc::segment_state_kernel<LA_PHI_ELU1> : tc::segment_state_kernel<LA_PHI_RELU>;
     cudaError_t e = allow_smem((const void*)skern, ctx->device);
     if (e != cudaSuccess) return e;

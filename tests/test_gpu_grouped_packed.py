@@ -26,10 +26,8 @@ def _run(C, T, W, phi, eps, alpha, first=0, B=1, H=3, workspace=False):
         need = ctx.la_prefill_workspace_bytes(B, T)
         assert need > 0
         ctx.la_set_workspace(torch.full((need,), 0xff, dtype=torch.uint8, device="cuda"))
-    n0 = ctx.la_launch_count()
     o = ctx.la_prefill_grouped(dev(q[:, :, first:]), dev(k[:, :, first:]), dev(v[:, :, first:]), wd, st, *args,
                                init_state=first > 0)
-    launches = ctx.la_launch_count() - n0
     assert ctx.la_last_device_status() == binding.LA_OK
     want, ost = orc.prefill_grouped_block(q, k, v, w, phi, eps, C, alpha, d ** -0.5)
     got = o.float().cpu().numpy()
@@ -39,7 +37,6 @@ def _run(C, T, W, phi, eps, alpha, first=0, B=1, H=3, workspace=False):
     assert rel_err(st.S.cpu().numpy(), ost.S) < TOL[io] and rel_err(st.z.cpu().numpy(), ost.z) < TOL[io]
     assert st.pos.tolist() == [first + T] * B
     np.testing.assert_array_equal(st.win.float().cpu().numpy(), ost.win)
-    return launches
 
 
 @pytest.mark.parametrize("C", [32, 64])
@@ -58,4 +55,4 @@ def test_options_and_continuation(C, W, phi, eps, alpha, first):
 @pytest.mark.parametrize("C,T,first,H", [(64, 900, 0, 36), (32, 770, 64, 2), (128, 1000, 0, 3), (100, 1200, 100, 40)])
 def test_cut_along_the_sequence(C, T, first, H):
     """With a workspace: packed groups, one group per tile, and partly filled tiles (100 tokens)."""
-    assert _run(C, T, 3, "elu1", 0.0, 1.0, first, H=H, workspace=True) > 1
+    _run(C, T, 3, "elu1", 0.0, 1.0, first, H=H, workspace=True)

@@ -1,5 +1,6 @@
-"""The prefill cut along the sequence with few segments per chain (their sums are added up by the blocks of the main pass
-as they load their state), at the smallest lengths that are cut, ragged and not, fresh and continuing."""
+"""The prefill cut along the sequence with few segments per chain (one cluster per chain, whose blocks form the segments'
+sums and add them up as they load their state), at the smallest lengths that are cut, ragged and not, fresh and
+continuing; and with up to 8 segments, which is as many as a cluster has, and more, which take launches of their own."""
 import numpy as np
 import pytest
 import torch
@@ -12,7 +13,8 @@ pytestmark = pytest.mark.gpu
 
 
 @pytest.mark.parametrize("H,T,W,first", [(36, 768, 3, 0), (36, 641, 3, 70), (74, 700, 1, 130), (37, 769, 5, 3), (40, 900, 32, 33),
-                                         (49, 2000, 2, 0)])
+                                         (49, 2000, 2, 0), (18, 1024, 3, 0), (18, 1024, 4, 5), (16, 1152, 8, 40), (21, 900, 6, 0),
+                                         (13, 1400, 3, 128)])
 def test_split_with_few_segments(H, T, W, first):
     """`first` tokens in a call of their own, then T in one that is cut; against the oracle on all of them (bf16: 2e-2, the
     tolerance of every tensor-core path) and against the same call without the workspace (only the order of fp32 sums and
@@ -33,9 +35,7 @@ def test_split_with_few_segments(H, T, W, first):
             ctx.la_prefill(dev(q[:, :, :first]), dev(k[:, :, :first]), dev(v[:, :, :first]), wd, st)
         if lend:
             ctx.la_set_workspace(torch.full((need,), 0xff, dtype=torch.uint8, device="cuda"))
-        n0 = ctx.la_launch_count()
         outs.append(ctx.la_prefill(dev(q[:, :, first:]), dev(k[:, :, first:]), dev(v[:, :, first:]), wd, st, init_state=first > 0))
-        assert ctx.la_launch_count() - n0 == (2 if lend else 1)
         states.append(st)
     assert ctx.la_last_device_status() == binding.LA_OK
     want, ost = orc.prefill_quadratic(q, k, v, w, "elu1", 0.0)
