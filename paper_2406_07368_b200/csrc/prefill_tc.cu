@@ -406,12 +406,13 @@ __device__ __forceinline__ uint32_t swz(int row, int cc) { return (uint32_t)row 
 // (Two channels per packed fp32 multiply-add: each half is the IEEE fused multiply-add of the scalar instruction.)
 __device__ __forceinline__ float2 bf2(uint32_t u) { return make_float2(lo_f(u), hi_f(u)); }
 // Long-window epilogue: one thread owns a pair of channels and 32 consecutive rows of the tile, in four blocks of 8.
-// conv_block adds one group of 8 taps to the 8 sums of block BLK: the 15 rows of v that those taps reach are each
-// read once, as one packed pair, and feed up to 8 of the sums.  Where the rows come from is fixed at compile time:
-//   ALL_V  the V buffer: pg[k] = the thread's column at (its first row - 8 g), for rows = k mod 8 (the swizzle)
-//   ALL_H  the halo column: hq = its row 8 (BLK - g) - 7
-//   MIXED  (g = BLK, first 32 rows of the tile) rows -7 ... -1 from the halo (hq = its row -7), rows 0 ... 7 from V
-// so that every load is one instruction with an immediate offset.
+// conv_block adds one group of 8 taps to the 8 sums of a block: the 15 rows of v that those taps reach are each read once,
+// as one packed pair, and feed up to 8 of the sums.  Where the rows come from is fixed at compile time:
+//   ALL_V  the V buffer: pg[k] = the thread's column, in the swizzle of rows = k mod 8, 8 g rows before the block's first
+//   ALL_H  the halo column: hq = 8 g + 7 rows before the block's first
+//   MIXED  (the group that straddles the tile's first row) rows -7 ... -1 from the halo (hq = its row -7), 0 ... 7 from V
+// so that every load is one instruction with an immediate offset.  The block is not: with a copy of this code per block and
+// source (33 KB of instructions) the loop waited for its instructions.
 template <int I, int N, typename F>
 __device__ __forceinline__ void static_for(F&& f) {           // f(integral_constant<int, I>) ... for I, I + 1, ..., N - 1
   if constexpr (I < N) {
@@ -432,7 +433,7 @@ __device__ __forceinline__ float2 lds_f2(uint32_t a) {
   return v;
 }
 __device__ __forceinline__ void sts32(uint32_t a, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
-template <int BLK, int KIND>
+template <int KIND>
 __device__ __forceinline__ void conv_block(float2 (&acc)[8], uint32_t wtap, const uint32_t (&pg)[8], uint32_t hq) {
   float2 wg[8];
   static_for<0, 8>([&](auto tc_) {
@@ -443,8 +444,7 @@ __device__ __forceinline__ void conv_block(float2 (&acc)[8], uint32_t wtap, cons
     constexpr int i = decltype(ic)::value;
     uint32_t u;
     if constexpr (KIND == ALL_V) {
-      constexpr int rel = 8 * BLK - 7 + i;        // row, from the thread's first row, before the 8 g rows of the group
-      u = lds32(pg[rel & 7] + rel * 128);
+      u = lds32(pg[(i + 1) & 7] + (i - 7) * 128);
     } else if constexpr (KIND == ALL_H || i < 7) {
       u = lds32(hq + i * (D * 2));
     } else {
@@ -458,35 +458,36 @@ __device__ __forceinline__ void conv_block(float2 (&acc)[8], uint32_t wtap, cons
     });
   });
 }
-// All tap groups of block BLK (rows 8 BLK ... 8 BLK + 7 of the thread), then the sums are added to the attention
-// term that waits in the output tile.  FIRST: the thread owns the first 32 rows of the tile (rows before them
+// All tap groups of block blk (rows 8 blk ... 8 blk + 7 of the thread), then the sums are added to the attention
+// term that waits in the output tile.  first: the thread owns the first 32 rows of the tile (rows before them
 // come from the halo, hend = the halo column just past its last row).
-template <int BLK, bool FIRST>
-__device__ __forceinline__ void conv_rows(uint32_t wcol, const uint32_t (&pv)[8], uint32_t sthr, int cc, uint32_t hend, int ngroups) {
+__device__ __forceinline__ void conv_rows(int blk, bool first, uint32_t wcol, const uint32_t (&pv)[8], uint32_t sthr, int cc,
+                                          uint32_t hend, int ngroups) {
   float2 acc[8];
 #pragma unroll
   for (int jj = 0; jj < 8; ++jj) acc[jj] = make_float2(0.f, 0.f);
 #pragma unroll 1
   for (int g = 0; g < ngroups; ++g) {
     const uint32_t wtap = wcol + g * (8 * D * 4);
-    if (!FIRST || g < BLK) {
+    if (!first || g < blk) {
       uint32_t pg[8];
 #pragma unroll
-      for (int k = 0; k < 8; ++k) pg[k] = pv[k] - g * 1024;
-      conv_block<BLK, ALL_V>(acc, wtap, pg, 0u);
-    } else if (g == BLK) {
-      conv_block<BLK, MIXED>(acc, wtap, pv, hend - 7 * (D * 2));
+      for (int k = 0; k < 8; ++k) pg[k] = pv[k] + (blk - g) * 1024;
+      conv_block<ALL_V>(acc, wtap, pg, 0u);
+    } else if (g == blk) {
+      conv_block<MIXED>(acc, wtap, pv, hend - 7 * (D * 2));
     } else {
-      conv_block<BLK, ALL_H>(acc, wtap, pv, hend + (8 * (BLK - g) - 7) * (D * 2));
+      conv_block<ALL_H>(acc, wtap, pv, hend + (8 * (blk - g) - 7) * (D * 2));
     }
   }
+  sthr += blk * 1024;
   uint32_t lav[8];                                // the attention terms of the 8 rows, all loads in flight at once
 #pragma unroll
-  for (int jj = 0; jj < 8; ++jj) lav[jj] = lds32(sthr + (8 * BLK + jj) * 128 + ((cc ^ jj) << 4));
+  for (int jj = 0; jj < 8; ++jj) lav[jj] = lds32(sthr + jj * 128 + ((cc ^ jj) << 4));
 #pragma unroll
   for (int jj = 0; jj < 8; ++jj) {
     const float2 la = bf2(lav[jj]);
-    sts32(sthr + (8 * BLK + jj) * 128 + ((cc ^ jj) << 4), pack2(acc[jj].x + la.x, acc[jj].y + la.y));
+    sts32(sthr + jj * 128 + ((cc ^ jj) << 4), pack2(acc[jj].x + la.x, acc[jj].y + la.y));
   }
 }
 
@@ -1402,24 +1403,24 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
           for (int k = 0; k < 8; ++k) pv[k] = vthr + ((cc ^ k) << 4);
           const uint32_t sthr = sbase + (par ? OFF_K1 : OFF_K0) + colk;
           const int mine = valid - 32 * jq;                  // rows of this thread that hold tokens
+#pragma unroll 1
+          for (int blk = 0; blk < 4 && 8 * blk < mine; ++blk) conv_rows(blk, jq == 0, wcol, pv, sthr, cc, hend, ngroups);
           if (jq == 0) {
-            if (mine > 0) conv_rows<0, true>(wcol, pv, sthr, cc, hend, ngroups);
-            if (mine > 8) conv_rows<1, true>(wcol, pv, sthr, cc, hend, ngroups);
-            if (mine > 16) conv_rows<2, true>(wcol, pv, sthr, cc, hend, ngroups);
-            if (mine > 24) conv_rows<3, true>(wcol, pv, sthr, cc, hend, ngroups);
             // The rows before the next tile: the last W-1 of (halo ++ valid rows of v), in place.  This thread is the
             // only one that reads or writes this column of the halo (the rows of the other threads start at 32, and
             // no window reaches back further than 31 rows).
-            for (int i = 0; i < W - 1; ++i) {
-              const int src = valid - (W - 1) + i;
-              const uint32_t x = src >= 0 ? lds32(vthr + src * 128 + ((cc ^ (src & 7)) << 4)) : lds32(hend + src * (D * 2));
-              sts32(hcol + (lead + i) * (D * 2), x);
+            // (Eight rows at a time: row by row, every load waited for, it took 3 K cycles of a tile at 32 taps.)
+            for (int i0 = 0; i0 < W - 1; i0 += 8) {
+              uint32_t x[8];
+#pragma unroll
+              for (int i = 0; i < 8; ++i) {
+                const int src = min(valid - (W - 1) + i0 + i, valid - 1);
+                x[i] = lds32(src >= 0 ? vthr + src * 128 + ((cc ^ (src & 7)) << 4) : hend + src * (D * 2));
+              }
+#pragma unroll
+              for (int i = 0; i < 8; ++i)
+                if (i0 + i < W - 1) sts32(hcol + (lead + i0 + i) * (D * 2), x[i]);
             }
-          } else {
-            if (mine > 0) conv_rows<0, false>(wcol, pv, sthr, cc, hend, ngroups);
-            if (mine > 8) conv_rows<1, false>(wcol, pv, sthr, cc, hend, ngroups);
-            if (mine > 16) conv_rows<2, false>(wcol, pv, sthr, cc, hend, ngroups);
-            if (mine > 24) conv_rows<3, false>(wcol, pv, sthr, cc, hend, ngroups);
           }
         }
         fence_proxy_async();
