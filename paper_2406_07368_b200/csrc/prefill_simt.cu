@@ -9,8 +9,8 @@
 // through distributed shared memory; then all segments run at once.  No workspace, one launch.  Cost: S += phi(K)^T V
 // of all but a segment's last chunk is formed twice (d^2 of about 3 d^2 + C d multiply-adds per token).
 //
-// What bounds it: fp32 multiply-adds and the shared-memory loads that feed them (two fifths of the fp32 peak on 48 chains
-// of 1000 tokens, d = 64: 67 us, where one CTA per chain that walked the tokens one by one took 520 us).  All products are register tiles (8 x 4 per thread at d = 64) fed by 128-bit
+// What bounds it: the latency of the shared-memory loads behind the multiply-adds at 12 warps per SM (two fifths of the
+// fp32 peak on 48 chains of 1000 tokens, d = 64: 67 us, where one CTA per chain that walked the tokens one by one took 520 us).  All products are register tiles (8 x 4 per thread at d = 64) fed by 128-bit
 // shared-memory loads, three wavefronts per thirty-two multiply-adds of a warp.
 #include <cooperative_groups.h>
 
@@ -140,9 +140,11 @@ prefill_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* _
                                    : make_float4(0.f, 0.f, 0.f, 0.f));
     }
   };
-  // S += phi(K)^T V of the chunk in shared memory, and the parts of z += colsum phi(K)
+  // S += phi(K)^T V of the chunk in shared memory, and the parts of z += colsum phi(K).  (Three loads feed 32 multiply-adds
+  // here, and 12 warps per SM do not hide them alone: eight tokens' loads in flight.  48 chains of 2000 tokens, d = 64:
+  // 144.9 us with 2, 134.5 with 4, 132.2 with 8, 132.5 with 16; the scores below, four steps instead of two: 131.6.)
   auto absorb = [&]() {
-#pragma unroll 4
+#pragma unroll 8
     for (int j = 0; j < C; ++j) {
       float4 kk[A], vv[G];
 #pragma unroll
@@ -272,7 +274,7 @@ prefill_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* _
     for (int r = 0; r < R; ++r)
 #pragma unroll
       for (int c = 0; c < CB; ++c) p[r][c] = 0.f;
-#pragma unroll 2
+#pragma unroll 4
     for (int a = 0; a < D; a += 4) {
       float4 kk[CB];
 #pragma unroll
