@@ -323,8 +323,6 @@ __device__ __forceinline__ void tmem_st8(uint32_t taddr, const uint32_t* r) {
                "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7])
                : "memory");
 }
-// TMEM column (from P_COL) where the packed bf16 of token c, a multiple of 16, begins.
-__device__ __forceinline__ uint32_t pk_col(int c) { return (uint32_t)((c & 64) + ((c & 63) >> 1)); }
 
 __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
@@ -503,7 +501,11 @@ __device__ __forceinline__ uint4 pack8(const uint32_t* v) {
 // GM = 1: one group per tile (partly filled where the group is shorter than 128), no intra-tile linear term.
 // GM = 2 (MULTI): 128 / gsz groups of gsz = 32 or 64 tokens per tile.  A row then also meets the earlier groups of its
 // tile, linearly: a product per group, phi(Q) with phi(K) of that group, puts those scores in the place of the raw ones
-// that nobody needs (the accumulator's other lanes are masked off), and they join P unscaled.  (One partly filled tile
+// that nobody needs (the accumulator's other lanes are masked off), and they join P unscaled, as two bf16 numbers each:
+// the rounding of a score, unlike that of an entry of S, is not averaged over the 128 features (rounded once, they left
+// the global branch of values that cancel 30 times further from its exact value than the state's copy does).  P of 16
+// tokens c ... c + 15 takes the place of their fp32 scores: columns c ... c + 7, and c + 8 ... c + 15 for what the rounding
+// of the linear ones left over, so that every thread overwrites only what it has read itself.  (One partly filled tile
 // per group of 64 took 200 us on 128 chains of 2048 tokens, as long per tile as a full one.)
 template <int PHI, int WT, int GM = 0>
 __global__ void __launch_bounds__(kThreads, 1)
@@ -968,8 +970,12 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
         tc_fence_after();
 #pragma unroll
         for (int ks = 0; ks < 8; ++ks)       // O += (P o M) V; 16 tokens of every row of P = 8 columns
-          mma_bf16_ts(tmem + O_COL, tmem + P_COL + (ks < 4 ? 8 * ks : 64 + 8 * (ks - 4)), desc64(v_mn + kstep_mnmajor(ks)),
-                      idesc(false, true, 128), (has_state && (!GRP || use_glob)) || ks > 0);
+          mma_bf16_ts(tmem + O_COL, tmem + P_COL + (MULTI ? 16 * ks : ks < 4 ? 8 * ks : 64 + 8 * (ks - 4)),
+                      desc64(v_mn + kstep_mnmajor(ks)), idesc(false, true, 128), (has_state && (!GRP || use_glob)) || ks > 0);
+        if (MULTI && use_glob)               // the remainders of the linear scores: rows behind the group of the 16 tokens
+          for (int ks = 0; 16 * ks < TILE - gsz; ++ks)
+            mma_bf16_ts_below(tmem + O_COL, tmem + P_COL + 16 * ks + 8, desc64(v_mn + kstep_mnmajor(ks)),
+                              idesc(false, true, 128), true, (16 * ks / gsz + 1) * gsz);
         mma_commit((bar0 + 8u * (B_MMA_O0 + par)));
         // P of the next tile overwrites the columns that the last product of this tile reads
         ok = mbar_wait((bar0 + 8u * (B_MMA_O0 + par)), (n >> 1) & 1, abort);
@@ -1171,12 +1177,12 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
       }
       if constexpr (MULTI) {
         // ---- P: causal softmax inside the row's group (the two threads of a row take half of its columns each), the
-        // linear scores against the earlier groups of the tile, zeros behind the group.  Everything a row has is read
-        // before the barrier and written, packed, after it.
+        // linear scores against the earlier groups of the tile, zeros behind the group.
         const float c2 = sm_scale * 1.4426950408889634f;       // scores -> exponents of two
         const int b0 = 32 * (wa & 3) / gsz * gsz, hw = gsz >> 1, d0 = b0 + hw * hf, l0 = (b0 >> 1) * hf;   // warp-uniform
         float m_run = -INFINITY, l_run = 0.f;
-        uint32_t v[32], lp[24];
+        const uint32_t pbase = tmem + P_COL + lane_addr;
+        uint32_t v[32];
         if (ok) {
           tc_fence_after();
           if (hw == 32) LA_TMEM_LD32(tmem + P_COL + lane_addr + d0, v);
@@ -1198,20 +1204,24 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
         }
 #pragma unroll
         for (int c = 0; c < 3; ++c)                             // 16 of this thread's b0 / 2 linear scores at a time
-          if (32 * c < b0) {
-            uint32_t x[16];
+          if (32 * c < b0 && ok) {
+            uint32_t x[16], hi[8], lo[8];
 #pragma unroll
             for (int e = 0; e < 16; ++e) x[e] = 0u;
-            if (ok && use_glob) {
+            if (use_glob) {
               tc_fence_after();
-              LA_TMEM_LD16(tmem + P_COL + lane_addr + l0 + 16 * c, x);
+              LA_TMEM_LD16(pbase + l0 + 16 * c, x);
               tmem_wait_ld();
             }
 #pragma unroll
             for (int e = 0; e < 8; ++e) {
-              lp[8 * c + e] = pack2(__uint_as_float(x[2 * e]), __uint_as_float(x[2 * e + 1]));
-              dg += __uint_as_float(x[2 * e]) + __uint_as_float(x[2 * e + 1]);
+              const float x0 = __uint_as_float(x[2 * e]), x1 = __uint_as_float(x[2 * e + 1]);
+              hi[e] = pack2(x0, x1);
+              lo[e] = pack2(x0 - lo_f(hi[e]), x1 - hi_f(hi[e]));
+              dg += x0 + x1;
             }
+            tmem_st8(pbase + l0 + 16 * c, hi);
+            if (use_glob) tmem_st8(pbase + l0 + 16 * c + 8, lo);
           }
         mlh[hf * D + r] = make_float2(m_run, l_run);
         dgh[hf * D + r] = dg;
@@ -1225,18 +1235,14 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
         const float rs = has_g ? den / alpha : 1.f, f = rs / l;
         if (ok) {
           tc_fence_after();
-          const uint32_t pbase = tmem + P_COL + lane_addr;
           uint32_t pk[16];
 #pragma unroll
           for (int e = 0; e < 16; ++e)
             pk[e] = pack2(ex2(__uint_as_float(v[2 * e]) - m) * f, ex2(__uint_as_float(v[2 * e + 1]) - m) * f);
-          if (hw == 32) LA_TMEM_ST16(pbase + pk_col(d0), pk);
-          else tmem_st8(pbase + pk_col(d0), pk);
-#pragma unroll
-          for (int c = 0; c < 3; ++c)
-            if (32 * c < b0) tmem_st8(pbase + pk_col(l0 + 16 * c), lp + 8 * c);
+          tmem_st8(pbase + d0, pk);
+          if (hw == 32) tmem_st8(pbase + d0 + 16, pk + 8);
           const uint32_t zero[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
-          for (int c = b0 + gsz + 16 * hf; c < TILE; c += 32) tmem_st8(pbase + pk_col(c), zero);
+          for (int c = b0 + gsz + 16 * hf; c < TILE; c += 32) tmem_st8(pbase + c, zero);
           denbuf[(par * 2 + hf) * D + r] = hf == 0 ? rs : 0.f;
           tmem_wait_st();
         }

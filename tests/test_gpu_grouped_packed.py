@@ -56,3 +56,26 @@ def test_options_and_continuation(C, W, phi, eps, alpha, first):
 def test_cut_along_the_sequence(C, T, first, H):
     """With a workspace: packed groups, one group per tile, and partly filled tiles (100 tokens)."""
     _run(C, T, 3, "elu1", 0.0, 1.0, first, H=H, workspace=True)
+
+
+@pytest.mark.parametrize("C", [32, 64])
+def test_scores_against_earlier_groups_of_a_tile_keep_the_precision_of_the_state(C):
+    """The global branch where its values cancel: the tokens of group 0 come in pairs of nearly equal keys and opposite
+    values, all other values are zero, so that the output of a later row of the tile is a small difference of large sums.
+    ReLU of bf16 is exact, and what is left is the output's own rounding (2^-9 of it) and that of the scores: 2^-17 each in
+    two bf16 parts, of a mean of values of size 1; one more bit for the sums."""
+    d, H, T = 128, 3, 128
+    g = np.random.default_rng(5)
+    bf = lambda x: torch.from_numpy(x.astype(np.float32)).to(torch.bfloat16)              # noqa: E731
+    q, k = bf(g.normal(0.5, 1.0, (1, H, T, d))), bf(g.normal(0.5, 1.0, (1, H, T, d)))
+    k[:, :, 1:C:2] = k[:, :, 0:C:2] + bf(g.normal(0.0, 0.05, (1, H, C // 2, d)))
+    v = torch.zeros(1, H, T, d, dtype=torch.bfloat16)
+    v[:, :, 0:C:2], v[:, :, 1:C:2] = 1.0, -1.0
+    ctx = binding.Context(H, d, 1, "relu", 1e-6, "bf16")
+    o = ctx.la_prefill_grouped(q.cuda(), k.cuda(), v.cuda(), torch.zeros(H, d, 1, device="cuda"), ctx.new_state(1), C, 1.0,
+                               d ** -0.5)
+    f = lambda x: x.double().numpy()                                                       # noqa: E731
+    want, _ = orc.prefill_grouped_block(f(q), f(k), f(v), np.zeros((H, d, 1)), "relu", 1e-6, C, 1.0, d ** -0.5)
+    got, want = o.double().cpu().numpy()[:, :, C:], np.asarray(want)[:, :, C:]
+    assert 1e-4 < np.abs(want).max() < 2e-2                      # small, as intended
+    assert (np.abs(got - want) <= 2.0 ** -9 * np.abs(want) + 2.0 ** -16).all()
