@@ -968,14 +968,33 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
         ok = mbar_wait((bar0 + 8u * (B_PDONE)), par, abort);               // masked P of tile n is in TMEM
         if (!ok) break;
         tc_fence_after();
+        if (MULTI) {
+          // A group's tokens meet its own rows and those below: the rows above are masked off, and not met with zeros, which
+          // would give them a NaN where v of a later group is not finite.  16 tokens of every row of P = 8 columns; then the
+          // remainders of the linear scores, for the rows below the group.
+          // (The masks as constants, a copy of the code per group size: as numbers of the run they cost 2 % of a pass.)
+          const int valid = min(TILE, T - n * TILE);
+          auto products = [&](auto gc) {
+            constexpr int G = decltype(gc)::value;
 #pragma unroll
-        for (int ks = 0; ks < 8; ++ks)       // O += (P o M) V; 16 tokens of every row of P = 8 columns
-          mma_bf16_ts(tmem + O_COL, tmem + P_COL + (MULTI ? 16 * ks : ks < 4 ? 8 * ks : 64 + 8 * (ks - 4)),
-                      desc64(v_mn + kstep_mnmajor(ks)), idesc(false, true, 128), (has_state && (!GRP || use_glob)) || ks > 0);
-        if (MULTI && use_glob)               // the remainders of the linear scores: rows behind the group of the 16 tokens
-          for (int ks = 0; 16 * ks < TILE - gsz; ++ks)
-            mma_bf16_ts_below(tmem + O_COL, tmem + P_COL + 16 * ks + 8, desc64(v_mn + kstep_mnmajor(ks)),
-                              idesc(false, true, 128), true, (16 * ks / gsz + 1) * gsz);
+            for (int ks = 0; ks < 8; ++ks)
+              if (16 * ks < valid)
+                mma_bf16_ts_below(tmem + O_COL, tmem + P_COL + 16 * ks, desc64(v_mn + kstep_mnmajor(ks)), idesc(false, true, 128),
+                                  (has_state && use_glob) || ks > 0, 16 * ks / G * G);
+#pragma unroll
+            for (int ks = 0; 16 * ks < TILE - G; ++ks)
+              if (use_glob && (16 * ks / G + 1) * G < valid)
+                mma_bf16_ts_below(tmem + O_COL, tmem + P_COL + 16 * ks + 8, desc64(v_mn + kstep_mnmajor(ks)),
+                                  idesc(false, true, 128), true, (16 * ks / G + 1) * G);
+          };
+          if (gsz == 64) products(std::integral_constant<int, 64>{});
+          else products(std::integral_constant<int, 32>{});
+        } else {
+#pragma unroll
+          for (int ks = 0; ks < 8; ++ks)     // O += (P o M) V; 16 tokens of every row of P = 8 columns
+            mma_bf16_ts(tmem + O_COL, tmem + P_COL + (ks < 4 ? 8 * ks : 64 + 8 * (ks - 4)), desc64(v_mn + kstep_mnmajor(ks)),
+                        idesc(false, true, 128), (has_state && (!GRP || use_glob)) || ks > 0);
+        }
         mma_commit((bar0 + 8u * (B_MMA_O0 + par)));
         // P of the next tile overwrites the columns that the last product of this tile reads
         ok = mbar_wait((bar0 + 8u * (B_MMA_O0 + par)), (n >> 1) & 1, abort);
@@ -1177,7 +1196,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
       }
       if constexpr (MULTI) {
         // ---- P: causal softmax inside the row's group (the two threads of a row take half of its columns each), the
-        // linear scores against the earlier groups of the tile, zeros behind the group.
+        // linear scores against the earlier groups of the tile (nothing behind the group: no product reads it).
         const float c2 = sm_scale * 1.4426950408889634f;       // scores -> exponents of two
         const int b0 = 32 * (wa & 3) / gsz * gsz, hw = gsz >> 1, d0 = b0 + hw * hf, l0 = (b0 >> 1) * hf;   // warp-uniform
         float m_run = -INFINITY, l_run = 0.f;
@@ -1241,8 +1260,6 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
             pk[e] = pack2(ex2(__uint_as_float(v[2 * e]) - m) * f, ex2(__uint_as_float(v[2 * e + 1]) - m) * f);
           tmem_st8(pbase + d0, pk);
           if (hw == 32) tmem_st8(pbase + d0 + 16, pk + 8);
-          const uint32_t zero[8] = {0u, 0u, 0u, 0u, 0u, 0u, 0u, 0u};
-          for (int c = b0 + gsz + 16 * hf; c < TILE; c += 32) tmem_st8(pbase + c, zero);
           denbuf[(par * 2 + hf) * D + r] = hf == 0 ? rs : 0.f;
           tmem_wait_st();
         }

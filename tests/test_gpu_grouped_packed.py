@@ -79,3 +79,21 @@ def test_scores_against_earlier_groups_of_a_tile_keep_the_precision_of_the_state
     got, want = o.double().cpu().numpy()[:, :, C:], np.asarray(want)[:, :, C:]
     assert 1e-4 < np.abs(want).max() < 2e-2                      # small, as intended
     assert (np.abs(got - want) <= 2.0 ** -9 * np.abs(want) + 2.0 ** -16).all()
+
+
+@pytest.mark.parametrize("C,T,W", [(32, 128, 3), (64, 128, 3), (32, 200, 8), (64, 250, 1)])
+@pytest.mark.parametrize("bad", [float("inf"), float("nan")])
+def test_values_that_are_not_finite_stay_behind_their_group(C, T, W, bad):
+    """A value of a later group, in the same tile or the next one, that is not finite: the groups before it do not change."""
+    d, H = 128, 2
+    q, k, v = (torch.from_numpy(x).to(torch.bfloat16).cuda() for x in wl.qkv(7, (1, H, T, d), 0.5, "bf16", v_mean=1.0))
+    w = torch.from_numpy(wl.conv_weights(7, H, d, W)).cuda()
+    ctx = binding.Context(H, d, W, "elu1", 0.0, "bf16")
+    clean = ctx.la_prefill_grouped(q, k, v, w, ctx.new_state(1), C, 1.0, d ** -0.5)
+    for tok in range(C, T, C + 5):
+        v2 = v.clone()
+        v2[0, 1, tok, 77] = bad
+        o = ctx.la_prefill_grouped(q, k, v2, w, ctx.new_state(1), C, 1.0, d ** -0.5)
+        end = tok // C * C
+        assert torch.equal(o[:, :, :end], clean[:, :, :end]), tok
+        assert torch.equal(o[:, 0], clean[:, 0]) and not o[0, 1, tok, 77].isfinite()
