@@ -19,10 +19,7 @@ template <> __device__ __forceinline__ __nv_bfloat16 from_f32<__nv_bfloat16>(flo
 
 // ---- feature map (Sec. 3: Sim(Q,K) ~ phi(Q) phi(K)^T) ------------------------------------
 template <int PHI> __device__ __forceinline__ float phi(float x) {
-  if (PHI == LA_PHI_ELU1) {                         // both sides always: a select, not a branch per element
-    const float e = expf(fminf(x, 0.f));
-    return x > 0.f ? x + 1.f : e;
-  }
+  if (PHI == LA_PHI_ELU1) return x > 0.f ? x + 1.f : expf(x);   // (a NaN is not above 0 and stays one)
   return fmaxf(x, 0.f);
 }
 

@@ -57,8 +57,15 @@ __device__ __forceinline__ void gst4(__nv_bfloat16* p, float4 x) {
   __nv_bfloat162 a = __floats2bfloat162_rn(x.x, x.y), b = __floats2bfloat162_rn(x.z, x.w);
   *reinterpret_cast<uint2*>(p) = make_uint2(*reinterpret_cast<uint32_t*>(&a), *reinterpret_cast<uint32_t*>(&b));
 }
+// phi with both sides formed always, a select and not a branch per element, for whole chunks at a time (few values, as in
+// decode and commit, are faster with the branch: 1024 units of d = 64 decode in 6.2 us with it, 6.9 without).
+template <int PHI> __device__ __forceinline__ float phi_both(float x) {
+  if (PHI != LA_PHI_ELU1) return phi<PHI>(x);
+  const float e = expf(x > 0.f ? 0.f : x);                   // (not fminf, which would drop a NaN)
+  return x > 0.f ? x + 1.f : e;
+}
 template <int PHI> __device__ __forceinline__ float4 phi4(float4 x) {
-  return make_float4(phi<PHI>(x.x), phi<PHI>(x.y), phi<PHI>(x.z), phi<PHI>(x.w));
+  return make_float4(phi_both<PHI>(x.x), phi_both<PHI>(x.y), phi_both<PHI>(x.z), phi_both<PHI>(x.w));
 }
 __device__ __forceinline__ void fma4(float4& acc, float a, float4 b) {
   acc.x = fmaf(a, b.x, acc.x);
