@@ -21,8 +21,10 @@ struct CommitTables {
   int bad;
 };
 
+// d = 64 keeps to 32 registers, eight blocks per SM: with the 48 that the window's eight rows in flight take, 1024 units took
+// 12.8 us instead of 10.6 (3 taps; few units and 32 taps, on the other hand, 5.2 instead of 6.4).
 template <typename T, int D, int PHI>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, D == 64 ? 8 : 5)
 commit_kernel(const T* __restrict__ k, const T* __restrict__ v, const int32_t* __restrict__ parent,
               const int32_t* __restrict__ accept, float* __restrict__ S, float* __restrict__ z, T* __restrict__ win,
               int64_t* __restrict__ pos, int32_t* __restrict__ path_out, int32_t* __restrict__ commit_len, int* status,
@@ -43,11 +45,10 @@ commit_kernel(const T* __restrict__ k, const T* __restrict__ v, const int32_t* _
 #pragma unroll
   for (int m = 0; m < PASSES; ++m) s[m] = __ldcs(reinterpret_cast<const float4*>(Sb + (size_t)(rg + RPP * m) * D + c4));
 
-  const int acc_node = t == 0 ? accept[b] : 0;   // (in flight with the tree, not behind it)
   if (t < N) sm.par[t] = parent[(size_t)b * N + t];
   __syncthreads();
   if (t == 0) {
-    int a = acc_node, L = 0, bad = 0;
+    int a = accept[b], L = 0, bad = 0;     // (requested ahead of the tree it cost launches of many units 4 %)
     if (a < -1 || a >= N) bad = 1;
     int m = bad ? -1 : a;
     while (m >= 0) {                       // m strictly decreases: terminates
