@@ -352,21 +352,23 @@ prefill_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* _
       for (int m = LPR / 2; m > 0; m >>= 1) den += __shfl_xor_sync(0xffffffffu, den, m);
       if (t % LPR == 0) sden[t / LPR] = den;
     }
-    // O += (P o M) V
+    // O += (P o M) V, TY tokens at a time, which meet TY rows on the diagonal and all those below.  The tokens behind a row are
+    // left out, not met with a zero: where v is not finite that would be a NaN in the rows before it.
 #pragma unroll
-    for (int b = 0; b < CB; ++b) {                           // tokens 16 b ... 16 b + 15 meet the rows from 16 b on
+    for (int b = 0; b < R; ++b) {
 #pragma unroll 2
-      for (int j = 16 * b; j < 16 * b + 16; j += 4) {
+      for (int j = 0; j < TY; j += 4) {
         float4 pp[R];
 #pragma unroll
-        for (int r = 16 * b / TY; r < R; ++r) pp[r] = ld4(sq + (ty + TY * r) * PS + j);
+        for (int r = b; r < R; ++r) pp[r] = ld4(sq + (ty + TY * r) * PS + TY * b + j);
 #pragma unroll
         for (int i = 0; i < 4; ++i)
 #pragma unroll
           for (int g = 0; g < G; ++g) {
-            const float4 vv = ld4(svc + (j + i) * D + 64 * g + 4 * tx);
+            const float4 vv = ld4(svc + (TY * b + j + i) * D + 64 * g + 4 * tx);
+            if (j + i <= ty) fma4(acc[b][g], comp(pp[b], i), vv);
 #pragma unroll
-            for (int r = 16 * b / TY; r < R; ++r) fma4(acc[r][g], comp(pp[r], i), vv);
+            for (int r = b + 1; r < R; ++r) fma4(acc[r][g], comp(pp[r], i), vv);
           }
       }
     }

@@ -68,3 +68,19 @@ def test_nan_in_q_or_k_reaches_the_outputs(io, d, cuda_cores):
     assert o[1, 0, 33].isnan().all() and o.isnan().sum() == d
     o = ctx.la_prefill_grouped(q, k, v, w, st, 16, 1.0, d ** -0.5)
     assert o[1, 0, 33].isnan().all() and o.isnan().sum() == d
+
+
+@pytest.mark.parametrize("io,d", [("f32", 64), ("f32", 128), ("bf16", 64)])
+@pytest.mark.parametrize("bad", [float("inf"), NAN])
+def test_value_that_is_not_finite_reaches_no_earlier_token(io, d, bad):
+    """The CUDA-core prefill: the outputs before a token whose value is not finite do not change."""
+    T = 150
+    ctx, q, k, v, w, st = _make(io, d, (T,))
+    clean = ctx.la_prefill(q, k, v, w, st)
+    for tok in (0, 1, 15, 16, 31, 32, 33, 47, 63, 64, 100, 127, 128, 149):
+        v2 = v.clone()
+        v2[0, 1, tok, 3] = bad
+        o = ctx.la_prefill(q, k, v2, w, st)
+        assert torch.equal(o[0, 1, :tok], clean[0, 1, :tok]) and torch.equal(o[1], clean[1]), tok
+        assert not o[0, 1, tok:, 3].isfinite().any(), tok
+        assert torch.equal(o[0, 1, :, :3], clean[0, 1, :, :3]) and torch.equal(o[0, 1, :, 4:], clean[0, 1, :, 4:])
