@@ -122,7 +122,8 @@ const char* la_status_str(la_status s);
  * rounded to bf16, and the sum rounded to bf16 (with fewer taps both terms meet in fp32).  fp32 io, and
  * d = 64 in either type, take a CUDA-core kernel: the same chunkwise form with every product an fp32
  * multiply-add, which is what the fp32 tolerance needs; chains too few to fill the GPU are cut along
- * the sequence over a cluster of thread blocks (no workspace needed).
+ * the sequence over a cluster of thread blocks (no workspace needed).  Calls of a few tokens, too few to fill
+ * its chunks, walk them one by one instead.
  */
 la_status la_prefill(la_ctx* ctx, int32_t B, int32_t T, const void* q, const void* k, const void* v,
                      const float* conv_w, int32_t init_state, la_state* st /*host struct*/, void* o,

@@ -155,6 +155,8 @@ cudaError_t launch_decode(la_ctx* ctx, int B, const void* q, const void* k, cons
                           const la_state& st, void* o, cudaStream_t s);
 cudaError_t launch_prefill_simt(la_ctx* ctx, int B, int T, const void* q, const void* k, const void* v,
                                 const float* w, int init_state, const la_state& st, void* o, cudaStream_t s);
+cudaError_t launch_prefill_walk(la_ctx* ctx, int B, int T, const void* q, const void* k, const void* v,
+                                const float* w, int init_state, const la_state& st, void* o, cudaStream_t s);
 cudaError_t launch_verify(la_ctx* ctx, int B, int N, const void* q, const void* k, const void* v,
                           const int32_t* parent, const float* w, const la_state& st, void* o, cudaStream_t s);
 cudaError_t launch_commit(la_ctx* ctx, int B, int N, const void* k, const void* v, const int32_t* parent,

@@ -49,3 +49,12 @@ def test_options_and_continuation(io, d, W, phi, eps, first):
 @pytest.mark.parametrize("d,B,H", [(64, 32, 7), (128, 10, 8)])
 def test_one_block_per_chain_when_chains_abound(d, B, H):
     _run("f32", d, 100, 3, "elu1", 0.0, B, H, 40)
+
+
+@pytest.mark.parametrize("d,B,H,edges", [(64, 1, 2, (26,)), (64, 25, 8, (28,)), (64, 64, 8, (41, 86)), (128, 1, 2, (14, 34)),
+                                         (128, 19, 8, (23, 52, 80)), (128, 50, 8, (19, 44))])
+def test_both_sides_of_the_lines_between_walking_and_chunks(d, B, H, edges):
+    """Short calls walk their tokens; the lines depend on the head dimension and on the number of chains.  A call on either
+    side of each line continues 5 tokens (which are walked) and must agree with the oracle."""
+    for T in (t + x for t in edges for x in (0, 1)):
+        _run("f32", d, T + 5, 3, "elu1", 0.0, B, H, 5)
