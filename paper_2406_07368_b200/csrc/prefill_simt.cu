@@ -235,6 +235,7 @@ prefill_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* _
       for (int r = 0; r < kMaxCluster; ++r)
         if (r < rank) zr += part[r];
     }
+    load_halo(seg0);                                         // (before anybody stores an output: o may lie on v)
     cluster.sync();                                          // the prefixes are in place
     if (rank > 0) {
 #pragma unroll
@@ -264,7 +265,7 @@ prefill_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* _
     float4 y[LD];
     fetch(x, k, seg0, n);
     fetch(y, q, seg0, n);
-    load_halo(seg0);
+    if (nrank == 1) load_halo(seg0);
     put_phi(x, sk, n);
     fetch(x, v, seg0, n);
     put_phi(y, sq, n);
@@ -408,8 +409,17 @@ prefill_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* _
     if (more) {
       put_phi(x, sq, nn);
       fetch(x, v, i0 + C, nn);
+      // The rows before the next chunk are the last W - 1 of this one: from shared memory, not from v, where the outputs may
+      // stand by now (a call in place, o = v).
+      constexpr int HP = (LA_MAX_TAPS - 1) * D / 4 / NT + 1; // pieces per thread
+      float4 y[HP];
+#pragma unroll
+      for (int it = 0; it < HP; ++it)
+        if (t + it * NT < (W - 1) * (D / 4)) y[it] = ld4(sv + C * D + (t + it * NT) * 4);
       __syncthreads();                                       // v has been read
-      load_halo(i0 + C);
+#pragma unroll
+      for (int it = 0; it < HP; ++it)
+        if (t + it * NT < (W - 1) * (D / 4)) st4(sv + (t + it * NT) * 4, y[it]);
       put_v(x);
     }
   }
@@ -426,10 +436,8 @@ prefill_simt_kernel(const T* __restrict__ q, const T* __restrict__ k, const T* _
       for (int c = 0; c < G; ++c) st4(Sb + (size_t)(4 * TY * g + 4 * ty + i) * D + 64 * c + 4 * tx, s[g][i][c]);
   if (t < D) {
     zb[t] = zr;
-    for (int i = 0; i < W - 1; ++i) {                        // ascending: the source lies above the target
-      const int tok = Tlen - (W - 1) + i;
-      wb[(size_t)i * D + t] = tok >= 0 ? v[base + (size_t)tok * D + t] : init ? wb[(size_t)(Tlen + i) * D + t] : from_f32<T>(0.f);
-    }
+    const float* tail = sv + ((seg1 - seg0 - 1) % C + 1) * D + t;   // behind the tokens of the last chunk
+    for (int i = 0; i < W - 1; ++i) wb[(size_t)i * D + t] = from_f32<T>(tail[i * D]);
   }
   if (h == 0 && t == 0) pos[bh / H] = (init ? pos[bh / H] : 0) + Tlen;
 }
