@@ -1072,6 +1072,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
             const int buf = blk < 3 ? 3 + 3 * (int)par + blk : (n + 1) % 3;
             *reinterpret_cast<uint4*>(hb + buf * halo_bytes(WT) + halo_at(i, lane & 15, WT)) = x[m];
           }
+          __syncwarp();                                     // (a short last tile reads rows that other lanes wrote here)
         }
         mbar_arrive((bar0 + 8u * (B_HALO0 + par)));
       }

@@ -554,3 +554,18 @@ def test_tiny_fp32_workload_end_to_end():
     np.testing.assert_array_equal(host(path), wpath)
     check_state(st, ost, TOL[io])
     assert int(st.pos[0]) == 256 + 16 + 2
+
+
+@pytest.mark.parametrize("W", [3, 4, 5])
+@pytest.mark.parametrize("T", [129, 130, 257, 258, 259, 385])
+def test_last_tile_shorter_than_the_window(T, W):
+    """The rows before the last tile, and the window behind it, reach back past a tile of one to three rows."""
+    io, d, B, H = "bf16", 128, 3, 8
+    q, k, v = wl.qkv(T + W, (B, H, T, d), d ** -0.5, io, v_mean=0.5)
+    w = wl.conv_weights(17, H, d, W)
+    ctx = binding.Context(H, d, W, "elu1", 0.0, io)
+    st = ctx.new_state(B)
+    o = ctx.la_prefill(dev(q, io), dev(k, io), dev(v, io), dev(w, "f32"), st)
+    want, _ = orc.prefill_quadratic(q, k, v, w, "elu1", 0.0)
+    assert rel_err(o[:, :, -6:].float().cpu().numpy(), want[:, :, -6:]) < TOL[io]
+    assert np.array_equal(st.win.float().cpu().numpy(), v[:, :, T - (W - 1):])
