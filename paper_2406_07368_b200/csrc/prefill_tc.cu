@@ -81,10 +81,9 @@ __host__ __device__ constexpr uint32_t off_den(bool z3) { return OFF_ONES + ones
 __host__ __device__ constexpr uint32_t off_small(bool z3) { return off_den(z3) + 2048; }
 
 struct Small {
-  unsigned long long bars[24];
+  unsigned long long bars[25];
   uint32_t tmem_base;
   int abort;
-  int pad[2];
 };
 // full_*: TMA landed.  PHI / PDONE / SB: arrivals of group A.  EPI0 / EPI1: arrivals of group B (the accumulator
 // has been read; tiles alternate between the two).
@@ -97,8 +96,8 @@ enum { B_FULL_K0 = 0, B_FULL_V0 = 1, B_FULL_V1 = 2, B_MMA_P = 3, B_MMA_S0 = 4, B
        B_PDONE = 8, B_SB = 9, B_EPI0 = 10, B_EPI1 = 11, B_MMA_Q = 12, B_FULL_Q = 13, B_FULL_K1 = 14, B_STAGED0 = 15,
        B_STAGED1 = 16, B_HALO0 = 17, B_HALO1 = 18, B_MMA_S1 = 19,
        B_MMA_L = 20 /* the scores against earlier groups of the tile */, 
-       B_ST_PHI = 21, B_ST_MMA0 = 22, B_ST_MMA1 = 23 /* the state pass */, kNumBars = 24 };
-static_assert(kNumBars <= 24, "Small::bars");
+       B_ST_PHI0 = 21, B_ST_PHI1 = 22, B_ST_MMA0 = 23, B_ST_MMA1 = 24 /* the state pass */, kNumBars = 25 };
+static_assert(kNumBars <= 25 && sizeof(Small) == 208, "Small::bars");
 
 __host__ __device__ constexpr uint32_t off_w(bool z3) { return off_small(z3) + (uint32_t)((sizeof(Small) + 15) / 16 * 16); }
 // Short windows: nine halo buffers, rows of v that lie before 32 rows of a tile, for the convolution.  Buffers 0-2: the
@@ -622,10 +621,12 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
     mbar_init((bar0 + 8u * (B_STAGED1)), kThreadsB);
     mbar_init((bar0 + 8u * (B_HALO0)), 32);
     mbar_init((bar0 + 8u * (B_HALO1)), 32);
+    for (int i = 0; i < 2; ++i) {
+      mbar_init((bar0 + 8u * (B_ST_MMA0 + i)), 1);
+      mbar_init((bar0 + 8u * (B_ST_PHI0 + i)), kThreadsA + kThreadsB);
+    }
     sm.abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    for (int i = 0; i < 2; ++i) mbar_init((bar0 + 8u * (B_ST_MMA0 + i)), 1);
-    mbar_init((bar0 + 8u * (B_ST_PHI)), kThreadsA + kThreadsB);
     // the first tile is requested at once (nothing below touches the rows that it brings); the others follow behind the
     // taps and the window, which would otherwise wait for them (20 MB over all blocks: 3 us)
     pdl_wait();
@@ -705,7 +706,9 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
       if (lane == 0)
         for (int n = 0; n < nchunks; ++n) {
           const uint32_t par = n & 1;
-          if (!mbar_wait((bar0 + 8u * (B_ST_PHI)), par, abort) || !mbar_wait((bar0 + 8u * (B_FULL_V0 + par)), (n >> 1) & 1, abort)) break;
+          // (phi(K) of tiles 0 and 1 may both be in place before this lane looks: a barrier per tile parity.  Its next phase
+          // needs tile n + 2, which is loaded behind the product below.)
+          if (!mbar_wait((bar0 + 8u * (B_ST_PHI0 + par)), (n >> 1) & 1, abort) || !mbar_wait((bar0 + 8u * (B_FULL_V0 + par)), (n >> 1) & 1, abort)) break;
           tc_fence_after();
           const uint32_t k_mn = desc_lo(sbase + (par ? OFF_K1 : OFF_K0), KBOX_BYTES), v_mn = desc_lo(sbase + vbox(par, 0), vstep(par));
 #pragma unroll
@@ -739,7 +742,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
           else phi_k(K4c{}, K8c{}, n, tid - kThreadsB);
         }
         fence_proxy_async();
-        mbar_arrive((bar0 + 8u * (B_ST_PHI)));
+        mbar_arrive((bar0 + 8u * (B_ST_PHI0 + (n & 1))));
       }
       const int l = nchunks - 1;                  // (the last product; its barrier is at most one phase behind here: tile l
                                                   // was loaded only after product l - 2 had completed)
@@ -1590,7 +1593,9 @@ constexpr uint32_t ST_OFF_VQ = TILE_BYTES, ST_OFF_ONES = ST_OFF_VQ + 6 * BOX_BYT
 __host__ __device__ constexpr uint32_t st_kbuf(uint32_t b) { return b ? 0u : ST_OFF_VQ + BOX_BYTES; }
 __host__ __device__ constexpr uint32_t st_vbox(uint32_t b, uint32_t half) { return ST_OFF_VQ + (b ? 0u : 4 * BOX_BYTES) + half * vstep(b); }
 constexpr uint32_t kStateSmem = ST_OFF_SMALL + 256 + 1024;
-enum { SB_FULL_K0 = 0, SB_FULL_K1, SB_FULL_V0, SB_FULL_V1, SB_PHI, SB_MMA, kStateBars };
+// All of them by tile parity: both of the first two tiles may be in place before the issuing lane looks, and both of the last
+// two products complete before a compute warp does.
+enum { SB_FULL_K0 = 0, SB_FULL_K1, SB_FULL_V0, SB_FULL_V1, SB_PHI0, SB_PHI1, SB_MMA0, SB_MMA1, kStateBars };
 
 template <int PHI>
 __global__ void __launch_bounds__(kStateThreads, 1)
@@ -1616,8 +1621,10 @@ segment_state_kernel(const __grid_constant__ CUtensorMap mk, const __grid_consta
 
   if (tid == 0) {
     for (int i = 0; i < 4; ++i) mbar_init((bar0 + 8u * (i)), 1);
-    mbar_init((bar0 + 8u * (SB_PHI)), 256);
-    mbar_init((bar0 + 8u * (SB_MMA)), 1);
+    mbar_init((bar0 + 8u * (SB_PHI0)), 256);
+    mbar_init((bar0 + 8u * (SB_PHI1)), 256);
+    mbar_init((bar0 + 8u * (SB_MMA0)), 1);
+    mbar_init((bar0 + 8u * (SB_MMA1)), 1);
     *abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
@@ -1653,15 +1660,15 @@ segment_state_kernel(const __grid_constant__ CUtensorMap mk, const __grid_consta
       for (int n = 0; n < 2 && n < nchunks; ++n) load_tile(n);
       for (int n = 0; n < nchunks; ++n) {
         const uint32_t b2 = n & 1;
-        if (!mbar_wait((bar0 + 8u * (SB_PHI)), n & 1, abort) || !mbar_wait((bar0 + 8u * (SB_FULL_V0 + b2)), (n >> 1) & 1, abort)) break;
+        if (!mbar_wait((bar0 + 8u * (SB_PHI0 + b2)), (n >> 1) & 1, abort) || !mbar_wait((bar0 + 8u * (SB_FULL_V0 + b2)), (n >> 1) & 1, abort)) break;
         tc_fence_after();
         const uint32_t k_mn = desc_lo(sbase + st_kbuf(b2), BOX_BYTES), v_mn = desc_lo(sbase + st_vbox(b2, 0), vstep(b2));
 #pragma unroll
         for (int ks = 0; ks < 8; ++ks)       // [dS | dz] += phi(K)^T [V | 1]
           mma_bf16(tmem + SCOL, desc64(k_mn + kstep_mnmajor(ks)), desc64(v_mn + kstep_mnmajor(ks)), idesc(true, true, 144),
                    n > 0 || ks > 0);
-        mma_commit((bar0 + 8u * (SB_MMA)));
-        if (!mbar_wait((bar0 + 8u * (SB_MMA)), n & 1, abort)) break;       // both buffers of this tile are free
+        mma_commit((bar0 + 8u * (SB_MMA0 + b2)));
+        if (!mbar_wait((bar0 + 8u * (SB_MMA0 + b2)), (n >> 1) & 1, abort)) break;       // both buffers of this tile are free
         if (n + 2 < nchunks) load_tile(n + 2);
       }
     }
@@ -1684,11 +1691,11 @@ segment_state_kernel(const __grid_constant__ CUtensorMap mk, const __grid_consta
         }
       }
       fence_proxy_async();
-      mbar_arrive((bar0 + 8u * (SB_PHI)));
+      mbar_arrive((bar0 + 8u * (SB_PHI0 + (n & 1))));
     }
-    // Wait for the last two products in turn (tile L was loaded only after product L-2 had completed, so the
-    // barrier is at phase L-1 or later here and a parity wait cannot be fooled by an older phase).
-    for (int n = max(0, nchunks - 2); n < nchunks; ++n) ok = ok && mbar_wait((bar0 + 8u * (SB_MMA)), n & 1, abort);
+    const int l = nchunks - 1;                      // (its barrier is at most one phase behind here: tile l was loaded only after
+                                                    // product l - 2 had completed)
+    ok = ok && mbar_wait((bar0 + 8u * (SB_MMA0 + (l & 1))), (l >> 1) & 1, abort);
     ok = __all_sync(0xffffffffu, ok);
     if (ok) {
       tc_fence_after();

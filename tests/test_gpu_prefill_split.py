@@ -46,3 +46,20 @@ def test_split_with_few_segments(H, T, W, first):
         assert rel_err(st.S.cpu().numpy(), ost.S) < 2e-2 and rel_err(st.z.cpu().numpy(), ost.z) < 2e-2
         assert st.pos.tolist() == [first + T]
     assert torch.equal(states[0].win, states[1].win)
+
+
+def test_state_sums_of_many_tiles_over_and_over():
+    """The passes that only form sums run ahead of the products as far as two buffers allow: segments of two tiles and more,
+    many calls, every one bit for bit the same and none with a wait that ran out."""
+    ctx = binding.Context(36, 128, 3, "elu1", 0.0, "bf16")
+    for T in (900, 2500, 6000):                                  # one launch of clusters; per-segment sums of 2 to 12 tiles
+        q, k, v = (torch.from_numpy(x).to(torch.bfloat16).cuda() for x in wl.qkv(T, (1, 36, T, 128), 0.1, "bf16"))
+        w = torch.from_numpy(wl.conv_weights(5, 36, 128, 3)).cuda()
+        ctx.la_set_workspace(torch.empty(ctx.la_prefill_workspace_bytes(1, T), dtype=torch.uint8, device="cuda"))
+        first = None
+        for _ in range(50):
+            st = ctx.new_state(1)
+            got = (ctx.la_prefill(q, k, v, w, st), st.S, *ctx.la_segment_state(k, v))
+            first = first or got
+            assert all(torch.equal(a, b) for a, b in zip(got, first))
+    assert ctx.la_last_device_status() == binding.LA_OK
