@@ -1883,9 +1883,13 @@ static void plan_split(const la_ctx* ctx, int BH, int T, int* nseg, int* seg_len
   // One wave of thread blocks: as many segments per chain as fit on the SMs at once.  (Measured on 32 chains of
   // 32768 tokens: 4 segments per chain 418 us, 9 segments (two waves) 432 us, 13: 456, 18: 483 -- a second wave
   // never fills as well as the first, and every segment costs a 64 KB state written and read back.)
-  int n = std::min(ctx->sm_count / BH, tiles);
-  tiles = (T + tile - 1) / tile;               // (shorter tiles, of the three-branch block, never mean more segments)
-  const int per = (tiles + n - 1) / n;
+  int n = std::min(ctx->sm_count / BH, tiles), per = (tiles + n - 1) / n;
+  n = (tiles + per - 1) / per;
+  // Shorter tiles (of the three-branch block) are shared out over at most as many segments: rounded on their own they could
+  // make more (8 chains of 2306 tokens: 10 segments of 128-token tiles, 13 of 96), and the caller's workspace, whose size is
+  // asked for without a group, would be too small.
+  tiles = (T + tile - 1) / tile;
+  per = (tiles + n - 1) / n;
   n = (tiles + per - 1) / per;
   if (n < 2) return;
   *nseg = n;

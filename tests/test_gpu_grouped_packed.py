@@ -25,10 +25,13 @@ def _run(C, T, W, phi, eps, alpha, first=0, B=1, H=3, workspace=False):
     if workspace:
         need = ctx.la_prefill_workspace_bytes(B, T)
         assert need > 0
-        ctx.la_set_workspace(torch.full((need,), 0xff, dtype=torch.uint8, device="cuda"))
+        ws = torch.full((need,), 0xff, dtype=torch.uint8, device="cuda")
+        ctx.la_set_workspace(ws)
     o = ctx.la_prefill_grouped(dev(q[:, :, first:]), dev(k[:, :, first:]), dev(v[:, :, first:]), wd, st, *args,
                                init_state=first > 0)
     assert ctx.la_last_device_status() == binding.LA_OK
+    if workspace:
+        assert (ws != 0xff).any()                                # the cut was made
     want, ost = orc.prefill_grouped_block(q, k, v, w, phi, eps, C, alpha, d ** -0.5)
     got = o.float().cpu().numpy()
     assert rel_err(got, want[:, :, first:]) < TOL[io]
@@ -97,3 +100,9 @@ def test_values_that_are_not_finite_stay_behind_their_group(C, T, W, bad):
         end = tok // C * C
         assert torch.equal(o[:, :, :end], clean[:, :, :end]), tok
         assert torch.equal(o[:, 0], clean[:, 0]) and not o[0, 1, tok, 77].isfinite()
+
+
+@pytest.mark.parametrize("C,T,first,H", [(100, 1280, 0, 18), (96, 2306, 96, 8), (33, 700, 0, 32), (48, 2048, 48, 16)])
+def test_cut_with_the_workspace_asked_for_without_a_group(C, T, first, H):
+    """Tiles of other than 128 tokens: the number of segments must fit the workspace that la_prefill_workspace_bytes names."""
+    _run(C, T, 3, "elu1", 0.0, 1.0, first, H=H, workspace=True)
