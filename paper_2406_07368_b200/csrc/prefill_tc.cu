@@ -1690,6 +1690,13 @@ segment_state_kernel(const __grid_constant__ CUtensorMap mk, const __grid_consta
           *reinterpret_cast<uint4*>(Kb + swz(j, ct & 7)) = j < valid ? phi8<PHI>(x[i]) : make_uint4(0u, 0u, 0u, 0u);
         }
       }
+      if (valid < TILE && y0 + T < Ttot) {          // rows of the next segment: zeros (0 times a v that is not finite is not 0)
+        ok = ok && mbar_wait((bar0 + 8u * (SB_FULL_V0 + (n & 1))), (n >> 1) & 1, abort);
+        ok = __all_sync(0xffffffffu, ok);
+        if (ok)
+          for (int idx = tid; idx < (TILE - valid) * 16; idx += 256)
+            *reinterpret_cast<uint4*>(smem + st_vbox(n & 1, (idx & 15) >> 3) + swz(valid + (idx >> 4), idx & 7)) = make_uint4(0u, 0u, 0u, 0u);
+      }
       fence_proxy_async();
       mbar_arrive((bar0 + 8u * (SB_PHI0 + (n & 1))));
     }

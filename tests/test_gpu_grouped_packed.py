@@ -106,3 +106,23 @@ def test_values_that_are_not_finite_stay_behind_their_group(C, T, W, bad):
 def test_cut_with_the_workspace_asked_for_without_a_group(C, T, first, H):
     """Tiles of other than 128 tokens: the number of segments must fit the workspace that la_prefill_workspace_bytes names."""
     _run(C, T, 3, "elu1", 0.0, 1.0, first, H=H, workspace=True)
+
+
+@pytest.mark.parametrize("bad", [float("inf"), float("nan")])
+def test_values_that_are_not_finite_stay_behind_their_segment(bad):
+    """Ten segments of seven 40-token groups, whose sums are formed in 128-token tiles by a launch of its own: the last tile of
+    a segment overlaps the next one's first groups, a value of which must not enter the segment's sums."""
+    C, T, H, d = 40, 2660, 8, 128
+    q, k, v = (torch.from_numpy(x).to(torch.bfloat16).cuda() for x in wl.qkv(7, (1, H, T, d), 0.5, "bf16", v_mean=1.0))
+    w = torch.from_numpy(wl.conv_weights(7, H, d, 3)).cuda()
+    ctx = binding.Context(H, d, 3, "elu1", 0.0, "bf16")
+    ws = torch.full((ctx.la_prefill_workspace_bytes(1, T),), 0xff, dtype=torch.uint8, device="cuda")
+    ctx.la_set_workspace(ws)
+    clean = ctx.la_prefill_grouped(q, k, v, w, ctx.new_state(1), C, 1.0, d ** -0.5)
+    assert (ws != 0xff).any()
+    for tok in (325, 370, 605):
+        v2 = v.clone()
+        v2[0, 1, tok, 77] = bad
+        o = ctx.la_prefill_grouped(q, k, v2, w, ctx.new_state(1), C, 1.0, d ** -0.5)
+        end = tok // C * C
+        assert torch.equal(o[:, :, :end], clean[:, :, :end]), tok
