@@ -1496,7 +1496,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
       if (WN > 1) ok = ok && mbar_wait((bar0 + 8u * (B_HALO0 + par)), (n >> 1) & 1, abort);
       ok = ok && mbar_wait((bar0 + 8u * (B_MMA_O0 + par)), (n >> 1) & 1, abort);   // also: every product that reads V is done
       ok = __all_sync(0xffffffffu, ok);
-      if (ok) {
+      if (ok && (!GRP || 32 * q4 < valid)) {      // (32 rows behind a partly filled tile's tokens: zeros already)
         tc_fence_after();
         const uint32_t oaddr = tmem + lane_addr + O_COL + 64 * hf;
         uint32_t a0[16], a1[16];                  // rows 0-15 and 16-31
