@@ -146,20 +146,31 @@ const at::Tensor& lead(PyObject* o, int64_t dims, const char* name) {
   return t;
 }
 
+// The state's four tensors.  They are held until the call is over: an attribute may be a property that makes a view anew.
 struct StateArg {
   la_state st;
+  PyObject* held[4] = {nullptr, nullptr, nullptr, nullptr};
   StateArg(const Plan* p, PyObject* state, int64_t B) {
-    st.S = (float*)field(state, s_S, at::kFloat, {B, p->H, p->d, p->d}, "state.S");
-    st.z = (float*)field(state, s_z, at::kFloat, {B, p->H, p->d}, "state.z");
-    st.win = field(state, s_win, p->io, {B, p->H, p->W - 1, p->d}, "state.win");
-    st.pos = (int64_t*)field(state, s_pos, at::kLong, {B}, "state.pos");
+    try {
+      st.S = (float*)field(0, state, s_S, at::kFloat, {B, p->H, p->d, p->d}, "state.S");
+      st.z = (float*)field(1, state, s_z, at::kFloat, {B, p->H, p->d}, "state.z");
+      st.win = field(2, state, s_win, p->io, {B, p->H, p->W - 1, p->d}, "state.win");
+      st.pos = (int64_t*)field(3, state, s_pos, at::kLong, {B}, "state.pos");
+    } catch (...) {
+      release();
+      throw;
+    }
     if (p->W == 1) st.win = nullptr;
   }
-  static void* field(PyObject* state, PyObject* attr, at::ScalarType dtype, Shape shape, const char* name) {
-    PyObject* o = PyObject_GetAttr(state, attr);
-    if (!o) throw Raised();
-    Py_DECREF(o);   // the state object keeps it alive
-    return ptr(o, dtype, shape, name);
+  StateArg(const StateArg&) = delete;
+  ~StateArg() { release(); }
+  void release() {
+    for (PyObject*& o : held) Py_CLEAR(o);
+  }
+  void* field(int i, PyObject* state, PyObject* attr, at::ScalarType dtype, Shape shape, const char* name) {
+    held[i] = PyObject_GetAttr(state, attr);
+    if (!held[i]) throw Raised();
+    return ptr(held[i], dtype, shape, name);
   }
 };
 

@@ -61,3 +61,21 @@ def test_calls_on_a_given_stream():
     got = ctx.la_prefill(q, k, v, w, st2, out=out, stream=s)
     s.synchronize()
     assert torch.equal(got, want)
+
+
+def test_state_whose_tensors_are_views_made_on_access():
+    """A state out of a larger pool: every access makes a new view, which nothing but the call itself keeps alive."""
+    ctx, q, k, v, w, st = _inputs()
+    want = ctx.la_prefill(q, k, v, w, st)
+    pool = ctx.new_state(6)
+
+    class Slice:
+        S = property(lambda self: pool.S[2:4])
+        z = property(lambda self: pool.z[2:4])
+        win = property(lambda self: pool.win[2:4])
+        pos = property(lambda self: pool.pos[2:4])
+
+    for _ in range(20):
+        assert torch.equal(ctx.la_prefill(q, k, v, w, Slice()), want)
+    assert torch.equal(pool.S[2:4], st.S) and torch.equal(pool.win[2:4], st.win) and pool.pos.tolist() == [0, 0, 8, 8, 0, 0]
+    assert not pool.S[:2].any() and not pool.S[4:].any()
