@@ -183,14 +183,20 @@ void* stream_of(PyObject* o) {
   if (PyErr_Occurred()) throw Raised();
   return s;
 }
+// int(o) and float(o): whatever those take (a group size computed as 64.0, a one-element tensor).
 long integer(PyObject* o) {
-  const long v = PyLong_AsLong(o);
+  PyObject* n = PyNumber_Long(o);
+  if (!n) throw Raised();
+  const long v = PyLong_AsLong(n);
+  Py_DECREF(n);
   if (v == -1 && PyErr_Occurred()) throw Raised();
   return v;
 }
 float real(PyObject* o) {
-  const double v = PyFloat_AsDouble(o);
-  if (v == -1.0 && PyErr_Occurred()) throw Raised();
+  PyObject* n = PyNumber_Float(o);
+  if (!n) throw Raised();
+  const double v = PyFloat_AS_DOUBLE(n);
+  Py_DECREF(n);
   return (float)v;
 }
 bool truth(PyObject* o) {

@@ -79,3 +79,14 @@ def test_state_whose_tensors_are_views_made_on_access():
         assert torch.equal(ctx.la_prefill(q, k, v, w, Slice()), want)
     assert torch.equal(pool.S[2:4], st.S) and torch.equal(pool.win[2:4], st.win) and pool.pos.tolist() == [0, 0, 8, 8, 0, 0]
     assert not pool.S[:2].any() and not pool.S[4:].any()
+
+
+def test_numbers_are_taken_as_int_and_float_take_them():
+    ctx, q, k, v, w, st = _inputs()
+    want = ctx.la_prefill_grouped(q, k, v, w, st, 32, 1.0, 0.5)
+    for group, alpha, scale in ((32.0, 1, np.float32(0.5)), (np.int64(32), torch.tensor(1.0), "0.5"), (torch.tensor(32), True, 0.5)):
+        assert torch.equal(ctx.la_prefill_grouped(q, k, v, w, st, group, alpha, scale), want)
+    with pytest.raises(TypeError):
+        ctx.la_prefill_grouped(q, k, v, w, st, None, 1.0, 0.5)
+    with pytest.raises(ValueError):
+        ctx.la_prefill_grouped(q, k, v, w, st, 32, "one", 0.5)
