@@ -32,13 +32,24 @@ def _newer(target: str, deps: list[str]) -> bool:
     return all(os.path.getmtime(d) <= t for d in deps)
 
 
-def _build_host(deps: list[str]) -> None:
-    """_host.so: links against libla_b200.so (found beside it) and the torch libraries of the running interpreter."""
-    src = os.path.join(CSRC, "host.cpp")
-    if _newer(HOST, [src, *deps]):
-        return
-    import sysconfig
+def _built_for(stamp: str, what: str) -> bool:
+    """Whether the last build noted in the file `stamp` was made for `what`."""
+    if not os.path.exists(stamp):
+        return False
+    with open(stamp) as f:
+        return f.read() == what
 
+
+def _build_host(deps: list[str]) -> None:
+    """_host.so: links against libla_b200.so (found beside it) and the torch libraries of the running interpreter.  Built
+    anew for another interpreter or another torch: it uses torch's C++ classes, whose layout changes between versions."""
+    import sysconfig
+    from importlib.metadata import version
+
+    src, stamp = os.path.join(CSRC, "host.cpp"), os.path.join(OBJ, "host.stamp")
+    what = f"python {sysconfig.get_config_var('SOABI')}, torch {version('torch')}"
+    if _newer(HOST, [src, *deps]) and _built_for(stamp, what):
+        return
     from torch.utils import cpp_extension
     inc = [f"-I{d}" for d in (*cpp_extension.include_paths("cuda"), sysconfig.get_paths()["include"], os.path.join(ROOT, "include"), CSRC)]
     libs = [f"-L{d}" for d in cpp_extension.library_paths("cuda")]
@@ -48,6 +59,8 @@ def _build_host(deps: list[str]) -> None:
     if r.returncode != 0:
         sys.stderr.write(r.stdout + r.stderr)
         raise RuntimeError("g++ failed on host.cpp")
+    with open(stamp, "w") as f:
+        f.write(what)
 
 
 def build(verbose: bool = False, force: bool = False) -> str:
