@@ -8,6 +8,10 @@ shared library is missing or a call fails, an exception is raised.
 The calls of a model's inner loop (prefill, decode, verify, accept, commit) go through _host.so, which checks the
 tensors and allocates missing outputs in C++: a small call is bound by this work, not by its kernel (csrc/host.cpp).
 Everything else is ctypes.
+
+Outputs of la_commit, la_accept_greedy and la_accept_threshold that the caller does not bring share one allocation per
+call: they do not overlap, but saving, resizing or sharing the storage of one concerns the others (clone it first, or
+bring a buffer).
 """
 from __future__ import annotations
 
@@ -261,7 +265,8 @@ class Context:
         return int(lib().la_prefill_workspace_bytes(self._h, B, T))
 
     def la_set_workspace(self, workspace: torch.Tensor | None) -> None:
-        """Lends a device buffer (any dtype, contiguous) to the context; it is kept alive by this object."""
+        """Lends a device buffer (any dtype, contiguous) to the context; it is kept alive by this object.  Prefills that may
+        overlap on the GPU, on different streams, need a context and a workspace each (see include/la.h)."""
         self._ws = workspace
         if workspace is None:
             _check("la_set_workspace", lib().la_set_workspace(self._h, None, 0))

@@ -133,13 +133,8 @@ static inline cudaError_t launch_cluster(int cluster, bool pdl, void (*kern)(KAr
   return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
 }
 template <typename... KArgs, typename... Args>
-static inline cudaError_t launch_maybe_pdl(bool pdl, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                                           Args... args) {
-  return launch_cluster(1, pdl, kern, grid, block, smem, s, args...);
-}
-template <typename... KArgs, typename... Args>
 static inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args... args) {
-  return launch_maybe_pdl(true, kern, grid, block, smem, s, args...);
+  return launch_cluster(1, true, kern, grid, block, smem, s, args...);
 }
 
 namespace la {

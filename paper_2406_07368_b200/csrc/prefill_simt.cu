@@ -9,8 +9,9 @@
 // through distributed shared memory; then all segments run at once.  No workspace, one launch.  Cost: S += phi(K)^T V
 // of all but a segment's last chunk is formed twice (d^2 of about 3 d^2 + C d multiply-adds per token).
 //
-// What bounds it: the latency of the shared-memory loads behind the multiply-adds at 12 warps per SM (two fifths of the
-// fp32 peak on 48 chains of 1000 tokens, d = 64: 67 us, where one CTA per chain that walked the tokens one by one took 520 us).  All products are register tiles (8 x 4 per thread at d = 64) fed by 128-bit
+// What bounds it: the latency of the shared-memory loads behind the multiply-adds at 12 warps per SM.  48 chains of 1000
+// tokens, d = 64: 64 us in a graph, where its multiply-adds alone need about 22 at the fp32 peak, and where one CTA per chain
+// that walked the tokens one by one took 443.  All products are register tiles (8 x 4 per thread at d = 64) fed by 128-bit
 // shared-memory loads, three wavefronts per thirty-two multiply-adds of a warp.
 #include <cooperative_groups.h>
 
@@ -452,7 +453,7 @@ static cudaError_t launch_t(la_ctx* ctx, int B, int Tlen, const void* q, const v
   cudaError_t e = allow_smem((const void*)kern, ctx->device);
   if (e != cudaSuccess) return e;
   // CTAs per chain, each a segment of whole chunks: a whole cluster, until the chains alone fill half of the places for
-  // CTAs.  (d = 64, 1000 tokens, us by CTAs per chain: 48 chains 196 with 1, 126 with 2, 94 with 4, 67 with 8; 192 chains
+  // CTAs.  (d = 64, 1000 tokens, us by CTAs per chain, as first measured: 48 chains 196 with 1, 126 with 2, 94 with 4, 67 with 8; 192 chains
   // 287, 254, 254, 254; 384 chains 374 and 480-510.  d = 128, 300 tokens: 48 chains 135, 95, 113, 86; 96 chains 135 and
   // 168-188.)
   const int BH = B * c.H, chunks = (Tlen + Sh::C - 1) / Sh::C;

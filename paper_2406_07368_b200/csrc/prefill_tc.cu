@@ -125,9 +125,8 @@ __host__ __device__ inline uint32_t off_grp(int W, bool lng) {
   return ((lng ? smem_bytes_long(W, true) : smem_bytes(W)) - 1024 + 15u) & ~15u;
 }
 __host__ __device__ inline uint32_t smem_bytes_grp(int W, bool lng) { return off_grp(W, lng) + kGrpScratch + 1024; }
-// Which windows take the long epilogue: above 5 taps it is the faster of the two (measured on 128 chains of 2048
-// tokens: 6 taps 126 us either way, 8 taps 132 against 154 us, 16 taps 126 against 254, 32 taps 162 against 686).
-// The three-branch mode compiles the short epilogue for 3 taps only.
+// Which windows take the long epilogue: above 5 taps the short one's nine halo buffers no longer fit (6 taps: 235 008 bytes
+// of shared memory, kMaxSmem is 232 448).  The three-branch mode compiles the short epilogue for 3 taps only.
 inline bool long_epilogue(int W, bool grouped = false) { return grouped ? W != 3 : W > 5; }
 
 // ---- PTX wrappers ------------------------------------------------------------------------
@@ -1966,7 +1965,7 @@ static cudaError_t launch_split(la_ctx* ctx, int BH, int T, int tile, const CUte
     cudaError_t e = allow_smem((const void*)skern, ctx->device);
     if (e != cudaSuccess) return e;
     ctx->launches += 1;
-    e = launch_maybe_pdl(true, skern, dim3(BH * (nseg - 1)), dim3(tc::kStateThreads), tc::kStateSmem, s, mk, mv, S_seg, z_seg,
+    e = launch_pdl(skern, dim3(BH * (nseg - 1)), dim3(tc::kStateThreads), tc::kStateSmem, s, mk, mv, S_seg, z_seg,
                          ctx->d_status, T, nseg, sp.seg_len, nseg - 1, init, (const float*)st.S, (const float*)st.z,
                          (const __nv_bfloat16*)st.win, win_seg, c.conv_taps);
     if (e != cudaSuccess) return e;
@@ -2038,7 +2037,7 @@ cudaError_t launch_segment_state_tc(la_ctx* ctx, int B, int T, const void* k, co
   cudaError_t e = allow_smem((const void*)skern, ctx->device);
   if (e != cudaSuccess) return e;
   ctx->launches += 1;
-  return launch_maybe_pdl(false, skern, dim3(BH), dim3(tc::kStateThreads), tc::kStateSmem, s, mk, mv, dS, dz, ctx->d_status, T,
+  return launch_cluster(1, false, skern, dim3(BH), dim3(tc::kStateThreads), tc::kStateSmem, s, mk, mv, dS, dz, ctx->d_status, T,
                           1, T, 1, 0, (const float*)nullptr, (const float*)nullptr, (const __nv_bfloat16*)nullptr,
                           (__nv_bfloat16*)nullptr, c.conv_taps);
 }
