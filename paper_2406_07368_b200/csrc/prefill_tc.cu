@@ -1879,7 +1879,8 @@ static cudaError_t launch_phi(la_ctx* ctx, int BH, int T, const CUtensorMap& mq,
 // long enough to cut (every segment a whole number of tiles).
 constexpr int kSplitMinTiles = 6;
 // Up to this many segments per chain the blocks of the main pass add up the sums before them as they load their state;
-// beyond it a launch of its own forms the prefixes.
+// beyond it a launch of its own forms the prefixes.  (Reached where clusters of that many are not all resident, as with 46 to
+// 49 chains in 3 segments: 900 tokens 28.0 us in place, 30.6 with the launch; 2000 tokens 47.0 and 48.5.)
 constexpr int kSumInPlace = 4;
 static void plan_split(const la_ctx* ctx, int BH, int T, int* nseg, int* seg_len, int tile = tc::TILE) {
   *nseg = 1;

@@ -56,11 +56,17 @@ def test_commit_outputs_of_skipped_sequences(given_path, given_len):
 def test_calls_on_a_given_stream():
     ctx, q, k, v, w, st = _inputs()
     want = ctx.la_prefill(q, k, v, w, st)
-    st2, out, s = ctx.new_state(2), torch.empty_like(q), torch.cuda.Stream()
+    st2, out, s = ctx.new_state(2), torch.full_like(q, 7.0), torch.cuda.Stream()
     s.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(s):
+        torch.cuda._sleep(200_000_000)                           # about 0.1 s in front of the call on its stream
     got = ctx.la_prefill(q, k, v, w, st2, out=out, stream=s)
+    before = out.clone()                                         # on the current stream, which the call must not be on
+    torch.cuda.current_stream().synchronize()
+    assert not s.query()
+    assert (before == 7.0).all()
     s.synchronize()
-    assert torch.equal(got, want)
+    assert got is out and torch.equal(got, want)
 
 
 def test_state_whose_tensors_are_views_made_on_access():
