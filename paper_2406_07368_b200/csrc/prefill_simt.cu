@@ -476,15 +476,16 @@ static cudaError_t launch_phi(la_ctx* ctx, int B, int Tlen, const void* q, const
 
 // Whether walking the tokens (prefill_walk.cu) is faster: a chunk costs the same however few tokens it holds.  One line per
 // number of chunks, in tokens, from both kernels at 50 lengths x 17 numbers of chains (fp32, 3 taps; us walked / in chunks):
-//   d = 64    up to one chain per SM: 26 tokens (26 14.3 / 14.8, 28 15.2 / 14.8).  Up to three, as many blocks as an SM holds: 28
-//             (256 chains: 26 17 / 18, 30 18.6 / 18).  Beyond, blocks wait for a place: 45 tokens per chunk (512 chains: 40
+//   d = 64    up to one chain per SM: 25 tokens (24 13.4 / 14.0, 26 14.3 / 14.8, 28 15.2 / 14.8; 1 tap: 24 12.5 / 13.1, 26 13.3 /
+//             13.2), 22 with ReLU, which is cheap for a whole chunk (22 13.8 / 13.8, 24 14.7 / 13.6).  Up to three, as many
+//             blocks as an SM holds: 28 and 25 (256 chains: 26 17 / 18, 30 18.6 / 18; ReLU: 25 17.8 / 17.9, 27 19 / 18.2).  Beyond, blocks wait for a place: 45 tokens per chunk (512 chains: 40
 //             tokens 34 / 37, 48 40 / 37; 82 66 / 75, 96 76 / 74; 129 102 / 113; 1024 chains: 40 60 / 58, 76 115 / 120)
 //   d = 128   up to one chain per SM, as many chunked blocks as an SM holds: 19.5 per chunk (14 tokens 12.6 / 13.0, 16 13.4 /
 //             12.8; 33 24 / 25.6).  Beyond: 28.5 (160 chains: 22 tokens 23.5 / 24, 24 25.6 / 24; 48 46 / 50; 161 144 / 160; 512
 //             chains: 48 95 / 102, 136 267 / 277), and 24.5 where the chains of the last pair of chunked waves, which is one
 //             wave walked, fill half of it (1024 chains: 18 tokens 85 / 88, 44 183 / 190)
-static bool walks(int d, int BH, int T, int sms) {
-  if (d == 64) return BH <= 3 * sms ? T <= (BH > sms ? 28 : 26) : T + 4 <= 45 * ((T + 63) / 64);
+static bool walks(int d, bool relu, int BH, int T, int sms) {
+  if (d == 64) return BH <= 3 * sms ? T <= (BH > sms ? (relu ? 25 : 28) : (relu ? 22 : 25)) : T + 4 <= 45 * ((T + 63) / 64);
   const int waves = (BH + sms - 1) / sms;
   return 2 * (T + 5) <= (waves == 1 ? 39 : waves % 2 == 0 ? 57 : 49) * ((T + 31) / 32);
 }
@@ -492,7 +493,7 @@ static bool walks(int d, int BH, int T, int sms) {
 cudaError_t launch_prefill_simt(la_ctx* ctx, int B, int Tlen, const void* q, const void* k, const void* v,
                                 const float* w, int init, const la_state& st, void* o, cudaStream_t s) {
   const la_config& c = ctx->cfg;
-  if (walks(c.d, B * c.H, Tlen, ctx->sm_count)) return launch_prefill_walk(ctx, B, Tlen, q, k, v, w, init, st, o, s);
+  if (walks(c.d, c.phi == LA_PHI_RELU, B * c.H, Tlen, ctx->sm_count)) return launch_prefill_walk(ctx, B, Tlen, q, k, v, w, init, st, o, s);
   if (c.io_dtype == LA_F32)
     return c.d == 64 ? simt::launch_phi<float, 64>(ctx, B, Tlen, q, k, v, w, init, st, o, s)
                      : simt::launch_phi<float, 128>(ctx, B, Tlen, q, k, v, w, init, st, o, s);

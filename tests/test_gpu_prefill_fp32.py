@@ -51,10 +51,11 @@ def test_one_block_per_chain_when_chains_abound(d, B, H):
     _run("f32", d, 100, 3, "elu1", 0.0, B, H, 40)
 
 
-@pytest.mark.parametrize("d,B,H,edges", [(64, 1, 2, (26,)), (64, 25, 8, (28,)), (64, 64, 8, (41, 86)), (128, 1, 2, (14, 34)),
-                                         (128, 19, 8, (23, 52, 80)), (128, 50, 8, (19, 44))])
-def test_both_sides_of_the_lines_between_walking_and_chunks(d, B, H, edges):
-    """Short calls walk their tokens; the lines depend on the head dimension and on the number of chains.  A call on either
+@pytest.mark.parametrize("d,phi,B,H,edges", [
+    (64, "elu1", 1, 2, (25,)), (64, "relu", 1, 2, (22,)), (64, "elu1", 25, 8, (28,)), (64, "relu", 25, 8, (25,)),
+    (64, "elu1", 64, 8, (41, 86)), (128, "elu1", 1, 2, (14, 34)), (128, "relu", 19, 8, (23, 52, 80)), (128, "elu1", 50, 8, (19, 44))])
+def test_both_sides_of_the_lines_between_walking_and_chunks(d, phi, B, H, edges):
+    """Short calls walk their tokens; the lines depend on the head dimension, the number of chains and phi.  A call on either
     side of each line continues 5 tokens (which are walked) and must agree with the oracle."""
     for T in (t + x for t in edges for x in (0, 1)):
-        _run("f32", d, T + 5, 3, "elu1", 0.0, B, H, 5)
+        _run("f32", d, T + 5, 3, phi, 1e-6 if phi == "relu" else 0.0, B, H, 5)
