@@ -23,8 +23,9 @@ struct CommitTables {
 
 // d = 64 keeps to 32 registers, eight blocks per SM: with the 48 that the window's eight rows in flight take, 1024 units took
 // 12.8 us instead of 10.6 (3 taps; few units and 32 taps, on the other hand, 5.2 instead of 6.4).
+// d = 128: 40 registers, six blocks per SM (48 and five: 1024 units 21.9 us instead of 20.4, 512 12.0 instead of 11.6).
 template <typename T, int D, int PHI>
-__global__ void __launch_bounds__(256, D == 64 ? 8 : 5)
+__global__ void __launch_bounds__(256, D == 64 ? 8 : 6)
 commit_kernel(const T* __restrict__ k, const T* __restrict__ v, const int32_t* __restrict__ parent,
               const int32_t* __restrict__ accept, float* __restrict__ S, float* __restrict__ z, T* __restrict__ win,
               int64_t* __restrict__ pos, int32_t* __restrict__ path_out, int32_t* __restrict__ commit_len, int* status,
