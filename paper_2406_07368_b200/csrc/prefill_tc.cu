@@ -401,14 +401,14 @@ __device__ __forceinline__ uint32_t swz(int row, int cc) { return (uint32_t)row 
 // ---- the kernel ------------------------------------------------------------------------------------
 // (Two channels per packed fp32 multiply-add: each half is the IEEE fused multiply-add of the scalar instruction.)
 __device__ __forceinline__ float2 bf2(uint32_t u) { return make_float2(lo_f(u), hi_f(u)); }
-// Long-window epilogue: one thread owns a pair of channels and 32 consecutive rows of the tile, in four blocks of 8.
-// conv_block adds one group of 8 taps to the 8 sums of a block: the 15 rows of v that those taps reach are each read once,
-// as one packed pair, and feed up to 8 of the sums.  Where the rows come from is fixed at compile time:
-//   ALL_V  the V buffer: pg[k] = the thread's column, in the swizzle of rows = k mod 8, 8 g rows before the block's first
-//   ALL_H  the halo column: hq = 8 g + 7 rows before the block's first
-//   MIXED  (the group that straddles the tile's first row) rows -7 ... -1 from the halo (hq = its row -7), 0 ... 7 from V
-// so that every load is one instruction with an immediate offset.  The block is not: with a copy of this code per block and
-// source (33 KB of instructions) the loop waited for its instructions.
+// Long-window epilogue: one thread owns a pair of channels and 32 consecutive rows of the tile, in two blocks of 16.
+// conv_block adds one group of 8 taps to the 16 sums of a block: the 23 rows of v that those taps reach are each read once,
+// as one packed pair, and feed up to 8 of the sums.  (Blocks of 8 rows read and unpack 15 rows for half as many sums: 32 taps, 128
+// chains of 2048 tokens, 139.4 us; 126.4 so.)
+// The rows come from the V buffer (pg[k]: the thread's column, in the swizzle of rows = k mod 8, 8 g rows before the block's
+// first), so that every load is one instruction with an immediate offset; HALO: the first nh of them from the halo column
+// (hq: the first of the 23).  Two copies of the loop and not one per nh, of which there are four: it has to stay in the
+// instruction cache (segments of 4 tiles, 9 taps: 40.3 us before, 44.1 with four copies, 40.9 with two).
 template <int I, int N, typename F>
 __device__ __forceinline__ void static_for(F&& f) {           // f(integral_constant<int, I>) ... for I, I + 1, ..., N - 1
   if constexpr (I < N) {
@@ -416,7 +416,6 @@ __device__ __forceinline__ void static_for(F&& f) {           // f(integral_cons
     static_for<I + 1, N>(f);
   }
 }
-enum { ALL_V = 0, MIXED = 1, ALL_H = 2 };
 // (Shared-memory addresses as 32-bit numbers and explicit ld.shared / st.shared: one register per address.)
 __device__ __forceinline__ uint32_t lds32(uint32_t a) {
   uint32_t v;
@@ -429,8 +428,59 @@ __device__ __forceinline__ float2 lds_f2(uint32_t a) {
   return v;
 }
 __device__ __forceinline__ void sts32(uint32_t a, uint32_t v) { asm volatile("st.shared.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory"); }
+template <bool HALO>
+__device__ __forceinline__ void conv_block(float2 (&acc)[16], uint32_t wtap, const uint32_t (&pg)[8], uint32_t hq, int nh) {
+  float2 wg[8];
+  static_for<0, 8>([&](auto tc_) {
+    constexpr int t = decltype(tc_)::value;
+    wg[t] = lds_f2(wtap + t * (D * 4));
+  });
+  static_for<0, 23>([&](auto ic) {
+    constexpr int i = decltype(ic)::value;
+    const uint32_t a = pg[(i + 1) & 7] + (i - 7) * 128, u = lds32(HALO && i < nh ? hq + i * (D * 2) : a);
+    const float2 x = bf2(u);
+    static_for<0, 8>([&](auto tc_) {
+      constexpr int tau = decltype(tc_)::value;   // tap (within the group) that links input row i to sum jj
+      constexpr int jj = i - 7 + tau;
+      if constexpr (jj >= 0 && jj < 16) acc[jj] = __ffma2_rn(wg[tau], x, acc[jj]);
+    });
+  });
+}
+// All tap groups of block blk (rows 16 blk ... 16 blk + 15 of the thread), then the sums are added to the attention
+// term that waits in the output tile.  first: the thread owns the first 32 rows of the tile (rows before them
+// come from the halo, hend = the halo column just past its last row).
+__device__ __forceinline__ void conv_rows(int blk, bool first, uint32_t wcol, const uint32_t (&pv)[8], uint32_t sthr, int cc,
+                                          uint32_t hend, int ngroups) {
+  float2 acc[16];
+#pragma unroll
+  for (int jj = 0; jj < 16; ++jj) acc[jj] = make_float2(0.f, 0.f);
+#pragma unroll 1
+  for (int g = 0; g < ngroups; ++g) {
+    const uint32_t wtap = wcol + g * (8 * D * 4), hq = hend + (16 * blk - 8 * g - 7) * (D * 2);
+    const int m = first ? g - 2 * blk : -1;
+    uint32_t pg[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) pg[k] = pv[k] + (2 * blk - g) * 1024;
+    if (m < 0) conv_block<false>(acc, wtap, pg, hq, 0);
+    else conv_block<true>(acc, wtap, pg, hq, 8 * m + 7);
+  }
+  sthr += blk * 2048;
+#pragma unroll
+  for (int j0 = 0; j0 < 16; j0 += 8) {
+    uint32_t lav[8];                              // the attention terms of 8 rows, all loads in flight at once
+#pragma unroll
+    for (int jj = 0; jj < 8; ++jj) lav[jj] = lds32(sthr + (j0 + jj) * 128 + ((cc ^ jj) << 4));
+#pragma unroll
+    for (int jj = 0; jj < 8; ++jj) {
+      const float2 la = bf2(lav[jj]);
+      sts32(sthr + (j0 + jj) * 128 + ((cc ^ jj) << 4), pack2(acc[j0 + jj].x + la.x, acc[j0 + jj].y + la.y));
+    }
+  }
+}
+
+enum { ALL_V = 0, MIXED = 1, ALL_H = 2 };
 template <int KIND>
-__device__ __forceinline__ void conv_block(float2 (&acc)[8], uint32_t wtap, const uint32_t (&pg)[8], uint32_t hq) {
+__device__ __forceinline__ void conv_block8(float2 (&acc)[8], uint32_t wtap, const uint32_t (&pg)[8], uint32_t hq) {
   float2 wg[8];
   static_for<0, 8>([&](auto tc_) {
     constexpr int t = decltype(tc_)::value;
@@ -454,10 +504,13 @@ __device__ __forceinline__ void conv_block(float2 (&acc)[8], uint32_t wtap, cons
     });
   });
 }
+// The same in blocks of 8 rows, whose code is half as long: for windows of one group of taps, which is gone through once per block
+// (segments of 4 tiles, 6 taps: 37.1 us, 39.6 in blocks of 16), and for the three-branch mode (16 taps, groups of 64: 52.7 and 55.6).
+// conv_block8: rows -7 ... 7 of a block all from the V buffer (ALL_V), all from the halo (ALL_H), or the negative ones (MIXED).
 // All tap groups of block blk (rows 8 blk ... 8 blk + 7 of the thread), then the sums are added to the attention
 // term that waits in the output tile.  first: the thread owns the first 32 rows of the tile (rows before them
 // come from the halo, hend = the halo column just past its last row).
-__device__ __forceinline__ void conv_rows(int blk, bool first, uint32_t wcol, const uint32_t (&pv)[8], uint32_t sthr, int cc,
+__device__ __forceinline__ void conv_rows8(int blk, bool first, uint32_t wcol, const uint32_t (&pv)[8], uint32_t sthr, int cc,
                                           uint32_t hend, int ngroups) {
   float2 acc[8];
 #pragma unroll
@@ -469,11 +522,11 @@ __device__ __forceinline__ void conv_rows(int blk, bool first, uint32_t wcol, co
       uint32_t pg[8];
 #pragma unroll
       for (int k = 0; k < 8; ++k) pg[k] = pv[k] + (blk - g) * 1024;
-      conv_block<ALL_V>(acc, wtap, pg, 0u);
+      conv_block8<ALL_V>(acc, wtap, pg, 0u);
     } else if (g == blk) {
-      conv_block<MIXED>(acc, wtap, pv, hend - 7 * (D * 2));
+      conv_block8<MIXED>(acc, wtap, pv, hend - 7 * (D * 2));
     } else {
-      conv_block<ALL_H>(acc, wtap, pv, hend + (8 * (blk - g) - 7) * (D * 2));
+      conv_block8<ALL_H>(acc, wtap, pv, hend + (8 * (blk - g) - 7) * (D * 2));
     }
   }
   sthr += blk * 1024;
@@ -1435,8 +1488,13 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
           for (int k = 0; k < 8; ++k) pv[k] = vthr + ((cc ^ k) << 4);
           const uint32_t sthr = sbase + (par ? OFF_K1 : OFF_K0) + colk;
           const int mine = valid - 32 * jq;                  // rows of this thread that hold tokens
+          if (GRP || ngroups == 1) {
 #pragma unroll 1
-          for (int blk = 0; blk < 4 && 8 * blk < mine; ++blk) conv_rows(blk, jq == 0, wcol, pv, sthr, cc, hend, ngroups);
+            for (int blk = 0; blk < 4 && 8 * blk < mine; ++blk) conv_rows8(blk, jq == 0, wcol, pv, sthr, cc, hend, ngroups);
+          } else {
+#pragma unroll 1
+            for (int blk = 0; blk < 2 && 16 * blk < mine; ++blk) conv_rows(blk, jq == 0, wcol, pv, sthr, cc, hend, ngroups);
+          }
           if (jq == 0) {
             // The rows before the next tile: the last W-1 of (halo ++ valid rows of v), in place.  This thread is the
             // only one that reads or writes this column of the halo (the rows of the other threads start at 32, and
