@@ -575,6 +575,12 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
   const uint32_t sbase = smem_u32(smem);
   constexpr bool GRP = GM > 0, MULTI = GM == 2;
   constexpr bool LONG = WT < 0;                  // the epilogue for longer tap windows
+  // The exact layer keeps its loops rolled: all roles' code of one tile has to stay in the SM's instruction cache.  (Unrolled,
+  // 23 KB of it came anew with every tile from the cache that a GPC shares, and two of a scheduler's five warps waited for
+  // instructions on average, 0.6 of them now: 128 chains of 2048 tokens, 3 taps, 76.0 us unrolled, 71.7 rolled; 32 chains of 1700
+  // tokens 37.3 and 35.2.)  Not the three-branch mode, whose phi lies on the longest chain of a tile (groups of 64: 95 us, 104
+  // rolled), nor a long window beside a ReLU (32 chains of 8000 tokens, 6 taps: 100.7 and 104.4).
+  constexpr bool kRoll = !GRP && !(LONG && PHI == LA_PHI_RELU);
   // Who copies the state between two tiles: group B has the time beside an elu + 1 (which keeps group A busy), group A beside
   // a ReLU or a long window (which keeps group B busy).
   constexpr bool SNAP_A = LONG || (PHI == LA_PHI_RELU && !GRP);
@@ -737,14 +743,27 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
     if constexpr (NI > 0) {
       const int valid = min(tstep, T - m * tstep);
       const int ct = ta & 15, rg = ta >> 4;                     // chunk column 0..15, row group 0..15
-      unsigned char* Kb = smem + ((m & 1) ? OFF_K1 : OFF_K0) + (ct >> 3) * KBOX_BYTES;
-      uint4 x[NI];                                              // all loads first: they do not wait for the stores
+      if constexpr (kRoll) {                                    // (16 rows further on the swizzle is the same)
+        unsigned char* Kb = smem + ((m & 1) ? OFF_K1 : OFF_K0) + (ct >> 3) * KBOX_BYTES + swz(rg + 16 * I0, ct & 7);
+        auto put = [&](int i, uint4 x) {
+          *reinterpret_cast<uint4*>(Kb + i * 2048) = rg + 16 * (I0 + i) < valid ? phi8<PHI>(x) : make_uint4(0u, 0u, 0u, 0u);
+        };
+#pragma unroll 1
+        for (int i = 0; i < NI; i += 2) {                       // two at a time, the loads first
+          const uint4 x = *reinterpret_cast<const uint4*>(Kb + i * 2048), y = *reinterpret_cast<const uint4*>(Kb + min(i + 1, NI - 1) * 2048);
+          put(i, x);
+          if (i + 1 < NI) put(i + 1, y);
+        }
+      } else {
+        unsigned char* Kb = smem + ((m & 1) ? OFF_K1 : OFF_K0) + (ct >> 3) * KBOX_BYTES;
+        uint4 x[NI];                                              // all loads first: they do not wait for the stores
 #pragma unroll
-      for (int i = 0; i < NI; ++i) x[i] = *reinterpret_cast<const uint4*>(Kb + swz(rg + 16 * (I0 + i), ct & 7));
+        for (int i = 0; i < NI; ++i) x[i] = *reinterpret_cast<const uint4*>(Kb + swz(rg + 16 * (I0 + i), ct & 7));
 #pragma unroll
-      for (int i = 0; i < NI; ++i) {
-        const int j = rg + 16 * (I0 + i);
-        *reinterpret_cast<uint4*>(Kb + swz(j, ct & 7)) = j < valid ? phi8<PHI>(x[i]) : make_uint4(0u, 0u, 0u, 0u);
+        for (int i = 0; i < NI; ++i) {
+          const int j = rg + 16 * (I0 + i);
+          *reinterpret_cast<uint4*>(Kb + swz(j, ct & 7)) = j < valid ? phi8<PHI>(x[i]) : make_uint4(0u, 0u, 0u, 0u);
+        }
       }
     }
   };
@@ -920,7 +939,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
       tc_fence_after();
       uint32_t zbits = 0u;
       if (hf == 0) zbits = tmem_ld1(tmem + lane_addr + Z_COL);
-#pragma unroll
+#pragma unroll (kRoll ? 1 : 2)
       for (int qq = 0; qq < 2; ++qq) {
         uint32_t v[32];
         LA_TMEM_LD32(tmem + lane_addr + S_COL + 64 * hf + 32 * qq, v);
@@ -1165,23 +1184,32 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
       ok = __all_sync(0xffffffffu, ok);
       if (GRP) sync_group_a();                    // every thread is done with the halves of the last tile (dgh, mlh)
       // phi(q) of row r, this thread's 64 channels: 32 packed pairs = 32 TMEM columns of lane r.
-      uint32_t fq[32];
+      uint32_t fq[kRoll ? 16 : 32];
       float dg = 0.f;
-      if (ok) {
+      auto phi_q = [&](int c0) {                  // pieces c0 ... of the row
 #pragma unroll
-        for (int cc = 0; cc < 8; ++cc) {
-          const uint4 f = phi8<PHI>(*reinterpret_cast<const uint4*>(Qb + swz(r, cc)));
+        for (int cc = 0; cc < (kRoll ? 4 : 8); ++cc) {
+          const uint4 f = phi8<PHI>(*reinterpret_cast<const uint4*>(Qb + swz(r, c0 + cc)));
           fq[4 * cc] = f.x; fq[4 * cc + 1] = f.y; fq[4 * cc + 2] = f.z; fq[4 * cc + 3] = f.w;
         }
-      }
+      };
+      if (ok && !kRoll) phi_q(0);
       if (!SNAP_A) {                              // the products of tile n-1 that read these columns are complete
         if (n > 0) ok = ok && mbar_wait((bar0 + 8u * (B_MMA_Q)), par ^ 1, abort);
         ok = __all_sync(0xffffffffu, ok);
         tc_fence_after();
       }
       if (ok) {
-        LA_TMEM_ST32(tmem + lane_addr + FQ_COL + 32 * hf, fq);
-        if (GRP) {                                // this half of phi(q) . z_prev, z in fp32
+        if constexpr (!kRoll) {
+          LA_TMEM_ST32(tmem + lane_addr + FQ_COL + 32 * hf, fq);
+        } else {
+#pragma unroll 1
+          for (int qq = 0; qq < 2; ++qq) {
+            phi_q(4 * qq);
+            LA_TMEM_ST16(tmem + lane_addr + FQ_COL + 32 * hf + 16 * qq, fq);
+          }
+        }
+        if constexpr (GRP) {                      // this half of phi(q) . z_prev, z in fp32
 #pragma unroll
           for (int e = 0; e < 32; e += 2) {
             const float4 z4 = *reinterpret_cast<const float4*>(zs + 64 * hf + 2 * e);
@@ -1218,7 +1246,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
       ok = __all_sync(0xffffffffu, ok);
       if (!GRP && ok) {
         tc_fence_after();
-#pragma unroll
+#pragma unroll (kRoll ? 1 : 2)
         for (int qq = 0; qq < 2; ++qq) {
           const int col0 = 64 * hf + 32 * qq;
           uint32_t v[32], pk[16];
@@ -1556,9 +1584,6 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
       if (ok && (!GRP || 32 * q4 < valid)) {      // (32 rows behind a partly filled tile's tokens: zeros already)
         tc_fence_after();
         const uint32_t oaddr = tmem + lane_addr + O_COL + 64 * hf;
-        uint32_t a0[16], a1[16];                  // rows 0-15 and 16-31
-        LA_TMEM_LD_FRAG4(oaddr, a0);
-        LA_TMEM_LD_FRAG4(oaddr + (16u << 16), a1);
         float rden[4];
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
@@ -1566,41 +1591,54 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
           const float* dr = denbuf + par * 2 * D + 32 * q4 + (lane >> 2) + 8 * m;
           rden[m] = 1.f / (dr[0] + dr[D] + (GRP ? 0.f : eps));  // (three-branch mode: those left the finished factor)
         }
+        auto piece = [&](int cc, const uint32_t* f0, const uint32_t* f1) {   // 8 channels: fragments of rows 0-15 and 16-31
+          float2 acc[4];
 #pragma unroll
-        for (int qq = 0; qq < 2; ++qq) {
-          tmem_wait_ld();
-#pragma unroll
-          for (int g = 0; g < 4; ++g) {
-            const int cc = 4 * qq + g;
-            float2 acc[4];
-#pragma unroll
-            for (int m = 0; m < 4; ++m) {
-              const uint32_t* src = (m < 2 ? a0 : a1) + 4 * g + 2 * (m & 1);
-              acc[m] = __fmul2_rn(make_float2(__uint_as_float(src[0]), __uint_as_float(src[1])), make_float2(rden[m], rden[m]));
-            }
-#pragma unroll
-            for (int t = 0; t < WN; ++t) {
-              uint32_t u[4];
-              ldmatrix4(vrow[t] ^ (uint32_t)(cc << 4), u);
-              const float2 wt = lds_f2(waddr + t * (D * 4) + cc * 32);
-#pragma unroll
-              for (int m = 0; m < 4; ++m) acc[m] = __ffma2_rn(wt, bf2(u[m]), acc[m]);
-            }
-            uint32_t out[4];
-#pragma unroll
-            for (int m = 0; m < 4; ++m) {
-              out[m] = pack2(acc[m].x, acc[m].y);
-              // a partly filled tile stays zero below its tokens
-              if (GRP && 32 * q4 + (lane >> 2) + 8 * m >= valid) out[m] = 0u;
-            }
-            stmatrix4(vrow[0] ^ (uint32_t)(cc << 4), out);
+          for (int m = 0; m < 4; ++m) {
+            const uint32_t* src = (m < 2 ? f0 : f1) + 2 * (m & 1);
+            acc[m] = __fmul2_rn(make_float2(__uint_as_float(src[0]), __uint_as_float(src[1])), make_float2(rden[m], rden[m]));
           }
-          if (qq == 0) {
+#pragma unroll
+          for (int t = 0; t < WN; ++t) {
+            uint32_t u[4];
+            ldmatrix4(vrow[t] ^ (uint32_t)(cc << 4), u);
+            const float2 wt = lds_f2(waddr + t * (D * 4) + cc * 32);
+#pragma unroll
+            for (int m = 0; m < 4; ++m) acc[m] = __ffma2_rn(wt, bf2(u[m]), acc[m]);
+          }
+          uint32_t out[4];
+#pragma unroll
+          for (int m = 0; m < 4; ++m) {
+            out[m] = pack2(acc[m].x, acc[m].y);
+            // a partly filled tile stays zero below its tokens
+            if (GRP && 32 * q4 + (lane >> 2) + 8 * m >= valid) out[m] = 0u;
+          }
+          stmatrix4(vrow[0] ^ (uint32_t)(cc << 4), out);
+        };
+        uint32_t a0[16], a1[16];                  // rows 0-15 and 16-31 of 32 channels
+        if (!kRoll) {
+          LA_TMEM_LD_FRAG4(oaddr, a0);
+          LA_TMEM_LD_FRAG4(oaddr + (16u << 16), a1);
+        }
+#pragma unroll (kRoll ? 1 : 2)
+        for (int qq = 0; qq < 2; ++qq) {
+          if (kRoll) {
+            LA_TMEM_LD_FRAG4(oaddr + 32 * qq, a0);
+            LA_TMEM_LD_FRAG4(oaddr + 32 * qq + (16u << 16), a1);
+          }
+          tmem_wait_ld();
+          if (kRoll && qq == 1) {
+            tc_fence_before();
+            mbar_arrive((bar0 + 8u * (B_EPI0 + par)));         // this accumulator has been read
+          }
+#pragma unroll
+          for (int g = 0; g < 4; ++g) piece(4 * qq + g, a0 + 4 * g, a1 + 4 * g);
+          if (!kRoll && qq == 0) {
             LA_TMEM_LD_FRAG4(oaddr + 32, a0);
             LA_TMEM_LD_FRAG4(oaddr + 32 + (16u << 16), a1);
             tmem_wait_ld();
             tc_fence_before();
-            mbar_arrive((bar0 + 8u * (B_EPI0 + par)));         // this accumulator has been read
+            mbar_arrive((bar0 + 8u * (B_EPI0 + par)));
           }
         }
       } else {
