@@ -685,8 +685,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
     }
     sm.abort = 0;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    // the first tile is requested at once (nothing below touches the rows that it brings); the others follow behind the
-    // taps and the window, which would otherwise wait for them (20 MB over all blocks: 3 us)
+    // the first tile is requested at once (nothing below touches the rows that it brings)
     pdl_wait();
     load_k(0);
     if (!fused) load_q0();
@@ -699,8 +698,11 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
   float* denbuf = reinterpret_cast<float*>(smem + off_den(z3));
-  for (int idx = tid; idx < (int)ones_bytes(z3) / 16; idx += kThreads)         // the block of ones <- 0
-    reinterpret_cast<uint4*>(smem + OFF_ONES)[idx] = make_uint4(0u, 0u, 0u, 0u);
+  for (int idx = tid; idx < (int)ones_bytes(z3) / 16; idx += kThreads) {       // the block of ones: column 0 <- 1, the others <- 0
+    const bool first = z3 ? (idx & 7) == ((idx >> 3) & 7) : (idx & 8) == 0;
+    reinterpret_cast<uint4*>(smem + OFF_ONES)[idx] = make_uint4(first ? 0x3f80u : 0u, 0u, 0u, 0u);
+  }
+  if (GRP && tid < TILE) zs[tid] = 0.f;
   if (GRP && tstep < TILE) {                                                   // partly filled tiles: rows tstep-127 of V <- 0
     const int per_box = (TILE - tstep) * 8;                                    // 16-byte pieces per box
     for (int idx = tid; idx < 4 * per_box; idx += kThreads)
@@ -708,32 +710,42 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
   }
   for (int idx = tid; idx < 4 * 1024 / 16; idx += kThreads)                    // rows 128-135 of the four K boxes <- 0
     reinterpret_cast<uint4*>(smem + OFF_K0 + (idx >> 6) * KBOX_BYTES + BOX_BYTES)[idx & 63] = make_uint4(0u, 0u, 0u, 0u);
-  pdl_wait();                                     // everything above touched shared memory and TMEM only
-  if (early) pdl_trigger();
-  for (int idx = tid; idx < (LONG ? (int)long_taps(W) : W) * D; idx += kThreads)
-    wsm[idx] = idx < W * D ? w[((size_t)h * D + (idx % D)) * W + idx / D] : 0.f;
-  if (LONG) {                                    // [long_taps - 1][128]: zeros, then the W-1 rows of the window
-    const int lead = ((int)long_taps(W) - W) * D;
-    for (int idx = tid; idx < ((int)long_taps(W) - 1) * D; idx += kThreads)
-      halo0[idx] = has_in && idx >= lead ? win_in[idx - lead] : __float2bfloat16_rn(0.f);
-  } else {
-    for (int idx = tid; idx < (W - 1) * 16; idx += kThreads)
-      *reinterpret_cast<uint4*>(smem + off_halo(W) + halo_at(idx >> 4, idx & 15, W)) =
-          has_in ? reinterpret_cast<const uint4*>(win_in)[idx] : make_uint4(0u, 0u, 0u, 0u);
-  }
-  __syncthreads();
-  if (tid == kCopyWarp * 32 && nchunks > 1) {
-    load_k(1);
-    load_v(1);
-  }
-  if (tid < TILE) {
-    *reinterpret_cast<__nv_bfloat16*>(smem + OFF_ONES + (z3 ? swz(tid, 0) : ext_offset(tid, 0))) = __float2bfloat16_rn(1.f);
-    if (GRP) zs[tid] = 0.f;
+  // The taps, for group B, and the rows before the first tile, for those who copy them: `nt` threads, t of them this one.
+  auto load_taps = [&](int t, int nt) {
+    for (int idx = t; idx < (LONG ? (int)long_taps(W) : W) * D; idx += nt)
+      wsm[idx] = idx < W * D ? w[((size_t)h * D + (idx % D)) * W + idx / D] : 0.f;
+  };
+  auto load_window = [&](int t, int nt) {
+    if (LONG) {                                  // [long_taps - 1][128]: zeros, then the W-1 rows of the window
+      const int lead = ((int)long_taps(W) - W) * D;
+      for (int idx = t; idx < ((int)long_taps(W) - 1) * D; idx += nt)
+        halo0[idx] = has_in && idx >= lead ? win_in[idx - lead] : __float2bfloat16_rn(0.f);
+    } else {
+      for (int idx = t; idx < (W - 1) * 16; idx += nt)
+        *reinterpret_cast<uint4*>(smem + off_halo(W) + halo_at(idx >> 4, idx & 15, W)) =
+            has_in ? reinterpret_cast<const uint4*>(win_in)[idx] : make_uint4(0u, 0u, 0u, 0u);
+    }
+  };
+  if constexpr (GRP) {                            // (by everybody, ahead of the barrier: the other way costs these kernels registers)
+    pdl_wait();
+    load_taps(tid, kThreads);
+    load_window(tid, kThreads);
   }
   fence_proxy_async();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
+  if (!GRP) pdl_wait();                           // everything above touched shared memory and TMEM only
+  if (early) pdl_trigger();
+  if (tid == kCopyWarp * 32 && nchunks > 1) {
+    load_k(1);
+    load_v(1);
+  }
+  if constexpr (!GRP) {                           // nobody else waits for these loads (group B: a barrier of its own)
+    if (warp < 8) load_taps(tid, kThreadsB);
+    if (LONG ? warp < 8 : warp == kHaloWarp) load_window(LONG ? tid : lane, LONG ? kThreadsB : 32);
+    __syncwarp();
+  }
   const uint32_t tmem = sm.tmem_base;
 
   // phi on rows 16 I0 ... 16 I1 - 1 of the K tile of tile m, in place, by 256 threads (ta); rows at or beyond the end of the
@@ -1451,6 +1463,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
   } else {
     // =============================== group B: epilogue (256 threads) ===============================
     if (TRADE && kRegsB > 96) regs_up<kRegsB>();
+    if (!GRP) sync_group_b();                     // the taps (long windows: and the rows before the first tile) are in place
     const int r = 32 * (warp & 3) + lane;         // tile row = TMEM lane
     const int hf = warp >> 2;                     // column half
     const uint32_t lane_addr = (uint32_t)(32 * (warp & 3)) << 16;
