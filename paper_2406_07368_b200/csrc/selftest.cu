@@ -5,7 +5,7 @@
 
 namespace la {
 
-__global__ void __launch_bounds__(64) wait_timeout_kernel(int* status, unsigned long long limit_ns, long long* waited_ns) {
+__global__ void __launch_bounds__(64) wait_timeout_kernel(int* status, uint32_t limit_ns, long long* waited_ns) {
   __shared__ unsigned long long barrier;
   __shared__ int abort_flag;
   const uint32_t bar = (uint32_t)__cvta_generic_to_shared(&barrier);
@@ -14,7 +14,7 @@ __global__ void __launch_bounds__(64) wait_timeout_kernel(int* status, unsigned 
     abort_flag = 0;
   }
   __syncthreads();
-  const unsigned long long t0 = global_ns();
+  const uint32_t t0 = global_ns();
   const bool ok = mbar_wait(bar, 0, &abort_flag, limit_ns);      // phase 0 never completes
   if (!ok && threadIdx.x == 0) {
     report(status, LA_ERR_TIMEOUT);
@@ -29,7 +29,7 @@ extern "C" la_status la_selftest_wait_timeout(la_ctx* ctx, uint32_t limit_us, in
   int prev = -1;
   if (cudaGetDevice(&prev) != cudaSuccess) return LA_ERR_CUDA;
   if (prev != ctx->device && cudaSetDevice(ctx->device) != cudaSuccess) return LA_ERR_CUDA;
-  la::wait_timeout_kernel<<<1, 64, 0, static_cast<cudaStream_t>(stream)>>>(ctx->d_status, 1000ull * limit_us,
+  la::wait_timeout_kernel<<<1, 64, 0, static_cast<cudaStream_t>(stream)>>>(ctx->d_status, 1000u * limit_us,
                                                                           reinterpret_cast<long long*>(waited_ns));
   const cudaError_t e = cudaGetLastError();
   ctx->launches += 1;
