@@ -575,12 +575,12 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
   const uint32_t sbase = smem_u32(smem);
   constexpr bool GRP = GM > 0, MULTI = GM == 2;
   constexpr bool LONG = WT < 0;                  // the epilogue for longer tap windows
-  // The exact layer keeps its loops rolled: all roles' code of one tile has to stay in the SM's instruction cache.  (Unrolled,
-  // 23 KB of it came anew with every tile from the cache that a GPC shares, and two of a scheduler's five warps waited for
-  // instructions on average, 0.6 of them now: 128 chains of 2048 tokens, 3 taps, 76.0 us unrolled, 71.7 rolled; 32 chains of 1700
-  // tokens 37.3 and 35.2.)  Not the three-branch mode, whose phi lies on the longest chain of a tile (groups of 64: 95 us, 104
-  // rolled), nor a long window beside a ReLU (32 chains of 8000 tokens, 6 taps: 100.7 and 104.4).
-  constexpr bool kRoll = !GRP && !(LONG && PHI == LA_PHI_RELU);
+  // The exact layer with a short window keeps its loops rolled: all roles' code of one tile has to stay in the SM's instruction
+  // cache.  (Unrolled, 23 KB of it came anew with every tile from the cache that a GPC shares, and two of a scheduler's five
+  // warps waited for instructions on average, 0.6 of them now: 128 chains of 2048 tokens, 3 taps, 71.7 us unrolled, 67.6 rolled;
+  // 32 chains of 1700 tokens 37.4 and 35.2.)  Not the three-branch mode, whose phi lies on the longest chain of a tile (groups of 64:
+  // 95 us, 104 rolled), nor long windows, whose tap sums leave little of the wait (32 taps: 127.2 us, 128.9 rolled).
+  constexpr bool kRoll = !LONG && !GRP;
   // Who copies the state between two tiles: group B has the time beside an elu + 1 (which keeps group A busy), group A beside
   // a ReLU or a long window (which keeps group B busy).
   constexpr bool SNAP_A = LONG || (PHI == LA_PHI_RELU && !GRP);
