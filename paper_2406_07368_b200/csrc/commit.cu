@@ -23,9 +23,8 @@ struct CommitTables {
 
 // d = 64 keeps to 32 registers, eight blocks per SM: with the 48 that the window's eight rows in flight take, 1024 units took
 // 12.8 us instead of 10.6 (3 taps; few units and 32 taps, on the other hand, 5.2 instead of 6.4).
-// d = 128: 40 registers, six blocks per SM (48 and five: 1024 units 21.9 us instead of 20.4, 512 12.0 instead of 11.6).
-template <typename T, int D, int PHI>
-__global__ void __launch_bounds__(256, D == 64 ? 8 : 6)
+template <typename T, int D, int PHI, int BLOCKS>
+__global__ void __launch_bounds__(256, BLOCKS)
 commit_kernel(const T* __restrict__ k, const T* __restrict__ v, const int32_t* __restrict__ parent,
               const int32_t* __restrict__ accept, float* __restrict__ S, float* __restrict__ z, T* __restrict__ win,
               int64_t* __restrict__ pos, int32_t* __restrict__ path_out, int32_t* __restrict__ commit_len, int* status,
@@ -129,18 +128,42 @@ commit_kernel(const T* __restrict__ k, const T* __restrict__ v, const int32_t* _
   if (h == 0 && part == 0 && t == 0) pos[b] += L;
 }
 
-template <typename T, int D, int PHI>
-static cudaError_t launch_t(la_ctx* ctx, int B, int N, const void* k, const void* v, const int32_t* parent,
+template <int D> static size_t commit_smem(const la_config& c) {
+  return (size_t)2 * c.max_depth * D * sizeof(float) + sizeof(CommitTables);
+}
+
+template <typename T, int D, int PHI, int BLOCKS>
+static cudaError_t launch_b(la_ctx* ctx, int B, int N, const void* k, const void* v, const int32_t* parent,
                             const int32_t* accept, const la_state& st, int32_t* path_out, int32_t* commit_len, int fresh,
                             cudaStream_t s) {
   const la_config& c = ctx->cfg;
-  auto kern = commit_kernel<T, D, PHI>;
-  const size_t smem = (size_t)2 * c.max_depth * D * sizeof(float) + sizeof(CommitTables);
+  auto kern = commit_kernel<T, D, PHI, BLOCKS>;
+  const size_t smem = commit_smem<D>(c);
   cudaError_t e = allow_smem((const void*)kern, ctx->device);
   if (e != cudaSuccess) return e;
   ctx->launches += 1;
   return launch_pdl(kern, dim3(B * c.H * kCommitSplit), dim3(256), smem, s, (const T*)k, (const T*)v, parent, accept, st.S,
                     st.z, (T*)st.win, st.pos, path_out, commit_len, ctx->d_status, c.H, N, c.conv_taps, c.max_depth, fresh);
+}
+
+template <typename T, int D, int PHI>
+static cudaError_t launch_t(la_ctx* ctx, int B, int N, const void* k, const void* v, const int32_t* parent,
+                            const int32_t* accept, const la_state& st, int32_t* path_out, int32_t* commit_len, int fresh,
+                            cudaStream_t s) {
+  if constexpr (D == 64) {
+    return launch_b<T, D, PHI, 8>(ctx, B, N, k, v, parent, accept, st, path_out, commit_len, fresh, s);
+  } else {
+    // Six blocks per SM (40 registers; a ReLU spills 4 bytes, measured with them) or five (48).  Six where the launch then takes one
+    // wave instead of two (a few blocks more find room as the first end), and from three waves of five on: 186 ... 228 units
+    // 0.89-0.99 of the time of five, 372 ... 1280 units 0.94-0.99 (3 taps, both types, both phi); between them, in two waves either
+    // way, 0.99-1.03; 128 ... 184 units are one wave of five, 1.05-1.08 of whose time six took.  And only while six blocks leave most
+    // of the SM's memory to the L1, through which everything else goes: 512 and 1024 units 0.97 and 0.94 up to max_depth 24, 0.98 and
+    // 0.98 at 26, 0.99 and 1.00 at 28, 1.08 and 1.20 at 32.
+    const int blocks = B * ctx->cfg.H * kCommitSplit, sms = ctx->sm_count;
+    const bool six = ((blocks > 5 * sms && 5 * blocks <= 31 * sms) || blocks > 10 * sms) && 6 * commit_smem<D>(ctx->cfg) <= 160u * 1024u;
+    return six ? launch_b<T, D, PHI, 6>(ctx, B, N, k, v, parent, accept, st, path_out, commit_len, fresh, s)
+               : launch_b<T, D, PHI, 5>(ctx, B, N, k, v, parent, accept, st, path_out, commit_len, fresh, s);
+  }
 }
 
 template <typename T, int D>

@@ -96,14 +96,17 @@ def test_segments_of_few_tiles(tiles, W, group):
 
 @pytest.mark.parametrize("io,d", [("f32", 64), ("f32", 128), ("bf16", 64), ("bf16", 128)])
 @pytest.mark.parametrize("W", [1, 3, 12])
-def test_commit_of_paths_of_every_length(io, d, W):
-    """Chains of 64 nodes, accepted up to every node there is (rank-1 updates in order, and the window's rows)."""
-    H, N = 2, 64
+@pytest.mark.parametrize("H,depth,phi", [(2, 64, "elu1"), (2, 64, "relu"), (10, 16, "relu"), (10, 33, "elu1"), (20, 16, "elu1")])
+def test_commit_of_paths_of_every_length(io, d, W, H, depth, phi):
+    """Chains of 64 nodes, accepted up to every node there is (rank-1 updates in order, and the window's rows).  With d = 128 on 148
+    SMs: 38 units fit in one wave of five blocks per SM, 190 in one of six (not with paths of 33), 380 take three waves of five."""
+    N = 64
     lens = [0, 1, 2, 3, 4, 5, 7, 8, 9, 12, 15, 16, 17, 31, 32, 33, 48, 63, 64]
+    lens = [min(n, depth) for n in lens]
     B = len(lens)
     _, k, v = wl.qkv(11, (B, H, N, d), 0.3, io)
     parent, accept = np.stack([wl.chain_tree(N)] * B), np.array(lens, dtype=np.int32) - 1
-    ctx = binding.Context(H, d, W, "elu1", 0.0, io, max_nodes=64, max_depth=64)
+    ctx = binding.Context(H, d, W, phi, 0.0, io, max_nodes=64, max_depth=depth)
     st = ctx.new_state(B)
     g = np.random.default_rng(3)
     S, z = g.normal(size=st.S.shape).astype(np.float32), g.uniform(1, 2, st.z.shape).astype(np.float32)
@@ -112,9 +115,9 @@ def test_commit_of_paths_of_every_length(io, d, W):
     path, n = ctx.la_commit(_dev(k, io), _dev(v, io), torch.from_numpy(parent).cuda(), torch.from_numpy(accept).cuda(), st)
     assert ctx.la_last_device_status() == binding.LA_OK
     assert n.tolist() == lens
-    fk = np.where(k > 0, k + 1.0, np.exp(np.minimum(k, 0.0)))
+    fk = np.where(k > 0, k + 1.0, np.exp(np.minimum(k, 0.0))) if phi == "elu1" else np.maximum(k, 0.0)
     for b, L in enumerate(lens):
-        assert path[b].tolist() == list(range(L)) + [-1] * (64 - L)
+        assert path[b].tolist() == list(range(L)) + [-1] * (depth - L)
         assert rel_err(st.S[b].cpu().numpy(), S[b] + np.einsum("hna,hnc->hac", fk[b, :, :L], v[b, :, :L])) < TOL["f32"]
         assert rel_err(st.z[b].cpu().numpy(), z[b] + fk[b, :, :L].sum(1)) < TOL["f32"]
         rows = np.concatenate([win[b], v[b, :, :L]], axis=1)
