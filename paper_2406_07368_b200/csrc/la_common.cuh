@@ -46,12 +46,17 @@ __device__ __forceinline__ uint32_t global_ns() {              // (the low word:
 }
 // (Few instructions, one loop: it stands inline at every wait, and the code of all of a kernel's roles shares the instruction
 // cache.  With a second loop inside and 64-bit times: 7 sequences, 8 taps, verify and commit 21.4 us, 20.8 so.)
+// TIGHT: with that second loop, which looks at the clock and at the flag after every 64th try only; for roles in which it measured
+// better (the prefill kernel says which).
+template <bool TIGHT = false>
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatile int* abort,
                                           uint32_t limit_ns = kWaitLimitNs) {
   if (mbar_try_wait(bar, parity)) return true;
   const uint32_t t0 = global_ns();
   do {
-    if (mbar_try_wait(bar, parity)) return true;
+#pragma unroll 1
+    for (int it = 0; it < (TIGHT ? 64 : 1); ++it)
+      if (mbar_try_wait(bar, parity)) return true;
   } while (!*abort && global_ns() - t0 <= limit_ns);
   *abort = 1;
   return false;

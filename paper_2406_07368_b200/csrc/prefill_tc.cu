@@ -408,7 +408,7 @@ __device__ __forceinline__ float2 bf2(uint32_t u) { return make_float2(lo_f(u), 
 // The rows come from the V buffer (pg[k]: the thread's column, in the swizzle of rows = k mod 8, 8 g rows before the block's
 // first), so that every load is one instruction with an immediate offset; HALO: the first nh of them from the halo column
 // (hq: the first of the 23).  Two copies of the loop and not one per nh, of which there are four: it has to stay in the
-// instruction cache (segments of 4 tiles, 9 taps: 40.3 us before, 44.1 with four copies, 40.9 with two).
+// instruction cache (segments of 4 tiles, 9 taps: 40.4 us in blocks of 8, 44.1 with four copies, 40.1 with two).
 template <int I, int N, typename F>
 __device__ __forceinline__ void static_for(F&& f) {           // f(integral_constant<int, I>) ... for I, I + 1, ..., N - 1
   if constexpr (I < N) {
@@ -505,7 +505,7 @@ __device__ __forceinline__ void conv_block8(float2 (&acc)[8], uint32_t wtap, con
   });
 }
 // The same in blocks of 8 rows, whose code is half as long: for windows of one group of taps, which is gone through once per block
-// (segments of 4 tiles, 6 taps: 37.1 us, 39.6 in blocks of 16), and for the three-branch mode (16 taps, groups of 64: 52.7 and 55.6).
+// (segments of 4 tiles, 6 taps: 36.1 us, 38.7 in blocks of 16; 128 whole chains of 2048 tokens 84.4 and 85.3), and for the three-branch mode (16 taps, groups of 64: 52.7 and 55.6).
 // conv_block8: rows -7 ... 7 of a block all from the V buffer (ALL_V), all from the halo (ALL_H), or the negative ones (MIXED).
 // All tap groups of block blk (rows 8 blk ... 8 blk + 7 of the thread), then the sums are added to the attention
 // term that waits in the output tile.  first: the thread owns the first 32 rows of the tile (rows before them
@@ -575,6 +575,9 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
   const uint32_t sbase = smem_u32(smem);
   constexpr bool GRP = GM > 0, MULTI = GM == 2;
   constexpr bool LONG = WT < 0;                  // the epilogue for longer tap windows
+  // One group of 8 taps (WT = -1) and more (-2) are kernels of their own: with both forms of the tap loop in one, 32 chains of 1700
+  // tokens, 9 to 16 taps, took 1 % longer than with either alone.  (Three-branch mode: one form, -1.)
+  constexpr bool ONE8 = WT == -1 && !GRP;
   // The exact layer with a short window keeps its loops rolled: all roles' code of one tile has to stay in the SM's instruction
   // cache.  (Unrolled, 23 KB of it came anew with every tile from the cache that a GPC shares, and two of a scheduler's five
   // warps waited for instructions on average, 0.6 of them now: 128 chains of 2048 tokens, 3 taps, 71.7 us unrolled, 67.6 rolled;
@@ -596,6 +599,9 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
   constexpr int kRegsA = LONG && !GRP && PHI == LA_PHI_RELU ? 88 : LONG && !MULTI ? 96 : LONG ? 104 : 112;
   constexpr int kRegsB = 208 - kRegsA;
   static_assert(kThreadsA == 256 && kThreadsB == 256 && kThreads == 640, "register split");
+  // Whose waits are the tight ones (see mbar_wait).  Long windows, elu + 1: those of the issuing, copying and halo warps (means over 12
+  // shapes: 6 to 8 taps 0.3-0.6 % faster, 9 to 32 taps 1.0-1.4 %; with ReLU 0.5-1.9 % slower from 9 taps on).
+  constexpr bool TIGHT_C = LONG && !GRP && PHI == LA_PHI_ELU1;
   const bool z3 = LONG ? z3_long(W, GRP) : true; // z rides in the state update's product
   Small& sm = *reinterpret_cast<Small*>(smem + off_small(z3));
   float* wsm = reinterpret_cast<float*>(smem + off_w(z3));                     // [W][128] ([W up to a multiple of 8][128] if LONG)
@@ -976,6 +982,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
 
   if (warp >= 16) {
   if (TRADE) regs_down<64>();
+  auto mbar_wait = [](uint32_t bar, uint32_t parity, volatile int* abort) { return la::mbar_wait<TIGHT_C>(bar, parity, abort); };
   if (warp == kCtrlWarp) {
     // =============================== MMA issue, the Q and K loads (one lane) ===============================
     if (lane == 0) {
@@ -1484,7 +1491,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
       const uint32_t hcol = sbase + off_halo_long(W, GRP) + 4u * cp;
       const uint32_t hend = hcol + (long_taps(W) - 1) * (D * 2);
       const uint32_t wcol = sbase + off_w(z3) + 8u * cp;
-      const int ngroups = (W + 7) >> 3;
+      const int ngroups = ONE8 ? 1 : (W + 7) >> 3;
       for (int n = 0; n < nchunks; ++n) {
         const uint32_t par = n & 1;
         if (!early && n + 1 == nchunks) pdl_trigger();
@@ -1529,7 +1536,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
           for (int k = 0; k < 8; ++k) pv[k] = vthr + ((cc ^ k) << 4);
           const uint32_t sthr = sbase + (par ? OFF_K1 : OFF_K0) + colk;
           const int mine = valid - 32 * jq;                  // rows of this thread that hold tokens
-          if (GRP || ngroups == 1) {
+          if constexpr (ONE8 || GRP) {
 #pragma unroll 1
             for (int blk = 0; blk < 4 && 8 * blk < mine; ++blk) conv_rows8(blk, jq == 0, wcol, pv, sthr, cc, hend, ngroups);
           } else {
@@ -1960,7 +1967,8 @@ static cudaError_t launch_w(la_ctx* ctx, int BH, int T, const CUtensorMap& mq, c
     case 3: kern = tc::prefill_tc_kernel<PHI, 3>; break;
     case 4: kern = tc::prefill_tc_kernel<PHI, 4>; break;
     case 5: kern = tc::prefill_tc_kernel<PHI, 5>; break;
-    default: kern = tc::prefill_tc_kernel<PHI, -1>; break;
+    case 6: case 7: case 8: kern = tc::prefill_tc_kernel<PHI, -1>; break;
+    default: kern = tc::prefill_tc_kernel<PHI, -2>; break;
   }
   cudaError_t e = allow_smem((const void*)kern, ctx->device);
   if (e != cudaSuccess) return e;
