@@ -601,7 +601,9 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
   static_assert(kThreadsA == 256 && kThreadsB == 256 && kThreads == 640, "register split");
   // Whose waits are the tight ones (see mbar_wait).  Long windows, elu + 1: those of the issuing, copying and halo warps (means over 12
   // shapes: 6 to 8 taps 0.3-0.6 % faster, 9 to 32 taps 1.0-1.4 %; with ReLU 0.5-1.9 % slower from 9 taps on).
-  constexpr bool TIGHT_C = LONG && !GRP && PHI == LA_PHI_ELU1;
+  // Three-branch mode, one group per tile: those of group A with 3 taps (54 shapes, groups of 33 to 128 tokens: 2-4 % faster), those of
+  // group B otherwise (3-5 %; without, these kernels spill 20 bytes).  Groups that share a tile: nobody's (0-4 % slower).
+  constexpr bool TIGHT_C = LONG && !GRP && PHI == LA_PHI_ELU1, TIGHT_A = GM == 1 && !LONG, TIGHT_B = GM == 1 && LONG;
   const bool z3 = LONG ? z3_long(W, GRP) : true; // z rides in the state update's product
   Small& sm = *reinterpret_cast<Small*>(smem + off_small(z3));
   float* wsm = reinterpret_cast<float*>(smem + off_w(z3));                     // [W][128] ([W up to a multiple of 8][128] if LONG)
@@ -950,6 +952,9 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
   auto snapshot = [&](int n, int r, int hf, uint32_t lane_addr, bool& ok) {
     const uint32_t par = n & 1;
     unsigned char* Sb = smem + OFF_S + hf * BOX_BYTES;
+    auto mbar_wait = [](uint32_t bar, uint32_t parity, volatile int* abort) {
+      return la::mbar_wait<(SNAP_A ? TIGHT_A : TIGHT_B)>(bar, parity, abort);
+    };
     // S_n is final after MMA_S; the old copy may be overwritten once O = phi(Q) S_prev has read it
     ok = ok && mbar_wait((bar0 + 8u * (par ? B_MMA_S1 : B_MMA_S0)), (n >> 1) & 1, abort) && mbar_wait((bar0 + 8u * (B_MMA_Q)), par, abort);
     ok = __all_sync(0xffffffffu, ok);
@@ -1173,6 +1178,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
   }
   } else if (warp >= 8) {
     // =============================== group A: phi, P, [S|z] snapshot (256 threads) ===============================
+    auto mbar_wait = [](uint32_t bar, uint32_t parity, volatile int* abort) { return la::mbar_wait<TIGHT_A>(bar, parity, abort); };
     if constexpr (TRADE) {
       if constexpr (kRegsA > 96) regs_up<kRegsA>();
       if constexpr (kRegsA < 96) regs_down<kRegsA>();
@@ -1469,6 +1475,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
     }
   } else {
     // =============================== group B: epilogue (256 threads) ===============================
+    auto mbar_wait = [](uint32_t bar, uint32_t parity, volatile int* abort) { return la::mbar_wait<TIGHT_B>(bar, parity, abort); };
     if (TRADE && kRegsB > 96) regs_up<kRegsB>();
     if (!GRP) sync_group_b();                     // the taps (long windows: and the rows before the first tile) are in place
     const int r = 32 * (warp & 3) + lane;         // tile row = TMEM lane
