@@ -583,7 +583,9 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
   // warps waited for instructions on average, 0.6 of them now: 128 chains of 2048 tokens, 3 taps, 71.7 us unrolled, 67.6 rolled;
   // 32 chains of 1700 tokens 37.4 and 35.2.)  Not the three-branch mode, whose phi lies on the longest chain of a tile (groups of 64:
   // 95 us, 104 rolled), nor long windows, whose tap sums leave little of the wait (32 taps: 127.2 us, 128.9 rolled).
-  constexpr bool kRoll = !LONG && !GRP;
+  // (phi(K) and the epilogue only beside an elu + 1: a ReLU has little code, and the loads that a rolled loop waits for show.  ReLU, 1 to 4
+  // taps: 128 and 256 chains of 1000 or 2048 tokens 0.4-0.9 % faster unrolled, 32 chains of 1700 2 %, one tile 0.5-1 %.)
+  constexpr bool kRoll = !LONG && !GRP, kRollE = kRoll && PHI == LA_PHI_ELU1;
   // Who copies the state between two tiles: group B has the time beside an elu + 1 (which keeps group A busy), group A beside
   // a ReLU or a long window (which keeps group B busy).
   constexpr bool SNAP_A = LONG || (PHI == LA_PHI_RELU && !GRP);
@@ -763,7 +765,7 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
     if constexpr (NI > 0) {
       const int valid = min(tstep, T - m * tstep);
       const int ct = ta & 15, rg = ta >> 4;                     // chunk column 0..15, row group 0..15
-      if constexpr (kRoll) {                                    // (16 rows further on the swizzle is the same)
+      if constexpr (kRollE) {                                   // (16 rows further on the swizzle is the same)
         unsigned char* Kb = smem + ((m & 1) ? OFF_K1 : OFF_K0) + (ct >> 3) * KBOX_BYTES + swz(rg + 16 * I0, ct & 7);
         auto put = [&](int i, uint4 x) {
           *reinterpret_cast<uint4*>(Kb + i * 2048) = rg + 16 * (I0 + i) < valid ? phi8<PHI>(x) : make_uint4(0u, 0u, 0u, 0u);
@@ -1643,24 +1645,24 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
           stmatrix4(vrow[0] ^ (uint32_t)(cc << 4), out);
         };
         uint32_t a0[16], a1[16];                  // rows 0-15 and 16-31 of 32 channels
-        if (!kRoll) {
+        if (!kRollE) {
           LA_TMEM_LD_FRAG4(oaddr, a0);
           LA_TMEM_LD_FRAG4(oaddr + (16u << 16), a1);
         }
-#pragma unroll (kRoll ? 1 : 2)
+#pragma unroll (kRollE ? 1 : 2)
         for (int qq = 0; qq < 2; ++qq) {
-          if (kRoll) {
+          if (kRollE) {
             LA_TMEM_LD_FRAG4(oaddr + 32 * qq, a0);
             LA_TMEM_LD_FRAG4(oaddr + 32 * qq + (16u << 16), a1);
           }
           tmem_wait_ld();
-          if (kRoll && qq == 1) {
+          if (kRollE && qq == 1) {
             tc_fence_before();
             mbar_arrive((bar0 + 8u * (B_EPI0 + par)));         // this accumulator has been read
           }
 #pragma unroll
           for (int g = 0; g < 4; ++g) piece(4 * qq + g, a0 + 4 * g, a1 + 4 * g);
-          if (!kRoll && qq == 0) {
+          if (!kRollE && qq == 0) {
             LA_TMEM_LD_FRAG4(oaddr + 32, a0);
             LA_TMEM_LD_FRAG4(oaddr + 32 + (16u << 16), a1);
             tmem_wait_ld();
