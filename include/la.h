@@ -115,7 +115,7 @@ const char* la_status_str(la_status s);
  *   conv_w      [H, d, W] fp32, tap 0 multiplies the current token
  *   init_state  0: start from an empty state (st is output only); 1: continue from st
  *   st          in-out; on return holds S, z, the window and pos after the T tokens
- *   o           [B, H, T, d] io type
+ *   o           [B, H, T, d] io type; may be q, k or v itself
  *
  * Kernels: bf16 io with d = 128 runs grouped on the tensor cores (128-token tiles); with more than
  * 5 taps its tap sum is formed in fp32, added to the attention term after that term has been
@@ -326,7 +326,8 @@ la_status la_set_prefill_kernel(la_ctx* ctx, int32_t which);
  * calls that use it have completed; NULL, 0 takes it back).  Calls that use it must be ordered on the
  * GPU, la_prefill and la_prefill_grouped alike: prefills that may overlap, on different streams, need a
  * context and a workspace each.  Without a large enough workspace la_prefill runs every chain in one
- * thread block; the results agree up to rounding order. */
+ * thread block; the results agree up to rounding order.  (A workspace without room for the rows of v before each segment, the last
+ * 2 (W - 1) d bytes per segment and chain of what is asked for, does for calls whose outputs do not take the place of v.) */
 la_status la_set_workspace(la_ctx* ctx, void* workspace, uint64_t bytes);
 uint64_t  la_prefill_workspace_bytes(const la_ctx* ctx, int32_t B, int32_t T);
 

@@ -566,7 +566,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
                   __nv_bfloat16* __restrict__ win, int64_t* __restrict__ pos,
                   int* status, int H, int Ttot, int W, float eps, int init, int nseg,
                   int seg_len, float* S_seg, float* z_seg,
-                  const __nv_bfloat16* __restrict__ win_seg, int prefixed, int fused, const __nv_bfloat16* __restrict__ vg, float alpha,
+                  const __nv_bfloat16* __restrict__ win_seg, int prefixed, int fused, const __nv_bfloat16* __restrict__ vg,
+                  int v_chain, int v_seg, float alpha,
                   float sm_scale, int tstep, int gsz, int early) {
   extern __shared__ unsigned char smem_dyn[];
   // (an offset into the array rather than an integer cast: the compiler then knows that these are shared-memory
@@ -634,7 +635,8 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
   const int nsum = sg > 0 && !prefixed ? sg : 1;          // how many parts it has
   const size_t slot = (size_t)bh * nseg + (fused ? 0 : sg == 0 ? nseg - 1 : prefixed ? sg - 1 : 0);
   const float *S_in = callers ? S + (size_t)bh * D * D : S_seg + slot * D * D, *z_in = callers ? z + (size_t)bh * D : z_seg + slot * D;
-  const __nv_bfloat16* win_in = sg > 0 ? vg + ((size_t)bh * Ttot + y0 - (W - 1)) * D
+  // (the rows before segment sg: row bh * v_chain + sg * v_seg - (W - 1) ... of vg, which is v or holds copies of just these rows)
+  const __nv_bfloat16* win_in = sg > 0 ? vg + ((size_t)bh * v_chain + sg * v_seg - (W - 1)) * D
                                        : (nseg > 1 && !fused ? win_seg : win) + (size_t)bh * (W - 1) * D;
   auto z_start = [&](int a) {
     float x = z_in[a];
@@ -1726,7 +1728,8 @@ __global__ void __launch_bounds__(kStateThreads, 1)
 segment_state_kernel(const __grid_constant__ CUtensorMap mk, const __grid_constant__ CUtensorMap mv,
                      float* __restrict__ S_out, float* __restrict__ z_out, int* status, int Ttot, int nseg,
                      int seg_len, int nrun, int init, const float* __restrict__ S, const float* __restrict__ z,
-                     const __nv_bfloat16* __restrict__ win, __nv_bfloat16* __restrict__ win_copy, int W) {
+                     const __nv_bfloat16* __restrict__ win, __nv_bfloat16* __restrict__ win_copy, int W,
+                     const __nv_bfloat16* __restrict__ v_save) {
   extern __shared__ unsigned char smem_dyn[];
   // (an offset into the array rather than an integer cast: the compiler then knows that these are shared-memory
   // addresses: 32-bit arithmetic, ld.shared / st.shared)
@@ -1863,6 +1866,12 @@ segment_state_kernel(const __grid_constant__ CUtensorMap mk, const __grid_consta
       if (base)
         for (int idx = tid; idx < (W - 1) * D; idx += 256)
           win_copy[(size_t)bh * (W - 1) * D + idx] = win[(size_t)bh * (W - 1) * D + idx];
+      // Where the outputs take the place of v: the rows that the next segment's window reaches back to.
+      if (v_save) {
+        const size_t chains = gridDim.x / nrun, from = ((size_t)bh * Ttot + y0 + T - (W - 1)) * D;
+        for (int idx = tid; idx < (W - 1) * D; idx += 256)
+          win_copy[(chains + (size_t)bh * (nseg - 1) + sg) * (W - 1) * D + idx] = v_save[from + idx];
+      }
     }
   }
   tc_fence_before();
@@ -1955,6 +1964,7 @@ struct Split {
   const __nv_bfloat16* win = nullptr;
   int prefixed = 0;
   int fused = 0;      // one cluster per chain, whose blocks form the segments' sums themselves
+  int saved = 0;      // the rows of v before each segment have been copied to the workspace
 };
 
 template <int PHI>
@@ -1989,7 +1999,8 @@ static cudaError_t launch_w(la_ctx* ctx, int BH, int T, const CUtensorMap& mq, c
   const int early = 2 * units <= ctx->sm_count;
   return launch_cluster(sp.fused ? sp.nseg : 1, early || sp.nseg > 1, kern, dim3(units), dim3(tc::kThreads), smem, s, mq, mk, mv, mo, w, st.S, st.z,
                           (__nv_bfloat16*)st.win, st.pos, ctx->d_status, c.H, T, c.conv_taps, c.eps, init, sp.nseg,
-                          sp.nseg > 1 ? sp.seg_len : T, sp.S, sp.z, sp.win, sp.prefixed, sp.fused, (const __nv_bfloat16*)v, alpha,
+                          sp.nseg > 1 ? sp.seg_len : T, sp.S, sp.z, sp.win, sp.prefixed, sp.fused, sp.saved ? sp.win + (size_t)BH * (c.conv_taps - 1) * tc::D : (const __nv_bfloat16*)v,
+                          sp.saved ? (sp.nseg - 1) * (c.conv_taps - 1) : T, sp.saved ? c.conv_taps - 1 : sp.seg_len, alpha,
                           sm_scale, tstep, gsz, early);
 }
 static cudaError_t launch_phi(la_ctx* ctx, int BH, int T, const CUtensorMap& mq, const CUtensorMap& mk, const CUtensorMap& mv,
@@ -2028,8 +2039,10 @@ static void plan_split(const la_ctx* ctx, int BH, int T, int* nseg, int* seg_len
   *nseg = n;
   *seg_len = per * tile;
 }
-static size_t split_bytes(const la_config& c, int BH, int nseg) {
-  return (size_t)BH * ((size_t)nseg * (tc::D * tc::D + tc::D) * 4 + (size_t)(c.conv_taps > 1 ? c.conv_taps - 1 : 1) * tc::D * 2);
+// `rows`: with room for the W - 1 rows of v before each segment but the first.
+static size_t split_bytes(const la_config& c, int BH, int nseg, bool rows) {
+  return (size_t)BH * ((size_t)nseg * (tc::D * tc::D + tc::D) * 4 + (size_t)(c.conv_taps > 1 ? c.conv_taps - 1 : 1) * tc::D * 2 +
+                       (rows ? (size_t)(nseg - 1) * (c.conv_taps - 1) * tc::D * 2 : 0));
 }
 
 size_t prefill_workspace_bytes(const la_ctx* ctx, int B, int T) {
@@ -2037,7 +2050,7 @@ size_t prefill_workspace_bytes(const la_ctx* ctx, int B, int T) {
   if (c.io_dtype != LA_BF16 || c.d != tc::D) return 0;
   int nseg, seg_len;
   plan_split(ctx, B * c.H, T, &nseg, &seg_len);
-  return nseg > 1 ? split_bytes(c, B * c.H, nseg) : 0;
+  return nseg > 1 ? split_bytes(c, B * c.H, nseg, true) : 0;
 }
 
 // How many clusters of n blocks, one block per SM, the device holds at once.
@@ -2069,11 +2082,17 @@ static int resident_clusters(la_ctx* ctx, int n) {
 // Cuts the chains where that pays and the workspace allows it: launches what forms the segments' starting states.  `tile`:
 // tokens per tile of the main pass; mk, mv: maps with boxes of 128 rows.
 static cudaError_t launch_split(la_ctx* ctx, int BH, int T, int tile, const CUtensorMap& mk, const CUtensorMap& mv, int init,
-                                const la_state& st, Split* out, cudaStream_t s) {
+                                const la_state& st, const void* v, const void* o, Split* out, cudaStream_t s) {
   Split& sp = *out;
   const la_config& c = ctx->cfg;
   plan_split(ctx, BH, T, &sp.nseg, &sp.seg_len, tile);
-  if (sp.nseg > 1 && (ctx->ws == nullptr || ctx->ws_bytes < split_bytes(c, BH, sp.nseg) || T < c.conv_taps)) sp = Split();
+  if (sp.nseg > 1 && (ctx->ws == nullptr || T < c.conv_taps)) sp = Split();
+  const bool fits = sp.nseg > 1 && sp.nseg <= kMaxCluster && BH <= resident_clusters(ctx, sp.nseg);   // one cluster per chain
+  // Outputs in the place of v: the blocks of a cluster read the rows before their segments ahead of a barrier that every store is
+  // behind; in a grid without one they would race with the stores of the segment before, so copies are made first.
+  const uintptr_t va = (uintptr_t)v, oa = (uintptr_t)o, bytes = (uintptr_t)BH * T * tc::D * 2;
+  const bool save = !fits && c.conv_taps > 1 && va < oa + bytes && oa < va + bytes;
+  if (sp.nseg > 1 && ctx->ws_bytes < split_bytes(c, BH, sp.nseg, save)) sp = Split();
   if (sp.nseg > 1) {
     // Sequence split: the sums of all segments but the last, then every segment as its own CTA.
     const int nseg = sp.nseg, units = BH * nseg;
@@ -2084,7 +2103,7 @@ static cudaError_t launch_split(la_ctx* ctx, int BH, int T, int tile, const CUte
     // Up to 8 segments (a portable cluster): one launch, provided that all the clusters are resident at once.  (32 chains of
     // 1700 tokens, 4 segments each: 40.7 us with the sums formed by a launch of their own, 37 so; 32 x 3000: 55 and
     // 50; 32 x 32768 no difference.)
-    if (nseg <= kMaxCluster && BH <= resident_clusters(ctx, nseg)) {
+    if (fits) {
       sp.fused = 1;
       return cudaSuccess;
     }
@@ -2094,7 +2113,8 @@ static cudaError_t launch_split(la_ctx* ctx, int BH, int T, int tile, const CUte
     ctx->launches += 1;
     e = launch_pdl(skern, dim3(BH * (nseg - 1)), dim3(tc::kStateThreads), tc::kStateSmem, s, mk, mv, S_seg, z_seg,
                          ctx->d_status, T, nseg, sp.seg_len, nseg - 1, init, (const float*)st.S, (const float*)st.z,
-                         (const __nv_bfloat16*)st.win, win_seg, c.conv_taps);
+                         (const __nv_bfloat16*)st.win, win_seg, c.conv_taps, save ? (const __nv_bfloat16*)v : nullptr);
+    sp.saved = save;
     if (e != cudaSuccess) return e;
     if (nseg > kSumInPlace) {
       sp.prefixed = 1;
@@ -2120,7 +2140,7 @@ cudaError_t launch_prefill_tc(la_ctx* ctx, int B, int T, const void* q, const vo
     return cudaErrorNotSupported;   // the driver cannot encode tensor maps: reported, never a silent slow path
   *handled = true;
   Split sp;
-  const cudaError_t e = launch_split(ctx, BH, T, tc::TILE, mk, mv, init, st, &sp, s);
+  const cudaError_t e = launch_split(ctx, BH, T, tc::TILE, mk, mv, init, st, v, o, &sp, s);
   if (e != cudaSuccess) return e;
   return launch_phi(ctx, BH, T, mq, mk, mv, mo, v, w, init, st, sp, s);
 }
@@ -2144,7 +2164,7 @@ cudaError_t launch_prefill_grouped_tc(la_ctx* ctx, int B, int T, const void* q, 
     return cudaErrorNotSupported;
   *handled = true;
   Split sp;
-  const cudaError_t e = launch_split(ctx, BH, T, tile, tile != tc::TILE ? mk1 : mk, tile != tc::TILE ? mv1 : mv, init, st, &sp, s);
+  const cudaError_t e = launch_split(ctx, BH, T, tile, tile != tc::TILE ? mk1 : mk, tile != tc::TILE ? mv1 : mv, init, st, v, o, &sp, s);
   if (e != cudaSuccess) return e;
   return launch_phi(ctx, BH, T, mq, mk, mv, mo, v, w, init, st, sp, s, true, alpha, scale, tile, gsz);
 }
@@ -2166,7 +2186,7 @@ cudaError_t launch_segment_state_tc(la_ctx* ctx, int B, int T, const void* k, co
   ctx->launches += 1;
   return launch_cluster(1, false, skern, dim3(BH), dim3(tc::kStateThreads), tc::kStateSmem, s, mk, mv, dS, dz, ctx->d_status, T,
                           1, T, 1, 0, (const float*)nullptr, (const float*)nullptr, (const __nv_bfloat16*)nullptr,
-                          (__nv_bfloat16*)nullptr, c.conv_taps);
+                          (__nv_bfloat16*)nullptr, c.conv_taps, (const __nv_bfloat16*)nullptr);
 }
 
 }  // namespace la
