@@ -66,7 +66,7 @@ def test_segments_of_few_tiles(tiles, W, group):
     """32 chains in four segments of `tiles` tiles, the last one ragged, continuing: as the call that is not cut (only the order
     of fp32 sums and the roundings behind it differ: a few bf16 ulps)."""
     H, d, tile = 32, 128, 100 if group == 100 else 128
-    T, first = 4 * tiles * tile - 37, 192 if group == 64 else 200
+    T, first = 4 * tiles * tile - 19, 192 if group == 64 else 200       # (781 tokens in tiles of 100 are still seven of 128)
     q, k, v = (_dev(x) for x in wl.qkv(tiles, (1, H, first + T, d), d ** -0.5, "bf16", v_mean=0.5))
     w = torch.from_numpy(wl.conv_weights(5, H, d, W)).cuda()
     ctx = binding.Context(H, d, W, "elu1", 0.0, "bf16")
@@ -87,7 +87,9 @@ def test_segments_of_few_tiles(tiles, W, group):
             ws = torch.full((ctx.la_prefill_workspace_bytes(1, T),), 0xff, dtype=torch.uint8, device="cuda")
             ctx.la_set_workspace(ws)
         got.append((call(first, first + T, st), st))
-    assert ctx.la_last_device_status() == binding.LA_OK and (ws != 0xff).any()
+    assert ctx.la_last_device_status() == binding.LA_OK
+    S_seg = ws[:32 * 4 * d * d * 4].view(32, 4, -1)                     # a state per chain and segment: the first three are formed
+    assert (S_seg[:, :3] != 0xff).any(-1).all()
     (a, sa), (b, sb) = got
     assert rel_err(a.float().cpu().numpy(), b.float().cpu().numpy()) < 1.2e-2
     assert rel_err(sa.S.cpu().numpy(), sb.S.cpu().numpy()) < 1e-4 and rel_err(sa.z.cpu().numpy(), sb.z.cpu().numpy()) < 1e-4
