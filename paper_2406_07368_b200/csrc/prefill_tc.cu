@@ -505,7 +505,8 @@ __device__ __forceinline__ void conv_block8(float2 (&acc)[8], uint32_t wtap, con
   });
 }
 // The same in blocks of 8 rows, whose code is half as long: for windows of one group of taps, which is gone through once per block
-// (segments of 4 tiles, 6 taps: 36.1 us, 38.7 in blocks of 16; 128 whole chains of 2048 tokens 84.4 and 85.3), and for the three-branch mode (16 taps, groups of 64: 52.7 and 55.6).
+// (segments of 4 tiles, 6 taps: 36.1 us, 38.7 in blocks of 16; 128 whole chains of 2048 tokens 84.4 and 85.3), and for the
+// three-branch mode (16 taps, groups of 64: 52.7 and 55.6).
 // conv_block8: rows -7 ... 7 of a block all from the V buffer (ALL_V), all from the halo (ALL_H), or the negative ones (MIXED).
 // All tap groups of block blk (rows 8 blk ... 8 blk + 7 of the thread), then the sums are added to the attention
 // term that waits in the output tile.  first: the thread owns the first 32 rows of the tile (rows before them
@@ -581,8 +582,9 @@ prefill_tc_kernel(const __grid_constant__ CUtensorMap mq, const __grid_constant_
   constexpr bool ONE8 = WT == -1 && !GRP;
   // The exact layer with a short window keeps its loops rolled: all roles' code of one tile has to stay in the SM's instruction
   // cache.  (Unrolled, 23 KB of it came anew with every tile from the cache that a GPC shares, and two of a scheduler's five
-  // warps waited for instructions on average, 0.6 of them now: 128 chains of 2048 tokens, 3 taps, 71.7 us unrolled, 67.6 rolled;
-  // 32 chains of 1700 tokens 37.4 and 35.2.)  Not the three-branch mode, whose phi lies on the longest chain of a tile (groups of 64:
+  // warps waited for instructions on average, 0.6 of them now: 128 chains of 2048 tokens, 3 taps, in runs too short for the power
+  // limit 66.8 us before, 61.6 since; back to back, where the clock gives way, 72.1 and 71.5.  32 chains of 1700 tokens 37.4 and
+  // 35.2.)  Not the three-branch mode, whose phi lies on the longest chain of a tile (groups of 64:
   // 95 us, 104 rolled), nor long windows, whose tap sums leave little of the wait (32 taps: 127.2 us, 128.9 rolled).
   // (phi(K) and the epilogue only beside an elu + 1: a ReLU has little code, and the loads that a rolled loop waits for show.  ReLU, 1 to 4
   // taps: 128 and 256 chains of 1000 or 2048 tokens 0.4-0.9 % faster unrolled, 32 chains of 1700 2 %, one tile 0.5-1 %.)
